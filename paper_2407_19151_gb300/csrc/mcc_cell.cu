@@ -794,6 +794,7 @@ __device__ void correct_interaction(const StepArgs& A, const Tile<V>& t, Shared&
                 if (carry >= Dabs) done = true;
             }
             if (!done) Dabs -= carry;
+            __syncthreads();  // the next pass pairs across this one's pairs
         }
         __syncthreads();
         if (!done && threadIdx.x == 0) sh.fail = 1;
