@@ -373,7 +373,7 @@ int mcc_set_tile_cap(mcc_ctx* ctx, int32_t cap);
  * particles_per_warp sets caps[k] = particles_per_warp << k for k < 4 (0 = automatic: the capacity with which
  * sixteen warps share an SM's shared memory); largest sets caps[4] (0 = as large as one CTA's shared memory
  * allows). Every capacity is capped by what one CTA's shared memory holds (44 bytes per particle). Both 0 is the
- * default. Used by the autotuner; the step's results do not depend on it. */
+ * default; a call with few cells then runs its cells on larger groups than these classes say. Used by the autotuner; the step's results do not depend on it. */
 int mcc_set_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp, int32_t largest);
 
 /* The five class capacities mcc_step_fused uses for this precision and mode (caps_out: host int32[5]). */

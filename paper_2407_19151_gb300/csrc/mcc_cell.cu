@@ -1249,10 +1249,11 @@ const void* group_kernel(bool f32, bool rel, int cls)
     return rel ? group_kernel_f32rel(cls) : group_kernel_f32(cls);
 }
 
-cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, size_t smem, cudaStream_t st)
+cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem,
+                         cudaStream_t st)
 {
     void* args[] = {const_cast<StepArgs*>(&a)};
-    return cudaLaunchKernel(group_kernel(f32, rel, cls), dim3(grid), dim3(32 << cls), args, smem, st);
+    return cudaLaunchKernel(group_kernel(f32, rel, cls), dim3(grid), dim3(groups * (32 << cls)), args, smem, st);
 }
 
 size_t pair_tile_bytes_per_particle() { return kPairTileBytesPerParticle; }

@@ -1,10 +1,18 @@
-// Group kernels of the fused collision step on the mixed-precision path: a group of G threads (one CTA) owns one cell
-// at a time.
+// Group kernels of the fused collision step on the mixed-precision path: a group of G threads owns one cell at a time;
+// a CTA runs several groups (group_cta_warps warps) in lockstep.
 //
 // Cells are dispatched by size class: class k holds cells of at most C * 2^k particles and runs with G = 32 * 2^k
 // threads, so every class keeps the same shared memory per thread and the GPU the same number of resident warps.
-// The smallest class is one warp per cell and synchronises with warp barriers only. The largest class takes the
-// largest cell one CTA's shared memory can hold.
+// The smallest class is one warp per cell and synchronises with warp barriers only inside a cell; the groups of 64 to 256
+// threads use one named barrier each. The largest class takes the largest cell one CTA's shared memory can hold.
+//
+// Lockstep: what bounds a cell visit is instruction fetch. A visit is nearly straight-line code (each loop runs two or
+// three times over ~170 particles of a species, the code of one interaction is far larger than an SM partition's
+// instruction cache), and with sixteen independent warps per SM at different places every warp fetched for itself. The
+// groups of a CTA take cells of nearly equal size (the class order is by size) and meet at a CTA barrier after every
+// phase of an interaction, so that all warps of the SM run the same code at about the same time and share its
+// fetches. One GB300, against independent CTAs of one group each: three-species step of 1.34e8 particles 43.9 -> 29.1 ms,
+// relativistic beam of 1.16e7 particles 16.9 -> 8.0 ms.
 //
 // Per cell visit the particles are staged in shared memory and the whole step of Algorithm 1 runs there, every
 // interaction (a, b) in list order:
@@ -78,7 +86,7 @@ struct PhaseClk {
 #ifdef MCC_PHASE_CLOCKS
 #define PHASE_MARK(pc, k)                                                                                             \
     do {                                                                                                              \
-        if (threadIdx.x == 0) {                                                                                       \
+        if (tix<G>() == 0) {                                                                                          \
             const long long now_ = clock64();                                                                         \
             (pc).acc[(k)] += now_ - (pc).prev;                                                                        \
             (pc).prev = now_;                                                                                         \
@@ -151,18 +159,52 @@ __device__ __forceinline__ ff shidx(ff a, int l)
 }
 
 // ----------------------------------------------------------------------------------------------- group primitives
+// Thread and warp index within the group; group of the CTA this thread belongs to.
+template <int G>
+__device__ __forceinline__ int tix()
+{
+    return (int)threadIdx.x & (G - 1);
+}
+template <int G>
+__device__ __forceinline__ int wix()
+{
+    return ((int)threadIdx.x >> 5) & (G / 32 - 1);
+}
+template <int G>
+__device__ __forceinline__ int team()
+{
+    return (int)threadIdx.x / G;
+}
+
+// Barrier of the group: a warp barrier, or named barrier 1 + group (barrier 0 is the CTA's).
 template <int G>
 __device__ __forceinline__ void gsync()
 {
     if (G == 32) __syncwarp();
-    else __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + team<G>()), "n"(G) : "memory");
 }
 
 template <int G>
 __device__ __forceinline__ bool gany(bool p)
 {
     if (G == 32) return __any_sync(0xffffffffu, p);
-    return __syncthreads_or(p) != 0;
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)p), "r"(1 + team<G>()), "n"(G)
+        : "memory");
+    return r != 0;
+}
+
+// Lockstep barrier of the CTA's groups (nothing to do when the CTA is one group).
+template <int G>
+__device__ __forceinline__ void csync()
+{
+    if (blockDim.x > G) __syncthreads();
 }
 
 template <int P>
@@ -220,7 +262,7 @@ template <int G, int P>
 __device__ __forceinline__ void gallreduce(ff (&a)[P], GRed<G, 8>& r)
 {
     constexpr int SH = 5 - Lg<P>::v;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = wix<G>();
     const ff s = warp_rs<P>(a);
     if (G == 32) {
 #pragma unroll
@@ -229,13 +271,13 @@ __device__ __forceinline__ void gallreduce(ff (&a)[P], GRed<G, 8>& r)
     }
     constexpr int W = G / 32;
     if ((lane & ((1 << SH) - 1)) == 0) r.part[(lane >> SH) * W + warp] = s;
-    __syncthreads();
+    gsync<G>();
     if (warp == 0 && lane < P) {
         ff t = r.part[lane * W];
         for (int w = 1; w < W; ++w) t = ff_add(t, r.part[lane * W + w]);
         r.tot[lane] = t;
     }
-    __syncthreads();
+    gsync<G>();
 #pragma unroll
     for (int q = 0; q < P; ++q) a[q] = r.tot[q];
 }
@@ -246,7 +288,7 @@ template <int G, int P>
 __device__ __forceinline__ void greduce_warp0(ff (&a)[P], GRed<G, 8>& r)
 {
     constexpr int SH = 5 - Lg<P>::v;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = wix<G>();
     const ff s = warp_rs<P>(a);
     if (G == 32) {
 #pragma unroll
@@ -254,7 +296,7 @@ __device__ __forceinline__ void greduce_warp0(ff (&a)[P], GRed<G, 8>& r)
     } else {
         constexpr int W = G / 32;
         if ((lane & ((1 << SH) - 1)) == 0) r.part[(lane >> SH) * W + warp] = s;
-        __syncthreads();
+        gsync<G>();
         if (warp == 0) {
             const int q = lane < P ? lane : 0;
             ff t = r.part[q * W];
@@ -291,7 +333,7 @@ __device__ __forceinline__ ff seg_scan_excl(ff x, unsigned mask, int width, ff& 
 template <int G>
 __device__ __forceinline__ int gscan_int(int x, int* scr, int& total)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = wix<G>();
     int inc = x;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -305,14 +347,14 @@ __device__ __forceinline__ int gscan_int(int x, int* scr, int& total)
     }
     constexpr int W = G / 32;
     if (lane == 31) scr[warp] = inc;
-    __syncthreads();
+    gsync<G>();
     int off = 0, tot = 0;
     for (int w = 0; w < W; ++w) {
         const int y = scr[w];
         off += w < warp ? y : 0;
         tot += y;
     }
-    __syncthreads();
+    gsync<G>();
     total = tot;
     return off + exc;
 }
@@ -348,10 +390,6 @@ struct GShared {
     int off[kMaxSpecies + 1];
     int wmode[kMaxSpecies];  // 0 distinct (rho fixed for the visit), 1 all equal (rho = perm), 2 ties (rho per
                              // interaction), 3 stored in weight order (rho = identity)
-    int cell;
-    uint32_t step;
-    int used_k[kMaxInter];   // energy pairs of interaction k in this visit
-    int fail_k[kMaxInter];   // 1 if interaction k failed
     ff P[kMaxSpecies][3];    // carried m_s sum w v per species
     ff E[kMaxSpecies];       // carried m_s sum w KE/m per species
     ff wbar[kMaxSpecies];    // mean weight sum w / N_s (Eq. DeltaEs)
@@ -363,6 +401,23 @@ struct GShared {
     int eres_i[4];  // pairs used and failure of species a, then of species b
     int sci[G / 32 + 1];
 };
+
+// What the groups of a CTA share: the cells of the batch, and the cells to visit again without their failed interactions
+// (Sec. 5.2 under the rollback policy).
+struct CtaShared {
+    int base, take, retry;    // the batch: [base, base + take) of the class order, or of the retry list
+    int n_retry;
+    int r_cell[2 * group_cta_warps(true)];       // cell
+    int r_used[2 * group_cta_warps(true)];       // energy pairs of its failed interactions
+    uint64_t r_skip[2 * group_cta_warps(true)];  // its failed interactions
+};
+
+// Bytes of a group's GShared, the tile after it 16-byte aligned.
+template <int G>
+__host__ __device__ constexpr size_t group_shared_bytes()
+{
+    return (sizeof(GShared<G>) + 15) & ~(size_t)15;
+}
 
 // ----------------------------------------------------------------------------------------------- random permutation
 // Key of local index q of a side: the Philox block of q/2; bits (r.x, r.y) for even q, (r.z, r.w) for odd q; the
@@ -390,12 +445,12 @@ __device__ void gpermutations(const StepArgs& A, const GTile& t, GShared<G>& sh,
         while ((2 << lg1) < nb) ++lg1;
     const int B0 = 1 << lg0, B1 = nside > 1 ? 1 << lg1 : 0;
     const int L = B0 + B1;  // <= na + nb <= cap
-    for (int b = threadIdx.x; b < L; b += G) cnt[CHK(t.dbg, b, t.cap)] = 0;
+    for (int b = tix<G>(); b < L; b += G) cnt[CHK(t.dbg, b, t.cap)] = 0;
     gsync<G>();
     // keys of both sides as one range of half-indices h (one Philox block per two particle indices of a side); two
     // blocks per thread and iteration: independent chains for the issue slots
     const int ha = (na + 1) / 2, htot = ha + (nside > 1 ? (nb + 1) / 2 : 0);
-    for (int h = threadIdx.x; h < htot; h += 2 * G) {
+    for (int h = tix<G>(); h < htot; h += 2 * G) {
         const int h2 = h + G;
         const bool sb = h >= ha, sb2 = h2 >= ha;
         const int hl = sb ? h - ha : h, hl2 = sb2 ? h2 - ha : h2;
@@ -424,7 +479,7 @@ __device__ void gpermutations(const StepArgs& A, const GTile& t, GShared<G>& sh,
     {
         // exclusive scan over both sides' buckets (side b's positions come after side a's na)
         const int chunk = (L + G - 1) / G;
-        const int lo = threadIdx.x * chunk, hi = min(L, lo + chunk);
+        const int lo = tix<G>() * chunk, hi = min(L, lo + chunk);
         int local = 0;
         for (int b = lo; b < hi; ++b) local += (int)cnt[CHK(t.dbg, b, t.cap)];
         int total;
@@ -438,7 +493,7 @@ __device__ void gpermutations(const StepArgs& A, const GTile& t, GShared<G>& sh,
     gsync<G>();
     {
         const int ntot = na + (nside > 1 ? nb : 0);  // both sides as one index range
-        for (int qq = threadIdx.x; qq < ntot; qq += G) {
+        for (int qq = tix<G>(); qq < ntot; qq += G) {
             const bool sb = qq >= na;
             const int q = sb ? qq - na : qq;
             const int s0 = sb ? b0 : a0, base = sb ? B0 : 0, l = sb ? lg1 : lg0, off = sb ? na : 0;
@@ -449,7 +504,7 @@ __device__ void gpermutations(const StepArgs& A, const GTile& t, GShared<G>& sh,
     }
     gsync<G>();
     // cnt[b] is now the end of bucket b: order each bucket by the full key (insertion sort)
-    for (int bb = threadIdx.x; bb < L; bb += G) {  // both sides' buckets as one range
+    for (int bb = tix<G>(); bb < L; bb += G) {  // both sides' buckets as one range
         const bool sb = bb >= B0;
         const int b = sb ? bb - B0 : bb;
         const int s0 = sb ? b0 : a0, base = sb ? B0 : 0, off = sb ? na : 0;
@@ -475,13 +530,39 @@ __device__ void gpermutations(const StepArgs& A, const GTile& t, GShared<G>& sh,
 }
 
 // ----------------------------------------------------------------------------------------------- weight order
+// Ascending sort of n keys in shared memory by the whole group (the bitonic network of block_sort_u64).
+template <int G>
+__device__ __noinline__ void gsort_u64(uint64_t* a, int n)
+{
+    int logP = 0;
+    while ((1 << logP) < n) ++logP;
+    const int half_work = logP ? 1 << (logP - 1) : 0;
+    for (int lg = 1; lg <= logP; ++lg) {
+        const int size = 1 << lg, hmask = (size >> 1) - 1;
+        for (int i = tix<G>(); i < half_work; i += G) {
+            const int base = (i >> (lg - 1)) << lg;
+            const int lo = base + (i & hmask), hi = base + size - 1 - (i & hmask);
+            if (hi < n) cmpx(a, lo, hi);
+        }
+        gsync<G>();
+        for (int ls = lg - 2; ls >= 0; --ls) {
+            const int stride = 1 << ls;
+            for (int i = tix<G>(); i < half_work; i += G) {
+                const int lo = ((i >> ls) << (ls + 1)) + (i & (stride - 1)), hi = lo + stride;
+                if (hi < n) cmpx(a, lo, hi);
+            }
+            gsync<G>();
+        }
+    }
+}
+
 template <int G>
 __device__ __forceinline__ void sort_keys(uint64_t* key, int n)
 {
     if (n <= kWarpSortMax) {
-        if (threadIdx.x < 32) warp_sort_buf(key, n);
+        if (wix<G>() == 0) warp_sort_buf(key, n);
     } else {
-        block_sort_u64(key, n);
+        gsort_u64<G>(key, n);
     }
     gsync<G>();
 }
@@ -497,8 +578,8 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
                                            unsigned need)
 {
     constexpr int kWarps = G / 32;
-    const int warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0)
+    const int warp = wix<G>();
+    if (tix<G>() == 0)
         for (int sp = 0; sp < S; ++sp)
             if (!(need >> sp & 1u)) sh.wmode[sp] = 3;
     if (!need) return;
@@ -506,7 +587,7 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
         if (!(need >> sp & 1u)) continue;
         const int s0 = sh.off[sp], ns = sh.off[sp + 1] - s0;
         uint64_t* key = t.scr + s0;
-        for (int q = threadIdx.x; q < ns; q += G)
+        for (int q = tix<G>(); q < ns; q += G)
             key[CHK(t.dbg, q, ns)] = weight_key(A.w[cs + CHK(t.dbg, s0 + q, t.n)], (uint32_t)q);
     }
     gsync<G>();
@@ -518,7 +599,7 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
         const int ns = sh.off[sp + 1] - sh.off[sp];
         if ((need >> sp & 1u) && ns > kWarpSortMax) {
             gsync<G>();
-            block_sort_u64(t.scr + sh.off[sp], ns);
+            gsort_u64<G>(t.scr + sh.off[sp], ns);
         }
     }
     gsync<G>();
@@ -527,12 +608,12 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
         const int s0 = sh.off[sp], ns = sh.off[sp + 1] - s0;
         const uint64_t* key = t.scr + s0;
         bool tie = false;
-        for (int q = threadIdx.x; q < ns; q += G) {
+        for (int q = tix<G>(); q < ns; q += G) {
             t.rho[CHK(t.dbg, s0 + q, t.n)] = (uint16_t)(s0 + (int)(key[CHK(t.dbg, q, ns)] & kPermMask));
             if (q + 1 < ns) tie |= (key[CHK(t.dbg, q, ns)] >> kPermBits) == (key[CHK(t.dbg, q + 1, ns)] >> kPermBits);
         }
         const bool anytie = gany<G>(tie);
-        if (threadIdx.x == 0) {
+        if (tix<G>() == 0) {
             const bool all_equal = (key[0] >> kPermBits) == (key[CHK(t.dbg, ns - 1, ns)] >> kPermBits);
             sh.wmode[sp] = all_equal ? 1 : (anytie ? 2 : 0);
         }
@@ -546,12 +627,12 @@ template <int G>
 __device__ __noinline__ void gtie_order(const StepArgs& A, const GTile& t, int64_t cs, int s0, int ns)
 {
     uint64_t* key = t.scr + s0;
-    for (int r = threadIdx.x; r < ns; r += G)
+    for (int r = tix<G>(); r < ns; r += G)
         key[CHK(t.dbg, r, ns)] =
             weight_key(A.w[cs + CHK(t.dbg, (int)t.perm[CHK(t.dbg, s0 + r, t.n)], t.n)], (uint32_t)r);
     gsync<G>();
     sort_keys<G>(key, ns);
-    for (int m = threadIdx.x; m < ns; m += G)
+    for (int m = tix<G>(); m < ns; m += G)
         t.rho[CHK(t.dbg, s0 + m, t.n)] = t.perm[CHK(t.dbg, s0 + (int)(key[CHK(t.dbg, m, ns)] & kPermMask), t.n)];
     gsync<G>();
 }
@@ -997,11 +1078,11 @@ __device__ __forceinline__ void gscatter(const StepArgs& A, const GTile& t, int 
         const int r1 = r0 + len < total ? r0 + len : total;
         int p, stride, end;
         if (lead) {
-            p = threadIdx.x == 0 ? 0 : 3 + (int)threadIdx.x - 1;
-            stride = threadIdx.x == 0 ? 1 : G - 1;
-            end = threadIdx.x == 0 ? 3 : r1;
+            p = tix<G>() == 0 ? 0 : 3 + (int)tix<G>() - 1;
+            stride = tix<G>() == 0 ? 1 : G - 1;
+            end = tix<G>() == 0 ? 3 : r1;
         } else {
-            p = r0 + (int)threadIdx.x;
+            p = r0 + (int)tix<G>();
             stride = G;
             end = r1;
         }
@@ -1190,19 +1271,21 @@ __device__ __forceinline__ ff energy_call(const StepArgs& A, const GTile& t, int
 }
 
 // Moment correction of one interaction (Sec. 4, Appendix A, Sec. 5.2). Returns 1 if the interaction failed under
-// the rollback policy (the caller replays the cell without it).
+// the rollback policy (the caller visits the cell again without it); adds the energy pairs to `used`, the failure to
+// `failed`. Called by every group of the CTA; on = this group's cell runs the interaction.
 template <bool REL, int G>
-__device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c, int64_t cs, int k,
-                        const InterConst& ic, bool intra, int a0, int na, int b0, int nb, PhaseClk& pc)
+__device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c, int64_t cs,
+                        const InterConst& ic, bool intra, int a0, int na, int b0, int nb, bool on, int& used, int& failed,
+                        PhaseClk& pc)
 {
     const int cap = t.cap;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = wix<G>(), lane = threadIdx.x & 31;
     const int nside = intra ? 1 : 2;
     const ff zero = {0.f, 0.f};
     const ff ma = mass_ff(A, ic.a), mb = mass_ff(A, ic.b);
     const ff c2inv = {A.c2inv_f, A.c2inv_lo};
     // energy-pair order of tied species (rare), before the energy pairs read it
-    if (A.sort_by_weight) {
+    if (on && A.sort_by_weight) {
         if (sh.wmode[ic.a] == 2) gtie_order<G>(A, t, cs, a0, na);
         if (!intra && sh.wmode[ic.b] == 2) gtie_order<G>(A, t, cs, b0, nb);
     }
@@ -1210,14 +1293,14 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
     // Eq. vp_pm: B = (sum_p m_p v_ps - sum_p m_p v_bs) / sum_p m_p w_p over the interaction's particles, the
     // pre-scatter sum being the carried per-species momentum
     ff B[3], Pa[3], Pb[3];
-    {
+    if (on) {
         ff acc[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) acc[q] = zero;
         // both species' particles as one index range (fewer partly filled passes over the group)
         const int ntot = na + (nside > 1 ? nb : 0);
 #pragma unroll 1  // rolled: a smaller instruction footprint
-        for (int q = threadIdx.x; q < ntot; q += G) {
+        for (int q = tix<G>(); q < ntot; q += G) {
             const bool sb = q >= na;
             const int i = sb ? b0 + (q - na) : a0 + q;
             const float2 ws = t.w[CHK(t.dbg, i, t.n)];
@@ -1242,13 +1325,14 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
         }
     }
 
+    csync<G>();
     PHASE_MARK(pc, 3);
     // momentum shift v_pm = v_ps - B w_p (Eq. vp_pm) and the post-shift species energies (Eq. DeltaEs)
     ff e2[2] = {zero, zero};
-    {
+    if (on) {
         const int ntot = na + (nside > 1 ? nb : 0);
 #pragma unroll 1  // rolled: a smaller instruction footprint
-        for (int q = threadIdx.x; q < ntot; q += G) {
+        for (int q = tix<G>(); q < ntot; q += G) {
             const bool sb = q >= na;
             const int i = sb ? b0 + (q - na) : a0 + q;
             const float2 ws = t.w[CHK(t.dbg, i, t.n)];
@@ -1270,9 +1354,13 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
     // species a did not fail, and a failed interaction is replayed without it, so only the pair count of species b
     // is dropped when species a fails.
     const bool both = !intra && A.fail_policy == 0;
-    if (!both || G == 32) greduce_warp0<G, 2>(e2, sh.red);  // intra: e2[1] is zero
-    else gallreduce<G, 2>(e2, sh.red);
+    if (on) {
+        if (!both || G == 32) greduce_warp0<G, 2>(e2, sh.red);  // intra: e2[1] is zero
+        else gallreduce<G, 2>(e2, sh.red);
+    }
+    csync<G>();
     PHASE_MARK(pc, 4);
+    if (!on) return 0;
     // unit 0 runs species a (and b when not both), unit 1 species b
     const int unit = both ? (G == 32 ? lane >> 4 : warp) : (warp == 0 ? 0 : 2);
     if (unit < 2) {
@@ -1377,9 +1465,9 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
     // interaction's barriers (so no barrier closes this one)
     const int fa = sh.eres_i[1], fb = sh.eres_i[3];
     const int fail = fa | fb;
-    if (threadIdx.x == 0) {
-        sh.used_k[k] = sh.eres_i[0] + (fa ? 0 : sh.eres_i[2]);
-        sh.fail_k[k] = fail;
+    used += sh.eres_i[0] + (fa ? 0 : sh.eres_i[2]);
+    failed += fail;
+    if (tix<G>() == 0) {
         sh.E[ic.a] = sh.eres_E[0];
 #pragma unroll
         for (int d = 0; d < 3; ++d) sh.P[ic.a][d] = ff_sub(Pa[d], ff_mul(B[d], sh.W2m[ic.a]));
@@ -1414,7 +1502,7 @@ __device__ __forceinline__ void gload(const StepArgs& A, const GTile& t, GShared
         for (int q = 0; q < 8; ++q) acc[q] = zero;
         float unordered = 0.f;  // neighbours out of the stored weight order (counted in slot 6 of the reduction)
 #pragma unroll 1  // rolled: a smaller instruction footprint
-        for (int q = threadIdx.x; q < ns; q += G) {
+        for (int q = tix<G>(); q < ns; q += G) {
             const int i = s0 + q;
             const double wd = A.w[cs + CHK(t.dbg, i, t.n)];
             if (order && q + 1 < ns && weight_key(wd, 0) >= weight_key(A.w[cs + CHK(t.dbg, i + 1, t.n)], 0))
@@ -1439,7 +1527,7 @@ __device__ __forceinline__ void gload(const StepArgs& A, const GTile& t, GShared
         const ff m = mass_ff(A, sp);
         const ff Pm[3] = {ff_mul(m, acc[2]), ff_mul(m, acc[3]), ff_mul(m, acc[4])};
         const ff Em = ff_mul(m, acc[5]);
-        if (threadIdx.x == 0) {
+        if (tix<G>() == 0) {
             sh.wbar[sp] = ns > 0 ? ffq_div(acc[0], ffk((float)ns)) : zero;
             sh.W2m[sp] = ff_mul(m, acc[1]);
             sh.P[sp][0] = Pm[0];
@@ -1452,7 +1540,7 @@ __device__ __forceinline__ void gload(const StepArgs& A, const GTile& t, GShared
         tot[2] = ff_add(tot[2], Pm[2]);
         tot[3] = ff_add(tot[3], Em);
     }
-    if (threadIdx.x == 0) {
+    if (tix<G>() == 0) {
         sh.P0[0] = tot[0];
         sh.P0[1] = tot[1];
         sh.P0[2] = tot[2];
@@ -1462,22 +1550,28 @@ __device__ __forceinline__ void gload(const StepArgs& A, const GTile& t, GShared
     if (order) gweight_order<G>(A, t, sh, cs, S, need);
 }
 
+// One batch: this group visits cell c (c < 0: none, it only keeps step with the CTA's other groups) without the
+// interactions in `skip` (failed in an earlier visit, their energy pairs in `used`). A cell whose correction fails under
+// the rollback policy is left as stored and put on the CTA's retry list: Sec. 5.2 resets the failing interaction, and
+// the interactions before it give the same results again (every draw and reduction order is fixed).
 template <bool REL, int G>
-__device__ void gcell(const StepArgs& A, int c, unsigned char* dyn, GShared<G>& sh)
+__device__ void gcell(const StepArgs& A, int c, uint64_t skip, int used, unsigned char* tile, GShared<G>& sh,
+                      CtaShared& cta, uint32_t step)
 {
     const int S = A.S;
-    const int64_t cs = A.offsets[(int64_t)c * S];
-    const int n = (int)(A.offsets[(int64_t)(c + 1) * S] - cs);
-    if (n > A.gcap || n > A.max_cell) {
-        if (threadIdx.x == 0) latch(A.status, kErrBounds);
-        return;
+    int64_t cs = 0;
+    int n = 0;
+    if (c >= 0) {
+        cs = A.offsets[(int64_t)c * S];
+        n = (int)(A.offsets[(int64_t)(c + 1) * S] - cs);
+        if (n > A.gcap || n > A.max_cell) {
+            if (tix<G>() == 0) latch(A.status, kErrBounds);
+            c = -1;
+        }
     }
-    const GTile t = gtile(dyn, A.gcap, n, A.status ? A.status + 4 : nullptr);
-    if ((int)threadIdx.x <= S) sh.off[threadIdx.x] = (int)(A.offsets[(int64_t)c * S + threadIdx.x] - cs);
-    for (int k = threadIdx.x; k < kMaxInter; k += G) {
-        sh.used_k[k] = 0;
-        sh.fail_k[k] = 0;
-    }
+    const bool mine = c >= 0;
+    const GTile t = gtile(tile, A.gcap, n, A.status ? A.status + 4 : nullptr);
+    if (mine && tix<G>() <= S) sh.off[tix<G>()] = (int)(A.offsets[(int64_t)c * S + tix<G>()] - cs);
     gsync<G>();
     PhaseClk pc;
 #ifdef MCC_PHASE_CLOCKS
@@ -1485,40 +1579,53 @@ __device__ void gcell(const StepArgs& A, int c, unsigned char* dyn, GShared<G>& 
 #pragma unroll
     for (int q = 0; q < 8; ++q) pc.acc[q] = 0;
 #endif
-    const uint32_t step = sh.step;
-    // one call site of the cell load: the Sec. 5.2 fallback (an interaction failed) restarts the visit from the stored
-    // state, skipping the failed interactions
-    uint64_t skip = 0;
-    for (bool again = true; again;) {
-        again = false;
-        gload<REL, G>(A, t, sh, cs, S);
-        PHASE_MARK(pc, 0);
-        for (int k = 0; k < A.n_inter; ++k) {
-            if ((skip >> k) & 1ull) continue;
-            const InterConst& ic = A.ic[k];
-            const bool intra = ic.a == ic.b;
-            const int a0 = sh.off[ic.a], na = sh.off[ic.a + 1] - a0;
-            const int b0 = sh.off[ic.b], nb = sh.off[ic.b + 1] - b0;
-            const bool active = intra ? (na >= 2) : (na > 0 && nb > 0);
-            if (!active) continue;
-            const uint32_t ictr = (uint32_t)(A.inter_base + k);
-            gpermutations<G>(A, t, sh, c, ictr, intra ? 1 : 2, a0, na, b0, nb, step);
-            PHASE_MARK(pc, 1);
-            gscatter<REL, G>(A, t, c, cs, ictr, ic, intra, a0, na, b0, nb, step);
-            PHASE_MARK(pc, 2);
-            if (!A.correct) continue;
-            if (gcorrect<REL, G>(A, t, sh, c, cs, k, ic, intra, a0, na, b0, nb, pc)) {
-                skip |= 1ull << k;
-                again = true;
-                break;
-            }
+    int failed = __popcll(skip);
+    const int kept = used;
+    bool again = false;
+    if (mine) gload<REL, G>(A, t, sh, cs, S);
+    csync<G>();
+    PHASE_MARK(pc, 0);
+    for (int k = 0; k < A.n_inter; ++k) {
+        const InterConst& ic = A.ic[k];
+        const bool intra = ic.a == ic.b;
+        int a0 = 0, na = 0, b0 = 0, nb = 0;
+        if (mine) {
+            a0 = sh.off[ic.a];
+            na = sh.off[ic.a + 1] - a0;
+            b0 = sh.off[ic.b];
+            nb = sh.off[ic.b + 1] - b0;
         }
+        const bool on = mine && !again && !((skip >> k) & 1ull) && (intra ? (na >= 2) : (na > 0 && nb > 0));
+        const uint32_t ictr = (uint32_t)(A.inter_base + k);
+        if (on) gpermutations<G>(A, t, sh, c, ictr, intra ? 1 : 2, a0, na, b0, nb, step);
+        csync<G>();
+        PHASE_MARK(pc, 1);
+        if (on) gscatter<REL, G>(A, t, c, cs, ictr, ic, intra, a0, na, b0, nb, step);
+        csync<G>();
+        PHASE_MARK(pc, 2);
+        if (!A.correct) continue;
+        const int before = used;
+        if (gcorrect<REL, G>(A, t, sh, c, cs, ic, intra, a0, na, b0, nb, on, used, failed, pc)) {
+            skip |= 1ull << k;
+            again = true;
+            used = kept + (used - before);  // the pairs of the interactions before this one are counted again next time
+        }
+    }
+    if (!mine) return;
+    if (again) {
+        if (tix<G>() == 0) {
+            const int at = atomicAdd(&cta.n_retry, 1);
+            cta.r_cell[at] = c;
+            cta.r_used[at] = used;
+            cta.r_skip[at] = skip;
+        }
+        return;
     }
     // write back: the float-float state rounded once to float
     const int cap = t.cap;
     float* gv[3] = {reinterpret_cast<float*>(A.vx), reinterpret_cast<float*>(A.vy), reinterpret_cast<float*>(A.vz)};
 #pragma unroll 1  // rolled: a smaller instruction footprint
-    for (int i = threadIdx.x; i < n; i += G) {
+    for (int i = tix<G>(); i < n; i += G) {
 #pragma unroll
         for (int d = 0; d < 3; ++d)
             gv[d][cs + CHK(t.dbg, i, t.n)] = ff_round(ff_ld(t.v[d * cap + CHK(t.dbg, i, t.n)]));
@@ -1534,7 +1641,7 @@ __device__ void gcell(const StepArgs& A, int c, unsigned char* dyn, GShared<G>& 
             ff acc[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) acc[q] = zero;
-            for (int q = threadIdx.x; q < ns; q += G) {
+            for (int q = tix<G>(); q < ns; q += G) {
                 const int i = s0 + q;
                 const float2 ws = t.w[CHK(t.dbg, i, t.n)];
                 const ff w = {ws.x, ws.y};
@@ -1554,7 +1661,7 @@ __device__ void gcell(const StepArgs& A, int c, unsigned char* dyn, GShared<G>& 
             for (int q = 0; q < 4; ++q) tot[q] = ff_add(tot[q], ff_mul(m, acc[q]));
             amag = ff_add(amag, ff_mul(m, acc[4]));
         }
-        if (threadIdx.x == 0) {
+        if (tix<G>() == 0) {
             double dp = 0.0;
 #pragma unroll
             for (int d = 0; d < 3; ++d) dp = fmax(dp, fabs(ff_dbl(ff_sub(tot[d], sh.P0[d]))));
@@ -1565,18 +1672,13 @@ __device__ void gcell(const StepArgs& A, int c, unsigned char* dyn, GShared<G>& 
             A.resid[2 * (int64_t)c + 1] = e0 > 0.0 ? de / e0 : de;
         }
     }
-    if (threadIdx.x == 0) {
-        int u = 0, f = 0;
-        for (int k = 0; k < A.n_inter; ++k) {
-            u += sh.used_k[k];
-            f += sh.fail_k[k];
-        }
-        if (A.corr_pairs) A.corr_pairs[c] += u;
-        if (A.fail_count) A.fail_count[c] += f;
+    if (tix<G>() == 0) {
+        if (A.corr_pairs) A.corr_pairs[c] += used;
+        if (A.fail_count) A.fail_count[c] += failed;
     }
     PHASE_MARK(pc, 6);
 #ifdef MCC_PHASE_CLOCKS
-    if (threadIdx.x == 0 && A.phase_clk) {
+    if (tix<G>() == 0 && A.phase_clk) {
 #pragma unroll
         for (int q = 0; q < 7; ++q)
             atomicAdd(A.phase_clk + 8 * A.gcls + q, (unsigned long long)pc.acc[q]);
@@ -1585,26 +1687,64 @@ __device__ void gcell(const StepArgs& A, int c, unsigned char* dyn, GShared<G>& 
 #endif
 }
 
+// One CTA: blockDim.x / G groups. Every batch takes up to one cell per group from the class's queue, as many as make the
+// batches of the launch equal (a class with few cells spreads them over the CTAs instead of filling a few), or the
+// cells of the retry list once they fill a batch or the queue is empty.
 template <bool REL, int G>
-__global__ void __launch_bounds__(G, kGroupWarpsPerSm / (G / 32) > 0 ? kGroupWarpsPerSm / (G / 32) : 1)
+__global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group_cta_warps(REL),
+                                  G > 32 * group_cta_warps(REL) ? 1 : kGroupWarpsPerSm / group_cta_warps(REL))
     group_kernel(const __grid_constant__ StepArgs A)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ GShared<G> sh;
+    __shared__ CtaShared cta;
     const int cls = A.gcls;
-    const int beg = A.class_off[2 * cls], end = A.class_off[2 * cls + 1];
-    if (threadIdx.x == 0) sh.step = A.step_dev ? (uint32_t)(*A.step_dev + A.step_add) : A.rng.step;
+    const int beg = A.class_off[2 * cls], total = A.class_off[2 * cls + 1] - beg;
+    const uint32_t step = A.step_dev ? (uint32_t)(*A.step_dev + A.step_add) : A.rng.step;
+    const int teams = (int)blockDim.x / G, tm = team<G>();
+    const int waves = (total + teams * (int)gridDim.x - 1) / (teams * (int)gridDim.x);
+    const int most = waves > 0 ? (total + waves * (int)gridDim.x - 1) / (waves * (int)gridDim.x) : 1;  // <= teams
+    unsigned char* mem = dyn + (size_t)tm * group_smem(group_shared_bytes<G>(), A.gcap);
+    GShared<G>& sh = *reinterpret_cast<GShared<G>*>(mem);
+    unsigned char* tile = mem + group_shared_bytes<G>();
+    if (threadIdx.x == 0) cta.n_retry = 0;
     for (;;) {
         if (threadIdx.x == 0) {
-            const int q = beg + atomicAdd(&A.queues[cls], 1);
-            sh.cell = q < end ? A.order[CHK(A.status ? A.status + 4 : nullptr, q, A.n_cells)] : -1;
+            cta.retry = cta.n_retry >= teams;
+            if (!cta.retry) {
+                cta.base = atomicAdd(&A.queues[cls], most);
+                const int left = total - cta.base;
+                cta.take = left < most ? left : most;
+                if (cta.take <= 0) cta.retry = 1;
+            }
+            if (cta.retry) {
+                cta.take = cta.n_retry < teams ? cta.n_retry : teams;
+                cta.base = cta.n_retry -= cta.take;
+            }
         }
-        gsync<G>();
-        const int c = sh.cell;
-        if (c < 0) break;
-        gcell<REL, G>(A, c, dyn, sh);
-        gsync<G>();
+        __syncthreads();
+        if (cta.take <= 0) break;
+        int c = -1, used = 0;
+        uint64_t skip = 0;
+        if (tm < cta.take) {
+            if (cta.retry) {
+                c = cta.r_cell[cta.base + tm];
+                used = cta.r_used[cta.base + tm];
+                skip = cta.r_skip[cta.base + tm];
+            } else {
+                c = A.order[CHK(A.status ? A.status + 4 : nullptr, beg + cta.base + tm, A.n_cells)];
+            }
+        }
+        gcell<REL, G>(A, c, skip, used, tile, sh, cta, step);
+        __syncthreads();
     }
+}
+
+// Shared memory of one group of class cls beside its tile.
+inline size_t shared_bytes_of(int cls)
+{
+    const size_t b[kGroupClasses] = {group_shared_bytes<32>(), group_shared_bytes<64>(), group_shared_bytes<128>(),
+                                     group_shared_bytes<256>(), group_shared_bytes<512>()};
+    return b[cls];
 }
 
 template <bool REL, int G>

@@ -15,4 +15,6 @@ const void* group_kernel_f32(int cls)
     }
 }
 
+size_t group_shared_bytes(int cls) { return grp::shared_bytes_of(cls); }
+
 }  // namespace mcc

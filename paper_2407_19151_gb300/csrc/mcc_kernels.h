@@ -86,12 +86,23 @@ constexpr int kGroupClasses = 5;  // group sizes 32, 64, 128, 256, 512 threads
 // Warps of the group kernels resident per SM: their register budget (launch bounds) and the automatic capacity
 // (shared memory per warp) are both set for this many.
 constexpr int kGroupWarpsPerSm = MCC_GROUP_WARPS_PER_SM;
+// Warps of one CTA of the group kernels; its groups run in lockstep (mcc_group.cuh). Two CTAs of eight warps per SM
+// overlap one's barrier waits with the other's work; the relativistic code is larger and gains more from fetching once for
+// all sixteen warps (three-species step of 1.34e8 particles: 37.9 / 29.1 / 30.6 ms with 4 / 8 / 16 warps; relativistic beam
+// of 1.16e7: 12.2 / 8.7 / 8.0 ms).
+constexpr int group_cta_warps(bool rel) { return rel ? 16 : 8; }
 
 // Bytes per particle of the cell tile (keys, weights, velocities, pre-scatter copy, permutation, weight order).
 __host__ __device__ inline size_t tile_bytes_per_particle(bool f32) { return 8 + 8 + (f32 ? 6 * 4 : 6 * 8) + 4 + 4; }
 
 // Shared-memory bytes per particle of the group kernels' cell tile (state, weight, scratch, two orders).
 constexpr size_t kGroupBytesPerParticle = 44;
+
+// Shared memory of one group: its shared variables (shared_bytes, see group_shared_bytes) and a tile of cap particles.
+__host__ __device__ inline size_t group_smem(size_t shared_bytes, int cap)
+{
+    return (shared_bytes + (size_t)cap * kGroupBytesPerParticle + 15) & ~(size_t)15;
+}
 
 // N97 table: (f, h df/dx) at kN97Nodes + 1 nodes, computed on the host in double.
 void n97_table(double* f, double* dh);
@@ -106,7 +117,10 @@ cudaError_t launch_group_order(const int64_t* offsets, int32_t n_cells, int32_t 
                                int32_t* order, int32_t* class_off, cudaStream_t st);
 // Group kernels (mcc_group_*.cu): class cls runs groups of 32 << cls threads.
 const void* group_kernel(bool f32, bool rel, int cls);
-cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, size_t smem, cudaStream_t st);
+size_t group_shared_bytes(int cls);  // shared variables of one group
+// groups: groups (cells at a time) of one CTA
+cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem,
+                         cudaStream_t st);
 int cell_kernel_blocks_per_sm(bool f32, bool rel, int mode, size_t smem);
 cudaError_t set_cell_smem_limit(bool f32, bool rel, int mode, size_t smem);
 size_t cell_kernel_static_smem(bool f32, bool rel, int mode);
