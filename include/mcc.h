@@ -364,7 +364,7 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* particles, const int64_t* 
                    int32_t* corr_pairs, int32_t* fail_count, void* ws, size_t ws_bytes, mcc_stream stream);
 
 /* Particles staged on chip per cell by the one-CTA kernel of mcc_step_fused, which takes the cells above the
- * largest group class (0 = automatic: the largest tile with which six CTAs share an SM's shared memory, or the
+ * largest group class (0 = automatic: the largest tile with which four CTAs share an SM's shared memory, or the
  * largest cell if smaller). Cells above it run from the workspace slabs. */
 int mcc_set_tile_cap(mcc_ctx* ctx, int32_t cap);
 

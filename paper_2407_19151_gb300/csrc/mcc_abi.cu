@@ -2,6 +2,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include <nvtx3/nvToolsExt.h>
@@ -23,7 +24,7 @@ struct NvtxRange {
 
 struct mcc_ctx {
     int device;
-    int32_t* dbuf;  // [0] status word, [1] work-queue counter, then the N97 tables
+    int32_t* dbuf;  // [0] status word, [1] work-queue counter, then the tables
     int64_t launches;
     int num_sms;
     size_t smem_optin;
@@ -39,64 +40,127 @@ namespace mcc {
 // Bytes per particle of the pairing mode's tile (defined with its kernel, mcc_cell.cu).
 size_t pair_tile_bytes_per_particle();
 
-// N97 table on the host, in double: A(s) solves G(A) = 1 - coth A + 1/A = 1 - e^-s (bisection to the last bit);
-// stored as f = ln(A s) and h df/dx at x = ln s, where df/dx = 1 + s e^-s / (A G'(A)) by implicit
-// differentiation, G'(A) = -(1/A^2 - 1/sinh^2 A).
+// Host tables. A(s) solves L(A) = coth A - 1/A = e^-s.
 namespace {
 
-void laurent(double A, double& L, double& dL)
+// L and dL/dA; below A = 3/2 from the power series of A coth A (radius pi), whose coefficients a_n follow from
+// (A coth A) (sinh A / A) = cosh A.
+template <class T>
+void langevin(T A, T& L, T& dL)
 {
-    // coth A - 1/A = sum_n 2^{2n} B_{2n} A^{2n-1} / (2n)!, for A < 1/2
-    static const double c[12] = {1.0 / 3.0,       -1.0 / 45.0,        2.0 / 945.0,        -1.0 / 4725.0,
-                                 2.0 / 93555.0,   -1382.0 / 638512875.0, 4.0 / 18243225.0, -3617.0 / 162820783125.0,
-                                 87734.0 / 38979295480125.0, -349222.0 / 1531329465290625.0,
-                                 310732.0 / 13447856940643125.0, -472728182.0 / 201919571963756521875.0};
-    L = 0.0;
-    dL = 0.0;
-    double p = A;
-    for (int n = 0; n < 12; ++n) {
-        L += c[n] * p;
-        dL += (2 * n + 1) * c[n] * (p / A);
-        p *= A * A;
+    if (A >= T(1.5)) {
+        const T sh = A < T(350) ? std::sinh(A) : T(1);
+        L = 1 / std::tanh(A) - 1 / A;
+        dL = 1 / (A * A) - (A < T(350) ? 1 / (sh * sh) : T(0));
+        return;
     }
+    constexpr int kTerms = 30;
+    static const struct Series {
+        T a[kTerms + 1];
+        Series()
+        {
+            T fact[2 * kTerms + 2];
+            fact[0] = 1;
+            for (int n = 1; n < 2 * kTerms + 2; ++n) fact[n] = fact[n - 1] * n;
+            for (int n = 0; n <= kTerms; ++n) {
+                a[n] = 1 / fact[2 * n];
+                for (int k = 0; k < n; ++k) a[n] -= a[k] / fact[2 * (n - k) + 1];
+            }
+        }
+    } series;
+    const T x2 = A * A;
+    L = 0;
+    dL = 0;
+    for (int n = kTerms; n >= 1; --n) {
+        L = L * x2 + series.a[n];
+        dL = dL * x2 + (2 * n - 1) * series.a[n];
+    }
+    L *= A;
 }
-double G_of(double A)
+
+// One Newton step for A(s): on 1 - L(A) = 1 - e^-s for short lengths (1 - L = 1/A - 2/expm1(2A) keeps its relative
+// precision), on L(A) = e^-s otherwise.
+template <class T>
+T n97_newton(T s, T A)
 {
-    if (A < 0.5) {
-        double L, dL;
-        laurent(A, L, dL);
-        return 1.0 - L;
-    }
-    return 1.0 / A - 2.0 / std::expm1(2.0 * A);
+    T L, dL;
+    langevin(A, L, dL);
+    const T f = s < T(0.7) ? -std::expm1(-s) - (1 / A - 2 / std::expm1(2 * A)) : L - std::exp(-s);
+    return A - f / dL;
 }
-double dG_of(double A)
+
+// A(s): from the short-length series or the long-length inversion, Newton to double precision, then one step in the
+// host's long double, so that the tables are correctly rounded up to an ulp.
+long double n97_root(long double s)
 {
-    if (A < 0.5) {
-        double L, dL;
-        laurent(A, L, dL);
-        return -dL;
+    const double sd = (double)s, y = std::exp(-sd);
+    double A = sd < 2.0 ? -1.0 / std::expm1(-sd) : 3.0 * y * (1.0 + 0.6 * y * y);
+    for (int it = 0; it < 60; ++it) {
+        double An = n97_newton(sd, A);
+        if (!(An > 0.0)) An = 0.5 * A;
+        if (An > 4.0 * A) An = 4.0 * A;
+        const double d = std::fabs(An - A);
+        A = An;
+        if (d <= 1e-14 * A) break;
     }
-    const double sh = std::sinh(A);
-    return -(1.0 / (A * A) - (A < 350.0 ? 1.0 / (sh * sh) : 0.0));
+    return n97_newton(s, (long double)A);
 }
+
 }  // namespace
 
-void n97_table(double* f, double* dh)
+void n97_table(float* g, float* dh)
 {
     for (int k = 0; k <= kN97Nodes; ++k) {
-        const double x = kN97X0 + kN97H * k;
-        const double s = std::exp(x);
-        const double z = -std::expm1(-s);
-        double lo = 0.0, hi = 1.0 / z + 1.0;
-        for (int it = 0; it < 2000; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            if (mid <= lo || mid >= hi) break;
-            if (G_of(mid) > z) lo = mid;
-            else hi = mid;
+        const double s = std::exp(kN97X0 + kN97H * k);
+        const double A = (double)n97_root(s);
+        double L, dL;
+        langevin(A, L, dL);
+        g[k] = (float)(A * s);  // d ln(A s)/dx = 1 - s e^-s / (A L'(A))
+        dh[k] = (float)(A * s * kN97H * (1.0 - s * std::exp(-s) / (A * dL)));
+    }
+}
+
+// Tables of mcc_pair64.cuh: Chebyshev interpolants of A(s) s as monomials in the interval's own variable t in [-1, 1],
+// multiples of 1/256 turn, and the reciprocals and logarithms of mantissas in [0.6875, 1.375).
+void f64_tables(double* out)
+{
+    constexpr int N = 8;
+    using T = long double;
+    T cosine[N][N], cheb[N][N];  // cosine[m][j] = T_m(node j); cheb[m]: monomial coefficients of T_m
+    for (int m = 0; m < N; ++m) {
+        for (int q = 0; q < N; ++q) cheb[m][q] = 0;
+        if (m < 2) cheb[m][m] = 1;
+        else
+            for (int q = 0; q < N; ++q) cheb[m][q] = (q ? 2 * cheb[m - 1][q - 1] : T(0)) - cheb[m - 2][q];
+        for (int j = 0; j < N; ++j) cosine[m][j] = std::cos(std::acos(T(-1)) * m * (2 * j + 1) / (2 * N));
+    }
+    for (int i = 0; i < kF64N97; ++i) {
+        const T w = std::ldexp(T(1) / 64, i / 64 - 5);  // interval width
+        const T a = std::ldexp(T(1), i / 64 - 5) + (i % 64) * w;
+        T f[N], c[N] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (int j = 0; j < N; ++j) {
+            const T s = a + w * (1 + cosine[1][j]) / 2;
+            f[j] = n97_root(s) * s;
         }
-        const double A = 0.5 * (lo + hi);
-        f[k] = std::log(A * s);
-        dh[k] = kN97H * (1.0 + s * std::exp(-s) / (A * dG_of(A)));
+        for (int m = 0; m < N; ++m) {
+            T b = 0;
+            for (int j = 0; j < N; ++j) b += f[j] * cosine[m][j];
+            b *= T(m ? 2 : 1) / N;
+            for (int q = 0; q < N; ++q) c[q] += b * cheb[m][q];
+        }
+        for (int q = 0; q < N; ++q) out[N * i + q] = (double)c[q];
+    }
+    double* turn = out + N * kF64N97;
+    for (int i = 0; i < kF64Turn; ++i) {
+        turn[2 * i] = i % 128 == 64 ? 0.0 : std::cos(2.0 * M_PI * i / kF64Turn);
+        turn[2 * i + 1] = i % 128 == 0 ? 0.0 : std::sin(2.0 * M_PI * i / kF64Turn);
+    }
+    double* ln = turn + 2 * kF64Turn;
+    for (int i = 0; i < kF64Ln; ++i) {  // mantissas below 1 come in steps of 1/256, above in steps of 1/128
+        const double m = i < 80 ? 0.6875 + (i + 0.5) / 256.0 : 1.0 + (i - 80 + 0.5) / 128.0;
+        const double r = i == 79 || i == 80 ? 1.0 : (double)(float)(1.0 / m);
+        ln[2 * i] = r;
+        ln[2 * i + 1] = r == 1.0 ? 0.0 : -std::log(r);
     }
 }
 
@@ -106,15 +170,16 @@ namespace {
 
 using mcc::StepArgs;
 
-constexpr size_t kTabOffset = 64;  // bytes into the context buffer where the N97 tables start
-constexpr size_t kTabDoubles = 2 * (mcc::kN97Nodes + 1);
-constexpr size_t kClkOffset = (kTabOffset + kTabDoubles * sizeof(double) + kTabDoubles * sizeof(float) + 63) & ~63;
+constexpr size_t kTabOffset = 64;  // bytes into the context buffer where the tables start: FP64 pairs, then float pairs
+constexpr size_t kTab64Bytes = mcc::kF64TabDoubles * sizeof(double);
+constexpr size_t kTab32Floats = 2 * (mcc::kN97Nodes + 1);
+constexpr size_t kClkOffset = (kTabOffset + kTab64Bytes + kTab32Floats * sizeof(float) + 63) & ~63;
 constexpr size_t kClkWords = 8 * mcc::kGroupClasses;  // phase cycles of the group kernels (phase-timing builds)
 constexpr size_t kCtxBytes = kClkOffset + kClkWords * sizeof(unsigned long long);
 
 constexpr size_t kStaticSmemReserve = 1024;  // margin above the cell kernel's static shared memory
 #ifndef MCC_AUTO_CTAS
-#define MCC_AUTO_CTAS 6
+#define MCC_AUTO_CTAS 4
 #endif
 constexpr int kAutoCtasPerSm = MCC_AUTO_CTAS;  // automatic tile: this many CTAs share one SM's shared memory
 constexpr int kMaxCtasPerSm = 2048 / mcc::kThreads;
@@ -191,6 +256,8 @@ int fill_args(StepArgs& a, const mcc_ctx* ctx, const mcc_particles* P, const int
             ic.kappa_mu2 = kappa / (mu * mu);
             ic.mu_ma = mu / ma;
             ic.mu_mb = mu / mb;
+            ic.inv_ma = 1.0 / ma;
+            ic.inv_mb = 1.0 / mb;
             ic.kappa_f = (float)ic.kappa;
             ic.kappa_mu2_f = (float)ic.kappa_mu2;
             ic.mu_ma_f = (float)ic.mu_ma;
@@ -227,9 +294,10 @@ int fill_args(StepArgs& a, const mcc_ctx* ctx, const mcc_particles* P, const int
     a.status = ctx->dbuf;
     a.queue = ctx->dbuf + 1;
     const char* base = reinterpret_cast<const char*>(ctx->dbuf) + kTabOffset;
-    a.n97_f = reinterpret_cast<const double*>(base);
-    a.n97_dh = a.n97_f + (mcc::kN97Nodes + 1);
-    a.n97_f32 = reinterpret_cast<const float*>(base + kTabDoubles * sizeof(double));
+    a.t64.n97 = reinterpret_cast<const double2*>(base);
+    a.t64.turn = a.t64.n97 + 4 * mcc::kF64N97;
+    a.t64.ln = a.t64.turn + mcc::kF64Turn;
+    a.n97_f32 = reinterpret_cast<const float*>(base + kTab64Bytes);
     a.n97_dh32 = a.n97_f32 + (mcc::kN97Nodes + 1);
     a.phase_clk = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(ctx->dbuf) + kClkOffset);
     return MCC_OK;
@@ -282,10 +350,22 @@ int run_cells(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, int cap, 
     return cuda_status(e);
 }
 
-// Grid of the adjoint kernel: one CTA per cell, at most two per SM (each holds a slab of the workspace).
-int adjoint_grid(const mcc_ctx* ctx, int32_t n_cells)
+// Whether the adjoint's working arrays for cells of max_cell particles fit one CTA's shared memory.
+bool adjoint_on_chip(const mcc_ctx* ctx, int32_t max_cell)
 {
-    const int g = ctx->num_sms * 2;
+    return mcc::adjoint_work_bytes(max_cell) + mcc::adjoint_static_smem() <= ctx->smem_optin;
+}
+
+// Grid of the adjoint kernel: one CTA per cell, at most as many as are resident. slab: bytes each CTA holds of the
+// workspace (0: the slabs are per cell); more than two CTAs per SM only while they hold less than 1 GiB in all.
+int adjoint_grid(const mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, size_t slab)
+{
+    const size_t cta = mcc::adjoint_static_smem() + ctx->smem_reserved +
+                       (adjoint_on_chip(ctx, max_cell) ? mcc::adjoint_work_bytes(max_cell) : 0);
+    int per_sm = mcc::adjoint_ctas_per_sm();
+    while (per_sm > 1 && cta * (size_t)per_sm > ctx->smem_per_sm) --per_sm;
+    while (per_sm > 2 && slab * (size_t)per_sm * (size_t)ctx->num_sms > ((size_t)1 << 30)) --per_sm;
+    const int g = ctx->num_sms * per_sm;
     return n_cells < g ? (n_cells > 0 ? n_cells : 1) : g;
 }
 
@@ -316,16 +396,14 @@ int mcc_create(mcc_ctx** out, int device)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     c->smem_optin = (size_t)optin;
     c->num_sms = sms;
-    // status word, queue counter and the N97 tables (double, then float), computed here once
-    double tab[kTabDoubles];
-    float tab32[kTabDoubles];
-    mcc::n97_table(tab, tab + (mcc::kN97Nodes + 1));
-    // float copy: g = A s = exp(f) and h dg/dx = exp(f) (h df/dx)
-    for (int k = 0; k <= mcc::kN97Nodes; ++k) {
-        const double g = std::exp(tab[k]);
-        tab32[k] = (float)g;
-        tab32[mcc::kN97Nodes + 1 + k] = (float)(g * tab[mcc::kN97Nodes + 1 + k]);
-    }
+    // status word, queue counter and the tables, computed here once
+    static double tab[mcc::kF64TabDoubles];
+    static float tab32[kTab32Floats];
+    static std::once_flag once;
+    std::call_once(once, [] {
+        mcc::f64_tables(tab);
+        mcc::n97_table(tab32, tab32 + (mcc::kN97Nodes + 1));
+    });
     if (cudaMalloc(&c->dbuf, kCtxBytes) != cudaSuccess || cudaMemset(c->dbuf, 0, kCtxBytes) != cudaSuccess ||
         cudaMemcpy(reinterpret_cast<char*>(c->dbuf) + kTabOffset, tab, sizeof tab, cudaMemcpyHostToDevice) !=
             cudaSuccess ||
@@ -788,8 +866,8 @@ int mcc_adjoint_workspace_size(mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, 
     if (max_cell > MCC_MAX_SEGMENT) return MCC_ERR_TOO_LARGE;
     const int32_t mc = max_cell > 0 ? max_cell : 1;
     const int32_t ep = max_corr_passes * (mc / 2 + 1) + 1;
-    const int grid = adjoint_grid(ctx, n_cells);
-    *bytes = mcc::adjoint_slab_bytes(mc, ep) * (size_t)grid;
+    const size_t slab = mcc::adjoint_slab_bytes(mc, ep, adjoint_on_chip(ctx, mc));
+    *bytes = slab * (size_t)adjoint_grid(ctx, n_cells, mc, slab);
     return MCC_OK;
 }
 
@@ -799,7 +877,7 @@ int mcc_adjoint_tape_size(mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, int32
     if (max_cell > MCC_MAX_SEGMENT) return MCC_ERR_TOO_LARGE;
     const int32_t mc = max_cell > 0 ? max_cell : 1;
     const int32_t ep = max_corr_passes * (mc / 2 + 1) + 1;
-    *bytes = mcc::adjoint_slab_bytes(mc, ep) * (size_t)(n_cells > 0 ? n_cells : 1);
+    *bytes = mcc::adjoint_slab_bytes(mc, ep, adjoint_on_chip(ctx, mc)) * (size_t)(n_cells > 0 ? n_cells : 1);
     return MCC_OK;
 }
 
@@ -830,9 +908,11 @@ int mcc_adjoint(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets, in
     if (!ws || ws_bytes < need) return MCC_ERR_WORKSPACE;
     const int32_t mc = max_cell > 0 ? max_cell : 1;
     const int32_t ep = p->max_corr_passes * (mc / 2 + 1) + 1;
+    const bool on_chip = adjoint_on_chip(ctx, mc);
+    const size_t slab = tape == MCC_ADJOINT_RECOMPUTE ? mcc::adjoint_slab_bytes(mc, ep, on_chip) : 0;
     const cudaError_t e = mcc::launch_adjoint(a, lnL[sa * n_species + sb], vx_out, vy_out, vz_out, gvx, gvy, gvz, gw,
-                                              glnL, reinterpret_cast<char*>(ws), mc, ep, tape,
-                                              adjoint_grid(ctx, n_cells), S(stream));
+                                              glnL, reinterpret_cast<char*>(ws), mc, ep, tape, on_chip,
+                                              adjoint_grid(ctx, n_cells, mc, slab), S(stream));
     ctx->launches += 1;
     return cuda_status(e);
 }

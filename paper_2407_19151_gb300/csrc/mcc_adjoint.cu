@@ -16,14 +16,26 @@
 // A Delta E_s that vanishes (equal weights, or below the rounding-noise threshold) is differentiated as its limit:
 // the first pair of the order as the crossing pair with U = Delta E_s = 0.
 // The kernel recomputes the interaction from the stored pre-interaction state, keeping a tape of every pair's inputs,
-// then runs the chain rule backwards through the tape (one CTA per cell, the cell's working arrays in a per-CTA slab
-// of the workspace). With a recorded tape the slabs are per cell and outlive the call: a recording call runs the
-// forward and keeps each cell's slab (the tape and the per-cell scalars of the correction); a later replaying call on
-// the same interaction runs only the reverse sweep from it.
-#include "mcc_kernels.h"
+// then runs the chain rule backwards through the tape (one CTA per cell; the tape in a per-CTA slab of the workspace).
+// With a recorded tape the slabs are per cell and outlive the call: a recording call runs the forward and keeps each
+// cell's slab (the tape and the per-cell scalars of the correction); a later replaying call on the same interaction
+// runs only the reverse sweep from it.
+//
+// What bounds it: the FP64 pipe for the pairs (mcc_pair64.cuh), once the serial parts are out of the way. The working
+// arrays that are read in random order (state or gradient, weights, sort keys, permutation, weight order: 64 B per
+// particle) live in shared memory, the permutations are counting sorts there, and both directions of the energy pairs
+// run 32 at a time (a pass's pairs are disjoint; the forward needs a prefix sum over their caps, the reverse only the
+// crossing pair's dL/dU, which comes first). Two recorded steps of 1024 cells x 512 with their reverse: 5.9 -> 2.75 ms, of which
+// 3.8 with the pair functions alone. The forward sums what the step kernel sums in its order, so a replay from a
+// checkpoint repeats the step's trajectory bit for bit (the closed-form gradients over 50 steps from checkpoints then hold as
+// closely as from tapes, 1e-11 where they held 3e-10).
+#include "mcc_pair64.cuh"
+#include "mcc_perm.cuh"
 
 namespace mcc {
 namespace {
+
+constexpr int kAdjCtasPerSm = 4;  // resident CTAs the kernel's registers are bounded for
 
 constexpr int kFlagTriplet = 1, kFlagUpdI = 2, kFlagUpdJ = 4, kFlagActive = 8;
 
@@ -43,6 +55,7 @@ struct AdjArgs {
     int32_t max_cell;
     int32_t max_epairs;
     int32_t tape;              // 0: per-CTA slabs, recompute; 1: per-cell slabs, record; 2: per-cell slabs, replay
+    int32_t on_chip;           // working arrays in shared memory (else in the slab)
 };
 
 // Per-cell scalars of the forward that the reverse sweep reads (kept at the end of a recorded slab).
@@ -51,39 +64,60 @@ struct TapeHead {
     double B[3], Sw, S[3], dE, Es[2], W1[2], D[2];
 };
 
-// Per-CTA working arrays (n = max_cell, E = max_epairs).
+// The tape of one cell (n = max_cell, E = max_epairs).
 struct Slab {
-    uint64_t* keys;
-    double* v;      // [3][n] working state
     double* vb;     // [3][n] before the interaction
     double* vp;     // [3][n] after the scatter
     double* vm;     // [3][n] after the momentum shift
-    double* g;      // [3][n] gradient of the current stage
-    double* gb;     // [3][n] gradient reaching v_before directly through the correction
-    double* gwl;    // [n] dL/dw of this interaction
     double* pv;     // [6][n] per scatter pair: v_i, v_j at the pair's turn
     double* ev;     // [6][E] per energy pair: v_1, v_2 at the pair's turn
     double* eU;     // [E]
     double* eK;     // [E]
-    int32_t* perm;  // [n] random permutation (cell-local indices, segment start included)
-    int32_t* rho;   // [n] energy-pair order
     int32_t* pi;    // [n] scatter pair particles and flags
     int32_t* pj;
     int32_t* pf;
-    int32_t* ei;    // [E] energy pair particles, capped flag
+    int32_t* ei;    // [E] energy pair particles; 2 pass + (1 if the pair took its cap)
     int32_t* ej;
     int32_t* ecap;
     TapeHead* head;
+    char* work;     // working arrays of cells too large for shared memory
     int n, E;
 };
 
+// Working arrays of the cell in progress: the forward's and, over the same bytes, the reverse sweep's.
+struct Work {
+    double* v;       // [3][n] forward: the state; reverse: gradient of the current stage
+    uint64_t* keys;  // [n] forward: sort keys
+    double* gwl;     // [n] reverse: dL/dw of this interaction (over keys)
+    uint32_t* cnt;   // [2 n] forward: bucket counters
+    int32_t* perm;   // [n] forward: random permutation (cell-local indices, segment start included)
+    int32_t* rho;    // [n] forward: energy-pair order
+    double* gb;      // [3][n] reverse: gradient reaching v_before directly through the correction (over cnt ..)
+    double* w;       // [n] weights
+};
+constexpr size_t kWorkBytesPerParticle = 24 + 8 + 24 + 8;
+
+__device__ __forceinline__ Work make_work(char* base, int n)
+{
+    Work k;
+    k.v = reinterpret_cast<double*>(base);
+    k.gwl = k.v + 3 * (size_t)n;
+    k.keys = reinterpret_cast<uint64_t*>(k.gwl);
+    k.gb = k.gwl + n;
+    k.cnt = reinterpret_cast<uint32_t*>(k.gb);
+    k.perm = reinterpret_cast<int32_t*>(k.gb + n);
+    k.rho = k.perm + n;
+    k.w = k.gb + 3 * (size_t)n;
+    return k;
+}
+
 __host__ __device__ inline size_t al8(size_t x) { return (x + 7) & ~(size_t)7; }
 
-__host__ __device__ inline size_t slab_bytes(int n, int E)
+__host__ __device__ inline size_t slab_bytes(int n, int E, bool on_chip)
 {
     const size_t dn = (size_t)n, de = (size_t)E;
-    return al8(8 * dn) + 6 * al8(24 * dn) + al8(8 * dn) + al8(48 * dn) + al8(48 * de) + 2 * al8(8 * de) +
-           5 * al8(4 * dn) + 3 * al8(4 * de) + al8(sizeof(TapeHead)) + 256;
+    return 3 * al8(24 * dn) + al8(48 * dn) + al8(48 * de) + 2 * al8(8 * de) + 3 * al8(4 * dn) + 3 * al8(4 * de) +
+           al8(sizeof(TapeHead)) + (on_chip ? 0 : kWorkBytesPerParticle * dn) + 256;
 }
 
 __device__ Slab make_slab(char* base, int n, int E)
@@ -97,20 +131,13 @@ __device__ Slab make_slab(char* base, int n, int E)
         o += al8(b);
         return p;
     };
-    s.keys = reinterpret_cast<uint64_t*>(take(8 * (size_t)n));
-    s.v = reinterpret_cast<double*>(take(24 * (size_t)n));
     s.vb = reinterpret_cast<double*>(take(24 * (size_t)n));
     s.vp = reinterpret_cast<double*>(take(24 * (size_t)n));
     s.vm = reinterpret_cast<double*>(take(24 * (size_t)n));
-    s.g = reinterpret_cast<double*>(take(24 * (size_t)n));
-    s.gb = reinterpret_cast<double*>(take(24 * (size_t)n));
-    s.gwl = reinterpret_cast<double*>(take(8 * (size_t)n));
     s.pv = reinterpret_cast<double*>(take(48 * (size_t)n));
     s.ev = reinterpret_cast<double*>(take(48 * (size_t)E));
     s.eU = reinterpret_cast<double*>(take(8 * (size_t)E));
     s.eK = reinterpret_cast<double*>(take(8 * (size_t)E));
-    s.perm = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
-    s.rho = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
     s.pi = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
     s.pj = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
     s.pf = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
@@ -118,107 +145,46 @@ __device__ Slab make_slab(char* base, int n, int E)
     s.ej = reinterpret_cast<int32_t*>(take(4 * (size_t)E));
     s.ecap = reinterpret_cast<int32_t*>(take(4 * (size_t)E));
     s.head = reinterpret_cast<TapeHead*>(take(sizeof(TapeHead)));
+    s.work = base + o;
     return s;
 }
 
 struct AdjShared {
     int off[kMaxSpecies + 1];
-    int fail;
+    int fail, fail0;  // the correction failed; no species could take a share
     int ne[2];        // energy pairs taped per side
     int e0[2];        // first tape entry of each side
     int zeroed[2];    // Delta E_s set to zero as rounding noise
     double B[3], Sw, S[3];
     double dE, Es[2], W1[2], D[2], gD[2], gB[3];
     double gS[3], gSw, gdE, gEs[2], gW1[2];
+    int iscan[kWarps + 1];
     alignas(16) unsigned char red_raw[8 * kThreads * 8];
     alignas(8) unsigned char red[8 * 8];
 };
 
 __device__ __forceinline__ Acc<double>* accp(unsigned char* p) { return reinterpret_cast<Acc<double>*>(p); }
 
-// Polar angle of one scatter pair with its derivatives: sin(Theta), 1 - cos(Theta) and d/ds of both.
-__device__ void angle_and_derivative(const StepArgs& A, double s, double U1, double U4, double& st, double& omc,
-                                     double& dst, double& domc)
-{
-    dst = 0.0;
-    domc = 0.0;
-    if (A.method == 0) {
-        // TA77: delta = sqrt(s/2) g; both branches of the forward are sin = 2d/(1+d^2), 1-cos = 2d^2/(1+d^2)
-        const double g = sqrt(-2.0 * log(U1)) * cospi(2.0 * U4);
-        const double d = sqrt(0.5 * s) * g;
-        const double den = 1.0 + d * d;
-        st = 2.0 * d / den;
-        omc = 2.0 * d * d / den;
-        const double dd = s > 0.0 ? d / (2.0 * s) : 0.0;
-        dst = 2.0 * (1.0 - d * d) / (den * den) * dd;
-        domc = 4.0 * d / (den * den) * dd;
-        return;
-    }
-    N97Tab<double> tab = {A.n97_f, A.n97_dh};
-    const double Aa = n97_A(s, tab);
-    double o, q;
-    bool diff = true;
-    if (Aa == 0.0) {
-        o = 2.0 * U1;
-        q = 2.0 * (1.0 - U1);
-        diff = false;
-    } else if (isinf(Aa)) {
-        o = 0.0;
-        q = 2.0;
-        diff = false;
-    } else {
-        const double x = -U1 * -expm1(-2.0 * Aa);
-        o = x > -0.5 ? -log1p(x) / Aa : -log((1.0 - U1) + U1 * exp(-2.0 * Aa)) / Aa;
-        q = o <= 1.0 ? 2.0 - o : log1p((1.0 - U1) * expm1(2.0 * Aa)) / Aa;
-    }
-    bool co = false, cq = false;
-    if (o < 0.0) { o = 0.0; co = true; }
-    if (o > 2.0) { o = 2.0; co = true; }
-    if (q < 0.0) { q = 0.0; cq = true; }
-    if (q > 2.0) { q = 2.0; cq = true; }
-    omc = o;
-    st = sqrt(o * q);
-    if (!diff) return;
-    // 1 - cos = -ln Y / A with Y = (1 - U1) + U1 e^-2A; 1 + cos = 2 - (1 - cos)
-    const double Y = (1.0 - U1) + U1 * exp(-2.0 * Aa);
-    const double do_dA = co ? 0.0 : (-o / Aa + 2.0 * U1 * exp(-2.0 * Aa) / (Aa * Y));
-    const double dq_dA = cq ? 0.0 : -(-o / Aa + 2.0 * U1 * exp(-2.0 * Aa) / (Aa * Y));
-    // G(A) = 1 - (coth A - 1/A) = 1 - e^-s  =>  dA/ds = e^-s / G'(A)
-    double G, dG;
-    n97_G_dG(Aa, G, dG);
-    const double dA_ds = exp(-s) / dG;
-    domc = do_dA * dA_ds;
-    dst = st > 0.0 ? (q * do_dA + o * dq_dA) / (2.0 * st) * dA_ds : 0.0;
-}
-
 // Forward of one scatter pair (the FP64 pair loop of the step kernel); returns the flags.
 __device__ int pair_forward(const StepArgs& A, const InterConst& ic, double vi[3], double vj[3], double wi, double wj,
                             int nmin, bool trip, uint4 r)
 {
     int flags = trip ? kFlagTriplet : 0;
-    const double ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
-    const double u2 = ux * ux + uy * uy + uz * uz;
     bool upd_i = true, upd_j = true;
     if (wi != wj) {
-        const bool moves = u23<double>(r.z) * fmax(wi, wj) < fmin(wi, wj);
+        const bool moves = u23_bits(r.z) * fmax(wi, wj) < fmin(wi, wj);
         if (wi > wj) upd_i = moves;
         else upd_j = moves;
     }
     if (upd_i) flags |= kFlagUpdI;
     if (upd_j) flags |= kFlagUpdJ;
-    if (u2 == 0.0) return flags;
+    const double wf = (wi > wj ? wi : wj) * (double)nmin;
+    double du[3];
+    if (!pair64(A.t64, A.method, (trip ? 0.5 : 1.0) * ic.kappa_mu2 * wf, vi, vj, r, du)) return flags;
     flags |= kFlagActive;
-    const double um = sqrt(u2);
-    const double wmax = wi > wj ? wi : wj;
-    double s = ic.kappa_mu2 * wmax * (double)nmin / (u2 * um);
-    if (trip) s *= 0.5;
-    double st, omc, dst, domc, sp, cp, d[3];
-    angle_and_derivative(A, s, u23<double>(r.x), u23<double>(r.w), st, omc, dst, domc);
-    sincospi(2.0 * u23<double>(r.y), &sp, &cp);
-    rotate<double>(ux, uy, uz, st, omc, cp, sp, d[0], d[1], d[2]);
     for (int k = 0; k < 3; ++k) {
-        if (upd_i) vi[k] += ic.mu_ma * d[k];
-        if (upd_j) vj[k] -= ic.mu_mb * d[k];
+        if (upd_i) vi[k] = fma(ic.mu_ma, du[k], vi[k]);
+        if (upd_j) vj[k] = fma(-ic.mu_mb, du[k], vj[k]);
     }
     return flags;
 }
@@ -235,29 +201,30 @@ __device__ void pair_reverse(const StepArgs& A, const InterConst& ic, double lnL
     if (gd[0] == 0.0 && gd[1] == 0.0 && gd[2] == 0.0) return;
     const double u[3] = {vi[0] - vj[0], vi[1] - vj[1], vi[2] - vj[2]};
     const double u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double um = sqrt(u2);
+    const double ru = rsqrt(u2), um = u2 * ru;
     const double wmax = wi > wj ? wi : wj;
-    double s = ic.kappa_mu2 * wmax * (double)nmin / (u2 * um);
+    double s = ic.kappa_mu2 * wmax * (double)nmin * (ru * ru * ru);
     if (flags & kFlagTriplet) s *= 0.5;
     double st, omc, dst, domc, sp, cp;
-    angle_and_derivative(A, s, u23<double>(r.x), u23<double>(r.w), st, omc, dst, domc);
-    sincospi(2.0 * u23<double>(r.y), &sp, &cp);
+    angle64<true>(A.t64, A.method, s, r, st, omc, dst, domc);
+    turn64(A.t64, r.y, cp, sp);
     // rotation du(u, st, omc) backwards
     double gst, gomc, gu[3];
-    const double uperp = sqrt(u[0] * u[0] + u[1] * u[1]);
+    const double up2 = u[0] * u[0] + u[1] * u[1];
     double gum;
-    if (uperp > 0.0) {
-        const double a = u[0] / uperp, b = u[1] / uperp;
+    if (up2 > 0.0) {
+        const double rp = rsqrt(up2), uperp = up2 * rp;
+        const double a = u[0] * rp, b = u[1] * rp;
         gst = gd[0] * (a * u[2] * cp - b * um * sp) + gd[1] * (b * u[2] * cp + a * um * sp) - gd[2] * uperp * cp;
         gomc = -(gd[0] * u[0] + gd[1] * u[1] + gd[2] * u[2]);
         const double ga = gd[0] * u[2] * st * cp + gd[1] * um * st * sp;
         const double gb = -gd[0] * um * st * sp + gd[1] * u[2] * st * cp;
         gum = -gd[0] * b * st * sp + gd[1] * a * st * sp;
         double gup = -gd[2] * st * cp;
-        gu[0] = -gd[0] * omc + ga / uperp;
-        gu[1] = -gd[1] * omc + gb / uperp;
+        gu[0] = -gd[0] * omc + ga * rp;
+        gu[1] = -gd[1] * omc + gb * rp;
         gu[2] = gd[0] * a * st * cp + gd[1] * b * st * cp - gd[2] * omc;
-        gup -= (ga * a + gb * b) / uperp;
+        gup -= (ga * a + gb * b) * rp;
         gu[0] += gup * a;
         gu[1] += gup * b;
     } else {
@@ -270,8 +237,8 @@ __device__ void pair_reverse(const StepArgs& A, const InterConst& ic, double lnL
     }
     // angle, then s = C w_max / um^3
     const double gs = gst * dst + gomc * domc;
-    gum += gs * (-3.0 * s / um);
-    for (int k = 0; k < 3; ++k) gu[k] += gum * u[k] / um;
+    gum = (gum - gs * 3.0 * s * ru) * ru;
+    for (int k = 0; k < 3; ++k) gu[k] += gum * u[k];
     const double gwmax = gs * s / wmax;
     if (wi > wj) gwi += gwmax;
     else gwj += gwmax;
@@ -296,37 +263,190 @@ __device__ __forceinline__ void st3(double* p, int n, int i, const double x[3])
 }
 
 // k-th TA77 pair (cell-local indices) with p mod N_min supplied (inter).
-__device__ __forceinline__ void pair_of(const Slab& sl, bool intra, int na, int nb, int a0, int b0, int p, int pm,
+__device__ __forceinline__ void pair_of(const int32_t* perm, bool intra, int na, int nb, int a0, int b0, int p, int pm,
                                         int& i, int& j, bool& trip)
 {
     trip = false;
     if (intra) {
         if (na & 1) {
             if (p < 3) {
-                i = sl.perm[a0 + p];
-                j = sl.perm[a0 + (p + 1) % 3];
+                i = perm[a0 + p];
+                j = perm[a0 + (p + 1) % 3];
                 trip = true;
                 return;
             }
-            i = sl.perm[a0 + 2 * p - 3];
-            j = sl.perm[a0 + 2 * p - 2];
+            i = perm[a0 + 2 * p - 3];
+            j = perm[a0 + 2 * p - 2];
             return;
         }
-        i = sl.perm[a0 + 2 * p];
-        j = sl.perm[a0 + 2 * p + 1];
+        i = perm[a0 + 2 * p];
+        j = perm[a0 + 2 * p + 1];
         return;
     }
     if (na >= nb) {
-        i = sl.perm[a0 + p];
-        j = sl.perm[b0 + pm];
+        i = perm[a0 + p];
+        j = perm[b0 + pm];
     } else {
-        i = sl.perm[a0 + pm];
-        j = sl.perm[b0 + p];
+        i = perm[a0 + pm];
+        j = perm[b0 + p];
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ AdjArgs G)
+// Energy pairs of one species forward (Algorithm 1, final loop), by one warp, 32 pairs of a pass at a time: caps fE K, a
+// prefix sum over them, capped pairs take their cap and the crossing pair the remainder of |D|. Every pair that
+// absorbed energy is taped from entry e0 on, in order; returns their number. D = 0: Delta E_s vanishes here (exactly,
+// or as rounding noise), so the step applies no pair; but it moves at first order with v and w, and then the first
+// pair of the order absorbs it as the crossing pair: that pair is taped with U = 0. done: D was absorbed.
+__device__ int energy_forward(const StepArgs& A, const Slab& sl, const Work& wk, int N, int s0, int ns, double msd,
+                              double D, int e0, bool& done)
 {
+    const int lane = threadIdx.x & 31;
+    const bool none = D == 0.0;
+    const double sgn = D > 0.0 ? 1.0 : -1.0;
+    double Dabs = fabs(D);
+    int used = 0;
+    done = none;
+    const int passes = none ? 1 : A.max_corr_passes;
+    bool stop = false;
+    for (int pass = 0; pass < passes && !stop; ++pass) {
+        const int o = pass & 1, np = (ns - o) / 2;
+        double carry = 0.0;
+        for (int base = 0; base < np && !stop; base += 32) {
+            const int m = base + lane;
+            int i = 0, j = 0;
+            double v1[3], v2[3], m1 = 1.0, m2 = 1.0, K = 0.0;
+            if (m < np) {
+                i = wk.rho[s0 + o + 2 * m];
+                j = wk.rho[s0 + o + 2 * m + 1];
+                ld3(wk.v, N, i, v1);
+                ld3(wk.v, N, j, v2);
+                m1 = msd * wk.w[i];
+                m2 = msd * wk.w[j];
+                K = pair_kecm<double, false>(A.c, m1, m2, v1, v2);
+            }
+            const bool ok = K > 0.0;
+            bool take;
+            double U = 0.0, capE = 0.0;
+            if (none) {
+                const unsigned b = __ballot_sync(0xffffffffu, ok);
+                take = ok && lane == __ffs(b) - 1;
+                stop = b != 0;
+            } else {
+                capE = ok ? A.fE * K : 0.0;
+                double inc = capE;
+#pragma unroll
+                for (int q = 1; q < 32; q <<= 1) {
+                    const double y = __shfl_up_sync(0xffffffffu, inc, q);
+                    if (lane >= q) inc += y;
+                }
+                double excl = __shfl_up_sync(0xffffffffu, inc, 1);
+                excl = (lane ? excl : 0.0) + carry;
+                take = ok && excl < Dabs;
+                const double rem = Dabs - excl;
+                U = sgn * (rem < capE ? rem : capE);
+                carry += __shfl_sync(0xffffffffu, inc, 31);
+                stop = done = carry >= Dabs;
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, take);
+            if (take) {
+                const int e = e0 + used + __popc(b & ((1u << lane) - 1u));
+                if (e < sl.E) {
+                    for (int k = 0; k < 3; ++k) {
+                        sl.ev[k * sl.E + e] = v1[k];
+                        sl.ev[(3 + k) * sl.E + e] = v2[k];
+                    }
+                    sl.ei[e] = i;
+                    sl.ej[e] = j;
+                    sl.eU[e] = U;
+                    sl.eK[e] = K;
+                    sl.ecap[e] = 2 * pass + (!none && fabs(U) == capE);
+                } else if (!none) {
+                    latch(A.status, kErrTooLarge);
+                }
+                if (!none) {
+                    energy_pair<double, false>(A.c, m1, m2, K, v1, v2, U);
+                    st3(wk.v, N, i, v1);
+                    st3(wk.v, N, j, v2);
+                }
+            }
+            used += __popc(b);
+            __syncwarp();
+        }
+        Dabs -= carry;
+    }
+    return used;
+}
+
+// The same pairs backwards, by one warp: from the last entry, up to 32 entries of one pass at a time (disjoint particles).
+// Adds to the gradients at the pairs' particles and weights; returns dL/dD of the species.
+__device__ double energy_reverse(const StepArgs& A, const Slab& sl, const Work& wk, int N, int e0, int cnt, double msd,
+                                 double D)
+{
+    const int lane = threadIdx.x & 31;
+    const double sgn = D > 0.0 ? 1.0 : -1.0;
+    double gUc = 0.0, gD = 0.0;
+    for (int left = cnt; left > 0;) {
+        const int k = e0 + left - 1 - lane;  // lane 0 takes the last entry
+        const int cap = lane < left ? sl.ecap[k] : -2;
+        const bool mine = (cap >> 1) == (__shfl_sync(0xffffffffu, cap, 0) >> 1);
+        const int n = __popc(__ballot_sync(0xffffffffu, mine));  // a pass's entries are consecutive
+        int i = 0, j = 0;
+        double vr[3], g1[3], g2[3], h[3], m1 = 1.0, m2 = 1.0, K = 1.0, x = 0.0, gg = 1.0, ggm1 = 0.0, g1vr = 0.0,
+                                                                  g2vr = 0.0, vr2 = 0.0;
+        if (mine) {
+            i = sl.ei[k];
+            j = sl.ej[k];
+            ld3(wk.v, N, i, g1);
+            ld3(wk.v, N, j, g2);
+            m1 = msd * wk.w[i];
+            m2 = msd * wk.w[j];
+            K = sl.eK[k];
+            x = sl.eU[k] / K;
+            gg = sqrt(1.0 - x);
+            const double rM = 1.0 / (m1 + m2);
+            for (int d = 0; d < 3; ++d) {
+                vr[d] = sl.ev[d * sl.E + k] - sl.ev[(3 + d) * sl.E + k];
+                h[d] = (m2 * g1[d] - m1 * g2[d]) * rM;
+                ggm1 += h[d] * vr[d];
+                g1vr += g1[d] * vr[d];
+                g2vr += g2[d] * vr[d];
+                vr2 += vr[d] * vr[d];
+            }
+        }
+        // the crossing pair: U = D - (earlier U); g - 1 depends on U and K. It is the last entry, if there is one.
+        const bool crossing = mine && !(cap & 1);
+        const double gU = crossing ? -ggm1 / (2.0 * gg * K) : 0.0;
+        if (left == cnt) {
+            gD = __shfl_sync(0xffffffffu, gU, 0);
+            gUc = gD;
+        }
+        if (mine) {
+            const double gm1 = -x / (1.0 + gg), rM = 1.0 / (m1 + m2);
+            const double gc1 = gm1 * g1vr, gc2 = -gm1 * g2vr;
+            // a capped pair has U = sign(D) fE K, so U/K is fixed; its K still feeds the crossing pair's U
+            const double gK = crossing ? -gU * x : -gUc * sgn * A.fE;
+            const double mu = m1 * m2 * rM, gmu = gK * 0.5 * vr2, rM2 = rM * rM;
+            const double gm1m = (gmu * m2 - gc1 + gc2) * m2 * rM2;
+            const double gm2m = (gmu * m1 + gc1 - gc2) * m1 * rM2;
+            wk.gwl[i] += msd * gm1m;
+            wk.gwl[j] += msd * gm2m;
+            for (int d = 0; d < 3; ++d) {
+                const double gv = gm1 * h[d] + gK * mu * vr[d];
+                g1[d] += gv;
+                g2[d] -= gv;
+            }
+            st3(wk.v, N, i, g1);
+            st3(wk.v, N, j, g2);
+        }
+        left -= n;
+        __syncwarp();
+    }
+    return gD;
+}
+
+__global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __grid_constant__ AdjArgs G)
+{
+    extern __shared__ __align__(16) char dyn[];
     __shared__ AdjShared sh;
     const StepArgs& A = G.a;
     const InterConst& ic = A.ic[0];
@@ -337,9 +457,11 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
     const double* gvy = reinterpret_cast<const double*>(A.vy);
     const double* gvz = reinterpret_cast<const double*>(A.vz);
     const uint32_t ictr = (uint32_t)A.inter_base;
+    const bool keep = G.gx || G.tape == 1;  // a forward that is neither reversed nor recorded needs no tape
     for (int c = blockIdx.x; c < A.n_cells; c += gridDim.x) {
         const Slab sl = make_slab(G.slab + (size_t)(G.tape ? c : (int)blockIdx.x) * (size_t)G.slab_stride, G.max_cell,
                                   G.max_epairs);
+        const Work wk = make_work(G.on_chip ? dyn : sl.work, G.max_cell);
         const int64_t cs = A.offsets[(int64_t)c * S];
         const int n = (int)(A.offsets[(int64_t)(c + 1) * S] - cs);
         const int N = sl.n;
@@ -349,12 +471,12 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
         }
         if ((int)threadIdx.x <= S) sh.off[threadIdx.x] = (int)(A.offsets[(int64_t)c * S + threadIdx.x] - cs);
         for (int i = threadIdx.x; i < n; i += kThreads) {
+            wk.w[i] = wg[cs + i];
             if (G.tape != 2) {  // a replaying call finds the state before the interaction in the tape
                 const double x[3] = {gvx[cs + i], gvy[cs + i], gvz[cs + i]};
-                st3(sl.v, N, i, x);
+                st3(wk.v, N, i, x);
                 st3(sl.vb, N, i, x);
             }
-            sl.gwl[i] = 0.0;
         }
         __syncthreads();
         const int a0 = sh.off[ic.a], na = sh.off[ic.a + 1] - a0;
@@ -383,16 +505,8 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
             }
             __syncthreads();
         } else if (active) {
-            // ---- forward: permutations (sorted Philox keys)
-            for (int side = 0; side < nside; ++side) {
-                const int s0 = side ? b0 : a0, ns = side ? nb : na;
-                for (int q = threadIdx.x; q < ns; q += kThreads)
-                    sl.keys[s0 + q] = perm_key(A.rng, (uint32_t)c, ictr, (uint32_t)side, (uint32_t)q);
-                __syncthreads();
-                block_sort_u64(sl.keys + s0, ns);
-                for (int q = threadIdx.x; q < ns; q += kThreads) sl.perm[s0 + q] = s0 + (int)(sl.keys[s0 + q] & kPermMask);
-                __syncthreads();
-            }
+            // ---- forward: permutations
+            cta_permutations(A.rng, A.rng.step, wk.keys, wk.cnt, wk.perm, sh.iscan, c, ictr, nside, a0, na, b0, nb);
             // ---- forward: scatter pairs in round order, inputs taped
             const int npairs = intra ? ((na & 1) ? (na + 3) / 2 : na / 2) : (na > nb ? na : nb);
             const int nmin = intra ? na - 1 : (na < nb ? na : nb);
@@ -404,56 +518,67 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                 while (p < r1) {
                     int i, j;
                     bool trip;
-                    pair_of(sl, intra, na, nb, a0, b0, p, p - r0, i, j, trip);
+                    pair_of(wk.perm, intra, na, nb, a0, b0, p, p - r0, i, j, trip);
                     double vi[3], vj[3];
-                    ld3(sl.v, N, i, vi);
-                    ld3(sl.v, N, j, vj);
-                    for (int k = 0; k < 3; ++k) {
-                        sl.pv[k * N + p] = vi[k];
-                        sl.pv[(3 + k) * N + p] = vj[k];
+                    ld3(wk.v, N, i, vi);
+                    ld3(wk.v, N, j, vj);
+                    if (keep) {
+                        for (int k = 0; k < 3; ++k) {
+                            sl.pv[k * N + p] = vi[k];
+                            sl.pv[(3 + k) * N + p] = vj[k];
+                        }
+                        sl.pi[p] = i;
+                        sl.pj[p] = j;
                     }
                     const uint4 rr = draw(A.rng, (uint32_t)p, (uint32_t)c, ictr, kTagScat);
-                    sl.pf[p] = pair_forward(A, ic, vi, vj, wg[cs + i], wg[cs + j], nmin, trip, rr);
-                    sl.pi[p] = i;
-                    sl.pj[p] = j;
-                    st3(sl.v, N, i, vi);
-                    st3(sl.v, N, j, vj);
+                    const int flags = pair_forward(A, ic, vi, vj, wk.w[i], wk.w[j], nmin, trip, rr);
+                    if (keep) sl.pf[p] = flags;
+                    st3(wk.v, N, i, vi);
+                    st3(wk.v, N, j, vj);
                     p = (p + 1 < lead) ? p + 1 : (p < lead ? lead + (int)threadIdx.x : p + kThreads);
                 }
                 __syncthreads();
             }
-            for (int i = threadIdx.x; i < n; i += kThreads) {
-                double x[3];
-                ld3(sl.v, N, i, x);
-                st3(sl.vp, N, i, x);
+            if (keep) {
+                for (int i = threadIdx.x; i < n; i += kThreads) {
+                    double x[3];
+                    ld3(wk.v, N, i, x);
+                    st3(sl.vp, N, i, x);
+                }
             }
-            __syncthreads();
             // ---- forward: moment correction
             if (A.correct) {
+                // the sums and coefficients of the step kernel, term for term and in its order
                 const double ms[2] = {A.m[ic.a], A.m[ic.b]};
                 {
-                    Acc<double> acc[8];
-                    for (int k = 0; k < 8; ++k) acc[k] = Acc<double>::zero();
+                    Acc<double> mom[6], wsum[4];
+                    for (int k = 0; k < 6; ++k) mom[k] = Acc<double>::zero();
+                    for (int k = 0; k < 4; ++k) wsum[k] = Acc<double>::zero();
                     for (int side = 0; side < nside; ++side) {
                         const int s0 = side ? b0 : a0, ns = side ? nb : na;
                         for (int q = threadIdx.x; q < ns; q += kThreads) {
                             const int i = s0 + q;
-                            const double w = wg[cs + i], mp = ms[side] * w;
-                            for (int k = 0; k < 3; ++k) acc[k].add(mp * (sl.v[k * N + i] - sl.vb[k * N + i]));
-                            acc[3].add(mp * w);
-                            acc[4 + side].add(w);
+                            const double w = wk.w[i];
+                            for (int k = 0; k < 3; ++k) mom[3 * side + k].add(w * (wk.v[k * N + i] - sl.vb[k * N + i]));
+                            wsum[2 * side].add(w);
+                            wsum[2 * side + 1].add(w * w);
                         }
                     }
-                    block_sum<double, 8>(acc, accp(sh.red_raw), accp(sh.red));
+                    block_sum<double, 4>(wsum, accp(sh.red_raw), accp(sh.red));
                     if (threadIdx.x == 0) {
                         const Acc<double>* r = accp(sh.red);
-                        sh.Sw = r[3].x;
+                        sh.W1[0] = r[0].x;
+                        sh.W1[1] = r[2].x;
+                        sh.Sw = ms[0] * r[1].x + (intra ? 0.0 : ms[1] * r[3].x);
+                    }
+                    __syncthreads();
+                    block_sum<double, 6>(mom, accp(sh.red_raw), accp(sh.red));
+                    if (threadIdx.x == 0) {
+                        const Acc<double>* r = accp(sh.red);
                         for (int k = 0; k < 3; ++k) {
-                            sh.S[k] = r[k].x;
-                            sh.B[k] = r[k].x / r[3].x;
+                            sh.S[k] = ms[0] * r[k].x + (intra ? 0.0 : ms[1] * r[3 + k].x);
+                            sh.B[k] = sh.S[k] / sh.Sw;
                         }
-                        sh.W1[0] = r[4].x;
-                        sh.W1[1] = r[5].x;
                     }
                     __syncthreads();
                 }
@@ -464,26 +589,26 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                         const int s0 = side ? b0 : a0, ns = side ? nb : na;
                         for (int q = threadIdx.x; q < ns; q += kThreads) {
                             const int i = s0 + q;
-                            const double w = wg[cs + i], mp = ms[side] * w;
+                            const double w = wk.w[i];
                             double dd = 0.0, v2 = 0.0;
                             for (int k = 0; k < 3; ++k) {
-                                const double x = sl.v[k * N + i] - sh.B[k] * w, y = sl.vb[k * N + i];
-                                sl.v[k * N + i] = x;
-                                sl.vm[k * N + i] = x;
+                                const double x = wk.v[k * N + i] - sh.B[k] * w, y = sl.vb[k * N + i];
+                                wk.v[k * N + i] = x;
+                                if (keep) sl.vm[k * N + i] = x;
                                 dd += (x - y) * (x + y);
                                 v2 += x * x;
                             }
-                            acc[0].add(0.5 * mp * dd);
-                            acc[1 + side].add(0.5 * mp * v2);
+                            acc[2 * side].add(0.5 * w * dd);
+                            acc[2 * side + 1].add(0.5 * w * v2);
                         }
                     }
                     block_sum<double, 4>(acc, accp(sh.red_raw), accp(sh.red));
                     if (threadIdx.x == 0) {
                         const Acc<double>* r = accp(sh.red);
-                        const double dE = r[0].x;
+                        const double dE = ms[0] * r[0].x + (intra ? 0.0 : ms[1] * r[2].x);
                         sh.dE = dE;
-                        sh.Es[0] = r[1].x;
-                        sh.Es[1] = r[2].x;
+                        sh.Es[0] = ms[0] * r[1].x;
+                        sh.Es[1] = intra ? 0.0 : ms[1] * r[3].x;
                         double D0 = dE, D1 = 0.0;
                         int fail = 0;
                         if (!intra) {
@@ -511,107 +636,58 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                         sh.zeroed[1] = fabs(D1) <= 0x1p-47 * (intra ? 0.0 : sh.Es[1]);
                         sh.D[0] = sh.zeroed[0] ? 0.0 : D0;
                         sh.D[1] = sh.zeroed[1] ? 0.0 : D1;
-                        sh.fail = fail;
+                        sh.fail = sh.fail0 = fail;
                     }
                     __syncthreads();
                 }
                 // energy-pair order of each side: the permutation, stably sorted by descending weight (optional)
                 for (int side = 0; side < nside; ++side) {
                     const int s0 = side ? b0 : a0, ns = side ? nb : na;
-                    if (A.sort_by_weight) {
+                    if (!A.sort_by_weight) {
+                        for (int r = threadIdx.x; r < ns; r += kThreads) wk.rho[s0 + r] = wk.perm[s0 + r];
+                        continue;
+                    }
+                    for (int r = threadIdx.x; r < ns; r += kThreads)
+                        wk.keys[s0 + r] = weight_key(wk.w[wk.perm[s0 + r]], (uint32_t)r);
+                }
+                __syncthreads();
+                if (A.sort_by_weight) {
+                    for (int side = 0; side < nside; ++side) block_sort_u64(wk.keys + (side ? b0 : a0), side ? nb : na);
+                    for (int side = 0; side < nside; ++side) {
+                        const int s0 = side ? b0 : a0, ns = side ? nb : na;
                         for (int r = threadIdx.x; r < ns; r += kThreads)
-                            sl.keys[s0 + r] = weight_key(wg[cs + sl.perm[s0 + r]], (uint32_t)r);
-                        __syncthreads();
-                        block_sort_u64(sl.keys + s0, ns);
-                        for (int r = threadIdx.x; r < ns; r += kThreads)
-                            sl.rho[s0 + r] = sl.perm[s0 + (int)(sl.keys[s0 + r] & kPermMask)];
-                    } else {
-                        for (int r = threadIdx.x; r < ns; r += kThreads) sl.rho[s0 + r] = sl.perm[s0 + r];
+                            wk.rho[s0 + r] = wk.perm[s0 + (int)(wk.keys[s0 + r] & kPermMask)];
                     }
                     __syncthreads();
                 }
-                // energy loops, in order, by one thread (the tape records every pair that absorbed energy)
-                if (threadIdx.x == 0) {
-                    int e = 0;
-                    for (int side = 0; side < nside; ++side) {
-                        sh.e0[side] = e;
-                        sh.ne[side] = 0;
-                        if (sh.fail) continue;
-                        const int s0 = side ? b0 : a0, ns = side ? nb : na;
-                        const double msd = ms[side];
-                        if (sh.D[side] == 0.0) {
-                            // Delta E_s vanishes here (exactly, or as rounding noise), so the step applies no energy
-                            // pair; but it moves at first order with v and w, and then the first pair of the order
-                            // absorbs it as the crossing pair. Tape that pair with U = 0 (no change in the forward).
-                            for (int t = 0; t + 1 < ns; t += 2) {
-                                const int i = sl.rho[s0 + t], j = sl.rho[s0 + t + 1];
-                                double v1[3], v2[3];
-                                ld3(sl.v, N, i, v1);
-                                ld3(sl.v, N, j, v2);
-                                const double K =
-                                    pair_kecm<double, false>(A.c, msd * wg[cs + i], msd * wg[cs + j], v1, v2);
-                                if (!(K > 0.0)) continue;
-                                if (e < sl.E) {
-                                    for (int k = 0; k < 3; ++k) {
-                                        sl.ev[k * sl.E + e] = v1[k];
-                                        sl.ev[(3 + k) * sl.E + e] = v2[k];
-                                    }
-                                    sl.ei[e] = i;
-                                    sl.ej[e] = j;
-                                    sl.eU[e] = 0.0;
-                                    sl.eK[e] = K;
-                                    sl.ecap[e] = 0;
-                                    ++e;
-                                    ++sh.ne[side];
-                                }
-                                break;
-                            }
-                            continue;
+                // energy pairs, one warp per side: at once under the rollback policy (a failure undoes both), else
+                // species b only if species a did not fail. Side b's tape starts after the most that side a can need.
+                const int turns = A.fail_policy == 0 ? 1 : nside;
+                const int passes = A.max_corr_passes > 0 ? A.max_corr_passes : 1;
+                for (int turn = 0; turn < turns; ++turn) {
+                    const int side = threadIdx.x >> 5;
+                    if (side < nside && (turns == 1 || side == turn)) {
+                        const int e0 = side ? passes * (na / 2) : 0;
+                        int used = 0;
+                        bool done = true;
+                        if (!(turns == 1 ? sh.fail0 : sh.fail))
+                            used = energy_forward(A, sl, wk, N, side ? b0 : a0, side ? nb : na, ms[side], sh.D[side], e0,
+                                                  done);
+                        if ((threadIdx.x & 31) == 0) {
+                            sh.e0[side] = e0;
+                            sh.ne[side] = used;
+                            if (!done) sh.fail = 1;
                         }
-                        double D = sh.D[side];
-                        for (int pass = 0; pass < A.max_corr_passes && D != 0.0; ++pass) {
-                            for (int t = pass & 1; t + 1 < ns && D != 0.0; t += 2) {
-                                const int i = sl.rho[s0 + t], j = sl.rho[s0 + t + 1];
-                                double v1[3], v2[3];
-                                ld3(sl.v, N, i, v1);
-                                ld3(sl.v, N, j, v2);
-                                const double m1 = msd * wg[cs + i], m2 = msd * wg[cs + j];
-                                const double K = pair_kecm<double, false>(A.c, m1, m2, v1, v2);
-                                if (!(K > 0.0)) continue;
-                                const double capE = A.fE * K;
-                                const double U = (D > 0.0 ? 1.0 : -1.0) * (fabs(D) < capE ? fabs(D) : capE);
-                                if (e < sl.E) {
-                                    for (int k = 0; k < 3; ++k) {
-                                        sl.ev[k * sl.E + e] = v1[k];
-                                        sl.ev[(3 + k) * sl.E + e] = v2[k];
-                                    }
-                                    sl.ei[e] = i;
-                                    sl.ej[e] = j;
-                                    sl.eU[e] = U;
-                                    sl.eK[e] = K;
-                                    sl.ecap[e] = !(fabs(D) < capE);
-                                } else {
-                                    latch(A.status, kErrTooLarge);
-                                }
-                                ++e;
-                                ++sh.ne[side];
-                                energy_pair<double, false>(A.c, m1, m2, K, v1, v2, U);
-                                st3(sl.v, N, i, v1);
-                                st3(sl.v, N, j, v2);
-                                D -= U;
-                            }
-                        }
-                        if (D != 0.0) sh.fail = 1;
                     }
+                    __syncthreads();
                 }
-                __syncthreads();
                 if (sh.fail && A.fail_policy == 0) {
                     for (int side = 0; side < nside; ++side) {
                         const int s0 = side ? b0 : a0, ns = side ? nb : na;
                         for (int q = threadIdx.x; q < ns; q += kThreads) {
                             double x[3];
                             ld3(sl.vb, N, s0 + q, x);
-                            st3(sl.v, N, s0 + q, x);
+                            st3(wk.v, N, s0 + q, x);
                         }
                     }
                 }
@@ -640,81 +716,35 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
         // ---- forward output
         if (G.ox) {
             for (int i = threadIdx.x; i < n; i += kThreads) {
-                G.ox[cs + i] = sl.v[i];
-                G.oy[cs + i] = sl.v[N + i];
-                G.oz[cs + i] = sl.v[2 * N + i];
+                G.ox[cs + i] = wk.v[i];
+                G.oy[cs + i] = wk.v[N + i];
+                G.oz[cs + i] = wk.v[2 * N + i];
             }
         }
         // ---- reverse
         if (G.gx && active && !(A.correct && sh.fail && A.fail_policy == 0)) {
+            __syncthreads();  // the forward's working arrays are read no more
             for (int i = threadIdx.x; i < n; i += kThreads) {
                 const double x[3] = {G.gx[cs + i], G.gy[cs + i], G.gz[cs + i]};
-                st3(sl.g, N, i, x);
+                st3(wk.v, N, i, x);
                 const double z[3] = {0.0, 0.0, 0.0};
-                st3(sl.gb, N, i, z);
+                st3(wk.gb, N, i, z);
+                wk.gwl[i] = 0.0;
             }
             __syncthreads();
             if (A.correct) {
                 const double ms[2] = {A.m[ic.a], A.m[ic.b]};
-                // energy pairs backwards (one thread; each side's pairs in reverse order)
-                if (threadIdx.x == 0) {
-                    for (int side = nside - 1; side >= 0; --side) {
-                        sh.gD[side] = 0.0;
+                // energy pairs backwards, one warp per side (their particles are disjoint)
+                {
+                    const int side = threadIdx.x >> 5;
+                    if (side < nside) {
                         const int cnt = sh.ne[side] < sl.E - sh.e0[side] ? sh.ne[side] : sl.E - sh.e0[side];
-                        if (cnt <= 0) continue;
-                        const double msd = ms[side];
-                        const double sgn = sh.D[side] > 0.0 ? 1.0 : -1.0;
-                        double gUc = 0.0;
-                        for (int k = sh.e0[side] + cnt - 1; k >= sh.e0[side]; --k) {
-                            const int i = sl.ei[k], j = sl.ej[k];
-                            double v1[3], v2[3], g1[3], g2[3], vr[3];
-                            for (int d = 0; d < 3; ++d) {
-                                v1[d] = sl.ev[d * sl.E + k];
-                                v2[d] = sl.ev[(3 + d) * sl.E + k];
-                                vr[d] = v1[d] - v2[d];
-                            }
-                            ld3(sl.g, N, i, g1);
-                            ld3(sl.g, N, j, g2);
-                            const double m1 = msd * wg[cs + i], m2 = msd * wg[cs + j], M = m1 + m2;
-                            const double c1 = m2 / M, c2 = m1 / M, mu = m1 * m2 / M;
-                            const double U = sl.eU[k], K = sl.eK[k];
-                            const double x = U / K, gg = sqrt(1.0 - x), gm1 = -x / (1.0 + gg);
-                            double h[3], ggm1 = 0.0, g1vr = 0.0, g2vr = 0.0, vr2 = 0.0;
-                            for (int d = 0; d < 3; ++d) {
-                                h[d] = c1 * g1[d] - c2 * g2[d];
-                                ggm1 += h[d] * vr[d];
-                                g1vr += g1[d] * vr[d];
-                                g2vr += g2[d] * vr[d];
-                                vr2 += vr[d] * vr[d];
-                            }
-                            double gvr[3] = {gm1 * h[0], gm1 * h[1], gm1 * h[2]};
-                            const double gc1 = gm1 * g1vr, gc2 = -gm1 * g2vr;
-                            double gK;
-                            if (!sl.ecap[k]) {
-                                // crossing pair: U = D - (earlier U); g - 1 depends on U and K
-                                const double gU = -ggm1 / (2.0 * gg * K);
-                                gK = ggm1 * x / (2.0 * gg * K);
-                                gUc = gU;
-                                sh.gD[side] += gU;
-                            } else {
-                                // capped pair: U = sign(D) fE K, so U/K is fixed; K still feeds the crossing U
-                                gK = -gUc * sgn * A.fE;
-                            }
-                            for (int d = 0; d < 3; ++d) gvr[d] += gK * mu * vr[d];
-                            const double gmu = gK * 0.5 * vr2;
-                            const double M2 = M * M;
-                            const double gm1m = gmu * m2 * m2 / M2 - gc1 * m2 / M2 + gc2 * m2 / M2;
-                            const double gm2m = gmu * m1 * m1 / M2 + gc1 * m1 / M2 - gc2 * m1 / M2;
-                            sl.gwl[i] += msd * gm1m;
-                            sl.gwl[j] += msd * gm2m;
-                            for (int d = 0; d < 3; ++d) {
-                                g1[d] += gvr[d];
-                                g2[d] -= gvr[d];
-                            }
-                            st3(sl.g, N, i, g1);
-                            st3(sl.g, N, j, g2);
-                        }
+                        const double gD = energy_reverse(A, sl, wk, N, sh.e0[side], cnt, ms[side], sh.D[side]);
+                        if ((threadIdx.x & 31) == 0) sh.gD[side] = gD;
                     }
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) {
                     // Delta E split backwards
                     double gdE = 0.0, gE0 = 0.0, gE1 = 0.0, gW0 = 0.0, gW1 = 0.0;
                     const double g0 = sh.gD[0];
@@ -759,16 +789,16 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                         const double msd = ms[side];
                         for (int q = threadIdx.x; q < ns; q += kThreads) {
                             const int i = s0 + q;
-                            const double w = wg[cs + i], mp = msd * w;
+                            const double w = wk.w[i], mp = msd * w;
                             double gm[3], xm[3], xb[3];
-                            ld3(sl.g, N, i, gm);
+                            ld3(wk.v, N, i, gm);
                             ld3(sl.vm, N, i, xm);
                             ld3(sl.vb, N, i, xb);
                             const double gE = sh.gEs[side];
                             double xm2 = 0.0, xb2 = 0.0, gwd = 0.0;
                             for (int d = 0; d < 3; ++d) {
                                 gm[d] += (sh.gdE + gE) * mp * xm[d];
-                                sl.gb[d * N + i] -= sh.gdE * mp * xb[d];
+                                wk.gb[d * N + i] -= sh.gdE * mp * xb[d];
                                 xm2 += xm[d] * xm[d];
                                 xb2 += xb[d] * xb[d];
                             }
@@ -777,8 +807,8 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                                 acc[d].add(-w * gm[d]);
                                 gwd -= sh.B[d] * gm[d];
                             }
-                            sl.gwl[i] += gwd;
-                            st3(sl.g, N, i, gm);
+                            wk.gwl[i] += gwd;
+                            st3(wk.v, N, i, gm);
                         }
                     }
                     block_sum<double, 3>(acc, accp(sh.red_raw), accp(sh.red));
@@ -799,14 +829,14 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                     const double msd = ms[side];
                     for (int q = threadIdx.x; q < ns; q += kThreads) {
                         const int i = s0 + q;
-                        const double w = wg[cs + i], mp = msd * w;
+                        const double w = wk.w[i], mp = msd * w;
                         double gwd = 2.0 * mp * sh.gSw;
                         for (int d = 0; d < 3; ++d) {
-                            sl.g[d * N + i] += mp * sh.gS[d];
-                            sl.gb[d * N + i] -= mp * sh.gS[d];
+                            wk.v[d * N + i] += mp * sh.gS[d];
+                            wk.gb[d * N + i] -= mp * sh.gS[d];
                             gwd += msd * (sl.vp[d * N + i] - sl.vb[d * N + i]) * sh.gS[d];
                         }
-                        sl.gwl[i] += gwd;
+                        wk.gwl[i] += gwd;
                     }
                 }
                 __syncthreads();
@@ -831,16 +861,16 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                             vi[k] = sl.pv[k * N + p];
                             vj[k] = sl.pv[(3 + k) * N + p];
                         }
-                        ld3(sl.g, N, i, g1);
-                        ld3(sl.g, N, j, g2);
+                        ld3(wk.v, N, i, g1);
+                        ld3(wk.v, N, j, g2);
                         const uint4 r = draw(A.rng, (uint32_t)p, (uint32_t)c, ictr, kTagScat);
                         double gwi = 0.0, gwj = 0.0;
-                        pair_reverse(A, ic, G.lnL, vi, vj, wg[cs + i], wg[cs + j], nmin, sl.pf[p], r, g1, g2, gwi, gwj,
+                        pair_reverse(A, ic, G.lnL, vi, vj, wk.w[i], wk.w[j], nmin, sl.pf[p], r, g1, g2, gwi, gwj,
                                      glnl);
-                        st3(sl.g, N, i, g1);
-                        st3(sl.g, N, j, g2);
-                        sl.gwl[i] += gwi;
-                        sl.gwl[j] += gwj;
+                        st3(wk.v, N, i, g1);
+                        st3(wk.v, N, j, g2);
+                        wk.gwl[i] += gwi;
+                        wk.gwl[j] += gwj;
                     };
                     if (lead && threadIdx.x == 0)
                         for (int p = lead - 1; p >= 0; --p) undo(p);
@@ -853,10 +883,10 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
                 const int s0 = side ? b0 : a0, ns = side ? nb : na;
                 for (int q = threadIdx.x; q < ns; q += kThreads) {
                     const int i = s0 + q;
-                    G.gx[cs + i] = sl.g[i] + sl.gb[i];
-                    G.gy[cs + i] = sl.g[N + i] + sl.gb[N + i];
-                    G.gz[cs + i] = sl.g[2 * N + i] + sl.gb[2 * N + i];
-                    if (G.gw) G.gw[cs + i] += sl.gwl[i];
+                    G.gx[cs + i] = wk.v[i] + wk.gb[i];
+                    G.gy[cs + i] = wk.v[N + i] + wk.gb[N + i];
+                    G.gz[cs + i] = wk.v[2 * N + i] + wk.gb[2 * N + i];
+                    if (G.gw) G.gw[cs + i] += wk.gwl[i];
                 }
             }
             {
@@ -871,11 +901,24 @@ __global__ void __launch_bounds__(kThreads) k_adjoint(const __grid_constant__ Ad
 
 }  // namespace
 
-size_t adjoint_slab_bytes(int32_t max_cell, int32_t max_epairs) { return (slab_bytes(max_cell, max_epairs) + 255) & ~(size_t)255; }
+size_t adjoint_slab_bytes(int32_t max_cell, int32_t max_epairs, bool on_chip)
+{
+    return (slab_bytes(max_cell, max_epairs, on_chip) + 255) & ~(size_t)255;
+}
+
+size_t adjoint_work_bytes(int32_t max_cell) { return kWorkBytesPerParticle * (size_t)max_cell; }
+
+size_t adjoint_static_smem()
+{
+    cudaFuncAttributes fa;
+    return cudaFuncGetAttributes(&fa, k_adjoint) == cudaSuccess ? fa.sharedSizeBytes : 16384;
+}
+
+int adjoint_ctas_per_sm() { return kAdjCtasPerSm; }
 
 cudaError_t launch_adjoint(const StepArgs& a, double lnL, double* ox, double* oy, double* oz, double* gx, double* gy,
                            double* gz, double* gw, double* glnL, char* slab, int32_t max_cell, int32_t max_epairs,
-                           int32_t tape, int grid, cudaStream_t st)
+                           int32_t tape, bool on_chip, int grid, cudaStream_t st)
 {
     AdjArgs g;
     g.a = a;
@@ -889,11 +932,15 @@ cudaError_t launch_adjoint(const StepArgs& a, double lnL, double* ox, double* oy
     g.gw = gw;
     g.glnL = glnL;
     g.slab = slab;
-    g.slab_stride = (int64_t)adjoint_slab_bytes(max_cell, max_epairs);
+    g.slab_stride = (int64_t)adjoint_slab_bytes(max_cell, max_epairs, on_chip);
     g.max_cell = max_cell;
     g.max_epairs = max_epairs;
     g.tape = tape;
-    k_adjoint<<<grid, kThreads, 0, st>>>(g);
+    g.on_chip = on_chip;
+    const size_t smem = on_chip ? adjoint_work_bytes(max_cell) : 0;
+    const cudaError_t e = cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_adjoint<<<grid, kThreads, smem, st>>>(g);
     return cudaGetLastError();
 }
 

@@ -16,10 +16,14 @@
 //
 // FP64 path: everything in double. Mixed path: float velocities and kinematics, float-float accumulation of the
 // per-cell sums, FP64 only for the per-cell coefficients (B, Delta E, its split) computed by one thread.
-#include "mcc_kernels.h"
+#include "mcc_pair64.cuh"
+#include "mcc_perm.cuh"
 
+// Resident CTAs per SM the registers are bounded for: four (128 registers, nothing spilled). With the FP64 pipe the limit,
+// more warps gain nothing and spills cost: FP64 three-species step of 4096 cells 2.38 / 2.41 / 2.39 ms and relativistic beam of
+// 2048 cells 2.21 / 2.31 / 3.17 ms at 4 / 5 / 6; 256-thread CTAs at three per SM 2.84 / 2.63 ms.
 #ifndef MCC_MIN_BLOCKS
-#define MCC_MIN_BLOCKS 6
+#define MCC_MIN_BLOCKS 4
 #endif
 
 namespace mcc {
@@ -146,9 +150,6 @@ template <>
 __device__ __forceinline__ double pick<double>(double d, float) { return d; }
 template <>
 __device__ __forceinline__ float pick<float>(double, float f) { return f; }
-
-__device__ __forceinline__ void n97_tab(const StepArgs& A, N97Tab<double>& t) { t = {A.n97_f, A.n97_dh}; }
-__device__ __forceinline__ void n97_tab(const StepArgs& A, N97Tab<float>& t) { t = {A.n97_f32, A.n97_dh32}; }
 
 struct Shared {
     int off[kMaxSpecies + 1];
@@ -278,92 +279,6 @@ __device__ __forceinline__ void partition_coef(const StepArgs& A, const InterCon
     sh.fail = fail;
 }
 
-// Random permutations of the interaction's one or two species segments: local indices ordered by their 64-bit
-// Philox keys (44 random bits above the index). The random bits are uniform, so a counting sort on their top
-// log2(B) bits (B = next power of two >= n buckets) already places almost every key; each bucket holding several
-// keys is finished by an insertion sort on the full key. The result is the sort by full key (keys are distinct).
-// One Philox block gives the keys of two consecutive indices, so each thread draws for a pair. The permutation is
-// stored as cell-local particle indices (segment start included).
-// Scratch: the pre-interaction copy vb (unused until after the permutations) holds the bucket counters.
-template <class V>
-__device__ void permutations(const StepArgs& A, const Tile<V>& t, Shared& sh, int c, uint32_t ictr, int nside,
-                             int a0, int na, int b0, int nb)
-{
-    uint32_t* cnt = t.cnt;
-    const int s0v[2] = {a0, b0}, nv[2] = {na, nb};
-    int lgB[2] = {0, 0}, Bv[2] = {0, 0};
-    for (int side = 0; side < nside; ++side) {
-        while ((1 << lgB[side]) < nv[side]) ++lgB[side];
-        Bv[side] = 1 << lgB[side];
-    }
-    const int base1 = Bv[0];
-    const int L = Bv[0] + (nside > 1 ? Bv[1] : 0);
-    for (int side = 0; side < nside; ++side) {
-        const int s0 = s0v[side], n = nv[side];
-        const uint32_t tag = side ? kTagPermB : kTagPermA;
-        for (int h = threadIdx.x; 2 * h < n; h += kThreads) {
-            const uint4 r = draw_at(A.rng, sh.step, (uint32_t)h, (uint32_t)c, ictr, tag);
-            t.keys[s0 + 2 * h] = ((((uint64_t)r.x << 32) | r.y) & ~kPermMask) | (uint64_t)(2 * h);
-            if (2 * h + 1 < n) t.keys[s0 + 2 * h + 1] = ((((uint64_t)r.z << 32) | r.w) & ~kPermMask) | (uint64_t)(2 * h + 1);
-        }
-    }
-    for (int b = threadIdx.x; b < L; b += kThreads) cnt[b] = 0;
-    __syncthreads();
-    for (int side = 0; side < nside; ++side) {
-        const int base = side ? base1 : 0;
-        for (int q = threadIdx.x; q < nv[side]; q += kThreads) {
-            const uint64_t k = t.keys[s0v[side] + q];
-            const int b = lgB[side] ? (int)(k >> (64 - lgB[side])) : 0;
-            atomicAdd(&cnt[base + b], 1u);
-        }
-    }
-    __syncthreads();
-    // exclusive scan over both sides' buckets (side 1's positions are offset by na)
-    {
-        const int chunk = (L + kThreads - 1) / kThreads;
-        const int lo = threadIdx.x * chunk, hi = min(L, lo + chunk);
-        int local = 0;
-        for (int b = lo; b < hi; ++b) local += (int)cnt[b];
-        int total;
-        int run = block_exclusive_scan<int>(local, sh.iscan, total);
-        for (int b = lo; b < hi; ++b) {
-            const int x = (int)cnt[b];
-            cnt[b] = (uint32_t)run;
-            run += x;
-        }
-    }
-    __syncthreads();
-    for (int side = 0; side < nside; ++side) {
-        const int base = side ? base1 : 0, off = side ? na : 0, s0 = s0v[side];
-        for (int q = threadIdx.x; q < nv[side]; q += kThreads) {
-            const uint64_t k = t.keys[s0 + q];
-            const int b = lgB[side] ? (int)(k >> (64 - lgB[side])) : 0;
-            const int pos = (int)atomicAdd(&cnt[base + b], 1u) - off;
-            t.perm[s0 + pos] = s0 + q;
-        }
-    }
-    __syncthreads();
-    // cnt[b] now holds the end of bucket b: finish buckets with several keys
-    for (int side = 0; side < nside; ++side) {
-        const int base = side ? base1 : 0, off = side ? na : 0, s0 = s0v[side];
-        for (int b = threadIdx.x; b < Bv[side]; b += kThreads) {
-            const int end = (int)cnt[base + b] - off;
-            const int start = b ? (int)cnt[base + b - 1] - off : 0;
-            for (int x = start + 1; x < end; ++x) {
-                const int v = t.perm[s0 + x];
-                const uint64_t kv = t.keys[v];
-                int y = x - 1;
-                while (y >= start && t.keys[t.perm[s0 + y]] > kv) {
-                    t.perm[s0 + y + 1] = t.perm[s0 + y];
-                    --y;
-                }
-                t.perm[s0 + y + 1] = v;
-            }
-        }
-    }
-    __syncthreads();
-}
-
 template <class V>
 __device__ __forceinline__ V* scan_scratch(Shared& sh);
 template <>
@@ -439,7 +354,7 @@ __device__ __forceinline__ bool nxn_slot(int na, int nb, bool intra, int k, int&
 __device__ __forceinline__ bool heavy_moves(const Tile<double>& t, const StepArgs&, int64_t, int i, int j,
                                             uint32_t r)
 {
-    const double U3 = u23<double>(r);
+    const double U3 = u23_bits(r);
     const double wi = t.w[i], wj = t.w[j];
     return U3 * fmax(wi, wj) < fmin(wi, wj);
 }
@@ -484,43 +399,125 @@ __device__ __forceinline__ void add_weight_sums(Acc<float>& a1, Acc<float>& a2, 
     a2.add(ff_mul(w, w));
 }
 
-// Relativistic pair, given its CM frame: scattering length with |p*|^2 v_rel* in place of mu^2 u^3, rotation of p*
-// through (Theta, phi), boost of the change back to the lab frame. Returns dp = p_i' - p_i.
-template <class V>
-__device__ __forceinline__ void rel_pair_dp_cm(const StepArgs& A, const InterConst& ic, const RelCM<V>& cm, V cc,
-                                               V wf, uint8_t f, V U1, V U2, V U4, V dp[3])
+// Velocities of a pair after its scatter; false if it does not scatter. FP64 by mcc_pair64.cuh, except with CHAIN: in the
+// order N x N pairing every particle is scattered by every partner in turn, and last-bit differences grow along the chain
+// (a change of its inputs by an ulp moves the oracle's own two-species result by 1e-12), so those pairs take correctly
+// rounded roots and quotients and the library functions.
+template <bool REL, bool CHAIN>
+__device__ __forceinline__ bool pair_out(const StepArgs& A, const InterConst& ic, const double vi[3], const double vj[3],
+                                         double wf, uint8_t f, const uint4& r, double ni[3], double nj[3])
 {
-    V s = pick<V>(ic.kappa, ic.kappa_f) * wf / (cm.pmag * cm.pmag * cm.vrel);
-    if (f & kPairTriplet) s *= (V)0.5;
-    V st, omc, sp, cp, dx, dy, dz;
-    N97Tab<V> tab;
-    n97_tab(A, tab);
-    sample_angle<V>(A.method, s, U1, U4, st, omc, tab);
-    sincospi_v((V)2 * U2, &sp, &cp);
-    rotate<V>(cm.px, cm.py, cm.pz, st, omc, cp, sp, dx, dy, dz);
-    const V coef_b = cm.gC * cm.gC / (cc * cc * (cm.gC + (V)1));
-    const V Vd = cm.Vx * dx + cm.Vy * dy + cm.Vz * dz;
-    dp[0] = dx + coef_b * Vd * cm.Vx;
-    dp[1] = dy + coef_b * Vd * cm.Vy;
-    dp[2] = dz + coef_b * Vd * cm.Vz;
+    const double half = (f & kPairTriplet) ? 0.5 : 1.0;
+    if (CHAIN) {
+        const double U1 = u23<double>(r.x), U2 = u23<double>(r.y), U4 = u23<double>(r.w);
+        double st, omc, sp, cp, dx, dy, dz;
+        if (!REL) {
+            const double ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
+            const double u2 = ux * ux + uy * uy + uz * uz;
+            if (u2 == 0.0) return false;
+            sample_angle(A.method, half * (ic.kappa_mu2 * wf / (u2 * sqrt(u2))), U1, U4, st, omc, A.t64);
+            sincospi(2.0 * U2, &sp, &cp);
+            rotate<double>(ux, uy, uz, st, omc, cp, sp, dx, dy, dz);
+            const double fa = ic.mu_ma, fb = ic.mu_mb;
+            ni[0] = vi[0] + fa * dx; ni[1] = vi[1] + fa * dy; ni[2] = vi[2] + fa * dz;
+            nj[0] = vj[0] - fb * dx; nj[1] = vj[1] - fb * dy; nj[2] = vj[2] - fb * dz;
+            return true;
+        }
+        if (vi[0] == vj[0] && vi[1] == vj[1] && vi[2] == vj[2]) return false;
+        const RelCM<double> cm = rel_cm<double>(A.c, A.ma[ic.a], A.ma[ic.b], vi, vj);
+        if (!(cm.pmag > 0.0)) return false;
+        sample_angle(A.method, half * (ic.kappa * wf / (cm.pmag * cm.pmag * cm.vrel)), U1, U4, st, omc, A.t64);
+        sincospi(2.0 * U2, &sp, &cp);
+        rotate<double>(cm.px, cm.py, cm.pz, st, omc, cp, sp, dx, dy, dz);
+        const double cb = cm.gC * cm.gC / (A.c * A.c * (cm.gC + 1.0));
+        const double Vd = cm.Vx * dx + cm.Vy * dy + cm.Vz * dz;
+        const double dp[3] = {dx + cb * Vd * cm.Vx, dy + cb * Vd * cm.Vy, dz + cb * Vd * cm.Vz};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ni[d] = vi[d] + dp[d] / A.ma[ic.a];
+            nj[d] = vj[d] - dp[d] / A.ma[ic.b];
+        }
+        return true;
+    }
+    if (REL) {
+        double dp[3];
+        if (vi[0] == vj[0] && vi[1] == vj[1] && vi[2] == vj[2]) return false;
+        if (!rel_pair64(A.t64, A.method, A.c * A.c, A.ma[ic.a], A.ma[ic.b], half * ic.kappa * wf, vi, vj, r, dp))
+            return false;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ni[d] = fma(dp[d], ic.inv_ma, vi[d]);
+            nj[d] = fma(-dp[d], ic.inv_mb, vj[d]);
+        }
+        return true;
+    }
+    double du[3];
+    if (!pair64(A.t64, A.method, half * ic.kappa_mu2 * wf, vi, vj, r, du)) return false;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ni[d] = fma(ic.mu_ma, du[d], vi[d]);
+        nj[d] = fma(-ic.mu_mb, du[d], vj[d]);
+    }
+    return true;
 }
 
-template <class V>
-__device__ __noinline__ void rel_pair_dp(const StepArgs& A, const InterConst& ic, const V vi[3], const V vj[3],
-                                         V wf, uint8_t f, V U1, V U2, V U4, V dp[3])
+// Float pairs (cells above every group class on the mixed path).
+template <bool REL, bool CHAIN>
+__device__ __forceinline__ bool pair_out(const StepArgs& A, const InterConst& ic, const float vi[3], const float vj[3],
+                                         float wf, uint8_t f, const uint4& r, float ni[3], float nj[3])
 {
-    const V cc = pick<V>(A.c, A.c_f);
-    const V ma = pick<V>(A.ma[ic.a], A.ma_f[ic.a]), mb = pick<V>(A.ma[ic.b], A.ma_f[ic.b]);
-    const RelCM<V> cm = rel_cm<V>(cc, ma, mb, vi, vj);
-    if (!(cm.pmag > (V)0)) {
-        dp[0] = dp[1] = dp[2] = (V)0;
-        return;
+    const float U1 = u23<float>(r.x), U2 = u23<float>(r.y), U4 = u23<float>(r.w);
+    const N97Tab<float> tab = {A.n97_f32, A.n97_dh32};
+    float st, omc, sp, cp, dx, dy, dz;
+    if (!REL) {
+        const float ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
+        const float u2 = ux * ux + uy * uy + uz * uz;
+        if (u2 == 0.f) return false;
+        const float um = sqrtf(u2);
+        float s = ic.kappa_mu2_f * wf / (u2 * um);
+        if (f & kPairTriplet) s *= 0.5f;
+        sample_angle<float>(A.method, s, U1, U4, st, omc, tab);
+        sincospi_v(2.f * U2, &sp, &cp);
+        rotate<float>(ux, uy, uz, st, omc, cp, sp, dx, dy, dz);
+        const float fa = ic.mu_ma_f, fb = ic.mu_mb_f;
+        ni[0] = vi[0] + fa * dx; ni[1] = vi[1] + fa * dy; ni[2] = vi[2] + fa * dz;
+        nj[0] = vj[0] - fb * dx; nj[1] = vj[1] - fb * dy; nj[2] = vj[2] - fb * dz;
+        return true;
     }
-    rel_pair_dp_cm<V>(A, ic, cm, cc, wf, f, U1, U2, U4, dp);
+    if (vi[0] == vj[0] && vi[1] == vj[1] && vi[2] == vj[2]) return false;
+    const float cc = A.c_f, ma = A.ma_f[ic.a], mb = A.ma_f[ic.b];
+    const RelCM<float> cm = rel_cm<float>(cc, ma, mb, vi, vj);
+    if (cm.gC > 2.f) {
+        // a fast-moving CM frame amplifies float rounding by ~gamma_C^2: this pair's kinematics run in double
+        const double vid[3] = {vi[0], vi[1], vi[2]}, vjd[3] = {vj[0], vj[1], vj[2]};
+        double di[3], dj[3];
+        if (!pair_out<true, CHAIN>(A, ic, vid, vjd, (double)wf, f, r, di, dj)) return false;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ni[d] = (float)di[d];
+            nj[d] = (float)dj[d];
+        }
+        return true;
+    }
+    if (!(cm.pmag > 0.f)) return false;
+    float s = ic.kappa_f * wf / (cm.pmag * cm.pmag * cm.vrel);
+    if (f & kPairTriplet) s *= 0.5f;
+    sample_angle<float>(A.method, s, U1, U4, st, omc, tab);
+    sincospi_v(2.f * U2, &sp, &cp);
+    rotate<float>(cm.px, cm.py, cm.pz, st, omc, cp, sp, dx, dy, dz);
+    const float coef_b = cm.gC * cm.gC / (cc * cc * (cm.gC + 1.f));
+    const float Vd = cm.Vx * dx + cm.Vy * dy + cm.Vz * dz;
+    const float dp[3] = {dx + coef_b * Vd * cm.Vx, dy + coef_b * Vd * cm.Vy, dz + coef_b * Vd * cm.Vz};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ni[d] = vi[d] + dp[d] / ma;
+        nj[d] = vj[d] - dp[d] / mb;
+    }
+    return true;
 }
 
 // One scattering pair (Algorithm 1 pair loop).
-template <class V, bool REL>
+template <class V, bool REL, bool CHAIN>
 __device__ __forceinline__ void scatter_pair(const StepArgs& A, const Tile<V>& t, int c, int64_t cs, uint32_t ictr,
                                              const InterConst& ic, int p, int i, int j, uint8_t f, int nmin,
                                              int nmax, int pm, uint32_t step)
@@ -534,54 +531,8 @@ __device__ __forceinline__ void scatter_pair(const StepArgs& A, const Tile<V>& t
     V wf = wmax * (V)nmin;
     if (A.weighting == 1 && nmax > 0) wf = wmax / (V)((nmax - 1 - pm) / nmin + 1) * (V)nmax;
     const uint4 r = draw_at(A.rng, step, (uint32_t)p, (uint32_t)c, ictr, kTagScat);
-    const V U1 = u23<V>(r.x), U2 = u23<V>(r.y), U4 = u23<V>(r.w);
-    V dvi[3], dvj[3];
-    if (!REL) {
-        const V ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
-        const V u2 = ux * ux + uy * uy + uz * uz;
-        if (u2 == (V)0) return;
-        const V um = sqrt(u2);
-        V s = pick<V>(ic.kappa_mu2, ic.kappa_mu2_f) * wf / (u2 * um);
-        if (f & kPairTriplet) s *= (V)0.5;
-        V st, omc, sp, cp, dx, dy, dz;
-        N97Tab<V> tab;
-        n97_tab(A, tab);
-        sample_angle<V>(A.method, s, U1, U4, st, omc, tab);
-        sincospi_v((V)2 * U2, &sp, &cp);
-        rotate<V>(ux, uy, uz, st, omc, cp, sp, dx, dy, dz);
-        const V fa = pick<V>(ic.mu_ma, ic.mu_ma_f), fb = pick<V>(ic.mu_mb, ic.mu_mb_f);
-        dvi[0] = fa * dx; dvi[1] = fa * dy; dvi[2] = fa * dz;
-        dvj[0] = -fb * dx; dvj[1] = -fb * dy; dvj[2] = -fb * dz;
-    } else {
-        V du2 = 0;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) du2 += (vi[d] - vj[d]) * (vi[d] - vj[d]);
-        if (du2 == (V)0) return;
-        const V cc = pick<V>(A.c, A.c_f);
-        const V ma = pick<V>(A.ma[ic.a], A.ma_f[ic.a]), mb = pick<V>(A.ma[ic.b], A.ma_f[ic.b]);
-        const RelCM<V> cm = rel_cm<V>(cc, ma, mb, vi, vj);
-        if (sizeof(V) == 4 && cm.gC > (V)2) {
-            // a fast-moving CM frame amplifies float rounding by ~gamma_C^2: this pair's kinematics run in double
-            const double vid[3] = {vi[0], vi[1], vi[2]}, vjd[3] = {vj[0], vj[1], vj[2]};
-            double dd[3];
-            rel_pair_dp<double>(A, ic, vid, vjd, (double)wf, f, u23<double>(r.x), u23<double>(r.y),
-                                u23<double>(r.w), dd);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                dvi[d] = (V)(dd[d] / A.ma[ic.a]);
-                dvj[d] = (V)(-dd[d] / A.ma[ic.b]);
-            }
-        } else {
-            if (!(cm.pmag > (V)0)) return;
-            V dp[3];
-            rel_pair_dp_cm<V>(A, ic, cm, cc, wf, f, U1, U2, U4, dp);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                dvi[d] = dp[d] / ma;
-                dvj[d] = -dp[d] / mb;
-            }
-        }
-    }
+    V ni[3], nj[3];
+    if (!pair_out<REL, CHAIN>(A, ic, vi, vj, wf, f, r, ni, nj)) return;
     bool upd_i = true, upd_j = true;
     if (!w_equal(t, i, j)) {
         const bool moves = heavy_moves(t, A, cs, i, j, r.z);
@@ -590,11 +541,11 @@ __device__ __forceinline__ void scatter_pair(const StepArgs& A, const Tile<V>& t
     }
     if (upd_i) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) t.v[d * t.vs + i] = vi[d] + dvi[d];
+        for (int d = 0; d < 3; ++d) t.v[d * t.vs + i] = ni[d];
     }
     if (upd_j) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) t.v[d * t.vs + j] = vj[d] + dvj[d];
+        for (int d = 0; d < 3; ++d) t.v[d * t.vs + j] = nj[d];
     }
 }
 
@@ -845,7 +796,7 @@ __device__ void interaction(const StepArgs& A, const Tile<V>& t, Shared& sh, int
         return;
     }
     // random permutation of each participating species (counter = {i/2, cell, step, inter<<8 | 1 + side})
-    if (MODE != kScatter) permutations<V>(A, t, sh, c, ictr, intra ? 1 : 2, a0, na, b0, nb);
+    if (MODE != kScatter) cta_permutations(A.rng, sh.step, t.keys, t.cnt, t.perm, sh.iscan, c, ictr, intra ? 1 : 2, a0, na, b0, nb);
     const int npairs = intra ? ((na & 1) ? (na + 3) / 2 : na / 2) : (na > nb ? na : nb);
     const int nmin = intra ? na - 1 : (na < nb ? na : nb);
     if (MODE == kPair) {
@@ -898,7 +849,7 @@ __device__ void interaction(const StepArgs& A, const Tile<V>& t, Shared& sh, int
                     int a, b;
                     if (!nxn_slot(na, nb, intra, r0 + q, a, b)) continue;
                     const int i = t.perm[a0 + a], j = intra ? t.perm[a0 + b] : t.perm[b0 + b];
-                    scatter_pair<V, REL>(A, t, c, cs, ictr, ic, r0 + q, i, j, 0, 1, 0, 0, sh.step);
+                    scatter_pair<V, REL, true>(A, t, c, cs, ictr, ic, r0 + q, i, j, 0, 1, 0, 0, sh.step);
                 }
                 __syncthreads();
             }
@@ -915,7 +866,7 @@ __device__ void interaction(const StepArgs& A, const Tile<V>& t, Shared& sh, int
                 int i, j;
                 uint8_t f;
                 get(p, p - r0, i, j, f);
-                scatter_pair<V, REL>(A, t, c, cs, ictr, ic, p, i, j, f, nmin, intra ? 0 : npairs, p - r0, sh.step);
+                scatter_pair<V, REL, false>(A, t, c, cs, ictr, ic, p, i, j, f, nmin, intra ? 0 : npairs, p - r0, sh.step);
                 p = (p + 1 < lead) ? p + 1 : (p < lead ? lead + (int)threadIdx.x : p + kThreads);
             }
             __syncthreads();

@@ -436,57 +436,10 @@ __device__ __forceinline__ V pair_kecm_du(V c, V m1, V m2, const V v1[3], const 
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// N97: A(s) solves L(A) = coth A - 1/A = exp(-s), taken in the equivalent form G(A) = 1 - L(A) = -expm1(-s) so that
-// small s (large A) keeps full relative precision. G is decreasing and convex, so Newton converges from any start
-// (one step from the left of the root lands right of it, then monotone). Below A = 1/2, L and L' come from the
-// Laurent series of coth (coefficients 2^{2n} B_{2n} / (2n)!); above, G = 1/A - 2/expm1(2A).
+// N97: A(s) solves L(A) = coth A - 1/A = exp(-s). Table of the float pairs over x = ln s in
+// [kN97X0, kN97X0 + kN97Nodes * kN97H]: node k holds g = A s and h dg/dx for cubic Hermite interpolation (error ~1e-9), built
+// on the host when a context is created. The FP64 pairs have their own (mcc_pair64.cuh).
 // ---------------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void n97_G_dG(double A, double& G, double& dG)
-{
-    if (A < 0.5) {
-        const double c[12] = {3.33333333333333315e-01,  -2.22222222222222231e-02, 2.11640211640211654e-03,
-                              -2.11640211640211649e-04, 2.13777991555769346e-05,  -2.16440428080639722e-06,
-                              2.19259478518737778e-07,  -2.22146087899796781e-08, 2.25078465168089944e-09,
-                              -2.28051512045921834e-10, 2.31064325990026242e-11,  -2.34117068198248822e-12};
-        const double x2 = A * A;
-        double p = c[11], q = 23.0 * c[11];
-#pragma unroll
-        for (int k = 10; k >= 0; --k) {
-            p = fma(p, x2, c[k]);
-            q = fma(q, x2, (double)(2 * k + 1) * c[k]);
-        }
-        G = 1.0 - p * A;
-        dG = -q;
-        return;
-    }
-    G = 1.0 / A - 2.0 / expm1(2.0 * A);
-    const double sh = sinh(A);
-    dG = -(1.0 / (A * A) - (A < 350.0 ? 1.0 / (sh * sh) : 0.0));
-}
-
-__device__ __forceinline__ void n97_G_dG(float A, float& G, float& dG)
-{
-    if (A < 0.5f) {
-        const float x2 = A * A;
-        const float p = fmaf(fmaf(fmaf(fmaf(2.13777991555769346e-05f, x2, -2.11640211640211649e-04f), x2,
-                                       2.11640211640211654e-03f), x2, -2.22222222222222231e-02f), x2,
-                             3.33333333333333315e-01f);
-        const float q = fmaf(fmaf(fmaf(fmaf(1.92400192400192391e-04f, x2, -1.48148148148148141e-03f), x2,
-                                       1.05820105820105814e-02f), x2, -6.66666666666666657e-02f), x2,
-                             3.33333333333333315e-01f);
-        G = 1.0f - p * A;
-        dG = -q;
-        return;
-    }
-    G = 1.0f / A - 2.0f / expm1f(2.0f * A);
-    const float sh = sinhf(A);
-    dG = -(1.0f / (A * A) - (A < 40.0f ? 1.0f / (sh * sh) : 0.0f));
-}
-
-// Table of f(x) = ln(A s) over x = ln s in [kN97X0, kN97X0 + kN97Nodes * kN97H]: node k holds (f, h df/dx) for
-// cubic Hermite interpolation (error ~1e-9). Built on the host when a context is created. The float copy holds
-// g = A s = exp(f) and h dg/dx instead: |f| reaches 8.5, where a float entry of f would carry ~5e-7 of A's relative
-// error, while a float entry of g carries 6e-8.
 constexpr int kN97Nodes = 512;
 constexpr double kN97X0 = -6.907755278982137;  // ln 1e-3
 constexpr double kN97X1 = 2.4849066497880004;  // ln 12
@@ -494,7 +447,7 @@ constexpr double kN97H = (kN97X1 - kN97X0) / kN97Nodes;
 
 template <class V>
 struct N97Tab {
-    const V* f;   // kN97Nodes + 1 values of ln(A s) (double) or A s (float)
+    const V* f;   // kN97Nodes + 1 values of A s
     const V* dh;  // kN97Nodes + 1 values of h times their derivative in ln s
 };
 
@@ -517,8 +470,7 @@ __device__ __forceinline__ V n97_A_table(V s, V z, const N97Tab<V>& tab)
     const V t2 = t * t, t3 = t2 * t;
     const V f = ((V)2 * t3 - (V)3 * t2 + (V)1) * f0 + (t3 - (V)2 * t2 + t) * d0 + ((V)-2 * t3 + (V)3 * t2) * f1 +
                 (t3 - t2) * d1;
-    if (sizeof(V) == 4) return f / s;  // the float table holds A s
-    return exp(f) / s;
+    return f / s;
 }
 
 template <class V>
@@ -527,30 +479,15 @@ __device__ __forceinline__ V n97_A(V s, const N97Tab<V>& tab)
     const V z = -expm1(-s);                  // 1 - exp(-s)
     if (!(z < (V)1)) return (V)0;            // exp(-s) underflows: isotropic limit
     if (!(z > (V)0)) return (V)CUDART_INF;   // s == 0: no scattering
-    V A = n97_A_table<V>(s, z, tab);
-    if (sizeof(V) == 4) return A;            // ~1e-9 from the table: below float resolution
-    // Newton converges quadratically: once a step is a few ulps the next would only chase rounding noise in G, so
-    // stop there (a step of 4 ulps leaves an error far below one ulp).
-    const int iters = 6;
-    const V tol = (V)1e-15;
-    for (int it = 0; it < iters; ++it) {
-        V G, dG;
-        n97_G_dG(A, G, dG);
-        V An = A - (G - z) / dG;
-        if (!(An > (V)0)) An = (V)0.5 * A;
-        const V d = fabs(An - A);
-        A = An;
-        if (d <= tol * A) break;
-    }
-    return A;
+    return n97_A_table<V>(s, z, tab);        // ~1e-9 from the table: below float resolution
 }
 
 // Centre-of-mass polar angle from the scattering length: sin(Theta) and 1 - cos(Theta).
 //  TA77: tan(Theta/2) = delta ~ N(0, s/2) by Box-Muller from (U1, U4).
 //  N97:  1 - cos chi = -log1p(U1 expm1(-2A)) / A (inverse CDF of the density proportional to exp(A cos chi)),
 //        1 + cos chi = log1p((1 - U1) expm1(2A)) / A.
-template <class V>
-__device__ __forceinline__ void sample_angle(int method, V s, V U1, V U4, V& sin_t, V& omc, const N97Tab<V>& tab)
+template <class V, class Tab>
+__device__ __forceinline__ void sample_angle(int method, V s, V U1, V U4, V& sin_t, V& omc, const Tab& tab)
 {
     if (method == 0) {
         const V g = sqrt((V)-2 * log(U1)) * cospi((V)2 * U4);

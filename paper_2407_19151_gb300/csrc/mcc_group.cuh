@@ -693,19 +693,6 @@ __device__ __forceinline__ RelCM<V> rel_cm_du(V c, V ma, V mb, const V ui[3], co
     return r;
 }
 
-template <class V>
-__device__ __forceinline__ void n97_tab_of(const StepArgs& A, N97Tab<V>& t);
-template <>
-__device__ __forceinline__ void n97_tab_of<double>(const StepArgs& A, N97Tab<double>& t)
-{
-    t = {A.n97_f, A.n97_dh};
-}
-template <>
-__device__ __forceinline__ void n97_tab_of<float>(const StepArgs& A, N97Tab<float>& t)
-{
-    t = {A.n97_f32, A.n97_dh32};
-}
-
 // Momentum change dp of particle i of a relativistic pair in its CM frame (rotation of p* through (Theta, phi) and
 // the boost of the change back to the lab frame); kappa = the interaction's q^2 q^2 lnL dt / (4 pi eps0^2 dV).
 template <class V>
@@ -715,8 +702,7 @@ __device__ __forceinline__ void rel_dp(const StepArgs& A, V kappa, const RelCM<V
     V s = kappa * wf / (cm.pmag * cm.pmag * cm.vrel);
     if (f & kPairTriplet) s *= (V)0.5;
     V st, omc, sp, cp, dx, dy, dz;
-    N97Tab<V> tab;
-    n97_tab_of<V>(A, tab);
+    const N97Tab<V> tab = {A.n97_f32, A.n97_dh32};
     sample_angle<V>(A.method, s, U1, U4, st, omc, tab);
     sincospi_v((V)2 * U2, &sp, &cp);
     rotate<V>(cm.px, cm.py, cm.pz, st, omc, cp, sp, dx, dy, dz);
@@ -973,8 +959,7 @@ __device__ __forceinline__ void gscatter_pair(const StepArgs& A, const GTile& t,
         float s = __fdividef(ic.kappa_mu2_f * wf, u2 * um);
         if (f & kPairTriplet) s *= 0.5f;
         float st, omc, sp, cp, dx, dy, dz;
-        N97Tab<float> tab;
-        n97_tab_of<float>(A, tab);
+        const N97Tab<float> tab = {A.n97_f32, A.n97_dh32};
         sample_angle_fast(A.method, s, U1, U4, st, omc, tab);
         sincospif(2.f * U2, &sp, &cp);
         rotate_fast(du[0], du[1], du[2], um, st, omc, cp, sp, dx, dy, dz);

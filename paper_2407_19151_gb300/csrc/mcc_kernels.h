@@ -16,9 +16,20 @@ struct InterConst {
     int32_t a, b;
     double kappa_mu2;  // q_a^2 q_b^2 lnL_ab dt / (4 pi eps0^2 dV) / mu^2: s = kappa_mu2 w_max N_min / u^3
     double kappa;      // same without 1/mu^2 (relativistic: s = kappa w_max N_min / (|p*|^2 v_rel*))
-    double mu_ma, mu_mb;
+    double mu_ma, mu_mb, inv_ma, inv_mb;
     float kappa_mu2_f, kappa_f, mu_ma_f, mu_mb_f;
 };
+
+// Tables of the FP64 pair kinematics (mcc_pair64.cuh), built on the host when a context is created.
+constexpr int kF64N97 = 9 * 64;  // intervals of A(s) s: 64 per octave of [2^-5, 16), eight coefficients each
+constexpr int kF64Turn = 256;    // (cos, sin) of multiples of 1/256 turn
+constexpr int kF64Ln = 128;      // (r_i, -ln r_i)
+struct F64Tab {
+    const double2* n97;
+    const double2* turn;
+    const double2* ln;
+};
+constexpr size_t kF64TabDoubles = 8 * kF64N97 + 2 * kF64Turn + 2 * kF64Ln;
 
 struct StepArgs {
     const int64_t* offsets;
@@ -48,9 +59,8 @@ struct StepArgs {
     RngKey rng;
     const uint64_t* step_dev;  // step index in device memory (null: rng.step); step = *step_dev + step_add
     uint32_t step_add;
-    const double* n97_f;   // N97 table (see mcc_device.cuh), double and float copies
-    const double* n97_dh;
-    const float* n97_f32;
+    F64Tab t64;            // tables of the FP64 pairs
+    const float* n97_f32;  // N97 table of the float pairs (see mcc_device.cuh)
     const float* n97_dh32;
     // unfused input / output
     int32_t* pair_i;
@@ -104,8 +114,9 @@ __host__ __device__ inline size_t group_smem(size_t shared_bytes, int cap)
     return (shared_bytes + (size_t)cap * kGroupBytesPerParticle + 15) & ~(size_t)15;
 }
 
-// N97 table: (f, h df/dx) at kN97Nodes + 1 nodes, computed on the host in double.
-void n97_table(double* f, double* dh);
+// N97 table of the float pairs: g = A s and h dg/dx (x = ln s) at kN97Nodes + 1 nodes; tables of the FP64 pairs.
+void n97_table(float* g, float* dh);
+void f64_tables(double* out);
 
 // Kernel launches (defined in mcc_cell.cu / mcc_bin.cu).
 cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, cudaStream_t st);
@@ -136,11 +147,13 @@ cudaError_t launch_bin_static(const int32_t* cell, const int32_t* species, int64
                               int32_t n_species, int32_t* perm, int64_t* offsets, cudaStream_t st);
 int64_t static_bin_max_keys();
 // Adjoint of one interaction (mcc_adjoint.cu).
-size_t adjoint_slab_bytes(int32_t max_cell, int32_t max_epairs);
+size_t adjoint_slab_bytes(int32_t max_cell, int32_t max_epairs, bool on_chip);
+size_t adjoint_work_bytes(int32_t max_cell);  // working arrays of one cell
+size_t adjoint_static_smem();
+int adjoint_ctas_per_sm();
 cudaError_t launch_adjoint(const StepArgs& a, double lnL, double* ox, double* oy, double* oz, double* gx, double* gy,
                            double* gz, double* gw, double* glnL, char* slab, int32_t max_cell, int32_t max_epairs,
-                           int32_t tape,
-                           int grid, cudaStream_t st);
+                           int32_t tape, bool on_chip, int grid, cudaStream_t st);
 cudaError_t launch_gather(const void* in, const int32_t* perm, int64_t n, int elem_bytes, void* out, cudaStream_t st);
 
 // Species masses for the per-species moments (mcc_species_moments).

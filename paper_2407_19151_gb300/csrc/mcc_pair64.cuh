@@ -1,0 +1,267 @@
+// FP64 kinematics of one scattering pair: the N97 / TA77 angle, the azimuth and the rotation, shared by the one-CTA step
+// kernel and the adjoint.
+//
+// The FP64 pipe bounds both (GB300 issues FP64 at 1/64 of the float rate; it was 81% busy while an SM worked), and most
+// of its instructions were the pair's: two Newton steps on the N97 root (expm1, sinh, three divisions each), expm1,
+// log1p, log, exp, sincospi and eight divisions, about 600 FP64 instructions per pair. Here the functions whose
+// arguments are known in form are table lookups with a short series, each within about an ulp:
+//   A(s) s      piecewise degree-7 polynomials in s (64 per octave of [2^-5, 16)); below, the Bernoulli series of
+//               s / (1 - e^-s), which equals A s there to 1e-27; above, the inversion of L(A) = A/3 - A^3/45
+//   ln u        u = 2^k m, ln m = -ln r_i + ln(m r_i) with tabulated r_i ~ 1/m (Tang, "Table-driven implementation of
+//               the logarithm function in IEEE floating-point arithmetic", 1990)
+//   azimuth     2 pi (k + 1/2) 2^-23 = nearest 1/256 turn, tabulated, + a remainder below pi/256 (addition theorem)
+// and uniforms are assembled from their bits instead of converted. About 190 instructions per pair. FP64 step of 4096
+// three-species cells (2.1e6 particles) 6.11 -> 2.38 ms, relativistic beam of 2048 cells 6.45 -> 2.23 ms; the difference from
+// 64-bit results is unchanged (1.4e-16 of the velocities).
+#pragma once
+
+#include "mcc_kernels.h"
+
+namespace mcc {
+
+// Uniform on (0, 1): ((r >> 9) + 1/2) 2^-23.
+__device__ __forceinline__ double u23_bits(uint32_t r)
+{
+    return __hiloint2double((int)(0x3FF00000u | (r >> 12)), (int)(((r << 20) & 0xE0000000u) | 0x10000000u)) - 1.0;
+}
+
+// cos and sin of 2 pi ((r >> 9) + 1/2) 2^-23: the nearest 1/256 turn plus the remainder. The zeros of both are table entries,
+// so a result next to a zero keeps its relative precision (TA77 multiplies it by the root of a large s).
+__device__ __forceinline__ void turn64(const F64Tab& T, uint32_t r, double& cs, double& sn)
+{
+    const uint32_t up = (r >> 23) & 1u;  // past the middle of the 1/256 turn: the next entry is nearer
+    const double2 a = __ldg(T.turn + (((r >> 24) + up) & 255u));  // cos, sin
+    const double m = __hiloint2double((int)(0x3FF00010u | ((r >> 4) & 0xFFFE0u)), 0);  // 1 + position within it
+    const double d = (m - (up ? 2.0 : 1.0)) * 0.02454369260617025968;                   // 2 pi / 256
+    const double d2 = d * d;
+    const double sd = d * fma(d2, fma(d2, fma(d2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), 1.0);
+    const double cm = d2 * fma(d2, fma(d2, -1.0 / 720.0, 1.0 / 24.0), -0.5);
+    cs = a.x + fma(a.x, cm, -a.y * sd);
+    sn = a.y + fma(a.y, cm, a.x * sd);
+}
+
+// ln u for a positive normal u.
+__device__ __forceinline__ double ln64(const F64Tab& T, double u)
+{
+    const int hi = __double2hiint(u);
+    const int ix = hi - 0x3FE60000;  // mantissas are taken in [0.6875, 1.375)
+    const int k = ix >> 20;
+    const double2 t = __ldg(T.ln + ((ix >> 13) & 127));  // r_i, -ln r_i
+    const double m = __hiloint2double(hi - (k << 20), __double2loint(u));
+    const double f = fma(m, t.x, -1.0);  // |f| < 0.008; r_i = 1 in the two intervals next to 1
+    double p = fma(f, -1.0 / 8.0, 1.0 / 7.0);
+    p = fma(f, p, -1.0 / 6.0);
+    p = fma(f, p, 1.0 / 5.0);
+    p = fma(f, p, -1.0 / 4.0);
+    p = fma(f, p, 1.0 / 3.0);
+    p = fma(f, p, -0.5);
+    const double l = fma(f * f, p, f);
+    return fma((double)k, 0.69314718055994530942, t.y + l);
+}
+
+// A(s) s of the N97 angle, s > 0.
+__device__ __forceinline__ double n97_As(const F64Tab& T, double s)
+{
+    if (s < 0.03125) {
+        const double s2 = s * s;
+        return fma(s2, fma(s2, fma(s2, 1.0 / 30240.0, -1.0 / 720.0), 1.0 / 12.0), fma(0.5, s, 1.0));
+    }
+    if (s >= 16.0) {
+        const double y = exp(-s);
+        return 3.0 * y * fma(0.6 * y, y, 1.0) * s;
+    }
+    const int hi = __double2hiint(s);
+    const double2* c = T.n97 + 4 * ((hi >> 14) - (0x3FA00000 >> 14));
+    const double m = __hiloint2double(0x3FF00000 | (hi & 0x3FFF), __double2loint(s));
+    const double t = fma(m, 128.0, -129.0);  // [-1, 1) over the interval
+    const double2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2), c3 = __ldg(c + 3);
+    double p = fma(t, c3.y, c3.x);
+    p = fma(t, p, c2.y);
+    p = fma(t, p, c2.x);
+    p = fma(t, p, c1.y);
+    p = fma(t, p, c1.x);
+    p = fma(t, p, c0.y);
+    return fma(t, p, c0.x);
+}
+
+// A(s) for sample_angle: 0 where 1 - e^-s rounds to 1 (isotropic), infinite at s = 0.
+__device__ __forceinline__ double n97_A(double s, const F64Tab& T)
+{
+    if (s > 36.7) return 0.0;
+    return s > 0.0 ? n97_As(T, s) / s : CUDART_INF;
+}
+
+// ln(1 + x) for x > -1, u = 1 + x rounded: the rounding error of u enters to first order.
+__device__ __forceinline__ double ln1p64(const F64Tab& T, double x, double u)
+{
+    return ln64(T, u) + (x - (u - 1.0)) / u;
+}
+
+// Polar angle of a pair, sin(Theta) and 1 - cos(Theta), from the scattering length s and the draws (r.x, r.w).
+// DERIV: also their derivatives in s.
+//  TA77: tan(Theta/2) = d = sqrt(s/2) g, g normal by Box-Muller; sin = 2 d / (1 + d^2), 1 - cos = 2 d^2 / (1 + d^2).
+//  N97:  1 - cos = -ln((1 - U) + U e^-2A) / A, 1 + cos = ln1p((1 - U) expm1(2A)) / A; s above 36.7 is isotropic.
+template <bool DERIV>
+__device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, const uint4& r, double& st, double& omc,
+                                        double& dst, double& domc)
+{
+    const double U = u23_bits(r.x);
+    if (DERIV) dst = domc = 0.0;
+    if (method == 0) {
+        double cs, sn;
+        turn64(T, r.w, cs, sn);
+        const double d = sqrt(fmin(-s * ln64(T, U), 1e200)) * cs;
+        const double d2 = d * d, q = 1.0 / (1.0 + d2);
+        st = 2.0 * d * q;
+        omc = 2.0 * d2 * q;
+        if (DERIV && s > 0.0) {  // d' = d / (2 s)
+            const double x = q * q / s;
+            dst = d * (1.0 - d2) * x;
+            domc = 2.0 * d2 * x;
+        }
+        return;
+    }
+    const double V = 1.0 - U;  // exact
+    double o, q;
+    if (s > 36.7) {
+        o = 2.0 * U;
+        q = 2.0 * V;
+    } else {
+        const double g = n97_As(T, s), rA = s / g;
+        double A = 0.0, E = 0.0, F = 1.0;  // E = e^-2A, F = 1 - E; A > 31 below s = 2^-5: E < 1e-27
+        if (s >= 0.03125) {
+            A = g / s;
+            if (A < 0.35) {
+                F = -expm1(-2.0 * A);
+                E = 1.0 - F;
+            } else {
+                E = exp(-2.0 * A);
+                F = 1.0 - E;
+            }
+        }
+        // ln(1 + x), x = -U F: from 1 + x while x is small, from the two positive terms (1 - U) + U E once it is not
+        const double x = -U * F;
+        const bool near1 = x > -0.5;
+        const double u = near1 ? 1.0 + x : fma(U, E, V);
+        double l = ln64(T, u);
+        if (near1) {
+            const double c = x - (u - 1.0);
+            l += fma(-c, x, c);
+        }
+        o = -l * rA;
+        q = 2.0 - o;
+        if (o > 1.0) {
+            const double y = V * (F / E);
+            q = ln1p64(T, y, 1.0 + y) * rA;
+        }
+        if (DERIV) {
+            // L(A) = coth A - 1/A = e^-s: dA/ds = -e^-s / L'(A), L' = 1 - L^2 - 2 L / A = 1/A^2 - 4 E / F^2
+            const double ys = exp(-s);
+            const double ra2 = rA * rA;
+            double dL = ra2 - (E > 0.0 ? 4.0 * E / (F * F) : 0.0);
+            if (s >= 0.03125 && A < 0.5) dL = 1.0 - ys * ys - 2.0 * ys * rA;
+            // d(1 - cos)/dA = (-(1 - cos) + 2 U E / (1 + x)) / A
+            const double dA = -ys / dL;
+            const double do_ds = rA * (2.0 * U * E / u - o) * dA;
+            const bool cl = o > 2.0;
+            domc = cl ? 0.0 : do_ds;
+            dst = (o * q > 0.0 && !cl) ? (q - o) * do_ds * (0.5 * rsqrt(o * q)) : 0.0;
+        }
+    }
+    o = o > 2.0 ? 2.0 : o;
+    q = q > 2.0 ? 2.0 : q;
+    omc = o;
+    st = sqrt(o * q);
+}
+
+// Rotation of u (magnitude um) through (Theta, phi) about its own direction; returns du = u' - u.
+__device__ __forceinline__ void rotate64(double ux, double uy, double uz, double um, double st, double omc, double cp,
+                                         double sp, double& dx, double& dy, double& dz)
+{
+    const double p2 = fma(ux, ux, uy * uy);
+    const double sc = st * cp, ss = st * sp;
+    if (p2 > 0.0) {
+        const double rp = rsqrt(p2);
+        const double ax = ux * rp, ay = uy * rp;
+        const double zc = uz * sc, us = um * ss;
+        dx = ax * zc - ay * us - ux * omc;
+        dy = ay * zc + ax * us - uy * omc;
+        dz = -(p2 * rp) * sc - uz * omc;
+    } else {
+        dx = um * sc;
+        dy = um * ss;
+        dz = -uz * omc;
+    }
+}
+
+// Change of the relative velocity u = v_i - v_j of a non-relativistic pair, s = cw / |u|^3; false if u vanishes. cw = kappa
+// / mu^2 w_max N_min, halved for a triplet. The step kernel and the adjoint's forward both run this and then fma(mu / m, du,
+// v), so that a replayed interaction repeats the step's velocities bit for bit.
+__device__ __forceinline__ bool pair64(const F64Tab& T, int method, double cw, const double vi[3], const double vj[3],
+                                       const uint4& r, double du[3])
+{
+    const double ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
+    const double u2 = fma(uz, uz, fma(uy, uy, ux * ux));
+    if (u2 == 0.0) return false;
+    const double ru = rsqrt(u2);
+    double st, omc, sp, cp, d0, d1;
+    angle64<false>(T, method, cw * (ru * ru * ru), r, st, omc, d0, d1);
+    turn64(T, r.y, cp, sp);
+    rotate64(ux, uy, uz, u2 * ru, st, omc, cp, sp, du[0], du[1], du[2]);
+    return true;
+}
+
+// Momentum change of particle i of a relativistic pair in the lab frame (proper velocities vi, vj, masses ma, mb): the
+// pair's centre-of-momentum frame (see rel_cm), s with |p*|^2 v_rel* in place of mu^2 u^3, the rotation of p* and the
+// boost of its change back. kw = kappa w_max N_min (halved for a triplet). False if p* vanishes.
+__device__ __forceinline__ bool rel_pair64(const F64Tab& T, int method, double c2, double ma, double mb, double kw,
+                                           const double vi[3], const double vj[3], const uint4& r, double dp[3])
+{
+    const double ic2 = 1.0 / c2;
+    const double gi = sqrt(fma(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2], ic2, 1.0));
+    const double gj = sqrt(fma(vj[0] * vj[0] + vj[1] * vj[1] + vj[2] * vj[2], ic2, 1.0));
+    const double M = ma * gi + mb * gj, rM = 1.0 / M;
+    double du[3], V[3], du2 = 0.0, ss = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        du[d] = vi[d] - vj[d];
+        V[d] = (ma * vi[d] + mb * vj[d]) * rM;
+        du2 += du[d] * du[d];
+        ss += du[d] * (vi[d] + vj[d]);
+    }
+    const double dg = ss * ic2 / (gi + gj);
+    const double grm1 = fmax(0.5 * (du2 * ic2 - dg * dg), 0.0);
+    const double sm = ma + mb;
+    const double gC = M * rsqrt(fma(sm, sm, 2.0 * ma * mb * grm1));
+    const double cb = gC * gC * ic2 / (gC + 1.0);
+    const double k = ma * mb * rM;
+    double p[3], Vq = 0.0, p2 = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        p[d] = k * (gj * du[d] - dg * vj[d]);
+        Vq += V[d] * p[d];
+    }
+    Vq *= cb;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        p[d] = fma(Vq, V[d], p[d]);
+        p2 += p[d] * p[d];
+    }
+    if (!(p2 > 0.0)) return false;
+    const double rp = rsqrt(p2);
+    const double pm = p2 * rp;
+    // v_rel* = |p*| (1 / (m_a gamma_a*) + 1 / (m_b gamma_b*)), m gamma* = sqrt(m^2 + |p*|^2 / c^2)
+    const double pc = p2 * ic2;
+    const double iv = rsqrt(fma(ma, ma, pc)) + rsqrt(fma(mb, mb, pc));
+    const double s = kw * (rp * rp * rp) / iv;
+    double st, omc, cp, sp, x0, x1, d[3];
+    angle64<false>(T, method, s, r, st, omc, x0, x1);
+    turn64(T, r.y, cp, sp);
+    rotate64(p[0], p[1], p[2], pm, st, omc, cp, sp, d[0], d[1], d[2]);
+    const double Vd = cb * (V[0] * d[0] + V[1] * d[1] + V[2] * d[2]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) dp[q] = fma(Vd, V[q], d[q]);
+    return true;
+}
+
+}  // namespace mcc
