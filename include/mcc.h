@@ -183,7 +183,8 @@ int mcc_bin(mcc_ctx* ctx, const int32_t* cell, const int32_t* species, int64_t n
             int32_t n_species, int32_t* perm_out, int64_t* offsets_out, void* ws, size_t ws_bytes,
             mcc_stream stream);
 
-/* Bytes of device workspace mcc_bin_weighted needs (mcc_bin's counters plus 8 bytes per particle). */
+/* Bytes of device workspace mcc_bin_weighted needs (mcc_bin's counters plus 8 bytes per particle; mcc_bin's own is the
+ * counters plus 4 bytes per particle). */
 int mcc_bin_weighted_workspace_size(int64_t n, int32_t n_cells, int32_t n_species, size_t* bytes);
 
 /*

@@ -1,17 +1,22 @@
 // Cell binning: stable counting sort of particles by key = cell * S + species (particles collide per cell of
 // volume dV, Sec. 2), and a gather through the resulting permutation.
 //
-// histogram (atomic counts) -> exclusive scan -> scatter with atomic cursors (order within a segment arbitrary)
-// -> per-segment sort of the particle indices, which restores the stable (index) order. The result does not depend
-// on the order in which the atomics were served. The atomics are warp-aggregated (lanes with equal keys add once),
-// which matters for nearly binned input such as a re-bin after a particle push; segments of up to 512 entries are
-// sorted by one warp in its slice of shared memory (warp barriers only), larger ones by a whole CTA.
+// histogram (atomic counts) -> exclusive scan -> scatter to the counted places (order within a segment arbitrary)
+// -> per-segment sort: by particle index, which restores the stable order, or straight by weight. The result does not
+// depend on the order in which the atomics were served. Lanes with equal keys in a row add once, which matters for nearly
+// binned input such as a re-bin after a particle push (a warp match over all lanes cost more than the atomics it saved on
+// shuffled input); the count's atomic also gives each particle its place in the segment, so the scatter needs none.
+// Segments of up to 512 entries are sorted by one warp in its slice of shared memory (warp barriers only), larger ones
+// by a whole CTA. What bounds it: atomics and random sectors on shuffled input (3.3e7 particles, 2e5 segments: 1.71 -> 1.14 ms,
+// of which count 0.46 -> 0.33, scatter 0.52 -> 0.35, index sorts 0.67 -> 0.40); the weight sorts after a push (1.7e7 particles,
+// 1e5 segments: 0.64 -> 0.29 ms). A two-pass radix sort of (key, index) pairs took 1.43 ms shuffled and lost on nearly
+// binned input, where a warp here has few atomics.
 #include <mutex>
 
 #include "mcc_kernels.h"
 
 // Counters of mcc_bin_static: every device that loads the library holds this array until the process exits.
-// counts | cursors | large-segment list, the layout launch_bin expects for kStaticBinKeys segments.
+// counts | cursors | large-segment list, the layout bin_core expects for kStaticBinKeys segments.
 constexpr int64_t kStaticBinKeys = 1 << 21;
 constexpr size_t kStaticBinHalf = ((size_t)kStaticBinKeys * sizeof(int32_t) + 255) & ~(size_t)255;
 constexpr size_t kStaticBinList = ((size_t)(kStaticBinKeys + 1) * sizeof(int32_t) + 255) & ~(size_t)255;
@@ -40,16 +45,49 @@ __device__ __forceinline__ long long bin_key(const int32_t* __restrict__ cell, c
     return (long long)c * S + s;
 }
 
-// All lanes of a warp run the same trips (the loop index is the warp's base), so the match below sees the full warp.
-__global__ void k_hist(const int32_t* __restrict__ cell, const int32_t* __restrict__ species, int64_t n,
-                       int32_t n_cells, int32_t S, int32_t* __restrict__ counts, int32_t* status)
+// Lanes of a warp with equal keys in a row: this lane's run starts at lane `lead` and is `len` lanes long.
+__device__ __forceinline__ void key_run(long long key, int& lead, int& len)
+{
+    const int lane = threadIdx.x & 31;
+    const long long prev = __shfl_up_sync(0xffffffffu, key, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || key != prev);
+    const unsigned upto = (2u << lane) - 1u;  // this lane and those below
+    lead = 31 - __clz(heads & upto);
+    const unsigned after = heads & ~upto;
+    len = (after ? __ffs(after) - 1 : 32) - lead;
+}
+
+// All lanes of a warp run the same trips (the loop index is the warp's base), so the shuffles see the full warp. Four
+// elements per thread and iteration: their keys first, then their atomics, so that several are in flight.
+// PLACE: place[i] = the particle's place in its segment, in the order the atomics were served.
+constexpr int kBinUnroll = 4;
+
+template <bool PLACE>
+__global__ void __launch_bounds__(kBinThreads) k_hist(const int32_t* __restrict__ cell, const int32_t* __restrict__ species,
+                                                      int64_t n, int32_t n_cells, int32_t S, int32_t* __restrict__ counts,
+                                                      int32_t* __restrict__ place, int32_t* status)
 {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const long long key = bin_key(cell, species, base + lane, n, n_cells, S, status);
-        const unsigned m = __match_any_sync(0xffffffffu, key);
-        if (key >= 0 && lane == __ffs(m) - 1) atomicAdd(&counts[key], __popc(m));
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += kBinUnroll * stride) {
+        long long key[kBinUnroll];
+        int lead[kBinUnroll], at[kBinUnroll];
+#pragma unroll
+        for (int u = 0; u < kBinUnroll; ++u) key[u] = bin_key(cell, species, base + u * stride + lane, n, n_cells, S, status);
+#pragma unroll
+        for (int u = 0; u < kBinUnroll; ++u) {
+            int len;
+            key_run(key[u], lead[u], len);
+            at[u] = 0;
+            if (key[u] >= 0 && lane == lead[u]) at[u] = atomicAdd(&counts[key[u]], len);
+        }
+        if (PLACE) {
+#pragma unroll
+            for (int u = 0; u < kBinUnroll; ++u) {
+                const int a = __shfl_sync(0xffffffffu, at[u], lead[u]) + lane - lead[u];
+                if (key[u] >= 0) place[base + u * stride + lane] = a;
+            }
+        }
     }
 }
 
@@ -137,20 +175,36 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_add(const int32_t* __rest
         if (base + j < nk) offsets[base + j] += pre;
 }
 
-__global__ void k_scatter(const int32_t* __restrict__ cell, const int32_t* __restrict__ species, int64_t n,
-                          int32_t n_cells, int32_t S, const int64_t* __restrict__ offsets,
-                          int32_t* __restrict__ cursor, int32_t* __restrict__ perm)
+// PLACE: each particle's place was counted (place); else it is taken from the segment's cursor.
+template <bool PLACE>
+__global__ void __launch_bounds__(kBinThreads) k_scatter(const int32_t* __restrict__ cell, const int32_t* __restrict__ species,
+                                                         int64_t n, int32_t n_cells, int32_t S,
+                                                         const int64_t* __restrict__ offsets, int32_t* __restrict__ cursor,
+                                                         const int32_t* __restrict__ place, int32_t* __restrict__ perm)
 {
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const long long key = bin_key(cell, species, base + lane, n, n_cells, S, nullptr);
-        const unsigned m = __match_any_sync(0xffffffffu, key);
-        const int leader = __ffs(m) - 1;
-        int32_t at = 0;
-        if (key >= 0 && lane == leader) at = atomicAdd(&cursor[key], __popc(m));
-        at = __shfl_sync(0xffffffffu, at, leader);
-        if (key >= 0) perm[offsets[key] + at + __popc(m & ((1u << lane) - 1u))] = (int32_t)(base + lane);
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += kBinUnroll * stride) {
+        long long key[kBinUnroll];
+        int at[kBinUnroll];
+#pragma unroll
+        for (int u = 0; u < kBinUnroll; ++u) {
+            const int64_t i = base + u * stride + lane;
+            key[u] = bin_key(cell, species, i, n, n_cells, S, nullptr);
+            at[u] = PLACE && key[u] >= 0 ? place[i] : 0;
+        }
+        if (!PLACE) {
+#pragma unroll
+            for (int u = 0; u < kBinUnroll; ++u) {
+                int lead, len;
+                key_run(key[u], lead, len);
+                if (key[u] >= 0 && lane == lead) at[u] = atomicAdd(&cursor[key[u]], len);
+                at[u] = __shfl_sync(0xffffffffu, at[u], lead) + lane - lead;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kBinUnroll; ++u)
+            if (key[u] >= 0) perm[offsets[key[u]] + at[u]] = (int32_t)(base + u * stride + lane);
     }
 }
 
@@ -189,59 +243,119 @@ __device__ __forceinline__ void warp_sort_smem(int n, Cmpx cmpx)
 }
 
 // Small segments (2 .. kWarpSeg entries), one warp each, sorted in the warp's shared-memory slice (the loop index is
-// warp-uniform, so whole warps take the same branches). w == nullptr: the entries by particle index. Otherwise
-// straight into the weight order of mcc_bin_weighted: pairs (weight key with a zero rank field, particle index)
-// sorted lexicographically, which is descending truncated weight with ties in increasing index. The ids of the
-// larger segments are appended to `large` (large[0] the count, zeroed before) for the CTA-wide sorts.
-// WEIGHTED: the weight-order keys need a second slab; the index-only sort keeps 2 KB per warp, so that more warps
-// fit an SM (the sorts are latency-bound).
+// warp-uniform, so whole warps take the same branches). Not WEIGHTED: by particle index. WEIGHTED: straight into the weight
+// order of mcc_bin_weighted, pairs (weight key with a zero rank field, particle index) in lexicographic order, which is
+// descending truncated weight with ties in increasing index. The ids of the larger segments are appended to `large` (large[0]
+// the count, zeroed before) for the CTA-wide sorts.
+// A segment in order already is left. Otherwise a counting sort on a linear map of the keys' top words (the indices) to n or
+// more buckets, then an insertion sort within a bucket. Indices of shuffled particles spread evenly, and so do weights over
+// decades, as the IEEE bits of a weight are nearly linear in its logarithm; a segment with a bucket above kBucketMost (after
+// a particle push most indices of a segment are neighbours) takes the bitonic network.
+constexpr int kOrderWarps = 4;   // warps per CTA
+constexpr int kBucketMost = 12;  // longest bucket for the insertion sort
+
 template <bool WEIGHTED>
-__global__ void __launch_bounds__(kBinThreads) k_segsort_warp(const int64_t* __restrict__ offsets, int64_t nk,
-                                                              const double* __restrict__ w, int32_t* __restrict__ perm,
-                                                              int32_t* __restrict__ large)
+__global__ void __launch_bounds__(32 * kOrderWarps) k_segsort_warp(const int64_t* __restrict__ offsets, int64_t nk,
+                                                                  const double* __restrict__ w,
+                                                                  int32_t* __restrict__ perm, int32_t* __restrict__ large)
 {
-    __shared__ uint64_t kslab[WEIGHTED ? kBinThreads / 32 : 1][WEIGHTED ? kWarpSeg : 1];
-    __shared__ int32_t islab[kBinThreads / 32][kWarpSeg];
-    const int lane = threadIdx.x & 31;
-    uint64_t* kb = kslab[WEIGHTED ? threadIdx.x >> 5 : 0];
-    int32_t* ib = islab[threadIdx.x >> 5];
-    const int64_t warp = ((int64_t)blockIdx.x * kBinThreads + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * kBinThreads) >> 5;
-    for (int64_t seg = warp; seg < nk; seg += nwarps) {
+    __shared__ uint64_t kslab[WEIGHTED ? kOrderWarps : 1][WEIGHTED ? kWarpSeg : 1];
+    __shared__ int32_t islab[kOrderWarps][kWarpSeg];
+    __shared__ uint32_t cslab[kOrderWarps][kWarpSeg];
+    __shared__ uint16_t oslab[kOrderWarps][kWarpSeg];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint64_t* kb = kslab[WEIGHTED ? wid : 0];
+    int32_t* ib = islab[wid];
+    uint32_t* cnt = cslab[wid];
+    uint16_t* ord = oslab[wid];
+    auto top = [&](int i) -> uint32_t { return WEIGHTED ? (uint32_t)(kb[i] >> 32) : (uint32_t)ib[i]; };
+    auto after = [&](int i, int j) -> bool {  // entry i comes after entry j
+        return WEIGHTED ? (kb[i] > kb[j] || (kb[i] == kb[j] && ib[i] > ib[j])) : ib[i] > ib[j];
+    };
+    const int64_t nwarps = (int64_t)gridDim.x * kOrderWarps;
+    for (int64_t seg = (int64_t)blockIdx.x * kOrderWarps + wid; seg < nk; seg += nwarps) {
         const int64_t b = offsets[seg];
         const int n = (int)(offsets[seg + 1] - b);
         if (n > kWarpSeg && lane == 0) large[1 + atomicAdd(&large[0], 1)] = (int32_t)seg;
         if (n < 2 || n > kWarpSeg) continue;
         int32_t* p = perm + b;
-        if (!WEIGHTED) {
-            for (int i = lane; i < n; i += 32) ib[i] = p[i];
-            __syncwarp();
-            warp_sort_smem(n, [ib](int lo, int hi) {
-                const int32_t x = ib[lo], y = ib[hi];
-                if (x > y) {
-                    ib[lo] = y;
-                    ib[hi] = x;
-                }
-            });
-        } else {
-            for (int i = lane; i < n; i += 32) {
-                const int32_t q = p[i];
-                ib[i] = q;
-                kb[i] = weight_key(w[q], 0u);
-            }
-            __syncwarp();
-            warp_sort_smem(n, [kb, ib](int lo, int hi) {
-                const uint64_t x = kb[lo], y = kb[hi];
-                const int32_t a = ib[lo], c = ib[hi];
-                if (x > y || (x == y && a > c)) {
-                    kb[lo] = y;
-                    kb[hi] = x;
-                    ib[lo] = c;
-                    ib[hi] = a;
-                }
-            });
+        uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+        for (int i = lane; i < n; i += 32) {
+            const int32_t q = p[i];
+            ib[i] = q;
+            if (WEIGHTED) kb[i] = weight_key(w[q], 0u);
+            lo = min(lo, top(i));
+            hi = max(hi, top(i));
         }
-        for (int i = lane; i < n; i += 32) p[i] = ib[i];
+        __syncwarp();
+        bool out = false;
+        for (int i = lane; i + 1 < n; i += 32) out |= after(i, i + 1);
+        if (!__any_sync(0xffffffffu, out)) continue;
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        int lg = 5;
+        while ((1 << lg) < n) ++lg;
+        const int nb = 1 << lg, per = nb / 32;  // nb <= kWarpSeg
+        // bucket = (key - lo) nb / (hi - lo + 1), rounded down: below nb, and never decreasing in the key
+        const uint32_t span = hi - lo;
+        const uint32_t mult = span < (uint32_t)nb ? 0u : (uint32_t)(((uint64_t)nb << 32) / ((uint64_t)span + 1u));
+        auto bucket = [&](int i) -> int { return (int)(mult ? __umulhi(top(i) - lo, mult) : top(i) - lo); };
+        for (int i = lane; i < nb; i += 32) cnt[i] = 0;
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) atomicAdd(&cnt[bucket(i)], 1u);
+        __syncwarp();
+        uint32_t sum = 0, most = 0;
+        for (int i = 0; i < per; ++i) {
+            const uint32_t x = cnt[lane * per + i];
+            sum += x;
+            most = max(most, x);
+        }
+        if (__reduce_max_sync(0xffffffffu, most) > kBucketMost) {
+            warp_sort_smem(n, [&](int x, int y) {
+                if (after(x, y)) {
+                    const int32_t a = ib[x];
+                    ib[x] = ib[y];
+                    ib[y] = a;
+                    if (WEIGHTED) {
+                        const uint64_t k = kb[x];
+                        kb[x] = kb[y];
+                        kb[y] = k;
+                    }
+                }
+            });
+            for (int i = lane; i < n; i += 32) p[i] = ib[i];
+            __syncwarp();
+            continue;
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        uint32_t run = inc - sum;
+        for (int i = 0; i < per; ++i) {
+            const uint32_t x = cnt[lane * per + i];
+            cnt[lane * per + i] = run;
+            run += x;
+        }
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) ord[atomicAdd(&cnt[bucket(i)], 1u)] = (uint16_t)i;
+        __syncwarp();
+        for (int i = lane; i < nb; i += 32) {  // cnt[i] is now the end of bucket i
+            const int end = (int)cnt[i], start = i ? (int)cnt[i - 1] : 0;
+            for (int x = start + 1; x < end; ++x) {
+                const uint16_t v = ord[x];
+                int y = x - 1;
+                while (y >= start && after(ord[y], v)) {
+                    ord[y + 1] = ord[y];
+                    --y;
+                }
+                ord[y + 1] = v;
+            }
+        }
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) p[i] = ib[ord[i]];
         __syncwarp();
     }
 }
@@ -326,47 +440,56 @@ int grid_for(int64_t n, int threads)
 
 }  // namespace
 
-// Workspace: counts | cursors (one int32 per segment each) | large-segment list (count, then segment ids).
+static size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Counters: counts | cursors (one int32 per segment each) | large-segment list (count, then segment ids). The workspace of
+// mcc_bin adds each particle's place in its segment (int32), that of mcc_bin_weighted the keys of large segments (64 bits,
+// over the places, which are done with by then).
+static size_t counter_bytes(int64_t n_keys)
+{
+    return 2 * up256((size_t)n_keys * sizeof(int32_t)) + up256((size_t)(n_keys + 1) * sizeof(int32_t));
+}
+
 size_t bin_workspace_bytes(int64_t n, int64_t n_keys)
 {
-    (void)n;
-    const size_t one = ((size_t)n_keys * sizeof(int32_t) + 255) & ~(size_t)255;
-    const size_t lst = ((size_t)(n_keys + 1) * sizeof(int32_t) + 255) & ~(size_t)255;
-    return 2 * one + lst;
+    return counter_bytes(n_keys) + up256((size_t)n * sizeof(int32_t));
 }
 
 static int32_t* large_list(void* ws, int64_t nk)
 {
-    const size_t one = ((size_t)nk * sizeof(int32_t) + 255) & ~(size_t)255;
-    return reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + 2 * one);
+    return reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + 2 * up256((size_t)nk * sizeof(int32_t)));
 }
 
 // hist -> scan -> scatter -> small segments by one warp each (index order, or with w the weight order directly)
-// -> large segments by index, one CTA each.
+// -> large segments by index, one CTA each. place: [n] or null (the scatter then takes its places from the cursors).
 static cudaError_t bin_core(const int32_t* cell, const int32_t* species, int64_t n, int32_t n_cells,
-                            int32_t n_species, const double* w, int32_t* perm, int64_t* offsets, void* ws,
+                            int32_t n_species, const double* w, int32_t* perm, int64_t* offsets, void* ws, int32_t* place,
                             int32_t* status, cudaStream_t st, int64_t* launches)
 {
     const int64_t nk = (int64_t)n_cells * n_species;
-    const size_t one = ((size_t)nk * sizeof(int32_t) + 255) & ~(size_t)255;
     int32_t* counts = reinterpret_cast<int32_t*>(ws);
-    int32_t* cursor = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + one);
+    int32_t* cursor = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + up256((size_t)nk * sizeof(int32_t)));
     int32_t* large = large_list(ws, nk);
-    cudaError_t e = cudaMemsetAsync(ws, 0, bin_workspace_bytes(n, nk), st);
+    cudaError_t e = cudaMemsetAsync(ws, 0, counter_bytes(nk), st);
     if (e != cudaSuccess) return e;
     const int g = grid_for(n, kBinThreads);
-    if (n > 0) k_hist<<<g, kBinThreads, 0, st>>>(cell, species, n, n_cells, n_species, counts, status);
+    if (n > 0) {
+        if (place) k_hist<true><<<g, kBinThreads, 0, st>>>(cell, species, n, n_cells, n_species, counts, place, status);
+        else k_hist<false><<<g, kBinThreads, 0, st>>>(cell, species, n, n_cells, n_species, counts, place, status);
+    }
     const int64_t tiles = (nk + kScanTile - 1) / kScanTile;
     k_scan_tile<<<(unsigned)tiles, kScanThreads, 0, st>>>(counts, nk, offsets, status);
     k_scan_top<<<1, kScanThreads, 0, st>>>(counts, nk, tiles, offsets);
     k_scan_add<<<(unsigned)tiles, kScanThreads, 0, st>>>(counts, nk, offsets);
     *launches += 3;
     if (n > 0) {
-        k_scatter<<<g, kBinThreads, 0, st>>>(cell, species, n, n_cells, n_species, offsets, cursor, perm);
-        if (w)
-            k_segsort_warp<true><<<grid_for(nk * 32, kBinThreads), kBinThreads, 0, st>>>(offsets, nk, w, perm, large);
+        if (place)
+            k_scatter<true><<<g, kBinThreads, 0, st>>>(cell, species, n, n_cells, n_species, offsets, cursor, place, perm);
         else
-            k_segsort_warp<false><<<grid_for(nk * 32, kBinThreads), kBinThreads, 0, st>>>(offsets, nk, w, perm, large);
+            k_scatter<false><<<g, kBinThreads, 0, st>>>(cell, species, n, n_cells, n_species, offsets, cursor, place, perm);
+        const int gw = grid_for(nk * 32, 32 * kOrderWarps);
+        if (w) k_segsort_warp<true><<<gw, 32 * kOrderWarps, 0, st>>>(offsets, nk, w, perm, large);
+        else k_segsort_warp<false><<<gw, 32 * kOrderWarps, 0, st>>>(offsets, nk, w, perm, large);
         k_segsort<<<grid_for(n / (kWarpSeg + 1) * kBinThreads, kBinThreads), kBinThreads, 0, st>>>(offsets, large,
                                                                                                  perm);
         *launches += 4;
@@ -377,12 +500,13 @@ static cudaError_t bin_core(const int32_t* cell, const int32_t* species, int64_t
 cudaError_t launch_bin(const int32_t* cell, const int32_t* species, int64_t n, int32_t n_cells, int32_t n_species,
                        int32_t* perm, int64_t* offsets, void* ws, int32_t* status, cudaStream_t st, int64_t* launches)
 {
-    return bin_core(cell, species, n, n_cells, n_species, nullptr, perm, offsets, ws, status, st, launches);
+    int32_t* place = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + counter_bytes((int64_t)n_cells * n_species));
+    return bin_core(cell, species, n, n_cells, n_species, nullptr, perm, offsets, ws, place, status, st, launches);
 }
 
 size_t bin_weighted_workspace_bytes(int64_t n, int64_t n_keys)
 {
-    return bin_workspace_bytes(n, n_keys) + (((size_t)n * sizeof(uint64_t) + 255) & ~(size_t)255);
+    return counter_bytes(n_keys) + up256((size_t)n * sizeof(uint64_t));
 }
 
 cudaError_t launch_bin_weighted(const int32_t* cell, const int32_t* species, const double* w, int64_t n,
@@ -390,9 +514,10 @@ cudaError_t launch_bin_weighted(const int32_t* cell, const int32_t* species, con
                                 int32_t* status, cudaStream_t st, int64_t* launches)
 {
     const int64_t nk = (int64_t)n_cells * n_species;
-    cudaError_t e = bin_core(cell, species, n, n_cells, n_species, w, perm, offsets, ws, status, st, launches);
+    uint64_t* keys = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + counter_bytes(nk));
+    cudaError_t e = bin_core(cell, species, n, n_cells, n_species, w, perm, offsets, ws, reinterpret_cast<int32_t*>(keys),
+                             status, st, launches);
     if (e != cudaSuccess || n == 0) return e;
-    uint64_t* keys = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + bin_workspace_bytes(n, nk));
     const int32_t* large = large_list(ws, nk);  // the segments above kWarpSeg, already in index order
     k_segsort_w<<<grid_for(n / (kWarpSeg + 1) * kBinThreads, kBinThreads), kBinThreads, 0, st>>>(offsets, large, w,
                                                                                                perm, keys);
@@ -433,9 +558,9 @@ cudaError_t launch_bin_static(const int32_t* cell, const int32_t* species, int64
     void* ws = static_bin_scratch(&err);
     if (err) return cudaErrorInvalidSymbol;
     int64_t launches = 0;
-    // launch_bin clears both counter arrays on the stream before its kernels; no status word (out-of-range
-    // particles are dropped, visible as offsets[last] < n)
-    return launch_bin(cell, species, n, n_cells, n_species, perm, offsets, ws, nullptr, st, &launches);
+    // bin_core clears both counter arrays on the stream before its kernels; no place array and no status word
+    // (out-of-range particles are dropped, visible as offsets[last] < n)
+    return bin_core(cell, species, n, n_cells, n_species, nullptr, perm, offsets, ws, nullptr, nullptr, st, &launches);
 }
 
 cudaError_t launch_gather(const void* in, const int32_t* perm, int64_t n, int elem_bytes, void* out, cudaStream_t st)
