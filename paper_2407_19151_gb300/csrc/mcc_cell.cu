@@ -921,6 +921,7 @@ __device__ void process_cell(const StepArgs& A, int c, unsigned char* dyn, Share
     const int S = A.S;
     const int64_t cs = A.offsets[(int64_t)c * S];
     const int n = (int)(A.offsets[(int64_t)(c + 1) * S] - cs);
+    if (MODE != kFused && (n <= A.above || (A.more && n > A.cap))) return;
     Tile<V> t;
     if (MODE == kPair) {
         if (n > A.cap) {

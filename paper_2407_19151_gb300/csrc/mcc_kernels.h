@@ -75,6 +75,8 @@ struct StepArgs {
     int32_t* queue;
     const int32_t* order;  // processing order of the cells (null: index order)
     int32_t cap;        // particles per cell staged in shared memory
+    int32_t above;      // cells of at most this many particles belong to another launch (-1: none do)
+    int32_t more;       // cells above cap belong to another launch (else they latch kErrBounds)
     char* slab;         // per-CTA global slabs for larger cells (may be null)
     int64_t slab_stride;
     int32_t slab_cap;
