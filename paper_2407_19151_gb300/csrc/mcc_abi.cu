@@ -642,7 +642,9 @@ namespace {
 // Workspace of mcc_step_fused: the cell order (n_cells int32), the class bounds and queue counters of the group
 // kernels, then, when some cell exceeds the largest group class, one slab per resident CTA of the one-CTA kernel.
 size_t order_bytes(int32_t n_cells) { return ((size_t)n_cells * sizeof(int32_t) + 255) & ~(size_t)255; }
-constexpr size_t kCtrlBytes = 256;  // class_off [2 (kGroupClasses + 1)] and queues [kGroupClasses + 1], int32
+// class_off [2 (kGroupClasses + 1)], queues [kGroupClasses + 1] and the order's bins, int32
+constexpr size_t kCtrlHist = 256;
+size_t ctrl_bytes() { return kCtrlHist + ((mcc::group_order_hist_bytes() + 255) & ~(size_t)255); }
 
 int tile_of(const mcc_ctx* ctx, bool f32)
 {
@@ -737,7 +739,7 @@ int mcc_step_workspace_size(mcc_ctx* ctx, int32_t prec, int32_t n_cells, int32_t
     const int32_t top = caps[mcc::kGroupClasses - 1] < caps_rel[mcc::kGroupClasses - 1]
                             ? caps[mcc::kGroupClasses - 1]
                             : caps_rel[mcc::kGroupClasses - 1];
-    size_t total = order_bytes(n_cells) + kCtrlBytes;
+    size_t total = order_bytes(n_cells) + ctrl_bytes();
     if (max_cell > top && max_cell > tile_of(ctx, f32))
         total += slab_stride_of(max_cell, f32) * (size_t)ctx->num_sms * kMaxCtasPerSm;
     *bytes = total;
@@ -793,9 +795,12 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     int32_t* class_off = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + order_bytes(n_cells));
     int32_t* queues = class_off + 2 * (mcc::kGroupClasses + 1);
     // cells by size class, largest first (the order is the same for every step of the call)
-    if (mcc::launch_group_order(offsets, n_cells, n_species, caps, order, class_off, S(stream)) != cudaSuccess)
+    int32_t* hist = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(class_off) + kCtrlHist);
+    if (cudaMemsetAsync(class_off, 0, kCtrlHist + mcc::group_order_hist_bytes(), S(stream)) != cudaSuccess)
         return MCC_ERR_CUDA;
-    ctx->launches += 1;
+    if (mcc::launch_group_order(offsets, n_cells, n_species, caps, order, class_off, hist, &ctx->launches, S(stream)) !=
+        cudaSuccess)
+        return MCC_ERR_CUDA;
     a.order = order;
     a.class_off = class_off;
     a.queues = queues;
@@ -807,10 +812,10 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     if (fallback) {
         big.order_range = class_off + 2 * mcc::kGroupClasses;
         if (max_cell > tile) {
-            big.slab = reinterpret_cast<char*>(ws) + order_bytes(n_cells) + kCtrlBytes;
+            big.slab = reinterpret_cast<char*>(ws) + order_bytes(n_cells) + ctrl_bytes();
             big.slab_stride = (int64_t)slab_stride_of(max_cell, f32);
             big.slab_cap = max_cell;
-            max_grid = (int)((ws_bytes - order_bytes(n_cells) - kCtrlBytes) / (size_t)big.slab_stride);
+            max_grid = (int)((ws_bytes - order_bytes(n_cells) - ctrl_bytes()) / (size_t)big.slab_stride);
         }
     }
     // under stream capture the marks become event-record nodes of the graph, so that a replay records them too
@@ -823,7 +828,8 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     for (int32_t t = 0; t < n_steps; ++t) {
         a.rng.step = (uint32_t)(p->step + (uint64_t)t);
         a.step_add = (uint32_t)t;
-        if (cudaMemsetAsync(queues, 0, sizeof(int32_t) * (mcc::kGroupClasses + 1), S(stream)) != cudaSuccess)
+        // (the first step's queues are zero)
+        if (t > 0 && cudaMemsetAsync(queues, 0, sizeof(int32_t) * (mcc::kGroupClasses + 1), S(stream)) != cudaSuccess)
             return MCC_ERR_CUDA;
         cudaEvent_t* ev = (p->launch_events && t == n_steps - 1) ? reinterpret_cast<cudaEvent_t*>(p->launch_events)
                                                                    : nullptr;

@@ -123,11 +123,12 @@ void f64_tables(double* out);
 // Kernel launches (defined in mcc_cell.cu / mcc_bin.cu).
 cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_step_advance(uint64_t* step, uint64_t by, cudaStream_t st);
-cudaError_t launch_cell_order(const int64_t* offsets, int32_t n_cells, int32_t S, int32_t* order, cudaStream_t st);
 // Cells ordered by group size class (largest class first; class kGroupClasses = cells above every class), largest
-// first within a class; class_off receives each class's [begin, end) in `order`.
+// first within a class; class_off receives each class's [begin, end) in `order`. hist: group_order_hist_bytes() of zeroed
+// device memory.
+size_t group_order_hist_bytes();
 cudaError_t launch_group_order(const int64_t* offsets, int32_t n_cells, int32_t S, const int32_t* caps,
-                               int32_t* order, int32_t* class_off, cudaStream_t st);
+                               int32_t* order, int32_t* class_off, int32_t* hist, int64_t* launches, cudaStream_t st);
 // Group kernels (mcc_group_*.cu): class cls runs groups of 32 << cls threads.
 const void* group_kernel(bool f32, bool rel, int cls);
 size_t group_shared_bytes(int cls);  // shared variables of one group
