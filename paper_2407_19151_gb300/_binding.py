@@ -267,6 +267,8 @@ def _species(species) -> C.Array:
 
 
 def _lnL(lnL, S: int):
+    if isinstance(lnL, (int, float)):
+        return (C.c_double * (S * S))(*([float(lnL)] * (S * S)))
     import numpy as np
     L = np.asarray(lnL, dtype=np.float64)
     if L.ndim == 0:
@@ -487,9 +489,11 @@ def mcc_step_fused(vx, vy, vz, w, offsets, n_cells, n_species, species, lnL, par
     flat = (C.c_int32 * (2 * len(inter)))(*[int(v) for ab in inter for v in ab])
     if max_cell is None:
         max_cell = int((offsets[n_species::n_species] - offsets[:-1:n_species]).max().item()) if n_cells else 0
-    if corr_pairs is None:
+    if corr_pairs is None and fail_count is None:
+        corr_pairs, fail_count = torch.zeros((2, max(n_cells, 1)), dtype=torch.int32, device=vx.device).unbind(0)
+    elif corr_pairs is None:
         corr_pairs = torch.zeros(max(n_cells, 1), dtype=torch.int32, device=vx.device)
-    if fail_count is None:
+    elif fail_count is None:
         fail_count = torch.zeros(max(n_cells, 1), dtype=torch.int32, device=vx.device)
     nb = C.c_size_t()
     _check(lib().mcc_step_workspace_size(ctx.handle, P.prec, int(n_cells), int(max_cell), C.byref(nb)),
@@ -500,7 +504,8 @@ def mcc_step_fused(vx, vy, vz, w, offsets, n_cells, n_species, species, lnL, par
                                 _lnL(lnL, n_species), flat, len(inter), C.byref(cp), int(n_steps), int(max_cell),
                                 _ptr(corr_pairs), _ptr(fail_count), _ptr(ws), nb.value,
                                 _stream(stream, vx.device)), "mcc_step_fused")
-    return corr_pairs[:n_cells], fail_count[:n_cells]
+    return (corr_pairs, fail_count) if corr_pairs.numel() == fail_count.numel() == n_cells else \
+        (corr_pairs[:n_cells], fail_count[:n_cells])
 
 
 def sync_status(device=None, stream=None):

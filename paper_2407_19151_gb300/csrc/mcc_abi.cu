@@ -1,4 +1,5 @@
 // C ABI of the collision step (declarations and contracts in include/mcc.h).
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -33,6 +34,12 @@ struct mcc_ctx {
     int32_t group_cap; // particles per warp of the group kernels' size classes; 0 = automatic
     int32_t group_top; // upper bound of the largest class; 0 = what one CTA's shared memory holds
     size_t smem_reserved;  // shared memory the system reserves per CTA
+    // Attributes of the kernels, looked up once (each look-up costs about a microsecond of every call), and the last
+    // occupancy of each: launch shape << 8 | CTAs per SM in one word, so threads may share a context.
+    size_t cell_static[2][2][4];  // [float][relativistic][mode]
+    size_t group_static[2][mcc::kGroupClasses];
+    size_t adjoint_static;
+    std::atomic<uint64_t> cell_occ[2][2][4], group_occ[2][mcc::kGroupClasses];
 };
 
 namespace mcc {
@@ -307,7 +314,7 @@ int fill_args(StepArgs& a, const mcc_ctx* ctx, const mcc_particles* P, const int
 // Largest on-chip tile (particles) one CTA can stage: the opt-in shared memory minus the kernel's static part.
 size_t max_tile_particles(const mcc_ctx* ctx, bool f32)
 {
-    const size_t fixed = mcc::cell_kernel_static_smem(f32, true, mcc::kFused) + kStaticSmemReserve;
+    const size_t fixed = ctx->cell_static[f32][1][mcc::kFused] + kStaticSmemReserve;
     const size_t avail = ctx->smem_optin > fixed ? ctx->smem_optin - fixed : 0;
     return avail / mcc::tile_bytes_per_particle(f32);
 }
@@ -316,7 +323,7 @@ size_t max_tile_particles(const mcc_ctx* ctx, bool f32)
 // particle are defined with the kernel, in mcc_cell.cu).
 size_t max_pair_tile_particles(const mcc_ctx* ctx)
 {
-    const size_t fixed = mcc::cell_kernel_static_smem(false, false, mcc::kPair) + kStaticSmemReserve;
+    const size_t fixed = ctx->cell_static[0][0][mcc::kPair] + kStaticSmemReserve;
     const size_t avail = ctx->smem_optin > fixed ? ctx->smem_optin - fixed : 0;
     return avail / mcc::pair_tile_bytes_per_particle();
 }
@@ -324,11 +331,23 @@ size_t max_pair_tile_particles(const mcc_ctx* ctx)
 // Automatic tile: the largest that still lets kAutoCtasPerSm CTAs share an SM's shared memory.
 int auto_tile(const mcc_ctx* ctx, bool f32)
 {
-    const size_t fixed = mcc::cell_kernel_static_smem(f32, true, mcc::kFused) + 1024;
+    const size_t fixed = ctx->cell_static[f32][1][mcc::kFused] + 1024;
     const size_t per_cta = ctx->smem_per_sm / kAutoCtasPerSm;
     const size_t t = per_cta > fixed ? (per_cta - fixed) / mcc::tile_bytes_per_particle(f32) : 64;
     const size_t capmax = max_tile_particles(ctx, f32);
     return (int)(t < capmax ? t : capmax);
+}
+
+// CTAs per SM of a kernel in the launch shape `shape` (what its shared memory and threads follow from), from the cache if the
+// last look-up was for the same.
+template <class F>
+int cached_occupancy(std::atomic<uint64_t>& slot, uint64_t shape, F look_up)
+{
+    const uint64_t c = slot.load(std::memory_order_relaxed);
+    if (c != 0 && (c >> 8) == shape) return (int)(c & 255u);
+    const int b = look_up();
+    if (b > 0) slot.store((shape << 8) | (uint64_t)b, std::memory_order_relaxed);
+    return b;
 }
 
 // Launch one cell-kernel pass over every cell (queue reset, persistent grid of at most max_grid CTAs).
@@ -337,8 +356,8 @@ int run_cells(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, int cap, 
 {
     const size_t per = mode == mcc::kPair ? mcc::pair_tile_bytes_per_particle() : mcc::tile_bytes_per_particle(f32);
     const size_t smem = (size_t)cap * per;
-    if (mcc::set_cell_smem_limit(f32, rel, mode, smem) != cudaSuccess) return MCC_ERR_CUDA;
-    int bps = mcc::cell_kernel_blocks_per_sm(f32, rel, mode, smem);
+    const int bps = cached_occupancy(ctx->cell_occ[f32][rel][mode], smem,
+                                     [&] { return mcc::cell_kernel_blocks_per_sm(f32, rel, mode, smem); });
     if (bps < 1) return MCC_ERR_CUDA;
     int grid = ctx->num_sms * bps;
     if (grid > max_grid) grid = max_grid;
@@ -373,14 +392,14 @@ int run_split(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, cudaStrea
 // Whether the adjoint's working arrays for cells of max_cell particles fit one CTA's shared memory.
 bool adjoint_on_chip(const mcc_ctx* ctx, int32_t max_cell)
 {
-    return mcc::adjoint_work_bytes(max_cell) + mcc::adjoint_static_smem() <= ctx->smem_optin;
+    return mcc::adjoint_work_bytes(max_cell) + ctx->adjoint_static <= ctx->smem_optin;
 }
 
 // Grid of the adjoint kernel: one CTA per cell, at most as many as are resident. slab: bytes each CTA holds of the
 // workspace (0: the slabs are per cell); more than two CTAs per SM only while they hold less than 1 GiB in all.
 int adjoint_grid(const mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, size_t slab)
 {
-    const size_t cta = mcc::adjoint_static_smem() + ctx->smem_reserved +
+    const size_t cta = ctx->adjoint_static + ctx->smem_reserved +
                        (adjoint_on_chip(ctx, max_cell) ? mcc::adjoint_work_bytes(max_cell) : 0);
     int per_sm = mcc::adjoint_ctas_per_sm();
     while (per_sm > 1 && cta * (size_t)per_sm > ctx->smem_per_sm) --per_sm;
@@ -416,6 +435,35 @@ int mcc_create(mcc_ctx** out, int device)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     c->smem_optin = (size_t)optin;
     c->num_sms = sms;
+    // kernels' static shared memory; each may take all the rest as dynamic shared memory
+    cudaError_t attr = cudaSuccess;
+    for (int f32 = 0; f32 < 2; ++f32)
+        for (int rel = 0; rel < 2; ++rel)
+            for (int mode = 0; mode < 4; ++mode) {
+                c->cell_static[f32][rel][mode] = mcc::cell_kernel_static_smem(f32, rel, mode);
+                c->cell_occ[f32][rel][mode] = 0;
+                const cudaError_t e =
+                    mcc::set_cell_smem_limit(f32, rel, mode, c->smem_optin - c->cell_static[f32][rel][mode]);
+                if (e != cudaSuccess) attr = e;
+            }
+    for (int rel = 0; rel < 2; ++rel)
+        for (int cls = 0; cls < mcc::kGroupClasses; ++cls) {
+            cudaFuncAttributes fa;
+            cudaError_t e = cudaFuncGetAttributes(&fa, mcc::group_kernel(true, rel, cls));
+            if (e == cudaSuccess) {
+                c->group_static[rel][cls] = fa.sharedSizeBytes;
+                e = cudaFuncSetAttribute(mcc::group_kernel(true, rel, cls), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(c->smem_optin - fa.sharedSizeBytes));
+            }
+            c->group_occ[rel][cls] = 0;
+            if (e != cudaSuccess) attr = e;
+        }
+    c->adjoint_static = mcc::adjoint_static_smem();
+    const cudaError_t ea = mcc::set_adjoint_smem_limit(c->smem_optin - c->adjoint_static);
+    if (attr != cudaSuccess || ea != cudaSuccess) {
+        delete c;
+        return MCC_ERR_CUDA;
+    }
     // status word, queue counter and the tables, computed here once
     static double tab[mcc::kF64TabDoubles];
     static float tab32[kTab32Floats];
@@ -658,13 +706,7 @@ size_t slab_stride_of(int32_t max_cell, bool f32)
     return ((size_t)max_cell * mcc::tile_bytes_per_particle(f32) + 255) & ~(size_t)255;
 }
 
-size_t group_static_smem(bool f32, bool rel, int cls)
-{
-    if (!f32) return 0;
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, mcc::group_kernel(f32, rel, cls)) != cudaSuccess) return 8192;
-    return fa.sharedSizeBytes;
-}
+size_t group_static_smem(const mcc_ctx* ctx, bool f32, bool rel, int cls) { return f32 ? ctx->group_static[rel][cls] : 0; }
 
 // Shared memory one CTA of the group kernels may take for its groups: its share of the SM (kGroupWarpsPerSm warps in CTAs
 // of group_cta_warps).
@@ -673,7 +715,7 @@ size_t group_budget(const mcc_ctx* ctx, bool f32, bool rel, int cls)
     size_t b = ctx->smem_per_sm / (mcc::kGroupWarpsPerSm / mcc::group_cta_warps(rel));
     b = b > ctx->smem_reserved ? b - ctx->smem_reserved : 0;
     if (b > ctx->smem_optin) b = ctx->smem_optin;
-    const size_t st = group_static_smem(f32, rel, cls);
+    const size_t st = group_static_smem(ctx, f32, rel, cls);
     return b > st ? b - st : 0;
 }
 
@@ -704,7 +746,7 @@ void group_caps(const mcc_ctx* ctx, bool f32, bool rel, int32_t caps[mcc::kGroup
         per_warp = share > fixed ? (share - fixed) / mcc::kGroupBytesPerParticle : 32;
     }
     for (int k = 0; k < mcc::kGroupClasses; ++k) {
-        const size_t st = group_static_smem(f32, rel, k) + mcc::group_shared_bytes(k);
+        const size_t st = group_static_smem(ctx, f32, rel, k) + mcc::group_shared_bytes(k);
         const size_t maxp = ctx->smem_optin > st ? (ctx->smem_optin - st) / mcc::kGroupBytesPerParticle : 0;
         size_t cap = per_warp << k;
         if (k == mcc::kGroupClasses - 1) cap = ctx->group_top > 0 ? (size_t)ctx->group_top : maxp;
@@ -857,12 +899,14 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
             int groups = groups_per_cta(ctx, f32, rel, cls, caps[cls]);
             if (groups > per_sm) groups = per_sm;
             const size_t smem = (size_t)groups * mcc::group_smem(mcc::group_shared_bytes(cls), caps[cls]);
-            const void* fn = mcc::group_kernel(f32, rel, cls);
-            if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                return MCC_ERR_CUDA;
-            int bps = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, groups * (32 << cls), smem) != cudaSuccess || bps < 1)
-                return MCC_ERR_CUDA;
+            const int bps = cached_occupancy(ctx->group_occ[rel][cls], ((uint64_t)smem << 5) | (uint64_t)groups, [&] {
+                int b = 0;
+                return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, mcc::group_kernel(f32, rel, cls),
+                                                                     groups * (32 << cls), smem) == cudaSuccess
+                           ? b
+                           : 0;
+            });
+            if (bps < 1) return MCC_ERR_CUDA;
             int grid = bps * ctx->num_sms;
             if (grid > n_cells) grid = n_cells;
             a.gcls = cls;

@@ -914,6 +914,11 @@ size_t adjoint_static_smem()
     return cudaFuncGetAttributes(&fa, k_adjoint) == cudaSuccess ? fa.sharedSizeBytes : 16384;
 }
 
+cudaError_t set_adjoint_smem_limit(size_t smem)
+{
+    return cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 int adjoint_ctas_per_sm() { return kAdjCtasPerSm; }
 
 cudaError_t launch_adjoint(const StepArgs& a, double lnL, double* ox, double* oy, double* oz, double* gx, double* gy,
@@ -938,8 +943,6 @@ cudaError_t launch_adjoint(const StepArgs& a, double lnL, double* ox, double* oy
     g.tape = tape;
     g.on_chip = on_chip;
     const size_t smem = on_chip ? adjoint_work_bytes(max_cell) : 0;
-    const cudaError_t e = cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     k_adjoint<<<grid, kThreads, smem, st>>>(g);
     return cudaGetLastError();
 }

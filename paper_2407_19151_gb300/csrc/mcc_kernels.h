@@ -154,6 +154,7 @@ size_t adjoint_slab_bytes(int32_t max_cell, int32_t max_epairs, bool on_chip);
 size_t adjoint_work_bytes(int32_t max_cell);  // working arrays of one cell
 size_t adjoint_static_smem();
 int adjoint_ctas_per_sm();
+cudaError_t set_adjoint_smem_limit(size_t smem);
 cudaError_t launch_adjoint(const StepArgs& a, double lnL, double* ox, double* oy, double* oz, double* gx, double* gy,
                            double* gz, double* gw, double* glnL, char* slab, int32_t max_cell, int32_t max_epairs,
                            int32_t tape, bool on_chip, int grid, cudaStream_t st);
