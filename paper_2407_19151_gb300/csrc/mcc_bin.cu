@@ -409,7 +409,9 @@ __global__ void __launch_bounds__(kBinThreads) k_segsort_w(const int64_t* __rest
     }
 }
 
-// Four elements per thread and iteration, their permuted reads issued together (more reads in flight).
+// Four elements per thread and iteration, their permuted reads issued together (more reads in flight). A shuffled
+// permutation reads a whole sector per element, so what bounds it is how much of `in` stays in L2: the permutation and the
+// output, touched once, are marked to leave first (3.3e7 shuffled particles, three floats and a double: 1.56 -> 1.52 ms).
 template <class T>
 __global__ void k_gather(const T* __restrict__ in, const int32_t* __restrict__ perm, int64_t n, T* __restrict__ out)
 {
@@ -419,12 +421,12 @@ __global__ void k_gather(const T* __restrict__ in, const int32_t* __restrict__ p
         int32_t p[U];
         T v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) p[u] = base + u * stride < n ? perm[base + u * stride] : 0;
+        for (int u = 0; u < U; ++u) p[u] = base + u * stride < n ? __ldcs(perm + base + u * stride) : 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) v[u] = base + u * stride < n ? __ldg(in + p[u]) : T(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (base + u * stride < n) out[base + u * stride] = v[u];
+            if (base + u * stride < n) __stcs(out + base + u * stride, v[u]);
     }
 }
 
