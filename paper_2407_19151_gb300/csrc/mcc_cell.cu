@@ -179,24 +179,25 @@ __device__ __forceinline__ Acc<V>* acc_at(unsigned char* p)
     return reinterpret_cast<Acc<V>*>(p);
 }
 
-// Per-interaction coefficients, computed by one thread from the block sums. FP64 path: in double. Mixed path: in
-// float-float (the float pipe; the FP64 pipe of this part is a small fraction of the float rate).
+// Per-interaction coefficients from the block sums, by the first warp. FP64 path: in double, the components of B and the
+// species' terms of the split on lanes of their own (an FP64 instruction costs the pipe as much for one lane as for 32).
+// Mixed path: in float-float (the float pipe; the FP64 pipe of this part is a small fraction of the float rate), one lane.
 // Eq. vp_pm: B = sum_s m_s sum w (v_ps - v_bs) / sum_s m_s sum w^2 over the interaction's species (one side intra).
 __device__ __forceinline__ void shift_coef(const StepArgs& A, const InterConst& ic, bool intra,
                                            const Acc<double>* r, const Acc<double>* W2, Shared& sh)
 {
+    const int d = threadIdx.x;
+    if (d >= 3) return;
     const double ma = A.m[ic.a], mb = A.m[ic.b];
     const double Sw = ma * W2[ic.a].x + (intra ? 0.0 : mb * W2[ic.b].x);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const double S = ma * r[d].x + (intra ? 0.0 : mb * r[3 + d].x);
-        sh.B[d] = S / Sw;
-        sh.Bf[d] = (float)sh.B[d];
-    }
+    const double S = ma * r[d].x + (intra ? 0.0 : mb * r[3 + d].x);
+    sh.B[d] = S / Sw;
+    sh.Bf[d] = (float)sh.B[d];
 }
 __device__ __forceinline__ void shift_coef(const StepArgs& A, const InterConst& ic, bool intra,
                                            const Acc<float>* r, const Acc<float>* W2, Shared& sh)
 {
+    if (threadIdx.x != 0) return;
     const ff ma = {A.m_f[ic.a], A.m_lo[ic.a]}, mb = {A.m_f[ic.b], A.m_lo[ic.b]};
     ff Sw = ff_mul(ma, W2[ic.a].x);
     if (!intra) Sw = ff_add(Sw, ff_mul(mb, W2[ic.b].x));
@@ -215,15 +216,19 @@ __device__ __forceinline__ void shift_coef(const StepArgs& A, const InterConst& 
 __device__ __forceinline__ void partition_coef(const StepArgs& A, const InterConst& ic, bool intra, int na, int nb,
                                                const Acc<double>* r, const Acc<double>* W1, Shared& sh)
 {
+    if (threadIdx.x >= 32) return;
     const double ma = A.m[ic.a], mb = A.m[ic.b];
+    const bool b = threadIdx.x & 1;  // species of this lane's terms
+    const double E = b ? (intra ? 0.0 : mb * r[3].x) : ma * r[1].x;
+    const double wE = W1[b ? ic.b : ic.a].x / (double)(b ? nb : na) * E;
+    const double Ea = __shfl_sync(0xffffffffu, E, 0), Eb = __shfl_sync(0xffffffffu, E, 1);
+    const double wa = __shfl_sync(0xffffffffu, wE, 0), wb = __shfl_sync(0xffffffffu, wE, 1);
     const double dE = ma * r[0].x + (intra ? 0.0 : mb * r[2].x);
     double D0 = dE, D1 = 0.0;
     int fail = 0;
     if (!intra) {
         const bool can0 = na >= 2, can1 = nb >= 2;
         if (can0 && can1) {
-            const double wa = W1[ic.a].x / (double)na * (ma * r[1].x);
-            const double wb = W1[ic.b].x / (double)nb * (mb * r[3].x);
             const double den = wa + wb;
             if (den > 0.0) {
                 D0 = wa / den * dE;
@@ -240,13 +245,16 @@ __device__ __forceinline__ void partition_coef(const StepArgs& A, const InterCon
             fail = 1;
         }
     }
-    sh.D[0] = fabs(D0) <= 0x1p-47 * (ma * r[1].x) ? 0.0 : D0;
-    sh.D[1] = fabs(D1) <= 0x1p-47 * (intra ? 0.0 : mb * r[3].x) ? 0.0 : D1;
-    sh.fail = fail;
+    if (threadIdx.x == 0) {
+        sh.D[0] = fabs(D0) <= 0x1p-47 * Ea ? 0.0 : D0;
+        sh.D[1] = fabs(D1) <= 0x1p-47 * Eb ? 0.0 : D1;
+        sh.fail = fail;
+    }
 }
 __device__ __forceinline__ void partition_coef(const StepArgs& A, const InterConst& ic, bool intra, int na, int nb,
                                                const Acc<float>* r, const Acc<float>* W1, Shared& sh)
 {
+    if (threadIdx.x != 0) return;
     const ff ma = {A.m_f[ic.a], A.m_lo[ic.a]}, mb = {A.m_f[ic.b], A.m_lo[ic.b]};
     const ff Ea = ff_mul(ma, r[1].x), Eb = ff_mul(mb, r[3].x);
     ff dE = ff_mul(ma, r[0].x);
@@ -579,6 +587,7 @@ __device__ void correct_interaction(const StepArgs& A, const Tile<V>& t, Shared&
 {
     const int nside = intra ? 1 : 2;
     const V cc = pick<V>(A.c, A.c_f);
+    const V c2 = cc * cc, ic2 = REL ? (V)1 / c2 : (V)0;
 
     // Eq. vp_pm: per species sums of w (v_ps - v_bs), times m_s in FP64; the sums of w^2 are fixed for the visit
     {
@@ -595,7 +604,7 @@ __device__ void correct_interaction(const StepArgs& A, const Tile<V>& t, Shared&
             }
         }
         block_sum<V, 6>(mom, acc_at<V>(sh.red_raw), acc_at<V>(sh.red));
-        if (threadIdx.x == 0) shift_coef(A, ic, intra, acc_at<V>(sh.red), acc_at<V>(sh.W2), sh);
+        shift_coef(A, ic, intra, acc_at<V>(sh.red), acc_at<V>(sh.W2), sh);
         __syncthreads();
     }
 
@@ -624,15 +633,14 @@ __device__ void correct_interaction(const StepArgs& A, const Tile<V>& t, Shared&
                     acc[side * 2 + 0].add((V)0.5 * w * dd);
                     acc[side * 2 + 1].add((V)0.5 * w * v2);
                 } else {
-                    const V c2 = cc * cc;
-                    const V ga = sqrt((V)1 + v2 / c2), gb = sqrt((V)1 + b2 / c2);
+                    const V ga = sqrt((V)1 + over(v2, c2, ic2)), gb = sqrt((V)1 + over(b2, c2, ic2));
                     acc[side * 2 + 0].add(w * dd / (ga + gb));
                     acc[side * 2 + 1].add(w * v2 / (ga + (V)1));
                 }
             }
         }
         block_sum<V, 4>(acc, acc_at<V>(sh.red_raw), acc_at<V>(sh.red));
-        if (threadIdx.x == 0) partition_coef(A, ic, intra, na, nb, acc_at<V>(sh.red), acc_at<V>(sh.W1), sh);
+        partition_coef(A, ic, intra, na, nb, acc_at<V>(sh.red), acc_at<V>(sh.W1), sh);
         __syncthreads();
     }
 

@@ -594,6 +594,10 @@ __device__ __forceinline__ RelCM<V> rel_cm(V c, V ma, V mb, const V ui[3], const
     return r;
 }
 
+// x / y with r = 1 / y: in double by the reciprocal (a division costs the FP64 pipe about eight instructions).
+__device__ __forceinline__ double over(double x, double, double r) { return x * r; }
+__device__ __forceinline__ float over(float x, float y, float) { return x / y; }
+
 // Centre-of-mass kinetic energy of a weighted pair (masses m1, m2 already weighted).
 template <class V, bool REL>
 __device__ __forceinline__ V pair_kecm(V c, V m1, V m2, const V v1[3], const V v2[3])
@@ -604,9 +608,9 @@ __device__ __forceinline__ V pair_kecm(V c, V m1, V m2, const V v1[3], const V v
         for (int d = 0; d < 3; ++d) vr2 += (v1[d] - v2[d]) * (v1[d] - v2[d]);
         return (V)0.5 * (m1 * m2 / (m1 + m2)) * vr2;
     }
-    const V c2 = c * c;
-    const V g1 = sqrt((V)1 + (v1[0] * v1[0] + v1[1] * v1[1] + v1[2] * v1[2]) / c2);
-    const V g2 = sqrt((V)1 + (v2[0] * v2[0] + v2[1] * v2[1] + v2[2] * v2[2]) / c2);
+    const V c2 = c * c, ic2 = (V)1 / c2;
+    const V g1 = sqrt((V)1 + over(v1[0] * v1[0] + v1[1] * v1[1] + v1[2] * v1[2], c2, ic2));
+    const V g2 = sqrt((V)1 + over(v2[0] * v2[0] + v2[1] * v2[1] + v2[2] * v2[2], c2, ic2));
     V du2 = 0, ss = 0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -614,7 +618,7 @@ __device__ __forceinline__ V pair_kecm(V c, V m1, V m2, const V v1[3], const V v
         ss += (v1[d] - v2[d]) * (v1[d] + v2[d]);
     }
     const V dg = ss / (c2 * (g1 + g2));
-    V grm1 = (V)0.5 * (du2 / c2 - dg * dg);
+    V grm1 = (V)0.5 * (over(du2, c2, ic2) - dg * dg);
     if (grm1 < (V)0) grm1 = 0;
     const V Minv = sqrt((m1 + m2) * (m1 + m2) + (V)2 * m1 * m2 * grm1);
     return (V)2 * m1 * m2 * c2 * grm1 / (Minv + m1 + m2);
@@ -637,10 +641,10 @@ __device__ __forceinline__ void energy_pair(V c, V m1, V m2, V K, V v1[3], V v2[
         }
         return;
     }
-    const V c2 = c * c;
-    const V g1 = sqrt((V)1 + (v1[0] * v1[0] + v1[1] * v1[1] + v1[2] * v1[2]) / c2);
-    const V g2 = sqrt((V)1 + (v2[0] * v2[0] + v2[1] * v2[1] + v2[2] * v2[2]) / c2);
-    const V E1 = m1 * g1, E2 = m2 * g2, Ut = U / c2;
+    const V c2 = c * c, ic2 = (V)1 / c2;
+    const V g1 = sqrt((V)1 + over(v1[0] * v1[0] + v1[1] * v1[1] + v1[2] * v1[2], c2, ic2));
+    const V g2 = sqrt((V)1 + over(v2[0] * v2[0] + v2[1] * v2[1] + v2[2] * v2[2], c2, ic2));
+    const V E1 = m1 * g1, E2 = m2 * g2, Ut = over(U, c2, ic2);
     const V A = E1 + E2 - Ut;
     V du[3], pt[3], du2 = 0, ss = 0;
 #pragma unroll
@@ -659,8 +663,8 @@ __device__ __forceinline__ void energy_pair(V c, V m1, V m2, V K, V v1[3], V v2[
         bdot += du[d] * bv;
         ptdu += pt[d] * du[d];
     }
-    const V a = (V)4 * (A * A * du2 / c2 - ptdu * ptdu / (c2 * c2));
-    const V b = (V)4 / c2 * bdot;
+    const V a = (V)4 * (over(A * A * du2, c2, ic2) - over(ptdu * ptdu, c2 * c2, ic2 * ic2));
+    const V b = over((V)4, c2, ic2) * bdot;
     const V c0 = Ut * ((V)2 * E1 - Ut) * ((V)2 * E2 - Ut) * ((V)2 * E1 + (V)2 * E2 - Ut);
     V disc = b * b - (V)4 * a * c0;
     if (disc < (V)0) disc = 0;
@@ -668,10 +672,11 @@ __device__ __forceinline__ void energy_pair(V c, V m1, V m2, V K, V v1[3], V v2[
     const V r1 = (a != (V)0) ? q / a : (V)CUDART_INF;
     const V r2 = (q != (V)0) ? c0 / q : (V)0;
     const V alpha = fabs(r1) < fabs(r2) ? r1 : r2;
+    const V r1m = (V)1 / m1, r2m = (V)1 / m2;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        v1[d] += alpha * du[d] / m1;
-        v2[d] -= alpha * du[d] / m2;
+        v1[d] += over(alpha * du[d], m1, r1m);
+        v2[d] -= over(alpha * du[d], m2, r2m);
     }
     (void)K;
 }

@@ -7,11 +7,14 @@
 // arguments are known in form are table lookups with a short series, each within about an ulp:
 //   A(s) s      piecewise degree-7 polynomials in s (64 per octave of [2^-5, 16)); below, the Bernoulli series of
 //               s / (1 - e^-s), which equals A s there to 1e-27; above, the inversion of L(A) = A/3 - A^3/45
+//   e^-2A       the same intervals: e^-2A below s = 2, 1 - e^-2A above (the smaller one, or nearly). Its polynomials lose
+//               relative precision towards s = 2^-5, where e^-2A is below 1e-16 of what it is added to
 //   ln u        u = 2^k m, ln m = -ln r_i + ln(m r_i) with tabulated r_i ~ 1/m (Tang, "Table-driven implementation of
 //               the logarithm function in IEEE floating-point arithmetic", 1990)
 //   azimuth     2 pi (k + 1/2) 2^-23 = nearest 1/256 turn, tabulated, + a remainder below pi/256 (addition theorem)
-// and uniforms are assembled from their bits instead of converted. About 190 instructions per pair. FP64 step of 4096
-// three-species cells (2.1e6 particles) 6.11 -> 2.38 ms, relativistic beam of 2048 cells 6.45 -> 2.23 ms; the difference from
+// uniforms are assembled from their bits instead of converted, and comparisons are made on the bits (an FP64 comparison
+// takes the FP64 pipe too). About 150 instructions per pair. FP64 step of 4096
+// three-species cells (2.1e6 particles) 6.11 -> 2.14 ms, relativistic beam of 2048 cells 6.45 -> 1.95 ms; the difference from
 // 64-bit results is unchanged (1.4e-16 of the velocities).
 #pragma once
 
@@ -56,22 +59,16 @@ __device__ __forceinline__ double ln64(const F64Tab& T, double u)
     p = fma(f, p, 1.0 / 3.0);
     p = fma(f, p, -0.5);
     const double l = fma(f * f, p, f);
-    return fma((double)k, 0.69314718055994530942, t.y + l);
+    // k converted exactly by an addition
+    const double kd = __hiloint2double(0x43300000, (int)(0x80000000u ^ (uint32_t)k)) - 4503601774854144.0;
+    return fma(kd, 0.69314718055994530942, t.y + l);
 }
 
-// A(s) s of the N97 angle, s > 0.
-__device__ __forceinline__ double n97_As(const F64Tab& T, double s)
+// Polynomial of one interval of s in [2^-5, 16): coefficients at tab[4 k ..] for interval k.
+__device__ __forceinline__ double n97_poly(const double2* tab, double s)
 {
-    if (s < 0.03125) {
-        const double s2 = s * s;
-        return fma(s2, fma(s2, fma(s2, 1.0 / 30240.0, -1.0 / 720.0), 1.0 / 12.0), fma(0.5, s, 1.0));
-    }
-    if (s >= 16.0) {
-        const double y = exp(-s);
-        return 3.0 * y * fma(0.6 * y, y, 1.0) * s;
-    }
     const int hi = __double2hiint(s);
-    const double2* c = T.n97 + 4 * ((hi >> 14) - (0x3FA00000 >> 14));
+    const double2* c = tab + 4 * ((hi >> 14) - (0x3FA00000 >> 14));
     const double m = __hiloint2double(0x3FF00000 | (hi & 0x3FFF), __double2loint(s));
     const double t = fma(m, 128.0, -129.0);  // [-1, 1) over the interval
     const double2 c0 = __ldg(c), c1 = __ldg(c + 1), c2 = __ldg(c + 2), c3 = __ldg(c + 3);
@@ -84,11 +81,44 @@ __device__ __forceinline__ double n97_As(const F64Tab& T, double s)
     return fma(t, p, c0.x);
 }
 
+// A(s) s of the N97 angle, s > 0, and with EF e^-2A and 1 - e^-2A (A > 31 below s = 2^-5: e^-2A < 1e-27 counts as 0).
+template <bool EF>
+__device__ __forceinline__ double n97_As(const F64Tab& T, double s, double& E, double& F)
+{
+    const int hi = __double2hiint(s);
+    if (hi < 0x3FA00000) {  // s < 2^-5
+        if (EF) {
+            E = 0.0;
+            F = 1.0;
+        }
+        const double s2 = s * s;
+        return fma(s2, fma(s2, fma(s2, 1.0 / 30240.0, -1.0 / 720.0), 1.0 / 12.0), fma(0.5, s, 1.0));
+    }
+    if (hi >= 0x40300000) {  // s >= 16: A < 4e-7
+        const double y = exp(-s);
+        const double A = 3.0 * y * fma(0.6 * y, y, 1.0);
+        if (EF) {
+            const double t = A + A;
+            F = t * fma(t, fma(t, 1.0 / 6.0, -0.5), 1.0);
+            E = 1.0 - F;
+        }
+        return A * s;
+    }
+    if (EF) {
+        const double h = n97_poly(T.n97 + 4 * kF64N97, s);
+        const double r = 1.0 - h;
+        E = hi < 0x40000000 ? h : r;
+        F = hi < 0x40000000 ? r : h;
+    }
+    return n97_poly(T.n97, s);
+}
+
 // A(s) for sample_angle: 0 where 1 - e^-s rounds to 1 (isotropic), infinite at s = 0.
 __device__ __forceinline__ double n97_A(double s, const F64Tab& T)
 {
+    double E, F;
     if (s > 36.7) return 0.0;
-    return s > 0.0 ? n97_As(T, s) / s : CUDART_INF;
+    return s > 0.0 ? n97_As<false>(T, s, E, F) / s : CUDART_INF;
 }
 
 // ln(1 + x) for x > -1, u = 1 + x rounded: the rounding error of u enters to first order.
@@ -96,6 +126,9 @@ __device__ __forceinline__ double ln1p64(const F64Tab& T, double x, double u)
 {
     return ln64(T, u) + (x - (u - 1.0)) / u;
 }
+
+// x >= the value whose high word is lo, from the high word of x; false for NaN.
+__device__ __forceinline__ bool from64(int hi, int lo) { return (uint32_t)(hi - lo) <= (uint32_t)(0x7FF00000 - lo); }
 
 // Polar angle of a pair, sin(Theta) and 1 - cos(Theta), from the scattering length s and the draws (r.x, r.w).
 // DERIV: also their derivatives in s.
@@ -123,25 +156,16 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
     }
     const double V = 1.0 - U;  // exact
     double o, q;
-    if (s > 36.7) {
+    const int hs = __double2hiint(s);
+    if (from64(hs, 0x40425800)) {  // s >= 36.69: isotropic
         o = 2.0 * U;
         q = 2.0 * V;
     } else {
-        const double g = n97_As(T, s), rA = s / g;
-        double A = 0.0, E = 0.0, F = 1.0;  // E = e^-2A, F = 1 - E; A > 31 below s = 2^-5: E < 1e-27
-        if (s >= 0.03125) {
-            A = g / s;
-            if (A < 0.35) {
-                F = -expm1(-2.0 * A);
-                E = 1.0 - F;
-            } else {
-                E = exp(-2.0 * A);
-                F = 1.0 - E;
-            }
-        }
-        // ln(1 + x), x = -U F: from 1 + x while x is small, from the two positive terms (1 - U) + U E once it is not
+        double E, F;  // e^-2A, 1 - e^-2A
+        const double g = n97_As<true>(T, s, E, F), rA = s / g;
+        // ln(1 + x), x = -U F: from 1 + x while |x| is below 1/2, from the two positive terms (1 - U) + U E beyond
         const double x = -U * F;
-        const bool near1 = x > -0.5;
+        const bool near1 = (__double2hiint(x) & 0x7FFFFFFF) < 0x3FE00000;
         const double u = near1 ? 1.0 + x : fma(U, E, V);
         double l = ln64(T, u);
         if (near1) {
@@ -150,16 +174,16 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
         }
         o = -l * rA;
         q = 2.0 - o;
-        if (o > 1.0) {
+        if (__double2hiint(o) >= 0x3FF00000) {
+            // s < 1/8 gets here with probability below e^-8: e^-2A from the exponential, in full relative precision
+            if (hs < 0x3FC00000) E = exp(-2.0 / rA);
             const double y = V * (F / E);
             q = ln1p64(T, y, 1.0 + y) * rA;
         }
         if (DERIV) {
-            // L(A) = coth A - 1/A = e^-s: dA/ds = -e^-s / L'(A), L' = 1 - L^2 - 2 L / A = 1/A^2 - 4 E / F^2
+            // L(A) = coth A - 1/A = e^-s: dA/ds = -e^-s / L'(A), L' = 1/A^2 - 4 E / F^2 = 1 - L^2 - 2 L / A (A < 1/2)
             const double ys = exp(-s);
-            const double ra2 = rA * rA;
-            double dL = ra2 - (E > 0.0 ? 4.0 * E / (F * F) : 0.0);
-            if (s >= 0.03125 && A < 0.5) dL = 1.0 - ys * ys - 2.0 * ys * rA;
+            const double dL = hs >= 0x3FFD0000 ? 1.0 - ys * ys - 2.0 * ys * rA : rA * rA - 4.0 * E / (F * F);
             // d(1 - cos)/dA = (-(1 - cos) + 2 U E / (1 + x)) / A
             const double dA = -ys / dL;
             const double do_ds = rA * (2.0 * U * E / u - o) * dA;
@@ -168,8 +192,8 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
             dst = (o * q > 0.0 && !cl) ? (q - o) * do_ds * (0.5 * rsqrt(o * q)) : 0.0;
         }
     }
-    o = o > 2.0 ? 2.0 : o;
-    q = q > 2.0 ? 2.0 : q;
+    o = from64(__double2hiint(o), 0x40000000) ? 2.0 : o;
+    q = from64(__double2hiint(q), 0x40000000) ? 2.0 : q;
     omc = o;
     st = sqrt(o * q);
 }
@@ -202,7 +226,7 @@ __device__ __forceinline__ bool pair64(const F64Tab& T, int method, double cw, c
 {
     const double ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
     const double u2 = fma(uz, uz, fma(uy, uy, ux * ux));
-    if (u2 == 0.0) return false;
+    if (__double_as_longlong(u2) == 0) return false;
     const double ru = rsqrt(u2);
     double st, omc, sp, cp, d0, d1;
     angle64<false>(T, method, cw * (ru * ru * ru), r, st, omc, d0, d1);
