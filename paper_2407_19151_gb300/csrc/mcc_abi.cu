@@ -127,7 +127,7 @@ void n97_table(float* g, float* dh)
     }
 }
 
-// Tables of mcc_pair64.cuh: Chebyshev interpolants of A(s) s and of e^-2A or 1 - e^-2A as monomials in the interval's own variable t in [-1, 1],
+// Tables of mcc_pair64.cuh: Chebyshev interpolants of 1 / A(s) and of e^-2A or 1 - e^-2A as monomials in the interval's own variable t in [-1, 1],
 // multiples of 1/256 turn, and the reciprocals and logarithms of mantissas in [0.6875, 1.375).
 void f64_tables(double* out)
 {
@@ -147,7 +147,7 @@ void f64_tables(double* out)
         T f[2][N];
         for (int j = 0; j < N; ++j) {
             const T s = a + w * (1 + cosine[1][j]) / 2, A = n97_root(s);
-            f[0][j] = A * s;
+            f[0][j] = 1 / A;
             f[1][j] = i / 64 < 6 ? std::exp(-2 * A) : -std::expm1(-2 * A);  // s < 2; s >= 2
         }
         for (int k = 0; k < 2; ++k) {

@@ -5,16 +5,17 @@
 // of its instructions were the pair's: two Newton steps on the N97 root (expm1, sinh, three divisions each), expm1,
 // log1p, log, exp, sincospi and eight divisions, about 600 FP64 instructions per pair. Here the functions whose
 // arguments are known in form are table lookups with a short series, each within about an ulp:
-//   A(s) s      piecewise degree-7 polynomials in s (64 per octave of [2^-5, 16)); below, the Bernoulli series of
-//               s / (1 - e^-s), which equals A s there to 1e-27; above, the inversion of L(A) = A/3 - A^3/45
+//   1 / A(s)    piecewise degree-7 polynomials in s (64 per octave of [2^-5, 16)); below, the series of 1 - e^-s, which
+//               equals 1 / A there to 1e-27; above, the inversion of L(A) = A/3 - A^3/45
 //   e^-2A       the same intervals: e^-2A below s = 2, 1 - e^-2A above (the smaller one, or nearly). Its polynomials lose
 //               relative precision towards s = 2^-5, where e^-2A is below 1e-16 of what it is added to
 //   ln u        u = 2^k m, ln m = -ln r_i + ln(m r_i) with tabulated r_i ~ 1/m (Tang, "Table-driven implementation of
 //               the logarithm function in IEEE floating-point arithmetic", 1990)
+//               one logarithm per pair: of whichever of 1 - cos and 1 + cos is smaller, the other being 2 minus it
 //   azimuth     2 pi (k + 1/2) 2^-23 = nearest 1/256 turn, tabulated, + a remainder below pi/256 (addition theorem)
 // uniforms are assembled from their bits instead of converted, and comparisons are made on the bits (an FP64 comparison
-// takes the FP64 pipe too). About 150 instructions per pair. FP64 step of 4096
-// three-species cells (2.1e6 particles) 6.11 -> 2.14 ms, relativistic beam of 2048 cells 6.45 -> 1.95 ms; the difference from
+// takes the FP64 pipe too). About 120 instructions per pair. FP64 step of 4096
+// three-species cells (2.1e6 particles) 6.11 -> 2.06 ms, relativistic beam of 2048 cells 6.45 -> 1.93 ms; the difference from
 // 64-bit results is unchanged (1.4e-16 of the velocities).
 #pragma once
 
@@ -43,8 +44,8 @@ __device__ __forceinline__ void turn64(const F64Tab& T, uint32_t r, double& cs, 
     sn = a.y + fma(a.y, cm, a.x * sd);
 }
 
-// ln u for a positive normal u.
-__device__ __forceinline__ double ln64(const F64Tab& T, double u)
+// ln(u + c) for a positive normal u and a c below its rounding (to first order).
+__device__ __forceinline__ double ln64(const F64Tab& T, double u, double c = 0.0)
 {
     const int hi = __double2hiint(u);
     const int ix = hi - 0x3FE60000;  // mantissas are taken in [0.6875, 1.375)
@@ -58,7 +59,9 @@ __device__ __forceinline__ double ln64(const F64Tab& T, double u)
     p = fma(f, p, -1.0 / 4.0);
     p = fma(f, p, 1.0 / 3.0);
     p = fma(f, p, -0.5);
-    const double l = fma(f * f, p, f);
+    // c / u with 2^-k r_i for 1 / u
+    const double ru = __hiloint2double(__double2hiint(t.x) - (k << 20), __double2loint(t.x));
+    const double l = fma(f * f, p, fma(c, ru, f));
     // k converted exactly by an addition
     const double kd = __hiloint2double(0x43300000, (int)(0x80000000u ^ (uint32_t)k)) - 4503601774854144.0;
     return fma(kd, 0.69314718055994530942, t.y + l);
@@ -81,9 +84,9 @@ __device__ __forceinline__ double n97_poly(const double2* tab, double s)
     return fma(t, p, c0.x);
 }
 
-// A(s) s of the N97 angle, s > 0, and with EF e^-2A and 1 - e^-2A (A > 31 below s = 2^-5: e^-2A < 1e-27 counts as 0).
+// 1 / A(s) of the N97 angle, s > 0, and with EF e^-2A and 1 - e^-2A (A > 31 below s = 2^-5: e^-2A < 1e-27 counts as 0).
 template <bool EF>
-__device__ __forceinline__ double n97_As(const F64Tab& T, double s, double& E, double& F)
+__device__ __forceinline__ double n97_rA(const F64Tab& T, double s, double& E, double& F)
 {
     const int hi = __double2hiint(s);
     if (hi < 0x3FA00000) {  // s < 2^-5
@@ -91,8 +94,13 @@ __device__ __forceinline__ double n97_As(const F64Tab& T, double s, double& E, d
             E = 0.0;
             F = 1.0;
         }
-        const double s2 = s * s;
-        return fma(s2, fma(s2, fma(s2, 1.0 / 30240.0, -1.0 / 720.0), 1.0 / 12.0), fma(0.5, s, 1.0));
+        double p = fma(s, -1.0 / 40320.0, 1.0 / 5040.0);
+        p = fma(s, p, -1.0 / 720.0);
+        p = fma(s, p, 1.0 / 120.0);
+        p = fma(s, p, -1.0 / 24.0);
+        p = fma(s, p, 1.0 / 6.0);
+        p = fma(s, p, -0.5);
+        return fma(s * s, p, s);
     }
     if (hi >= 0x40300000) {  // s >= 16: A < 4e-7
         const double y = exp(-s);
@@ -102,7 +110,7 @@ __device__ __forceinline__ double n97_As(const F64Tab& T, double s, double& E, d
             F = t * fma(t, fma(t, 1.0 / 6.0, -0.5), 1.0);
             E = 1.0 - F;
         }
-        return A * s;
+        return 1.0 / A;
     }
     if (EF) {
         const double h = n97_poly(T.n97 + 4 * kF64N97, s);
@@ -118,13 +126,7 @@ __device__ __forceinline__ double n97_A(double s, const F64Tab& T)
 {
     double E, F;
     if (s > 36.7) return 0.0;
-    return s > 0.0 ? n97_As<false>(T, s, E, F) / s : CUDART_INF;
-}
-
-// ln(1 + x) for x > -1, u = 1 + x rounded: the rounding error of u enters to first order.
-__device__ __forceinline__ double ln1p64(const F64Tab& T, double x, double u)
-{
-    return ln64(T, u) + (x - (u - 1.0)) / u;
+    return s > 0.0 ? 1.0 / n97_rA<false>(T, s, E, F) : CUDART_INF;
 }
 
 // x >= the value whose high word is lo, from the high word of x; false for NaN.
@@ -162,23 +164,27 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
         q = 2.0 * V;
     } else {
         double E, F;  // e^-2A, 1 - e^-2A
-        const double g = n97_As<true>(T, s, E, F), rA = s / g;
-        // ln(1 + x), x = -U F: from 1 + x while |x| is below 1/2, from the two positive terms (1 - U) + U E beyond
+        const double rA = n97_rA<true>(T, s, E, F);
+        // 1 - cos = -ln(1 + x) / A, x = -U F: 1 + x itself while |x| is below 1/2, the two positive terms (1 - U) + U E
+        // beyond. Where that exceeds 1, 1 + cos = ln(1 + y) / A, y = (1 - U) (e^2A - 1), takes its place.
         const double x = -U * F;
         const bool near1 = (__double2hiint(x) & 0x7FFFFFFF) < 0x3FE00000;
         const double u = near1 ? 1.0 + x : fma(U, E, V);
-        double l = ln64(T, u);
-        if (near1) {
-            const double c = x - (u - 1.0);
-            l += fma(-c, x, c);
-        }
-        o = -l * rA;
-        q = 2.0 - o;
-        if (__double2hiint(o) >= 0x3FF00000) {
+        const bool far = __double_as_longlong(u * u) < __double_as_longlong(E);  // 1 + x < e^-A
+        double z = x, a = u;
+        if (far) {
             // s < 1/8 gets here with probability below e^-8: e^-2A from the exponential, in full relative precision
             if (hs < 0x3FC00000) E = exp(-2.0 / rA);
-            const double y = V * (F / E);
-            q = ln1p64(T, y, 1.0 + y) * rA;
+            z = V * (F / E);
+            a = 1.0 + z;
+        }
+        const double l = ln64(T, a, near1 || far ? z - (a - 1.0) : 0.0);
+        o = (far ? l : -l) * rA;
+        q = 2.0 - o;
+        if (far) {
+            const double y = o;
+            o = q;
+            q = y;
         }
         if (DERIV) {
             // L(A) = coth A - 1/A = e^-s: dA/ds = -e^-s / L'(A), L' = 1/A^2 - 4 E / F^2 = 1 - L^2 - 2 L / A (A < 1/2)
