@@ -127,7 +127,7 @@ void n97_table(float* g, float* dh)
     }
 }
 
-// Tables of mcc_pair64.cuh: Chebyshev interpolants of 1 / A(s) and of e^-2A or 1 - e^-2A as monomials in the interval's own variable t in [-1, 1],
+// Tables of mcc_pair64.cuh: Chebyshev interpolants of 1 / A(s), of e^-2A or 1 - e^-2A and of s A' / A as monomials in the interval's own variable t in [-1, 1],
 // multiples of 1/256 turn, and the reciprocals and logarithms of mantissas in [0.6875, 1.375).
 void f64_tables(double* out)
 {
@@ -144,13 +144,16 @@ void f64_tables(double* out)
     for (int i = 0; i < kF64N97; ++i) {
         const T w = std::ldexp(T(1) / 64, i / 64 - 5);  // interval width
         const T a = std::ldexp(T(1), i / 64 - 5) + (i % 64) * w;
-        T f[2][N];
+        T f[3][N];
         for (int j = 0; j < N; ++j) {
             const T s = a + w * (1 + cosine[1][j]) / 2, A = n97_root(s);
             f[0][j] = 1 / A;
             f[1][j] = i / 64 < 6 ? std::exp(-2 * A) : -std::expm1(-2 * A);  // s < 2; s >= 2
+            T L, dL;
+            langevin(A, L, dL);
+            f[2][j] = -s * std::exp(-s) / (A * dL);  // s A' / A
         }
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < 3; ++k) {
             T c[N] = {0, 0, 0, 0, 0, 0, 0, 0};
             for (int m = 0; m < N; ++m) {
                 T b = 0;
@@ -161,7 +164,7 @@ void f64_tables(double* out)
             for (int q = 0; q < N; ++q) out[N * (kF64N97 * k + i) + q] = (double)c[q];
         }
     }
-    double* turn = out + 2 * N * kF64N97;
+    double* turn = out + 3 * N * kF64N97;
     for (int i = 0; i < kF64Turn; ++i) {
         turn[2 * i] = i % 128 == 64 ? 0.0 : std::cos(2.0 * M_PI * i / kF64Turn);
         turn[2 * i + 1] = i % 128 == 0 ? 0.0 : std::sin(2.0 * M_PI * i / kF64Turn);
@@ -307,7 +310,7 @@ int fill_args(StepArgs& a, const mcc_ctx* ctx, const mcc_particles* P, const int
     a.queue = ctx->dbuf + 1;
     const char* base = reinterpret_cast<const char*>(ctx->dbuf) + kTabOffset;
     a.t64.n97 = reinterpret_cast<const double2*>(base);
-    a.t64.turn = a.t64.n97 + 8 * mcc::kF64N97;
+    a.t64.turn = a.t64.n97 + 12 * mcc::kF64N97;
     a.t64.ln = a.t64.turn + mcc::kF64Turn;
     a.n97_f32 = reinterpret_cast<const float*>(base + kTab64Bytes);
     a.n97_dh32 = a.n97_f32 + (mcc::kN97Nodes + 1);

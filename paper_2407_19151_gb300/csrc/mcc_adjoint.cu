@@ -15,7 +15,7 @@
 //   rollback (Sec. 5.2) when the correction fails: v_after = v_before.
 // A Delta E_s that vanishes (equal weights, or below the rounding-noise threshold) is differentiated as its limit:
 // the first pair of the order as the crossing pair with U = Delta E_s = 0.
-// The kernel recomputes the interaction from the stored pre-interaction state, keeping a tape of every pair's inputs,
+// The kernel recomputes the interaction from the stored pre-interaction state, keeping a tape of every pair's angles,
 // then runs the chain rule backwards through the tape (one CTA per cell; the tape in a per-CTA slab of the workspace).
 // With a recorded tape the slabs are per cell and outlive the call: a recording call runs the forward and keeps each
 // cell's slab (the tape and the per-cell scalars of the correction); a later replaying call on the same interaction
@@ -25,8 +25,8 @@
 // arrays that are read in random order (state or gradient, weights, sort keys, permutation, weight order: 64 B per
 // particle) live in shared memory, the permutations are counting sorts there, and both directions of the energy pairs
 // run 32 at a time (a pass's pairs are disjoint; the forward needs a prefix sum over their caps, the reverse only the
-// crossing pair's dL/dU, which comes first). Two recorded steps of 1024 cells x 512 with their reverse: 5.9 -> 2.75 ms, of which
-// 3.8 with the pair functions alone. The forward sums what the step kernel sums in its order, so a replay from a
+// crossing pair's dL/dU, which comes first). Two recorded steps of 1024 cells x 512 with their reverse: 5.9 -> 2.3 ms (3.8 with
+// the pair functions alone, 2.6 before the pairs' angles were taped with their derivatives). The forward sums what the step kernel sums in its order, so a replay from a
 // checkpoint repeats the step's trajectory bit for bit (the closed-form gradients over 50 steps from checkpoints then hold as
 // closely as from tapes, 1e-11 where they held 3e-10).
 #include "mcc_pair64.cuh"
@@ -37,7 +37,7 @@ namespace {
 
 constexpr int kAdjCtasPerSm = 4;  // resident CTAs the kernel's registers are bounded for
 
-constexpr int kFlagTriplet = 1, kFlagUpdI = 2, kFlagUpdJ = 4, kFlagActive = 8;
+constexpr int kFlagUpdI = 1 << 28, kFlagUpdJ = 1 << 29, kFlagActive = 1 << 30, kPairIndex = kFlagUpdI - 1;
 
 struct AdjArgs {
     StepArgs a;                // state before the interaction (vx, vy, vz: double), w, constants of ic[0]
@@ -67,15 +67,13 @@ struct TapeHead {
 // The tape of one cell (n = max_cell, E = max_epairs).
 struct Slab {
     double* vb;     // [3][n] before the interaction
-    double* vp;     // [3][n] after the scatter
     double* vm;     // [3][n] after the momentum shift
-    double* pv;     // [6][n] per scatter pair: v_i, v_j at the pair's turn
+    double* pv;     // [kPairTape][n] per scatter pair, see pair64
     double* ev;     // [6][E] per energy pair: v_1, v_2 at the pair's turn
     double* eU;     // [E]
     double* eK;     // [E]
-    int32_t* pi;    // [n] scatter pair particles and flags
+    int32_t* pi;    // [n] scatter pair particles; the flags in the top bits of the first
     int32_t* pj;
-    int32_t* pf;
     int32_t* ei;    // [E] energy pair particles; 2 pass + (1 if the pair took its cap)
     int32_t* ej;
     int32_t* ecap;
@@ -116,7 +114,7 @@ __host__ __device__ inline size_t al8(size_t x) { return (x + 7) & ~(size_t)7; }
 __host__ __device__ inline size_t slab_bytes(int n, int E, bool on_chip)
 {
     const size_t dn = (size_t)n, de = (size_t)E;
-    return 3 * al8(24 * dn) + al8(48 * dn) + al8(48 * de) + 2 * al8(8 * de) + 3 * al8(4 * dn) + 3 * al8(4 * de) +
+    return 2 * al8(24 * dn) + al8(8 * kPairTape * dn) + al8(48 * de) + 2 * al8(8 * de) + 2 * al8(4 * dn) + 3 * al8(4 * de) +
            al8(sizeof(TapeHead)) + (on_chip ? 0 : kWorkBytesPerParticle * dn) + 256;
 }
 
@@ -132,15 +130,13 @@ __device__ Slab make_slab(char* base, int n, int E)
         return p;
     };
     s.vb = reinterpret_cast<double*>(take(24 * (size_t)n));
-    s.vp = reinterpret_cast<double*>(take(24 * (size_t)n));
     s.vm = reinterpret_cast<double*>(take(24 * (size_t)n));
-    s.pv = reinterpret_cast<double*>(take(48 * (size_t)n));
+    s.pv = reinterpret_cast<double*>(take(8 * kPairTape * (size_t)n));
     s.ev = reinterpret_cast<double*>(take(48 * (size_t)E));
     s.eU = reinterpret_cast<double*>(take(8 * (size_t)E));
     s.eK = reinterpret_cast<double*>(take(8 * (size_t)E));
     s.pi = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
     s.pj = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
-    s.pf = reinterpret_cast<int32_t*>(take(4 * (size_t)n));
     s.ei = reinterpret_cast<int32_t*>(take(4 * (size_t)E));
     s.ej = reinterpret_cast<int32_t*>(take(4 * (size_t)E));
     s.ecap = reinterpret_cast<int32_t*>(take(4 * (size_t)E));
@@ -165,11 +161,11 @@ struct AdjShared {
 
 __device__ __forceinline__ Acc<double>* accp(unsigned char* p) { return reinterpret_cast<Acc<double>*>(p); }
 
-// Forward of one scatter pair (the FP64 pair loop of the step kernel); returns the flags.
+// Forward of one scatter pair (the FP64 pair loop of the step kernel); returns the flags. pt: its tape (null: none).
 __device__ int pair_forward(const StepArgs& A, const InterConst& ic, double vi[3], double vj[3], double wi, double wj,
-                            int nmin, bool trip, uint4 r)
+                            int nmin, bool trip, uint4 r, double* pt, size_t n)
 {
-    int flags = trip ? kFlagTriplet : 0;
+    int flags = 0;
     bool upd_i = true, upd_j = true;
     if (wi != wj) {
         const bool moves = u23_bits(r.z) * fmax(wi, wj) < fmin(wi, wj);
@@ -180,7 +176,7 @@ __device__ int pair_forward(const StepArgs& A, const InterConst& ic, double vi[3
     if (upd_j) flags |= kFlagUpdJ;
     const double wf = (wi > wj ? wi : wj) * (double)nmin;
     double du[3];
-    if (!pair64(A.t64, A.method, (trip ? 0.5 : 1.0) * ic.kappa_mu2 * wf, vi, vj, r, du)) return flags;
+    if (!pair64<true>(A.t64, A.method, (trip ? 0.5 : 1.0) * ic.kappa_mu2 * wf, vi, vj, r, du, pt, n)) return flags;
     flags |= kFlagActive;
     for (int k = 0; k < 3; ++k) {
         if (upd_i) vi[k] = fma(ic.mu_ma, du[k], vi[k]);
@@ -189,64 +185,56 @@ __device__ int pair_forward(const StepArgs& A, const InterConst& ic, double vi[3
     return flags;
 }
 
-// Reverse of one scatter pair: g1, g2 (dL/d outputs) -> dL/d inputs in place; dL/dw of the heavier particle and
-// dL/dlnL accumulated.
-__device__ void pair_reverse(const StepArgs& A, const InterConst& ic, double lnL, const double vi[3],
-                             const double vj[3], double wi, double wj, int nmin, int flags, uint4 r, double g1[3],
-                             double g2[3], double& gwi, double& gwj, double& glnL)
+// Reverse of one scatter pair from its tape (at pv, one value every N): g1, g2 (dL/d outputs) -> dL/d inputs in place; dL/dw
+// of the heavier particle accumulated; returns s dL/ds
+// (not a number for lnL = 0: s carries no derivative in it then). The angles are taped with their derivatives: taking them again
+// cost more than half of the sweep's FP64 instructions (two recorded steps of 1024 cells x 512 with their reverse: 2.62 -> 2.30 ms).
+__device__ double pair_reverse(const InterConst& ic, double lnL, const double* pv, int N, double wi, double wj,
+                               int flags, double g1[3], double g2[3], double& gwi, double& gwj)
 {
-    if (!(flags & kFlagActive)) return;
+    if (!(flags & kFlagActive)) return 0.0;
     const double fa = (flags & kFlagUpdI) ? ic.mu_ma : 0.0, fb = (flags & kFlagUpdJ) ? ic.mu_mb : 0.0;
     const double gd[3] = {fa * g1[0] - fb * g2[0], fa * g1[1] - fb * g2[1], fa * g1[2] - fb * g2[2]};
-    if (gd[0] == 0.0 && gd[1] == 0.0 && gd[2] == 0.0) return;
-    const double u[3] = {vi[0] - vj[0], vi[1] - vj[1], vi[2] - vj[2]};
-    const double u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const double ru = rsqrt(u2), um = u2 * ru;
-    const double wmax = wi > wj ? wi : wj;
-    double s = ic.kappa_mu2 * wmax * (double)nmin * (ru * ru * ru);
-    if (flags & kFlagTriplet) s *= 0.5;
-    double st, omc, dst, domc, sp, cp;
-    angle64<true>(A.t64, A.method, s, r, st, omc, dst, domc);
-    turn64(A.t64, r.y, cp, sp);
+    if (gd[0] == 0.0 && gd[1] == 0.0 && gd[2] == 0.0) return 0.0;
+    const double u[3] = {pv[0], pv[N], pv[2 * (size_t)N]};
+    const double ru = pv[3 * (size_t)N], st = pv[4 * (size_t)N], omc = pv[5 * (size_t)N];
+    const double cp = pv[8 * (size_t)N], sp = pv[9 * (size_t)N];
+    const double um = (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * ru;
     // rotation du(u, st, omc) backwards
-    double gst, gomc, gu[3];
+    double gst, gu[3], gum;
+    const double gomc = -(gd[0] * u[0] + gd[1] * u[1] + gd[2] * u[2]);
     const double up2 = u[0] * u[0] + u[1] * u[1];
-    double gum;
+    const double uc = u[2] * cp, us = um * sp, tc = st * cp, ts = st * sp;
     if (up2 > 0.0) {
-        const double rp = rsqrt(up2), uperp = up2 * rp;
+        const double rp = rsqrt(up2);
         const double a = u[0] * rp, b = u[1] * rp;
-        gst = gd[0] * (a * u[2] * cp - b * um * sp) + gd[1] * (b * u[2] * cp + a * um * sp) - gd[2] * uperp * cp;
-        gomc = -(gd[0] * u[0] + gd[1] * u[1] + gd[2] * u[2]);
-        const double ga = gd[0] * u[2] * st * cp + gd[1] * um * st * sp;
-        const double gb = -gd[0] * um * st * sp + gd[1] * u[2] * st * cp;
-        gum = -gd[0] * b * st * sp + gd[1] * a * st * sp;
-        double gup = -gd[2] * st * cp;
-        gu[0] = -gd[0] * omc + ga * rp;
-        gu[1] = -gd[1] * omc + gb * rp;
-        gu[2] = gd[0] * a * st * cp + gd[1] * b * st * cp - gd[2] * omc;
-        gup -= (ga * a + gb * b) * rp;
-        gu[0] += gup * a;
-        gu[1] += gup * b;
+        const double g01 = gd[0] * a + gd[1] * b, g10 = gd[1] * a - gd[0] * b;
+        gst = g01 * uc + g10 * us - gd[2] * (up2 * rp) * cp;
+        gum = g10 * ts;
+        const double x = u[2] * tc, y = um * ts;
+        const double ga = gd[0] * x + gd[1] * y, gb = gd[1] * x - gd[0] * y;
+        const double gup = -gd[2] * tc - (ga * a + gb * b) * rp;
+        gu[0] = ga * rp + gup * a - gd[0] * omc;
+        gu[1] = gb * rp + gup * b - gd[1] * omc;
+        gu[2] = g01 * tc - gd[2] * omc;
     } else {
         gst = (gd[0] * cp + gd[1] * sp) * um;
-        gomc = -gd[2] * u[2];
-        gum = (gd[0] * cp + gd[1] * sp) * st;
+        gum = gd[0] * tc + gd[1] * ts;
         gu[0] = 0.0;
         gu[1] = 0.0;
         gu[2] = -gd[2] * omc;
     }
     // angle, then s = C w_max / um^3
-    const double gs = gst * dst + gomc * domc;
-    gum = (gum - gs * 3.0 * s * ru) * ru;
-    for (int k = 0; k < 3; ++k) gu[k] += gum * u[k];
-    const double gwmax = gs * s / wmax;
-    if (wi > wj) gwi += gwmax;
-    else gwj += gwmax;
-    glnL += gs * s / lnL;
+    const double gss = gst * pv[6 * (size_t)N] + gomc * pv[7 * (size_t)N];
+    gum = (gum - 3.0 * gss * ru) * ru;
     for (int k = 0; k < 3; ++k) {
-        g1[k] += gu[k];
-        g2[k] -= gu[k];
+        const double x = fma(gum, u[k], gu[k]);
+        g1[k] += x;
+        g2[k] -= x;
     }
+    if (wi > wj) gwi += gss / wi;
+    else gwj += gss / wj;
+    return lnL == 0.0 ? CUDART_NAN : gss;
 }
 
 __device__ __forceinline__ void ld3(const double* p, int n, int i, double x[3])
@@ -522,29 +510,18 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
                     double vi[3], vj[3];
                     ld3(wk.v, N, i, vi);
                     ld3(wk.v, N, j, vj);
+                    const uint4 rr = draw(A.rng, (uint32_t)p, (uint32_t)c, ictr, kTagScat);
+                    const int flags = pair_forward(A, ic, vi, vj, wk.w[i], wk.w[j], nmin, trip, rr,
+                                                   keep ? sl.pv + p : nullptr, (size_t)N);
                     if (keep) {
-                        for (int k = 0; k < 3; ++k) {
-                            sl.pv[k * N + p] = vi[k];
-                            sl.pv[(3 + k) * N + p] = vj[k];
-                        }
-                        sl.pi[p] = i;
+                        sl.pi[p] = i | flags;
                         sl.pj[p] = j;
                     }
-                    const uint4 rr = draw(A.rng, (uint32_t)p, (uint32_t)c, ictr, kTagScat);
-                    const int flags = pair_forward(A, ic, vi, vj, wk.w[i], wk.w[j], nmin, trip, rr);
-                    if (keep) sl.pf[p] = flags;
                     st3(wk.v, N, i, vi);
                     st3(wk.v, N, j, vj);
                     p = (p + 1 < lead) ? p + 1 : (p < lead ? lead + (int)threadIdx.x : p + kThreads);
                 }
                 __syncthreads();
-            }
-            if (keep) {
-                for (int i = threadIdx.x; i < n; i += kThreads) {
-                    double x[3];
-                    ld3(wk.v, N, i, x);
-                    st3(sl.vp, N, i, x);
-                }
             }
             // ---- forward: moment correction
             if (A.correct) {
@@ -834,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
                         for (int d = 0; d < 3; ++d) {
                             wk.v[d * N + i] += mp * sh.gS[d];
                             wk.gb[d * N + i] -= mp * sh.gS[d];
-                            gwd += msd * (sl.vp[d * N + i] - sl.vb[d * N + i]) * sh.gS[d];
+                            gwd += msd * ((sl.vm[d * N + i] - sl.vb[d * N + i]) + sh.B[d] * w) * sh.gS[d];  // v_ps = v_pm + B w
                         }
                         wk.gwl[i] += gwd;
                     }
@@ -842,7 +819,7 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
                 __syncthreads();
             }
             // scatter pairs backwards: rounds in reverse, the odd triplet in reverse by thread 0
-            double glnl = 0.0;
+            double glnl = 0.0;  // lnL dL/dlnL
             {
                 const int npairs = intra ? ((na & 1) ? (na + 3) / 2 : na / 2) : (na > nb ? na : nb);
                 const int nmin = intra ? na - 1 : (na < nb ? na : nb);
@@ -855,18 +832,12 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
                     // the triplet (0, 1, 2) shares particles: thread 0 undoes it in reverse; the other pairs of the round
                     // are disjoint from it and from each other
                     auto undo = [&](int p) {
-                        const int i = sl.pi[p], j = sl.pj[p];
-                        double vi[3], vj[3], g1[3], g2[3];
-                        for (int k = 0; k < 3; ++k) {
-                            vi[k] = sl.pv[k * N + p];
-                            vj[k] = sl.pv[(3 + k) * N + p];
-                        }
+                        const int f = sl.pi[p], i = f & kPairIndex, j = sl.pj[p];
+                        double g1[3], g2[3];
                         ld3(wk.v, N, i, g1);
                         ld3(wk.v, N, j, g2);
-                        const uint4 r = draw(A.rng, (uint32_t)p, (uint32_t)c, ictr, kTagScat);
                         double gwi = 0.0, gwj = 0.0;
-                        pair_reverse(A, ic, G.lnL, vi, vj, wk.w[i], wk.w[j], nmin, sl.pf[p], r, g1, g2, gwi, gwj,
-                                     glnl);
+                        glnl += pair_reverse(ic, G.lnL, sl.pv + p, N, wk.w[i], wk.w[j], f, g1, g2, gwi, gwj);
                         st3(wk.v, N, i, g1);
                         st3(wk.v, N, j, g2);
                         wk.gwl[i] += gwi;
@@ -892,7 +863,7 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
             {
                 Acc<double> acc[1] = {Acc<double>{glnl}};
                 block_sum<double, 1>(acc, accp(sh.red_raw), accp(sh.red));
-                if (threadIdx.x == 0 && G.glnL) atomicAdd(G.glnL, accp(sh.red)[0].x);
+                if (threadIdx.x == 0 && G.glnL) atomicAdd(G.glnL, accp(sh.red)[0].x != 0.0 ? accp(sh.red)[0].x / G.lnL : 0.0);
             }
         }
         __syncthreads();

@@ -460,7 +460,7 @@ __device__ __forceinline__ bool pair_out(const StepArgs& A, const InterConst& ic
         return true;
     }
     double du[3];
-    if (!pair64(A.t64, A.method, half * ic.kappa_mu2 * wf, vi, vj, r, du)) return false;
+    if (!pair64<false>(A.t64, A.method, half * ic.kappa_mu2 * wf, vi, vj, r, du)) return false;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         ni[d] = fma(ic.mu_ma, du[d], vi[d]);

@@ -21,8 +21,8 @@ struct InterConst {
 };
 
 // Tables of the FP64 pair kinematics (mcc_pair64.cuh), built on the host when a context is created.
-constexpr int kF64N97 = 9 * 64;  // intervals of s: 64 per octave of [2^-5, 16); eight coefficients each of 1 / A(s) and of
-                                 // e^-2A (s < 2) or 1 - e^-2A
+constexpr int kF64N97 = 9 * 64;  // intervals of s: 64 per octave of [2^-5, 16); eight coefficients each of 1 / A(s), of
+                                 // e^-2A (s < 2) or 1 - e^-2A, and of s A'(s) / A(s)
 constexpr int kF64Turn = 256;    // (cos, sin) of multiples of 1/256 turn
 constexpr int kF64Ln = 128;      // (r_i, -ln r_i)
 struct F64Tab {
@@ -30,7 +30,7 @@ struct F64Tab {
     const double2* turn;
     const double2* ln;
 };
-constexpr size_t kF64TabDoubles = 16 * kF64N97 + 2 * kF64Turn + 2 * kF64Ln;
+constexpr size_t kF64TabDoubles = 24 * kF64N97 + 2 * kF64Turn + 2 * kF64Ln;
 
 struct StepArgs {
     const int64_t* offsets;

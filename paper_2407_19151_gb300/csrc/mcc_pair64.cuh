@@ -45,7 +45,7 @@ __device__ __forceinline__ void turn64(const F64Tab& T, uint32_t r, double& cs, 
 }
 
 // ln(u + c) for a positive normal u and a c below its rounding (to first order).
-__device__ __forceinline__ double ln64(const F64Tab& T, double u, double c = 0.0)
+__device__ __forceinline__ double ln64(const F64Tab& T, double u, double c)
 {
     const int hi = __double2hiint(u);
     const int ix = hi - 0x3FE60000;  // mantissas are taken in [0.6875, 1.375)
@@ -132,27 +132,43 @@ __device__ __forceinline__ double n97_A(double s, const F64Tab& T)
 // x >= the value whose high word is lo, from the high word of x; false for NaN.
 __device__ __forceinline__ bool from64(int hi, int lo) { return (uint32_t)(hi - lo) <= (uint32_t)(0x7FF00000 - lo); }
 
+// s A'(s) / A(s), the logarithmic derivative of the N97 root, s > 0.
+__device__ __forceinline__ double n97_W(const F64Tab& T, double s)
+{
+    const int hi = __double2hiint(s);
+    if (hi < 0x3FA00000) {  // -s / (e^s - 1)
+        const double s2 = s * s;
+        return fma(s2, fma(s2, fma(s2, -1.0 / 30240.0, 1.0 / 720.0), -1.0 / 12.0), fma(0.5, s, -1.0));
+    }
+    if (hi >= 0x40300000) {  // A = 3 y (1 + 3 y^2 / 5), y = e^-s
+        const double y = exp(-s);
+        return -s * fma(1.2 * y, y, 1.0);
+    }
+    return n97_poly(T.n97 + 8 * kF64N97, s);
+}
+
 // Polar angle of a pair, sin(Theta) and 1 - cos(Theta), from the scattering length s and the draws (r.x, r.w).
-// DERIV: also their derivatives in s.
+// DERIV and want: also s times their derivatives in s.
 //  TA77: tan(Theta/2) = d = sqrt(s/2) g, g normal by Box-Muller; sin = 2 d / (1 + d^2), 1 - cos = 2 d^2 / (1 + d^2).
 //  N97:  1 - cos = -ln((1 - U) + U e^-2A) / A, 1 + cos = ln1p((1 - U) expm1(2A)) / A; s above 36.7 is isotropic.
+// The products whose rounding the two callers have to share are kept from being contracted.
 template <bool DERIV>
 __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, const uint4& r, double& st, double& omc,
-                                        double& dst, double& domc)
+                                        bool want, double& sdst, double& sdomc)
 {
     const double U = u23_bits(r.x);
-    if (DERIV) dst = domc = 0.0;
+    if (DERIV) sdst = sdomc = 0.0;
     if (method == 0) {
         double cs, sn;
         turn64(T, r.w, cs, sn);
-        const double d = sqrt(fmin(-s * ln64(T, U), 1e200)) * cs;
-        const double d2 = d * d, q = 1.0 / (1.0 + d2);
+        const double d = sqrt(fmin(-s * ln64(T, U, 0.0), 1e200)) * cs;
+        const double d2 = __dmul_rn(d, d), q = 1.0 / (1.0 + d2);
         st = 2.0 * d * q;
         omc = 2.0 * d2 * q;
-        if (DERIV && s > 0.0) {  // d' = d / (2 s)
-            const double x = q * q / s;
-            dst = d * (1.0 - d2) * x;
-            domc = 2.0 * d2 * x;
+        if (DERIV && want) {  // s d' = d / 2
+            const double x = q * q;
+            sdst = d * (1.0 - d2) * x;
+            sdomc = 2.0 * d2 * x;
         }
         return;
     }
@@ -167,7 +183,7 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
         const double rA = n97_rA<true>(T, s, E, F);
         // 1 - cos = -ln(1 + x) / A, x = -U F: 1 + x itself while |x| is below 1/2, the two positive terms (1 - U) + U E
         // beyond. Where that exceeds 1, 1 + cos = ln(1 + y) / A, y = (1 - U) (e^2A - 1), takes its place.
-        const double x = -U * F;
+        const double x = __dmul_rn(-U, F);
         const bool near1 = (__double2hiint(x) & 0x7FFFFFFF) < 0x3FE00000;
         const double u = near1 ? 1.0 + x : fma(U, E, V);
         const bool far = __double_as_longlong(u * u) < __double_as_longlong(E);  // 1 + x < e^-A
@@ -175,27 +191,18 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
         if (far) {
             // s < 1/8 gets here with probability below e^-8: e^-2A from the exponential, in full relative precision
             if (hs < 0x3FC00000) E = exp(-2.0 / rA);
-            z = V * (F / E);
+            z = __dmul_rn(V, F / E);
             a = 1.0 + z;
         }
-        const double l = ln64(T, a, near1 || far ? z - (a - 1.0) : 0.0);
-        o = (far ? l : -l) * rA;
-        q = 2.0 - o;
-        if (far) {
-            const double y = o;
-            o = q;
-            q = y;
-        }
-        if (DERIV) {
-            // L(A) = coth A - 1/A = e^-s: dA/ds = -e^-s / L'(A), L' = 1/A^2 - 4 E / F^2 = 1 - L^2 - 2 L / A (A < 1/2)
-            const double ys = exp(-s);
-            const double dL = hs >= 0x3FFD0000 ? 1.0 - ys * ys - 2.0 * ys * rA : rA * rA - 4.0 * E / (F * F);
+        const double l = __dmul_rn(ln64(T, a, near1 || far ? z - (a - 1.0) : 0.0), rA);
+        o = far ? 2.0 - l : -l;
+        q = far ? l : 2.0 + l;
+        if (DERIV && want) {
             // d(1 - cos)/dA = (-(1 - cos) + 2 U E / (1 + x)) / A
-            const double dA = -ys / dL;
-            const double do_ds = rA * (2.0 * U * E / u - o) * dA;
-            const bool cl = o > 2.0;
-            domc = cl ? 0.0 : do_ds;
-            dst = (o * q > 0.0 && !cl) ? (q - o) * do_ds * (0.5 * rsqrt(o * q)) : 0.0;
+            sdomc = (2.0 * U * E / u - o) * n97_W(T, s);
+            const double p = o * q;
+            sdst = p > 0.0 ? (q - o) * sdomc * (0.5 * rsqrt(p)) : 0.0;
+            if (from64(__double2hiint(o), 0x40000000)) sdomc = sdst = 0.0;
         }
     }
     o = from64(__double2hiint(o), 0x40000000) ? 2.0 : o;
@@ -227,16 +234,25 @@ __device__ __forceinline__ void rotate64(double ux, double uy, double uz, double
 // Change of the relative velocity u = v_i - v_j of a non-relativistic pair, s = cw / |u|^3; false if u vanishes. cw = kappa
 // / mu^2 w_max N_min, halved for a triplet. The step kernel and the adjoint's forward both run this and then fma(mu / m, du,
 // v), so that a replayed interaction repeats the step's velocities bit for bit.
+// TAPE and pt: what the reverse of the pair reads goes to pt, one value every n: u = v_i - v_j (3), 1 / |u|, sin(Theta),
+// 1 - cos(Theta), s times their derivatives in s, cos(phi), sin(phi).
+constexpr int kPairTape = 10;
+template <bool TAPE>
 __device__ __forceinline__ bool pair64(const F64Tab& T, int method, double cw, const double vi[3], const double vj[3],
-                                       const uint4& r, double du[3])
+                                       const uint4& r, double du[3], double* pt = nullptr, size_t n = 0)
 {
     const double ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
     const double u2 = fma(uz, uz, fma(uy, uy, ux * ux));
     if (__double_as_longlong(u2) == 0) return false;
     const double ru = rsqrt(u2);
     double st, omc, sp, cp, d0, d1;
-    angle64<false>(T, method, cw * (ru * ru * ru), r, st, omc, d0, d1);
+    angle64<TAPE>(T, method, cw * (ru * ru * ru), r, st, omc, pt != nullptr, d0, d1);
     turn64(T, r.y, cp, sp);
+    if (TAPE && pt) {
+        const double x[kPairTape] = {ux, uy, uz, ru, st, omc, d0, d1, cp, sp};
+#pragma unroll
+        for (int k = 0; k < kPairTape; ++k) pt[k * n] = x[k];
+    }
     rotate64(ux, uy, uz, u2 * ru, st, omc, cp, sp, du[0], du[1], du[2]);
     return true;
 }
@@ -285,7 +301,7 @@ __device__ __forceinline__ bool rel_pair64(const F64Tab& T, int method, double c
     const double iv = rsqrt(fma(ma, ma, pc)) + rsqrt(fma(mb, mb, pc));
     const double s = kw * (rp * rp * rp) / iv;
     double st, omc, cp, sp, x0, x1, d[3];
-    angle64<false>(T, method, s, r, st, omc, x0, x1);
+    angle64<false>(T, method, s, r, st, omc, false, x0, x1);
     turn64(T, r.y, cp, sp);
     rotate64(p[0], p[1], p[2], pm, st, omc, cp, sp, d[0], d[1], d[2]);
     const double Vd = cb * (V[0] * d[0] + V[1] * d[1] + V[2] * d[2]);
