@@ -25,10 +25,10 @@
 // arrays that are read in random order (state or gradient, weights, sort keys, permutation, weight order: 64 B per
 // particle) live in shared memory, the permutations are counting sorts there, and both directions of the energy pairs
 // run 32 at a time (a pass's pairs are disjoint; the forward needs a prefix sum over their caps, the reverse only the
-// crossing pair's dL/dU, which comes first). Two recorded steps of 1024 cells x 512 with their reverse: 5.9 -> 2.3 ms (3.8 with
-// the pair functions alone, 2.6 before the pairs' angles were taped with their derivatives). The forward sums what the step kernel sums in its order, so a replay from a
-// checkpoint repeats the step's trajectory bit for bit (the closed-form gradients over 50 steps from checkpoints then hold as
-// closely as from tapes, 1e-11 where they held 3e-10).
+// crossing pair's dL/dU, which comes first). Two recorded steps of 1024 cells x 512 with their reverse: 5.9 -> 2.3 ms
+// (3.8 with the pair functions alone, 2.6 before the pairs' angles were taped with their derivatives). The forward sums
+// what the step kernel sums in its order, so a replay from a checkpoint repeats the step's trajectory bit for bit (the
+// closed-form gradients over 50 steps from checkpoints then hold as closely as from tapes, 1e-11 where they held 3e-10).
 #include "mcc_pair64.cuh"
 #include "mcc_perm.cuh"
 
