@@ -37,9 +37,9 @@ struct mcc_ctx {
     // Attributes of the kernels, looked up once (each look-up costs about a microsecond of every call), and the last
     // occupancy of each: launch shape << 8 | CTAs per SM in one word, so threads may share a context.
     size_t cell_static[2][2][4];  // [float][relativistic][mode]
-    size_t group_static[2][mcc::kGroupClasses];
+    size_t group_static[2][mcc::kOrderClasses];
     size_t adjoint_static;
-    std::atomic<uint64_t> cell_occ[2][2][4], group_occ[2][mcc::kGroupClasses];
+    std::atomic<uint64_t> cell_occ[2][2][4], group_occ[2][mcc::kOrderClasses];
 };
 
 namespace mcc {
@@ -454,7 +454,8 @@ int mcc_create(mcc_ctx** out, int device)
                 if (e != cudaSuccess) attr = e;
             }
     for (int rel = 0; rel < 2; ++rel)
-        for (int cls = 0; cls < mcc::kGroupClasses; ++cls) {
+        for (int cls = 0; cls < mcc::kOrderClasses; ++cls) {
+            if (cls == mcc::kRestClass) continue;
             cudaFuncAttributes fa;
             cudaError_t e = cudaFuncGetAttributes(&fa, mcc::group_kernel(true, rel, cls));
             if (e == cudaSuccess) {
@@ -697,7 +698,7 @@ namespace {
 // Workspace of mcc_step_fused: the cell order (n_cells int32), the class bounds and queue counters of the group
 // kernels, then, when some cell exceeds the largest group class, one slab per resident CTA of the one-CTA kernel.
 size_t order_bytes(int32_t n_cells) { return ((size_t)n_cells * sizeof(int32_t) + 255) & ~(size_t)255; }
-// class_off [2 (kGroupClasses + 1)], queues [kGroupClasses + 1] and the order's bins, int32
+// class_off [2 kOrderClasses], queues [kOrderClasses] and the order's bins, int32
 constexpr size_t kCtrlHist = 256;
 size_t ctrl_bytes() { return kCtrlHist + ((mcc::group_order_hist_bytes() + 255) & ~(size_t)255); }
 
@@ -729,7 +730,7 @@ size_t group_budget(const mcc_ctx* ctx, bool f32, bool rel, int cls)
 // Groups of one CTA of class cls with tiles of cap particles: group_cta_warps warps, or as many groups as fit.
 int groups_per_cta(const mcc_ctx* ctx, bool f32, bool rel, int cls, int cap)
 {
-    const int most = mcc::group_cta_warps(rel) >> cls;
+    const int most = 32 * mcc::group_cta_warps(rel) / mcc::group_threads(cls);
     const int fit = (int)(group_budget(ctx, f32, rel, cls) / mcc::group_smem(mcc::group_shared_bytes(cls), cap));
     const int g = fit < most ? fit : most;
     return g > 1 ? g : 1;
@@ -838,16 +839,20 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     int32_t caps[mcc::kGroupClasses];
     group_caps(ctx, f32, rel, caps);
     if (ctx->group_cap == 0) few_cells_caps(ctx, n_cells, caps);
+    // two small cells to a warp, with automatic capacities, if they fill every warp's halves (a launch of its own costs the
+    // time of a visit, 0.1 ms)
+    int32_t half_min = 2 * mcc::kGroupWarpsPerSm * ctx->num_sms;
+    if (!f32 || ctx->group_cap > 0 || caps[0] < mcc::kHalfCells || n_cells < half_min) half_min = 0;
     // the group kernels serve the mixed path; the FP64 path runs every cell on the one-CTA kernel
     const bool fallback = !f32 || max_cell > caps[mcc::kGroupClasses - 1];
     int32_t* order = reinterpret_cast<int32_t*>(ws);
     int32_t* class_off = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws) + order_bytes(n_cells));
-    int32_t* queues = class_off + 2 * (mcc::kGroupClasses + 1);
+    int32_t* queues = class_off + 2 * mcc::kOrderClasses;
     // cells by size class, largest first (the order is the same for every step of the call)
     int32_t* hist = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(class_off) + kCtrlHist);
     if (cudaMemsetAsync(class_off, 0, kCtrlHist + mcc::group_order_hist_bytes(), S(stream)) != cudaSuccess)
         return MCC_ERR_CUDA;
-    if (mcc::launch_group_order(offsets, n_cells, n_species, caps, order, class_off, hist, &ctx->launches, S(stream)) !=
+    if (mcc::launch_group_order(offsets, n_cells, n_species, caps, half_min, order, class_off, hist, &ctx->launches, S(stream)) !=
         cudaSuccess)
         return MCC_ERR_CUDA;
     a.order = order;
@@ -874,11 +879,34 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
         if (cudaStreamIsCapturing(S(stream), &cs) != cudaSuccess) return MCC_ERR_CUDA;
         if (cs == cudaStreamCaptureStatusActive) rec_flags = cudaEventRecordExternal;
     }
+    // one launch of a size class with tiles of cap particles
+    auto run_class = [&](int cls, int32_t cap) -> int {
+        // fewer cells than groups: spread them over the SMs
+        const int per_sm = (n_cells + ctx->num_sms - 1) / ctx->num_sms;
+        int groups = groups_per_cta(ctx, f32, rel, cls, cap);
+        if (groups > per_sm) groups = per_sm;
+        const size_t smem = (size_t)groups * mcc::group_smem(mcc::group_shared_bytes(cls), cap);
+        const int bps = cached_occupancy(ctx->group_occ[rel][cls], ((uint64_t)smem << 6) | (uint64_t)groups, [&] {
+            int b = 0;
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, mcc::group_kernel(f32, rel, cls),
+                                                                 groups * mcc::group_threads(cls), smem) == cudaSuccess
+                       ? b
+                       : 0;
+        });
+        if (bps < 1) return MCC_ERR_CUDA;
+        int grid = bps * ctx->num_sms;
+        if (grid > n_cells) grid = n_cells;
+        a.gcls = cls;
+        a.gcap = cap;
+        const cudaError_t e = mcc::launch_group(f32, rel, cls, a, grid, groups, smem, S(stream));
+        ctx->launches += 1;
+        return e == cudaSuccess ? MCC_OK : MCC_ERR_CUDA;
+    };
     for (int32_t t = 0; t < n_steps; ++t) {
         a.rng.step = (uint32_t)(p->step + (uint64_t)t);
         a.step_add = (uint32_t)t;
         // (the first step's queues are zero)
-        if (t > 0 && cudaMemsetAsync(queues, 0, sizeof(int32_t) * (mcc::kGroupClasses + 1), S(stream)) != cudaSuccess)
+        if (t > 0 && cudaMemsetAsync(queues, 0, sizeof(int32_t) * mcc::kOrderClasses, S(stream)) != cudaSuccess)
             return MCC_ERR_CUDA;
         cudaEvent_t* ev = (p->launch_events && t == n_steps - 1) ? reinterpret_cast<cudaEvent_t*>(p->launch_events)
                                                                    : nullptr;
@@ -901,26 +929,9 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
                 mark(cls, 1);
                 continue;
             }
-            // fewer cells than groups: spread them over the SMs
-            const int per_sm = (n_cells + ctx->num_sms - 1) / ctx->num_sms;
-            int groups = groups_per_cta(ctx, f32, rel, cls, caps[cls]);
-            if (groups > per_sm) groups = per_sm;
-            const size_t smem = (size_t)groups * mcc::group_smem(mcc::group_shared_bytes(cls), caps[cls]);
-            const int bps = cached_occupancy(ctx->group_occ[rel][cls], ((uint64_t)smem << 5) | (uint64_t)groups, [&] {
-                int b = 0;
-                return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, mcc::group_kernel(f32, rel, cls),
-                                                                     groups * (32 << cls), smem) == cudaSuccess
-                           ? b
-                           : 0;
-            });
-            if (bps < 1) return MCC_ERR_CUDA;
-            int grid = bps * ctx->num_sms;
-            if (grid > n_cells) grid = n_cells;
-            a.gcls = cls;
-            a.gcap = caps[cls];
-            const cudaError_t e = mcc::launch_group(f32, rel, cls, a, grid, groups, smem, S(stream));
-            ctx->launches += 1;
-            if (e != cudaSuccess) return MCC_ERR_CUDA;
+            rc = run_class(cls, caps[cls]);
+            if (rc == MCC_OK && cls == 0 && half_min > 0) rc = run_class(mcc::kHalfClass, max_cell < mcc::kHalfCells ? max_cell : mcc::kHalfCells);
+            if (rc != MCC_OK) return rc;
             mark(cls, 1);
         }
     }

@@ -185,10 +185,10 @@ __device__ int pair_forward(const StepArgs& A, const InterConst& ic, double vi[3
     return flags;
 }
 
-// Reverse of one scatter pair from its tape (at pv, one value every N): g1, g2 (dL/d outputs) -> dL/d inputs in place; dL/dw
-// of the heavier particle accumulated; returns s dL/ds
-// (not a number for lnL = 0: s carries no derivative in it then). The angles are taped with their derivatives: taking them again
-// cost more than half of the sweep's FP64 instructions (two recorded steps of 1024 cells x 512 with their reverse: 2.62 -> 2.30 ms).
+// Reverse of one scatter pair from its tape (at pv, one value every N): g1, g2 (dL/d outputs) -> dL/d inputs in place;
+// dL/dw of the heavier particle accumulated; returns s dL/ds (not a number for lnL = 0: s carries no derivative in it
+// then). The angles are taped with their derivatives: taking them again cost more than half of the sweep's FP64
+// instructions (two recorded steps of 1024 cells x 512 with their reverse: 2.62 -> 2.30 ms).
 __device__ double pair_reverse(const InterConst& ic, double lnL, const double* pv, int N, double wi, double wj,
                                int flags, double g1[3], double g2[3], double& gwi, double& gwj)
 {

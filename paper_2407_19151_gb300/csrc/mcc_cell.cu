@@ -1080,19 +1080,24 @@ __device__ __forceinline__ void scan_bins(int* hist, int* warp_tot)
     __syncthreads();
 }
 
-// Begin and end of each class in the order, from the scanned bins.
-__device__ __forceinline__ void write_class_off(const int* hist, int32_t n_cells, int32_t* class_off)
+// Begin and end of each class in the order, from the scanned bins; the small cells of class 0 are its last bins.
+__device__ __forceinline__ void write_class_off(const int* hist, int32_t n_cells, int32_t half_min, int32_t* class_off)
 {
-    if (threadIdx.x <= kGroupClasses) {
+    constexpr int kLg = 31 - __builtin_clz(kHalfCells);
+    constexpr int kHalfBin = kGroupClasses * kGroupSub + kGroupSub - (8 * kLg + ((kHalfCells >> (kLg - 3)) & 7));
+    if (threadIdx.x < kOrderClasses) {
         const int cls = threadIdx.x;
-        const int b0 = (kGroupClasses - cls) * kGroupSub;
-        class_off[2 * cls] = hist[b0];
-        class_off[2 * cls + 1] = b0 + kGroupSub < kGroupBins ? hist[b0 + kGroupSub] : n_cells;
+        const int b0 = cls == kHalfClass ? kHalfBin : (kGroupClasses - cls) * kGroupSub;
+        const bool half = half_min > 0 && n_cells - hist[kHalfBin] >= half_min;
+        const int b1 = cls == 0 && half ? kHalfBin : (cls == kHalfClass ? kGroupBins : b0 + kGroupSub);
+        class_off[2 * cls + 1] = b1 < kGroupBins ? hist[b1] : n_cells;
+        class_off[2 * cls] = cls == kHalfClass && !half ? n_cells : hist[b0];
     }
 }
 
 __global__ void __launch_bounds__(kOrderThreads) k_group_order(const int64_t* __restrict__ offsets, int32_t n_cells,
-                                                              int32_t S, GroupCaps caps, int32_t* __restrict__ order,
+                                                              int32_t S, GroupCaps caps, int32_t half_min,
+                                                              int32_t* __restrict__ order,
                                                               int32_t* __restrict__ class_off)
 {
     __shared__ int hist[kGroupBins];
@@ -1103,7 +1108,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_group_order(const int64_t* __
         atomicAdd(&hist[group_bin(offsets[(int64_t)(c + 1) * S] - offsets[(int64_t)c * S], caps.cap)], 1);
     __syncthreads();
     scan_bins(hist, warp_tot);
-    write_class_off(hist, n_cells, class_off);
+    write_class_off(hist, n_cells, half_min, class_off);
     __syncthreads();
     for (int c = threadIdx.x; c < n_cells; c += kOrderThreads) {
         const int b = group_bin(offsets[(int64_t)(c + 1) * S] - offsets[(int64_t)c * S], caps.cap);
@@ -1126,7 +1131,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_count(const int64_t* __
         if (h[b]) atomicAdd(&hist[b], h[b]);
 }
 
-__global__ void __launch_bounds__(kOrderThreads) k_order_scan(int32_t* __restrict__ hist, int32_t n_cells,
+__global__ void __launch_bounds__(kOrderThreads) k_order_scan(int32_t* __restrict__ hist, int32_t n_cells, int32_t half_min,
                                                              int32_t* __restrict__ class_off)
 {
     __shared__ int h[kGroupBins];
@@ -1135,7 +1140,7 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_scan(int32_t* __restric
     __syncthreads();
     scan_bins(h, warp_tot);
     for (int b = threadIdx.x; b < kGroupBins; b += kOrderThreads) hist[b] = h[b];
-    write_class_off(h, n_cells, class_off);
+    write_class_off(h, n_cells, half_min, class_off);
 }
 
 __global__ void __launch_bounds__(kOrderThreads) k_order_place(const int64_t* __restrict__ offsets, int32_t n_cells, int32_t S,
@@ -1214,19 +1219,19 @@ constexpr int32_t kOrderOneCta = 16384;
 
 size_t group_order_hist_bytes() { return kGroupBins * sizeof(int32_t); }
 
-cudaError_t launch_group_order(const int64_t* offsets, int32_t n_cells, int32_t S, const int32_t* caps,
+cudaError_t launch_group_order(const int64_t* offsets, int32_t n_cells, int32_t S, const int32_t* caps, int32_t half_min,
                                int32_t* order, int32_t* class_off, int32_t* hist, int64_t* launches, cudaStream_t st)
 {
     GroupCaps gc;
     for (int k = 0; k < kGroupClasses; ++k) gc.cap[k] = caps[k];
     if (n_cells <= kOrderOneCta) {
-        k_group_order<<<1, kOrderThreads, 0, st>>>(offsets, n_cells, S, gc, order, class_off);
+        k_group_order<<<1, kOrderThreads, 0, st>>>(offsets, n_cells, S, gc, half_min, order, class_off);
         *launches += 1;
         return cudaGetLastError();
     }
     const int grid = n_cells / 4096 < 64 ? n_cells / 4096 : 64;
     k_order_count<<<grid, kOrderThreads, 0, st>>>(offsets, n_cells, S, gc, hist);
-    k_order_scan<<<1, kOrderThreads, 0, st>>>(hist, n_cells, class_off);
+    k_order_scan<<<1, kOrderThreads, 0, st>>>(hist, n_cells, half_min, class_off);
     k_order_place<<<grid, kOrderThreads, 0, st>>>(offsets, n_cells, S, gc, hist, order);
     *launches += 3;
     return cudaGetLastError();
@@ -1245,7 +1250,7 @@ cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int gri
                          cudaStream_t st)
 {
     void* args[] = {const_cast<StepArgs*>(&a)};
-    return cudaLaunchKernel(group_kernel(f32, rel, cls), dim3(grid), dim3(groups * (32 << cls)), args, smem, st);
+    return cudaLaunchKernel(group_kernel(f32, rel, cls), dim3(grid), dim3(groups * group_threads(cls)), args, smem, st);
 }
 
 size_t pair_tile_bytes_per_particle() { return kPairTileBytesPerParticle; }

@@ -3,8 +3,9 @@
 //
 // Cells are dispatched by size class: class k holds cells of at most C * 2^k particles and runs with G = 32 * 2^k
 // threads, so every class keeps the same shared memory per thread and the GPU the same number of resident warps.
-// The smallest class is one warp per cell and synchronises with warp barriers only inside a cell; the groups of 64 to 256
-// threads use one named barrier each. The largest class takes the largest cell one CTA's shared memory can hold.
+// The smallest class is one warp per cell and synchronises with warp barriers only inside a cell, its smallest cells two
+// to a warp (groups of 16 threads: half warps with masks of their own); the groups of 64 to 256 threads use one named
+// barrier each. The largest class takes the largest cell one CTA's shared memory can hold.
 //
 // Lockstep: what bounds a cell visit is instruction fetch. A visit is nearly straight-line code (each loop runs two or
 // three times over ~170 particles of a species, the code of one interaction is far larger than an SM partition's
@@ -145,19 +146,6 @@ __device__ __forceinline__ ff ff_ld(float2 s) { return {s.x, s.y}; }
 __device__ __forceinline__ float2 ff_st(ff x) { return make_float2(x.hi, x.lo); }
 __device__ __forceinline__ ff mass_ff(const StepArgs& A, int s) { return {A.m_f[s], A.m_lo[s]}; }
 
-__device__ __forceinline__ ff shx(ff a, int m)
-{
-    return {__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
-}
-__device__ __forceinline__ ff shup(ff a, int m)
-{
-    return {__shfl_up_sync(0xffffffffu, a.hi, m), __shfl_up_sync(0xffffffffu, a.lo, m)};
-}
-__device__ __forceinline__ ff shidx(ff a, int l)
-{
-    return {__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
-}
-
 // ----------------------------------------------------------------------------------------------- group primitives
 // Thread and warp index within the group; group of the CTA this thread belongs to.
 template <int G>
@@ -168,7 +156,36 @@ __device__ __forceinline__ int tix()
 template <int G>
 __device__ __forceinline__ int wix()
 {
-    return ((int)threadIdx.x >> 5) & (G / 32 - 1);
+    return G > 32 ? ((int)threadIdx.x >> 5) & (G / 32 - 1) : 0;
+}
+// Lanes of a warp that belong to one group (G = 16: two groups to a warp), this thread's lane among them, their mask.
+template <int G>
+constexpr int kLanes = G < 32 ? G : 32;
+template <int G>
+__device__ __forceinline__ int lix()
+{
+    return (int)threadIdx.x & (kLanes<G> - 1);
+}
+// Mask of the aligned run of `lanes` lanes this thread is in.
+__device__ __forceinline__ unsigned lane_mask(int lanes)
+{
+    return lanes == 32 ? 0xffffffffu : ((1u << lanes) - 1u) << (threadIdx.x & (32 - lanes));
+}
+template <int G>
+__device__ __forceinline__ unsigned gmask()
+{
+    return lane_mask(kLanes<G>);
+}
+template <int G>
+__device__ __forceinline__ ff shx(ff a, int m)
+{
+    return {__shfl_xor_sync(gmask<G>(), a.hi, m), __shfl_xor_sync(gmask<G>(), a.lo, m)};
+}
+// from lane l of the group's lanes
+template <int G>
+__device__ __forceinline__ ff shidx(ff a, int l)
+{
+    return {__shfl_sync(gmask<G>(), a.hi, l, kLanes<G>), __shfl_sync(gmask<G>(), a.lo, l, kLanes<G>)};
 }
 template <int G>
 __device__ __forceinline__ int team()
@@ -180,14 +197,14 @@ __device__ __forceinline__ int team()
 template <int G>
 __device__ __forceinline__ void gsync()
 {
-    if (G == 32) __syncwarp();
+    if (G <= 32) __syncwarp(gmask<G>());
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + team<G>()), "n"(G) : "memory");
 }
 
 template <int G>
 __device__ __forceinline__ bool gany(bool p)
 {
-    if (G == 32) return __any_sync(0xffffffffu, p);
+    if (G <= 32) return __any_sync(gmask<G>(), p);
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
@@ -204,50 +221,32 @@ __device__ __forceinline__ bool gany(bool p)
 template <int G>
 __device__ __forceinline__ void csync()
 {
+    if (G < 32) __syncwarp();  // both groups of the warp
     if (blockDim.x > G) __syncthreads();
 }
 
-template <int P>
-struct Lg;
-template <>
-struct Lg<1> {
-    static constexpr int v = 0;
-};
-template <>
-struct Lg<2> {
-    static constexpr int v = 1;
-};
-template <>
-struct Lg<4> {
-    static constexpr int v = 2;
-};
-template <>
-struct Lg<8> {
-    static constexpr int v = 3;
-};
-
-// Warp reduce-scatter of P (1, 2, 4 or 8) float-float values per lane: rounds with lane masks 16, 8, ... halve the
-// set of quantities each lane keeps (the lane with the mask bit set keeps the upper half and adds its partner's
+// Warp reduce-scatter of P (2 or 8) float-float values per lane over the group's W lanes: rounds with lane masks W/2, ... halve
+// the set of quantities each lane keeps (the lane with the mask bit set keeps the upper half and adds its partner's
 // values of it), then a butterfly on the one kept quantity. Afterwards every lane holds the warp total of quantity
-// lane >> (5 - log2 P); the lanes holding one quantity have the same bits (the butterfly's additions are symmetric),
+// lane / (W / P); the lanes holding one quantity have the same bits (the butterfly's additions are symmetric),
 // and the order of additions is fixed.
-template <int P>
+template <int G, int P>
 __device__ __forceinline__ ff warp_rs(ff (&a)[P])
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = lix<G>();
 #pragma unroll
-    for (int h = P / 2, m = 16; h >= 1; h >>= 1, m >>= 1) {
+    for (int h = P / 2, m = kLanes<G> / 2; h >= 1; h >>= 1, m >>= 1) {
         const bool up = (lane & m) != 0;
 #pragma unroll
         for (int k = 0; k < h; ++k) {
             const ff send = up ? a[k] : a[k + h];
             const ff keep = up ? a[k + h] : a[k];
-            a[k] = ff_add(keep, shx(send, m));
+            a[k] = ff_add(keep, shx<G>(send, m));
         }
     }
     ff s = a[0];
 #pragma unroll
-    for (int m = 16 / P; m >= 1; m >>= 1) s = ff_add(s, shx(s, m));
+    for (int m = kLanes<G> / 2 / P; m >= 1; m >>= 1) s = ff_add(s, shx<G>(s, m));
     return s;
 }
 
@@ -255,27 +254,27 @@ __device__ __forceinline__ ff warp_rs(ff (&a)[P])
 // group has met at the barrier inside the other.
 template <int G>
 struct GRed {
-    ff part[8 * (G / 32)];
+    ff part[8 * (G > 32 ? G / 32 : 1)];
 };
 
-// Group sum of P values per thread. Each lane gets the total of one quantity, q = lane >> (5 - log2 P), the same bits in
+// Group sum of P values per thread. Each lane gets the total of one quantity, q = lane / (lanes / P), the same bits in
 // every warp: the coefficients that follow are then computed for all quantities at once, a lane group each, where every
 // lane used to compute all of them (three-species step 29.2 -> 28.5 ms, relativistic beam 7.81 -> 7.61).
 template <int G, int P>
 __device__ __forceinline__ ff greduce(ff (&a)[P], GRed<G>& r)
 {
-    constexpr int SH = 5 - Lg<P>::v, W = G / 32;
-    const int lane = threadIdx.x & 31, warp = wix<G>(), q = lane >> SH;
-    const ff s = warp_rs<P>(a);
-    if (G == 32) return s;
-    if ((lane & ((1 << SH) - 1)) == 0) r.part[q * W + warp] = s;
+    constexpr int L = kLanes<G> / P, W = G / 32;
+    const int lane = lix<G>(), warp = wix<G>(), q = lane / L;
+    const ff s = warp_rs<G, P>(a);
+    if (G <= 32) return s;
+    if ((lane & (L - 1)) == 0) r.part[q * W + warp] = s;
     gsync<G>();
     ff t = r.part[q * W];
     for (int w = 1; w < W; ++w) t = ff_add(t, r.part[q * W + w]);
     return t;
 }
 
-// Exclusive prefix sum of one value per lane in lane order over a segment of W (16 or 32) lanes of the warp (lanes
+// Exclusive prefix sum of one value per lane in lane order over a segment of W (8, 16 or 32) lanes of the warp (lanes
 // given by mask), and the segment total. W = WIDTH, or the runtime width when WIDTH is 0 (one copy of the code serves
 // both segment widths).
 template <int WIDTH>
@@ -301,16 +300,16 @@ __device__ __forceinline__ ff seg_scan_excl(ff x, unsigned mask, int width, ff& 
 template <int G>
 __device__ __forceinline__ int gscan_int(int x, int* scr, int& total)
 {
-    const int lane = threadIdx.x & 31, warp = wix<G>();
+    const int lane = lix<G>(), warp = wix<G>();
     int inc = x;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    for (int o = 1; o < kLanes<G>; o <<= 1) {
+        const int y = __shfl_up_sync(gmask<G>(), inc, o, kLanes<G>);
         if (lane >= o) inc += y;
     }
     const int exc = inc - x;
-    if (G == 32) {
-        total = __shfl_sync(0xffffffffu, inc, 31);
+    if (G <= 32) {
+        total = __shfl_sync(gmask<G>(), inc, kLanes<G> - 1, kLanes<G>);
         return exc;
     }
     constexpr int W = G / 32;
@@ -368,17 +367,18 @@ struct GShared {
     ff eres_E[2];   // energy phase results: carried energy of species a, b after their energy pairs
     int eres_i[4];  // pairs used and failure of species a, then of species b
     int sci[G / 32 + 1];
-    uint32_t wrange[kMaxSpecies][G / 32][2];  // per warp: smallest and largest top key word of a species (weight order)
+    uint32_t wrange[kMaxSpecies][G > 32 ? G / 32 : 1][2];  // per warp: smallest and largest top key word of a species (weight order)
 };
 
 // What the groups of a CTA share: the cells of the batch, and the cells to visit again without their failed interactions
 // (Sec. 5.2 under the rollback policy).
+constexpr int kMostTeams = 2 * group_cta_warps(true);
 struct CtaShared {
     int base, take, retry;    // the batch: [base, base + take) of the class order, or of the retry list
     int n_retry;
-    int r_cell[2 * group_cta_warps(true)];       // cell
-    int r_used[2 * group_cta_warps(true)];       // energy pairs of its failed interactions
-    uint64_t r_skip[2 * group_cta_warps(true)];  // its failed interactions
+    int r_cell[2 * kMostTeams];       // cell
+    int r_used[2 * kMostTeams];       // energy pairs of its failed interactions
+    uint64_t r_skip[2 * kMostTeams];  // its failed interactions
 };
 
 // Bytes of a group's GShared, the tile after it 16-byte aligned.
@@ -528,7 +528,7 @@ __device__ __noinline__ void gsort_u64(uint64_t* a, int n)
 template <int G>
 __device__ __forceinline__ void sort_keys(uint64_t* key, int n)
 {
-    if (n <= kWarpSortMax) {
+    if (G >= 32 && n <= kWarpSortMax) {
         if (wix<G>() == 0) warp_sort_buf(key, n);
     } else {
         gsort_u64<G>(key, n);
@@ -552,7 +552,7 @@ template <int G>
 __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GShared<G>& sh, int64_t cs, int S,
                                            unsigned need)
 {
-    const int lane = threadIdx.x & 31, warp = wix<G>();
+    const int lane = lix<G>(), warp = wix<G>();
     if (tix<G>() == 0)
         for (int sp = 0; sp < S; ++sp)
             if (!(need >> sp & 1u)) sh.wmode[sp] = 3;
@@ -574,14 +574,14 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
             differ |= (k ^ first) >> kPermBits != 0;
             t.perm[CHK(t.dbg, s0 + q, t.n)] = 0;
         }
-        lo = __reduce_min_sync(0xffffffffu, lo);
-        hi = __reduce_max_sync(0xffffffffu, hi);
+        lo = __reduce_min_sync(gmask<G>(), lo);
+        hi = __reduce_max_sync(gmask<G>(), hi);
         if (G > 32 && lane == 0) {
             sh.wrange[sp][warp][0] = lo;
             sh.wrange[sp][warp][1] = hi;
         }
         if (!gany<G>(differ)) need &= ~(1u << sp);  // all equal
-        if (G == 32 && lane == 0) {
+        if (G <= 32 && lane == 0) {
             sh.wrange[sp][0][0] = lo;
             sh.wrange[sp][0][1] = hi;
         }
@@ -1217,7 +1217,7 @@ __device__ __forceinline__ ff ke_per_mass(const ff v[3], ff c2inv)
 }
 
 // ----------------------------------------------------------------------------------------------- correction
-// Energy-correction loop of one species (Algorithm 1, final loop) by a segment of W lanes (a warp, or a half warp;
+// Energy-correction loop of one species (Algorithm 1, final loop) by a segment of W lanes (a warp, a half or a quarter;
 // W = WIDTH, or the runtime width when WIDTH is 0): pairs of adjacent particles of the order rho, pass p from offset
 // p mod 2, in chunks of W pairs; each pair takes U = fE KE_cm (its cap) up to
 // the crossing pair, which takes the remainder of |Delta E_s| (a prefix sum over the caps gives every pair the sum
@@ -1231,7 +1231,7 @@ __device__ ff energy_loop(const StepArgs& A, const GTile& t, int64_t cs, int s0,
 {
     const int W = WIDTH ? WIDTH : width;
     const int lane = threadIdx.x & (W - 1);
-    const unsigned mask = W == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
+    const unsigned mask = lane_mask(W);
     const int cap = t.cap;
     const ff ms = mass_ff(A, spc);
     const ff fE = {A.fE_f, A.fE_lo};
@@ -1345,7 +1345,7 @@ template <bool REL, int G>
 __device__ __forceinline__ ff energy_call(const StepArgs& A, const GTile& t, int64_t cs, int s0, int ns, int spc,
                                           int mode, ff D, int width, int& used, bool& done)
 {
-    return energy_loop_ool<REL, G == 32 ? 0 : 32>(A, t, cs, s0, ns, spc, mode, D, width, used, done);
+    return energy_loop_ool<REL, G <= 32 ? 0 : 32>(A, t, cs, s0, ns, spc, mode, D, width, used, done);
 }
 
 // Moment correction of one interaction (Sec. 4, Appendix A, Sec. 5.2). Returns 1 if the interaction failed under
@@ -1357,7 +1357,8 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
                         PhaseClk& pc)
 {
     const int cap = t.cap;
-    const int warp = wix<G>(), lane = threadIdx.x & 31;
+    const int warp = wix<G>(), lane = lix<G>();
+    constexpr int kHalf = kLanes<G> / 2, kQ = kLanes<G> / 8;  // lanes of one of two and of one of eight quantities
     const int nside = intra ? 1 : 2;
     const ff zero = {0.f, 0.f};
     const ff ma = mass_ff(A, ic.a), mb = mass_ff(A, ic.b);
@@ -1371,7 +1372,7 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
     // Eq. vp_pm: B = (sum_p m_p v_ps - sum_p m_p v_bs) / sum_p m_p w_p over the interaction's particles, the
     // pre-scatter sum being the carried per-species momentum
     ff B[3], Pnew = zero;
-    const int grp = lane >> 2;  // the quantity this lane holds: momentum of species a (0..2), of species b (3..5)
+    const int grp = lane / kQ;  // the quantity this lane holds: momentum of species a (0..2), of species b (3..5)
     if (on) {
         ff acc[8];
 #pragma unroll
@@ -1398,12 +1399,13 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
         const bool has = grp < (intra ? 3 : 6);
         const int spc = sb ? ic.b : ic.a, comp = sb ? grp - 3 : grp;
         ff dP = has ? ff_sub(P, sh.car[spc][kMom + comp]) : zero;
-        dP = ff_add(dP, {__shfl_down_sync(0xffffffffu, dP.hi, 12), __shfl_down_sync(0xffffffffu, dP.lo, 12)});
+        dP = ff_add(dP, {__shfl_down_sync(gmask<G>(), dP.hi, 3 * kQ, kLanes<G>),
+                           __shfl_down_sync(gmask<G>(), dP.lo, 3 * kQ, kLanes<G>)});
         const ff W2 = sh.car[ic.a][kW2m];
         const ff inv = ffq_div(ffk(1.f), intra ? W2 : ff_add(W2, sh.car[ic.b][kW2m]));
-        const ff Bl = ff_mul(dP, inv);  // lanes 0..11
+        const ff Bl = ff_mul(dP, inv);  // the first 3 kQ lanes
 #pragma unroll
-        for (int d = 0; d < 3; ++d) B[d] = shidx(Bl, 4 * d);
+        for (int d = 0; d < 3; ++d) B[d] = shidx<G>(Bl, kQ * d);
         // carried momentum after the shift, written once the correction is done
         if (has) Pnew = ff_sub(P, ff_mul(comp == 0 ? B[0] : (comp == 1 ? B[1] : B[2]), sh.car[spc][kW2m]));
     }
@@ -1437,32 +1439,32 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
     // species a did not fail, and a failed interaction is replayed without it, so only the pair count of species b
     // is dropped when species a fails.
     const bool both = !intra && A.fail_policy == 0;
-    ff Es = zero;  // lanes 0..15: species a, 16..31: species b (intra: zero)
+    ff Es = zero;  // first half of the lanes: species a, second: species b (intra: zero)
     if (on) Es = greduce<G, 2>(e2, sh.red[1]);
     csync<G>();
     PHASE_MARK(pc, 4);
     if (!on) return 0;
     // unit 0 runs species a (and b when not both), unit 1 species b
-    const int unit = both ? (G == 32 ? lane >> 4 : warp) : (warp == 0 ? 0 : 2);
+    const int unit = both ? (G <= 32 ? lane / kHalf : warp) : (warp == 0 ? 0 : 2);
     if (unit < 2) {
         // Eq. Econs: Delta E = E_pm - E_bs, the pre-interaction energies carried; Eq. DeltaEs: its split in proportion
         // to mean weight times post-shift energy. A species with fewer than two particles cannot take a share; no
         // eligible species with Delta E != 0 fails. |Delta E_s| at or below 2^-47 of the species' post-shift energy
         // counts as zero (rounding noise). Each half warp computes its species' terms.
-        const bool hb = lane >= 16;
+        const bool hb = lane >= kHalf;
         const bool has = !(intra && hb);
         const int hs = hb ? ic.b : ic.a;
         const ff Epm = has ? ff_mul(hb ? mb : ma, Es) : zero;
         ff dE = has ? ff_sub(Epm, sh.car[hs][kEn]) : zero;
-        if (!intra) dE = ff_add(dE, shx(dE, 16));
+        if (!intra) dE = ff_add(dE, shx<G>(dE, kHalf));
         ff D0 = dE, D1 = zero;
         int fail = 0;
         if (!intra) {
             const bool can0 = na >= 2, can1 = nb >= 2;
             if (can0 && can1) {
                 const ff wx = ff_mul(sh.car[hs][kWbar], Epm);
-                const ff wa = shidx(wx, 0);
-                const ff den = ff_add(wx, shx(wx, 16));
+                const ff wa = shidx<G>(wx, 0);
+                const ff den = ff_add(wx, shx<G>(wx, kHalf));
                 if (den.hi > 0.f) {
                     D0 = ff_mul(ffq_div(wa, den), dE);
                     D1 = ff_sub(dE, D0);
@@ -1478,9 +1480,9 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
                 fail = 1;
             }
         } else {
-            D0 = shidx(dE, 0);
+            D0 = shidx<G>(dE, 0);
         }
-        const ff Epm0 = shidx(Epm, 0), Epm1 = shidx(Epm, 16);
+        const ff Epm0 = shidx<G>(Epm, 0), Epm1 = shidx<G>(Epm, kHalf);
         if (fabsf(D0.hi) <= 0x1p-47f * Epm0.hi) D0 = zero;
         if (fabsf(D1.hi) <= 0x1p-47f * Epm1.hi) D1 = zero;
         ff Eaft0 = Epm0, Eaft1 = Epm1;
@@ -1494,7 +1496,7 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
                 const int s0 = side ? b0 : a0, ns = side ? nb : na, spc = side ? ic.b : ic.a;
                 const int mode = A.sort_by_weight ? sh.wmode[spc] : 1;
                 int u = 0;
-                const ff ab = energy_call<REL, G>(A, t, cs, s0, ns, spc, mode, Ds, G == 32 ? 16 : 32, u, done);
+                const ff ab = energy_call<REL, G>(A, t, cs, s0, ns, spc, mode, Ds, G <= 32 ? kHalf : 32, u, done);
                 if (side) {
                     Eaft1 = ff_sub(Eaft1, ab);
                     used1 = u;
@@ -1510,19 +1512,19 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
             if (!fail && !ff_is0(D0)) {
                 bool done;
                 const int mode = A.sort_by_weight ? sh.wmode[ic.a] : 1;
-                Eaft0 = ff_sub(Eaft0, energy_call<REL, G>(A, t, cs, a0, na, ic.a, mode, D0, 32, used0, done));
+                Eaft0 = ff_sub(Eaft0, energy_call<REL, G>(A, t, cs, a0, na, ic.a, mode, D0, kLanes<G>, used0, done));
                 if (!done) fail0 = 1;
             }
             if (!fail && !fail0 && !intra && !ff_is0(D1)) {
                 bool done;
                 const int mode = A.sort_by_weight ? sh.wmode[ic.b] : 1;
-                Eaft1 = ff_sub(Eaft1, energy_call<REL, G>(A, t, cs, b0, nb, ic.b, mode, D1, 32, used1, done));
+                Eaft1 = ff_sub(Eaft1, energy_call<REL, G>(A, t, cs, b0, nb, ic.b, mode, D1, kLanes<G>, used1, done));
                 if (!done) fail1 = 1;
             }
         }
         // per unit: lane totals of the pair counts, then the unit's first lane publishes its species' results
-        const unsigned mask = (both && G == 32) ? (0xffffu << (threadIdx.x & 16)) : 0xffffffffu;
-        const int width = (both && G == 32) ? 16 : 32;
+        const int width = (both && G <= 32) ? kHalf : kLanes<G>;
+        const unsigned mask = lane_mask(width);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             if (o < width) {
@@ -1560,7 +1562,7 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
         if (!intra) sh.car[ic.b][kEn] = sh.eres_E[1];
         if (fail && A.fail_policy == 2) latch(A.status, kErrCorrectionFailed);
     }
-    if (warp == 0 && (lane & 3) == 0 && grp < (intra ? 3 : 6))
+    if (warp == 0 && (lane & (kQ - 1)) == 0 && grp < (intra ? 3 : 6))
         sh.car[grp >= 3 ? ic.b : ic.a][kMom + (grp >= 3 ? grp - 3 : grp)] = Pnew;
     PHASE_MARK(pc, 5);
     return (fail && A.fail_policy == 0) ? 1 : 0;
@@ -1576,7 +1578,8 @@ __device__ __forceinline__ void gload(const StepArgs& A, const GTile& t, GShared
                           reinterpret_cast<const float*>(A.vz)};
     const ff zero = {0.f, 0.f};
     const ff c2inv = {A.c2inv_f, A.c2inv_lo};
-    const int lane = threadIdx.x & 31, grp = lane >> 2;
+    constexpr int kQ = kLanes<G> / 8;  // lanes of one of eight quantities
+    const int lane = lix<G>(), grp = lane / kQ;
     const bool order = A.correct && A.sort_by_weight;
     unsigned need = 0;  // species whose segment is not stored in strictly descending weight
     for (int sp = 0; sp < S; ++sp) {
@@ -1607,10 +1610,10 @@ __device__ __forceinline__ void gload(const StepArgs& A, const GTile& t, GShared
         }
         acc[6] = ffk(unordered);
         const ff sum = greduce<G, 8>(acc, sh.red[sp & 1]);  // quantity grp
-        if (__shfl_sync(0xffffffffu, sum.hi, 24) > 0.f) need |= 1u << sp;
+        if (__shfl_sync(gmask<G>(), sum.hi, 6 * kQ, kLanes<G>) > 0.f) need |= 1u << sp;
         const ff mean = ns > 0 ? ffq_div(sum, ffk((float)ns)) : zero;
         const ff massed = ff_mul(mass_ff(A, sp), sum);
-        if (wix<G>() == 0 && (lane & 3) == 0 && grp < 6) sh.car[sp][grp] = grp == kWbar ? mean : massed;
+        if (wix<G>() == 0 && (lane & (kQ - 1)) == 0 && grp < 6) sh.car[sp][grp] = grp == kWbar ? mean : massed;
     }
     gsync<G>();
     if (A.resid && tix<G>() == 0) {
@@ -1733,8 +1736,8 @@ __device__ void gcell(const StepArgs& A, int c, uint64_t skip, int used, unsigne
             }
             const ff x = ff_mul(mass_ff(A, sp), greduce<G, 8>(acc, sh.red[sp & 1]));
 #pragma unroll
-            for (int q = 0; q < 4; ++q) tot[q] = ff_add(tot[q], shidx(x, 4 * q));
-            amag = ff_add(amag, shidx(x, 16));
+            for (int q = 0; q < 4; ++q) tot[q] = ff_add(tot[q], shidx<G>(x, kLanes<G> / 8 * q));
+            amag = ff_add(amag, shidx<G>(x, kLanes<G> / 2));
         }
         if (tix<G>() == 0) {
             double dp = 0.0;
@@ -1756,8 +1759,8 @@ __device__ void gcell(const StepArgs& A, int c, uint64_t skip, int used, unsigne
     if (tix<G>() == 0 && A.phase_clk) {
 #pragma unroll
         for (int q = 0; q < 7; ++q)
-            atomicAdd(A.phase_clk + 8 * A.gcls + q, (unsigned long long)pc.acc[q]);
-        atomicAdd(A.phase_clk + 8 * A.gcls + 7, 1ull);  // cells
+            atomicAdd(A.phase_clk + 8 * (A.gcls < kGroupClasses ? A.gcls : 0) + q, (unsigned long long)pc.acc[q]);
+        atomicAdd(A.phase_clk + 8 * (A.gcls < kGroupClasses ? A.gcls : 0) + 7, 1ull);  // cells
     }
 #endif
 }
@@ -1810,6 +1813,7 @@ __global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group
             }
         }
         gcell<REL, G>(A, c, skip, used, tile, sh, cta, step);
+        if (G < 32) __syncwarp();
         __syncthreads();
     }
 }
@@ -1817,9 +1821,14 @@ __global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group
 // Shared memory of one group of class cls beside its tile.
 inline size_t shared_bytes_of(int cls)
 {
-    const size_t b[kGroupClasses] = {group_shared_bytes<32>(), group_shared_bytes<64>(), group_shared_bytes<128>(),
-                                     group_shared_bytes<256>(), group_shared_bytes<512>()};
-    return b[cls];
+    switch (cls) {
+    case 0: return group_shared_bytes<32>();
+    case 1: return group_shared_bytes<64>();
+    case 2: return group_shared_bytes<128>();
+    case 3: return group_shared_bytes<256>();
+    case 4: return group_shared_bytes<512>();
+    default: return group_shared_bytes<16>();
+    }
 }
 
 template <bool REL, int G>

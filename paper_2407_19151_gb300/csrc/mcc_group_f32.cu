@@ -11,7 +11,8 @@ const void* group_kernel_f32(int cls)
     case 1: return grp::group_kernel_ptr<false, 64>();
     case 2: return grp::group_kernel_ptr<false, 128>();
     case 3: return grp::group_kernel_ptr<false, 256>();
-    default: return grp::group_kernel_ptr<false, 512>();
+    case 4: return grp::group_kernel_ptr<false, 512>();
+    default: return grp::group_kernel_ptr<false, 16>();
     }
 }
 

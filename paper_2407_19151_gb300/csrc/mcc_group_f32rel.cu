@@ -11,7 +11,8 @@ const void* group_kernel_f32rel(int cls)
     case 1: return grp::group_kernel_ptr<true, 64>();
     case 2: return grp::group_kernel_ptr<true, 128>();
     case 3: return grp::group_kernel_ptr<true, 256>();
-    default: return grp::group_kernel_ptr<true, 512>();
+    case 4: return grp::group_kernel_ptr<true, 512>();
+    default: return grp::group_kernel_ptr<true, 16>();
     }
 }
 

@@ -83,8 +83,8 @@ struct StepArgs {
     int32_t slab_cap;
     const int32_t* order_range;  // one-CTA kernel: [begin, end) of `order` to take cells from (null: every cell)
     // group kernels (mcc_group.cuh)
-    const int32_t* class_off;  // [2 * kGroupClasses + 2]: begin / end of each size class in `order` (last: the rest)
-    int32_t* queues;           // [kGroupClasses + 1] work-queue counters, one per class
+    const int32_t* class_off;  // [2 * kOrderClasses]: begin / end of each size class in `order`
+    int32_t* queues;           // [kOrderClasses] work-queue counters, one per class
     int32_t gcls;              // size class of the launch
     int32_t gcap;              // particles one group stages on chip in this class
     int32_t max_cell;          // the caller's bound on particles per cell (larger cells latch kErrBounds)
@@ -93,6 +93,16 @@ struct StepArgs {
 };
 
 constexpr int kGroupClasses = 5;  // group sizes 32, 64, 128, 256, 512 threads
+// Beside them in the order of the cells: the cells above every class (the one-CTA kernel's), and the cells of class 0 below
+// kHalfCells particles, run two to a warp if there are enough. A visit of a small cell takes nearly the same time
+// whatever its size (serial phases, few lanes busy), so two at once nearly halve it. Measured
+// per step, three species, one / two to a warp: 40000 cells of 30: 1.62 / 1.05 ms, of 90: 1.65 / 1.26, of 120: 1.74 / 1.62;
+// 2e5 of 30: 7.23 / 4.12; relativistic beam of 65536 cells 7.54 / 6.25. At 128 particles a warp's two tiles still fit its
+// share of the shared memory; lines at 160 and 224, where fewer warps are resident, take 1.09 and 1.31 ms at 30 particles.
+constexpr int kRestClass = kGroupClasses, kHalfClass = kGroupClasses + 1, kOrderClasses = kGroupClasses + 2;
+constexpr int kHalfCells = 128;  // a multiple of an eighth of its octave (the order's steps)
+// Threads of a group of class cls.
+constexpr int group_threads(int cls) { return cls == kHalfClass ? 16 : 32 << cls; }
 #ifndef MCC_GROUP_WARPS_PER_SM
 #define MCC_GROUP_WARPS_PER_SM 16
 #endif
@@ -125,12 +135,14 @@ void f64_tables(double* out);
 cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_step_advance(uint64_t* step, uint64_t by, cudaStream_t st);
 // Cells ordered by group size class (largest class first; class kGroupClasses = cells above every class), largest
-// first within a class; class_off receives each class's [begin, end) in `order`. hist: group_order_hist_bytes() of zeroed
+// first within a class; class_off receives each class's [begin, end) in `order`.
+// half_min: class kHalfClass takes class 0's cells below kHalfCells
+// if they are at least so many (0: never). hist: group_order_hist_bytes() of zeroed
 // device memory.
 size_t group_order_hist_bytes();
 cudaError_t launch_group_order(const int64_t* offsets, int32_t n_cells, int32_t S, const int32_t* caps,
-                               int32_t* order, int32_t* class_off, int32_t* hist, int64_t* launches, cudaStream_t st);
-// Group kernels (mcc_group_*.cu): class cls runs groups of 32 << cls threads.
+                               int32_t half_min, int32_t* order, int32_t* class_off, int32_t* hist, int64_t* launches, cudaStream_t st);
+// Group kernels (mcc_group_*.cu): class cls runs groups of group_threads(cls) threads.
 const void* group_kernel(bool f32, bool rel, int cls);
 size_t group_shared_bytes(int cls);  // shared variables of one group
 // groups: groups (cells at a time) of one CTA
