@@ -880,6 +880,7 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
         if (cs == cudaStreamCaptureStatusActive) rec_flags = cudaEventRecordExternal;
     }
     // one launch of a size class with tiles of cap particles
+    bool after = false;  // the launch before is a class of this step
     auto run_class = [&](int cls, int32_t cap) -> int {
         // fewer cells than groups: spread them over the SMs
         const int per_sm = (n_cells + ctx->num_sms - 1) / ctx->num_sms;
@@ -898,7 +899,8 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
         if (grid > n_cells) grid = n_cells;
         a.gcls = cls;
         a.gcap = cap;
-        const cudaError_t e = mcc::launch_group(f32, rel, cls, a, grid, groups, smem, S(stream));
+        const cudaError_t e = mcc::launch_group(f32, rel, cls, a, grid, groups, smem, after, S(stream));
+        after = !p->launch_events;  // (an event between two kernels orders them)
         ctx->launches += 1;
         return e == cudaSuccess ? MCC_OK : MCC_ERR_CUDA;
     };
@@ -922,6 +924,7 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
             if (rc != MCC_OK) return rc;
         }
         mark(mcc::kGroupClasses, 1);
+        after = false;
         for (int cls = mcc::kGroupClasses - 1; cls >= 0; --cls) {
             mark(cls, 0);
             // no cell can be in this class

@@ -1246,11 +1246,21 @@ const void* group_kernel(bool f32, bool rel, int cls)
     return rel ? group_kernel_f32rel(cls) : group_kernel_f32(cls);
 }
 
-cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem,
+cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem, bool after,
                          cudaStream_t st)
 {
     void* args[] = {const_cast<StepArgs*>(&a)};
-    return cudaLaunchKernel(group_kernel(f32, rel, cls), dim3(grid), dim3(groups * group_threads(cls)), args, smem, st);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(groups * group_threads(cls));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = after ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, group_kernel(f32, rel, cls), args);
 }
 
 size_t pair_tile_bytes_per_particle() { return kPairTileBytesPerParticle; }

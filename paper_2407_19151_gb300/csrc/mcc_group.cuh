@@ -1785,6 +1785,10 @@ __global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group
     GShared<G>& sh = *reinterpret_cast<GShared<G>*>(mem);
     unsigned char* tile = mem + group_shared_bytes<G>();
     if (threadIdx.x == 0) cta.n_retry = 0;
+    // The next class's CTAs may start where this one's have finished (its cells are others): a class otherwise left the GPU idle
+    // for the better part of a visit at its end. Three-species steps, one after another / overlapped: 1500 cells of 500 0.70 /
+    // 0.47 ms, 20000 of 300 1.83 / 1.59, 2^18 of 512 28.28 / 28.08; relativistic beam of 65536 cells 6.25 / 6.03.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (;;) {
         if (threadIdx.x == 0) {
             cta.retry = cta.n_retry >= teams;
@@ -1816,6 +1820,8 @@ __global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group
         if (G < 32) __syncwarp();
         __syncthreads();
     }
+    // done only when the classes before it are: what follows the step waits for its last class alone
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Shared memory of one group of class cls beside its tile.

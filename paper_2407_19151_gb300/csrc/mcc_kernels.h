@@ -145,8 +145,9 @@ cudaError_t launch_group_order(const int64_t* offsets, int32_t n_cells, int32_t 
 // Group kernels (mcc_group_*.cu): class cls runs groups of group_threads(cls) threads.
 const void* group_kernel(bool f32, bool rel, int cls);
 size_t group_shared_bytes(int cls);  // shared variables of one group
-// groups: groups (cells at a time) of one CTA
-cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem,
+// groups: groups (cells at a time) of one CTA; after: the launch before it on the stream is a class of the same step, and
+// this one may overlap it
+cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem, bool after,
                          cudaStream_t st);
 int cell_kernel_blocks_per_sm(bool f32, bool rel, int mode, size_t smem);
 cudaError_t set_cell_smem_limit(bool f32, bool rel, int mode, size_t smem);
