@@ -10,10 +10,12 @@
 // Lockstep: what bounds a cell visit is instruction fetch. A visit is nearly straight-line code (each loop runs two or
 // three times over ~170 particles of a species, the code of one interaction is far larger than an SM partition's
 // instruction cache), and with sixteen independent warps per SM at different places every warp fetched for itself. The
-// groups of a CTA take cells of nearly equal size (the class order is by size) and meet at a CTA barrier after every
-// phase of an interaction, so that all warps of the SM run the same code at about the same time and share its
-// fetches. One GB300, against independent CTAs of one group each: three-species step of 1.34e8 particles 43.9 -> 29.1 ms,
-// relativistic beam of 1.16e7 particles 16.9 -> 8.0 ms.
+// groups of a CTA take cells of nearly equal size (the class order is by size) and meet at a CTA barrier in every
+// interaction, after its pair loop, so that all warps of the SM run the same code at about the same time and share its
+// fetches. One GB300, against independent CTAs of one group each: three-species step of 1.34e8 particles 43.9 -> 27.4 ms,
+// relativistic beam of 1.16e7 particles 16.9 -> 5.9 ms (with two small cells to a warp). A barrier after every phase takes
+// 28.1 ms, after the permutations or before the shift instead of after the pairs 28.3 and 27.6, in every second
+// interaction 27.9, none within a visit 31.5.
 //
 // Per cell visit the particles are staged in shared memory and the whole step of Algorithm 1 runs there, every
 // interaction (a, b) in list order:
@@ -217,11 +219,18 @@ __device__ __forceinline__ bool gany(bool p)
     return r != 0;
 }
 
+// The two groups of a warp together again (G = 16).
+template <int G>
+__device__ __forceinline__ void hsync()
+{
+    if (G < 32) __syncwarp();
+}
+
 // Lockstep barrier of the CTA's groups (nothing to do when the CTA is one group).
 template <int G>
 __device__ __forceinline__ void csync()
 {
-    if (G < 32) __syncwarp();  // both groups of the warp
+    hsync<G>();
     if (blockDim.x > G) __syncthreads();
 }
 
@@ -367,7 +376,8 @@ struct GShared {
     ff eres_E[2];   // energy phase results: carried energy of species a, b after their energy pairs
     int eres_i[4];  // pairs used and failure of species a, then of species b
     int sci[G / 32 + 1];
-    uint32_t wrange[kMaxSpecies][G > 32 ? G / 32 : 1][2];  // per warp: smallest and largest top key word of a species (weight order)
+    // per warp: smallest and largest top key word of a species (weight order)
+    uint32_t wrange[kMaxSpecies][G > 32 ? G / 32 : 1][2];
 };
 
 // What the groups of a CTA share: the cells of the batch, and the cells to visit again without their failed interactions
@@ -544,8 +554,8 @@ __device__ __forceinline__ void sort_keys(uint64_t* key, int n)
 // buckets as fit the species' slots of the (still unused) permutation, then an insertion sort within a bucket. The IEEE
 // bits of a weight are nearly linear in its logarithm, so weights spread over decades fill the buckets evenly. A species
 // with a bucket above kBucketMost takes the bitonic network instead; equal weights are found without a sort.
-// Against one-warp bitonic sorts: equilibration steps (tied electron weights, unordered ions, 2.1e6 particles, two steps) 0.77 ->
-// 0.64 ms, relativistic beam (unordered) 7.98 -> 7.81 ms.
+// Against one-warp bitonic sorts: equilibration steps (tied electron weights, unordered ions, 2.1e6 particles, two steps)
+// 0.77 -> 0.64 ms, relativistic beam (unordered) 7.98 -> 7.81 ms.
 constexpr int kBucketMost = 12;
 
 template <int G>
@@ -1410,7 +1420,7 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
         if (has) Pnew = ff_sub(P, ff_mul(comp == 0 ? B[0] : (comp == 1 ? B[1] : B[2]), sh.car[spc][kW2m]));
     }
 
-    csync<G>();
+    hsync<G>();
     PHASE_MARK(pc, 3);
     // momentum shift v_pm = v_ps - B w_p (Eq. vp_pm) and the post-shift species energies (Eq. DeltaEs)
     ff e2[2] = {zero, zero};
@@ -1441,7 +1451,8 @@ __device__ int gcorrect(const StepArgs& A, const GTile& t, GShared<G>& sh, int c
     const bool both = !intra && A.fail_policy == 0;
     ff Es = zero;  // first half of the lanes: species a, second: species b (intra: zero)
     if (on) Es = greduce<G, 2>(e2, sh.red[1]);
-    csync<G>();
+    if (on && G <= 32) gsync<G>();
+    hsync<G>();
     PHASE_MARK(pc, 4);
     if (!on) return 0;
     // unit 0 runs species a (and b when not both), unit 1 species b
@@ -1662,7 +1673,7 @@ __device__ void gcell(const StepArgs& A, int c, uint64_t skip, int used, unsigne
     const int kept = used;
     bool again = false;
     if (mine) gload<REL, G>(A, t, sh, cs, S);
-    csync<G>();
+    hsync<G>();
     PHASE_MARK(pc, 0);
     for (int k = 0; k < A.n_inter; ++k) {
         const InterConst& ic = A.ic[k];
@@ -1677,7 +1688,7 @@ __device__ void gcell(const StepArgs& A, int c, uint64_t skip, int used, unsigne
         const bool on = mine && !again && !((skip >> k) & 1ull) && (intra ? (na >= 2) : (na > 0 && nb > 0));
         const uint32_t ictr = (uint32_t)(A.inter_base + k);
         if (on) gpermutations<G>(A, t, sh, c, ictr, intra ? 1 : 2, a0, na, b0, nb, step);
-        csync<G>();
+        hsync<G>();
         PHASE_MARK(pc, 1);
         if (on) gscatter<REL, G>(A, t, c, cs, ictr, ic, intra, a0, na, b0, nb, step);
         csync<G>();
@@ -1785,9 +1796,10 @@ __global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group
     GShared<G>& sh = *reinterpret_cast<GShared<G>*>(mem);
     unsigned char* tile = mem + group_shared_bytes<G>();
     if (threadIdx.x == 0) cta.n_retry = 0;
-    // The next class's CTAs may start where this one's have finished (its cells are others): a class otherwise left the GPU idle
-    // for the better part of a visit at its end. Three-species steps, one after another / overlapped: 1500 cells of 500 0.70 /
-    // 0.47 ms, 20000 of 300 1.83 / 1.59, 2^18 of 512 28.28 / 28.08; relativistic beam of 65536 cells 6.25 / 6.03.
+    // The next class's CTAs may start where this one's have finished (its cells are others): a class otherwise left the
+    // GPU idle for the better part of a visit at its end. Three-species steps, one after another / overlapped: 1500 cells
+    // of 500 0.70 / 0.47 ms, 20000 of 300 1.83 / 1.59, 2^18 of 512 28.28 / 28.08; relativistic beam of 65536 cells
+    // 6.25 / 6.03 ms.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1817,7 +1829,7 @@ __global__ void __launch_bounds__(G > 32 * group_cta_warps(REL) ? G : 32 * group
             }
         }
         gcell<REL, G>(A, c, skip, used, tile, sh, cta, step);
-        if (G < 32) __syncwarp();
+        hsync<G>();
         __syncthreads();
     }
     // done only when the classes before it are: what follows the step waits for its last class alone

@@ -111,8 +111,8 @@ constexpr int group_threads(int cls) { return cls == kHalfClass ? 16 : 32 << cls
 constexpr int kGroupWarpsPerSm = MCC_GROUP_WARPS_PER_SM;
 // Warps of one CTA of the group kernels; its groups run in lockstep (mcc_group.cuh). Two CTAs of eight warps per SM
 // overlap one's barrier waits with the other's work; the relativistic code is larger and gains more from fetching once for
-// all sixteen warps (three-species step of 1.34e8 particles: 37.9 / 29.1 / 30.6 ms with 4 / 8 / 16 warps; relativistic beam
-// of 1.16e7: 12.2 / 8.7 / 8.0 ms).
+// all sixteen warps (three-species step of 1.34e8 particles: 27.4 / 28.5 ms with 8 / 16 warps, four were 30% slower than
+// eight; relativistic beam of 1.16e7: 6.7 / 5.9 ms).
 constexpr int group_cta_warps(bool rel) { return rel ? 16 : 8; }
 
 // Bytes per particle of the cell tile (keys, weights, velocities, pre-scatter copy, permutation, weight order).
