@@ -345,8 +345,10 @@ int mcc_step_workspace_size(mcc_ctx* ctx, int32_t prec, int32_t n_cells, int32_t
 /*
  * mcc_step_fused: n_steps whole collision steps (Algorithm 1 for every interaction in list order, each step with
  * index params->step + t). A small kernel orders the cells once per call by size class (mcc_group_capacities),
- * largest first; each step then launches one persistent kernel per non-empty class, in which a group of 32 << k
- * threads takes cells from the class's work queue, stages the cell in shared memory, runs pairing, scatter and
+ * largest first; each step then launches one persistent kernel per possible class (a class kernel may overlap the one
+ * before it, unless params->launch_events are recorded between them), in which a group of 32 << k threads (half a
+ * warp for cells below 128 particles, when there are many) takes cells from the class's work queue, stages the cell
+ * in shared memory, runs pairing, scatter and
  * correction for every interaction and writes the cell back. Cells above every class run on a one-CTA kernel (from
  * its workspace slab when larger than its on-chip tile). For MCC_F64 the result equals the sequence
  * mcc_pair / mcc_scatter / mcc_correct over the interactions (up to rounding). For MCC_F32_MIXED the velocities of
@@ -374,7 +376,9 @@ int mcc_set_tile_cap(mcc_ctx* ctx, int32_t cap);
  * particles_per_warp sets caps[k] = particles_per_warp << k for k < 4 (0 = automatic: the capacity with which
  * sixteen warps share an SM's shared memory); largest sets caps[4] (0 = as large as one CTA's shared memory
  * allows). Every capacity is capped by what one CTA's shared memory holds (44 bytes per particle). Both 0 is the
- * default; a call with few cells then runs its cells on larger groups than these classes say. Used by the autotuner; the step's results do not depend on it. */
+ * default; a call with few cells then runs its cells on larger groups than these classes say, and one with many small
+ * cells runs those on half warps. Used by the autotuner; the step's results do not depend on it beyond the order of
+ * float-float sums. */
 int mcc_set_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp, int32_t largest);
 
 /* The five class capacities mcc_step_fused uses for this precision and mode (caps_out: host int32[5]). */

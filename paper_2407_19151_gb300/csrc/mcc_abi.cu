@@ -767,11 +767,13 @@ void group_caps(const mcc_ctx* ctx, bool f32, bool rel, int32_t caps[mcc::kGroup
 // one launch serves what would be several (the classes run one after another). Cells go up to class 3; class k is taken
 // while n_cells groups of it fit the GPU. Measured per step, 152 SMs, two species (us by group size 64 / 128 / 256 / 512):
 // 100 cells of 300: 43.6 / 35.2 / 32.8 / 36.2; 100 of 1000: 84.8 / 54.6 / 42.9 / 43.3; 600 of 300: 47.4 / 44.3 / 68 / 134;
-// 1200 of 300: 56.7 / 85 / 130 / 262.
-void few_cells_caps(const mcc_ctx* ctx, int32_t n_cells, int32_t caps[mcc::kGroupClasses])
+// 1200 of 300: 56.7 / 85 / 130 / 262. Not on more threads than half the largest cell's particles: 500 three-species
+// cells of 50 take 133 us per call with one-warp groups and 142 with 128 threads.
+void few_cells_caps(const mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, int32_t caps[mcc::kGroupClasses])
 {
     int k = 0;
-    while (k < 3 && ((int64_t)n_cells << (k + 1)) <= (int64_t)mcc::kGroupWarpsPerSm * ctx->num_sms) ++k;
+    while (k < 3 && ((int64_t)n_cells << (k + 1)) <= (int64_t)mcc::kGroupWarpsPerSm * ctx->num_sms && (128 << k) <= max_cell)
+        ++k;
     for (int j = 0; j < k; ++j) caps[j] = -1;  // not even empty cells
 }
 }  // namespace
@@ -838,7 +840,7 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     if (!ws || ws_bytes < need) return MCC_ERR_WORKSPACE;
     int32_t caps[mcc::kGroupClasses];
     group_caps(ctx, f32, rel, caps);
-    if (ctx->group_cap == 0) few_cells_caps(ctx, n_cells, caps);
+    if (ctx->group_cap == 0) few_cells_caps(ctx, n_cells, max_cell, caps);
     // two small cells to a warp, with automatic capacities, if they fill every warp's halves (a launch of its own costs the
     // time of a visit, 0.1 ms)
     int32_t half_min = 2 * mcc::kGroupWarpsPerSm * ctx->num_sms;
