@@ -36,10 +36,10 @@ struct mcc_ctx {
     size_t smem_reserved;  // shared memory the system reserves per CTA
     // Attributes of the kernels, looked up once (each look-up costs about a microsecond of every call), and the last
     // occupancy of each: launch shape << 8 | CTAs per SM in one word, so threads may share a context.
-    size_t cell_static[2][2][4];  // [float][relativistic][mode]
+    size_t cell_static[2][2][mcc::kModes];  // [float][relativistic][mode]
     size_t group_static[2][mcc::kOrderClasses];
     size_t adjoint_static;
-    std::atomic<uint64_t> cell_occ[2][2][4], group_occ[2][mcc::kOrderClasses];
+    std::atomic<uint64_t> cell_occ[2][2][mcc::kModes], group_occ[2][mcc::kOrderClasses];
 };
 
 namespace mcc {
@@ -446,7 +446,7 @@ int mcc_create(mcc_ctx** out, int device)
     cudaError_t attr = cudaSuccess;
     for (int f32 = 0; f32 < 2; ++f32)
         for (int rel = 0; rel < 2; ++rel)
-            for (int mode = 0; mode < 4; ++mode) {
+            for (int mode = 0; mode < mcc::kModes; ++mode) {
                 c->cell_static[f32][rel][mode] = mcc::cell_kernel_static_smem(f32, rel, mode);
                 c->cell_occ[f32][rel][mode] = 0;
                 const cudaError_t e =
@@ -922,7 +922,8 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
             big.rng.step = a.rng.step;
             big.step_add = a.step_add;
             const int cap = max_cell <= tile ? max_cell : tile;
-            rc = run_cells(ctx, big, f32, rel, mcc::kFused, cap, S(stream), max_grid);
+            const bool small = !f32 && max_cell <= mcc::kSmallCells && n_cells > 4 * ctx->num_sms;
+            rc = run_cells(ctx, big, f32, rel, small ? mcc::kFusedSmall : mcc::kFused, cap, S(stream), max_grid);
             if (rc != MCC_OK) return rc;
         }
         mark(mcc::kGroupClasses, 1);

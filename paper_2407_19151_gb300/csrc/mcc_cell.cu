@@ -25,9 +25,15 @@
 #ifndef MCC_MIN_BLOCKS
 #define MCC_MIN_BLOCKS 4
 #endif
+// Small cells are not bound by the FP64 pipe but by the latency of a visit (barriers, serial phases): six CTAs per SM
+// (kSmallMinBlocks) for FP64 steps whose cells hold at most kSmallCells particles, if there are more than four per SM. Four /
+// six per SM, per call: 5000 cells of one species, 24 / 100 / 200 particles, TA77: 251 / 338 / 502 -> 205 / 268 / 427 us;
+// three species of 50: 1471 -> 1343; of 200 (cells to ~800) 1729 -> 1801, so these keep four.
 
 namespace mcc {
 namespace {
+
+constexpr int kSmallMinBlocks = 6;
 
 template <class V>
 struct WStore;
@@ -997,8 +1003,8 @@ __device__ void process_cell(const StepArgs& A, int c, unsigned char* dyn, Share
     }
 }
 
-template <class V, bool REL, int MODE>
-__global__ void __launch_bounds__(kThreads, MCC_MIN_BLOCKS) cell_kernel(const __grid_constant__ StepArgs A)
+template <class V, bool REL, int MODE, int MIN_BLOCKS = MCC_MIN_BLOCKS>
+__global__ void __launch_bounds__(kThreads, MIN_BLOCKS) cell_kernel(const __grid_constant__ StepArgs A)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ Shared sh;
@@ -1160,14 +1166,19 @@ __global__ void __launch_bounds__(kOrderThreads) k_order_place(const int64_t* __
         order[atomicAdd(&h[group_bin(offsets[(int64_t)(c + 1) * S] - offsets[(int64_t)c * S], caps.cap)], 1)] = c;
 }
 
-template <class V, bool REL, int MODE>
+template <class V, bool REL, int MODE, int MIN_BLOCKS = MCC_MIN_BLOCKS>
 const void* kernel_ptr()
 {
-    return reinterpret_cast<const void*>(&cell_kernel<V, REL, MODE>);
+    return reinterpret_cast<const void*>(&cell_kernel<V, REL, MODE, MIN_BLOCKS>);
 }
 
 const void* select_kernel(bool f32, bool rel, int mode)
 {
+    if (mode == kFusedSmall) {
+        if (f32) mode = kFused;
+        else if (rel) return kernel_ptr<double, true, kFused, kSmallMinBlocks>();
+        else return kernel_ptr<double, false, kFused, kSmallMinBlocks>();
+    }
 #define MCC_SEL(V, R)                                   \
     switch (mode) {                                     \
     case kFused: return kernel_ptr<V, R, kFused>();     \

@@ -9,7 +9,8 @@
 
 namespace mcc {
 
-enum Mode { kFused = 0, kPair = 1, kScatter = 2, kCorrect = 3 };
+enum Mode { kFused = 0, kPair = 1, kScatter = 2, kCorrect = 3, kFusedSmall = 4, kModes = 5 };
+constexpr int kSmallCells = 320;  // largest cell of kFusedSmall (mcc_cell.cu)
 
 // Per-interaction constants, precomputed on the host in FP64 (and rounded once for the mixed path).
 struct InterConst {
