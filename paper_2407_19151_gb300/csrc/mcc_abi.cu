@@ -127,8 +127,8 @@ void n97_table(float* g, float* dh)
     }
 }
 
-// Tables of mcc_pair64.cuh: Chebyshev interpolants of 1 / A(s), of e^-2A or 1 - e^-2A and of s A' / A as monomials in the interval's own variable t in [-1, 1],
-// multiples of 1/256 turn, and the reciprocals and logarithms of mantissas in [0.6875, 1.375).
+// Tables of mcc_pair64.cuh: Chebyshev interpolants of 1 / A(s), of e^-2A or 1 - e^-2A and of s A' / A as monomials in the
+// interval's own variable t in [-1, 1], multiples of 1/256 turn, and the reciprocals and logarithms of mantissas in [0.6875, 1.375).
 void f64_tables(double* out)
 {
     constexpr int N = 8;
@@ -884,10 +884,13 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     // one launch of a size class with tiles of cap particles
     bool after = false;  // the launch before is a class of this step
     auto run_class = [&](int cls, int32_t cap) -> int {
-        // fewer cells than groups: spread them over the SMs
+        // Fewer cells than groups: spread them over the SMs. Up to four groups per SM get a CTA each: so few warps fetch little,
+        // and in lockstep each waits for the slowest (us per call, in a CTA per SM / a CTA each: 600 relativistic beam cells
+        // 368 / 315, 500 three-species cells of 100 126 / 121; 1200 cells of 50, eight per SM, 152 / 205).
         const int per_sm = (n_cells + ctx->num_sms - 1) / ctx->num_sms;
         int groups = groups_per_cta(ctx, f32, rel, cls, cap);
         if (groups > per_sm) groups = per_sm;
+        if (per_sm <= 4) groups = 1;
         const size_t smem = (size_t)groups * mcc::group_smem(mcc::group_shared_bytes(cls), cap);
         const int bps = cached_occupancy(ctx->group_occ[rel][cls], ((uint64_t)smem << 6) | (uint64_t)groups, [&] {
             int b = 0;
@@ -936,7 +939,8 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
                 continue;
             }
             rc = run_class(cls, caps[cls]);
-            if (rc == MCC_OK && cls == 0 && half_min > 0) rc = run_class(mcc::kHalfClass, max_cell < mcc::kHalfCells ? max_cell : mcc::kHalfCells);
+            if (rc == MCC_OK && cls == 0 && half_min > 0)
+                rc = run_class(mcc::kHalfClass, max_cell < mcc::kHalfCells ? max_cell : mcc::kHalfCells);
             if (rc != MCC_OK) return rc;
             mark(cls, 1);
         }
