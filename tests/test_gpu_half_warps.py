@@ -55,3 +55,41 @@ def test_half_warps(case):
     np.testing.assert_array_equal(runs[0][1], runs[1][1])
     np.testing.assert_array_equal(runs[0][2], runs[1][2])
     assert velocity_error(runs[0][0], runs[1][0], wl.offsets).max() <= 2.0 ** -22
+
+
+def test_overlapped_classes_captured():
+    # every size class in one step, whose kernels overlap: a captured step replayed twice gives the two steps of a direct call, and
+    # so does a call that records events between the kernels, bit for bit
+    import paper_2407_19151_gb300 as mcc
+    wl = W.three_species(n_cells=_cells(), mean_count=110.0, sigma=0.9, data_seed=12).weight_ordered()
+    species, mc = list(zip(wl.q, wl.m)), int(np.diff(wl.offsets[:: wl.n_species]).max())
+    assert mc > 1500
+    kw = dict(method=wl.method, dt=wl.dt, fE=wl.fE, seed=wl.seed)
+
+    def step(v, p, n):
+        return mcc.mcc_step_fused(*v, w, off, wl.n_cells, wl.n_species, species, wl.lnL, p, n_steps=n, max_cell=mc)
+
+    v0, w, off = device_state(wl, "f32")
+    v1, v2 = [x.clone() for x in v0], [x.clone() for x in v0]
+    warm = [x.clone() for x in v0]
+    step(v0, mcc.Params(step=4, **kw), 2)
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2 * (mcc.GROUP_CLASSES + 1))]
+    for e in ev:
+        e.record()
+    step(v2, mcc.Params(step=4, launch_events=ev, **kw), 2)
+    counter = torch.tensor([4], dtype=torch.int64, device="cuda")
+    pd = mcc.Params(step=0, **kw)
+    pd.step_device = counter
+    step(warm, pd, 1)
+    torch.cuda.synchronize()
+    counter.fill_(4)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        step(v1, pd, 1)
+    g.replay()
+    g.replay()
+    torch.cuda.synchronize()
+    mcc.sync_status(0)
+    assert int(counter.item()) == 6
+    for a, b, c in zip(v0, v1, v2):
+        assert torch.equal(a, b) and torch.equal(a, c)
