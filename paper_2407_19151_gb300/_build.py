@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 SOURCES = ["mcc_abi.cu", "mcc_cell.cu", "mcc_bin.cu", "mcc_adjoint.cu", "mcc_pic.cu", "mcc_group_f32.cu",
            "mcc_group_f32rel.cu", "mcc_moments.cu"]
-HEADERS = ["mcc_device.cuh", "mcc_pair64.cuh", "mcc_perm.cuh", "mcc_kernels.h", "mcc_pic.h", "mcc_group.cuh"]
+HEADERS = ["mcc_device.cuh", "mcc_tables.h", "mcc_pair64.cuh", "mcc_perm.cuh", "mcc_kernels.h", "mcc_pic.h", "mcc_group.cuh"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc" if os.path.exists("/usr/local/cuda/bin/nvcc") else "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]

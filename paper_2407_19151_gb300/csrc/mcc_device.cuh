@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "mcc_tables.h"
+
 namespace mcc {
 
 #ifndef MCC_THREADS
@@ -440,11 +442,6 @@ __device__ __forceinline__ V pair_kecm_du(V c, V m1, V m2, const V v1[3], const 
 // [kN97X0, kN97X0 + kN97Nodes * kN97H]: node k holds g = A s and h dg/dx for cubic Hermite interpolation (error ~1e-9), built
 // on the host when a context is created. The FP64 pairs have their own (mcc_pair64.cuh).
 // ---------------------------------------------------------------------------------------------------------------
-constexpr int kN97Nodes = 512;
-constexpr double kN97X0 = -6.907755278982137;  // ln 1e-3
-constexpr double kN97X1 = 2.4849066497880004;  // ln 12
-constexpr double kN97H = (kN97X1 - kN97X0) / kN97Nodes;
-
 template <class V>
 struct N97Tab {
     const V* f;   // kN97Nodes + 1 values of A s

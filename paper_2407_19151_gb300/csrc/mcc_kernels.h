@@ -21,17 +21,12 @@ struct InterConst {
     float kappa_mu2_f, kappa_f, mu_ma_f, mu_mb_f;
 };
 
-// Tables of the FP64 pair kinematics (mcc_pair64.cuh), built on the host when a context is created.
-constexpr int kF64N97 = 9 * 64;  // intervals of s: 64 per octave of [2^-5, 16); eight coefficients each of 1 / A(s), of
-                                 // e^-2A (s < 2) or 1 - e^-2A, and of s A'(s) / A(s)
-constexpr int kF64Turn = 256;    // (cos, sin) of multiples of 1/256 turn
-constexpr int kF64Ln = 128;      // (r_i, -ln r_i)
+// Tables of the FP64 pair kinematics (mcc_pair64.cuh; sizes and entries: mcc_tables.h).
 struct F64Tab {
     const double2* n97;
     const double2* turn;
     const double2* ln;
 };
-constexpr size_t kF64TabDoubles = 24 * kF64N97 + 2 * kF64Turn + 2 * kF64Ln;
 
 struct StepArgs {
     const int64_t* offsets;
@@ -127,10 +122,6 @@ __host__ __device__ inline size_t group_smem(size_t shared_bytes, int cap)
 {
     return (shared_bytes + (size_t)cap * kGroupBytesPerParticle + 15) & ~(size_t)15;
 }
-
-// N97 table of the float pairs: g = A s and h dg/dx (x = ln s) at kN97Nodes + 1 nodes; tables of the FP64 pairs.
-void n97_table(float* g, float* dh);
-void f64_tables(double* out);
 
 // Kernel launches (defined in mcc_cell.cu / mcc_bin.cu).
 cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, cudaStream_t st);
