@@ -591,8 +591,13 @@ __device__ __forceinline__ RelCM<V> rel_cm(V c, V ma, V mb, const V ui[3], const
     return r;
 }
 
-// x / y with r = 1 / y: in double by the reciprocal (a division costs the FP64 pipe about eight instructions).
-__device__ __forceinline__ double over(double x, double, double r) { return x * r; }
+// x / y with r = 1 / y: in double by the reciprocal and one correction from the exactly formed remainder (three instructions, the
+// accuracy of a division, which costs the FP64 pipe about eight).
+__device__ __forceinline__ double over(double x, double y, double r)
+{
+    const double q = x * r;
+    return fma(fma(-q, y, x), r, q);
+}
 __device__ __forceinline__ float over(float x, float y, float) { return x / y; }
 
 // Centre-of-mass kinetic energy of a weighted pair (masses m1, m2 already weighted).

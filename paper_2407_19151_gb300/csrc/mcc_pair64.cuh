@@ -14,9 +14,11 @@
 //               one logarithm per pair: of whichever of 1 - cos and 1 + cos is smaller, the other being 2 minus it
 //   azimuth     2 pi (k + 1/2) 2^-23 = nearest 1/256 turn, tabulated, + a remainder below pi/256 (addition theorem)
 // uniforms are assembled from their bits instead of converted, and comparisons are made on the bits (an FP64 comparison
-// takes the FP64 pipe too). About 120 instructions per pair. FP64 step of 4096
-// three-species cells (2.1e6 particles) 6.11 -> 2.06 ms, relativistic beam of 2048 cells 6.45 -> 1.93 ms; the difference from
-// 64-bit results is unchanged (1.4e-16 of the velocities).
+// takes the FP64 pipe too). Roots and quotients taken through reciprocals get one correction from their exactly formed residual, so
+// a pair's velocity change is as close to extended precision as the same formulas in plain double (rms 1.5e-16 of itself for N97,
+// 1.9e-16 for TA77; uncorrected 1.9e-16 and 2.2e-16). About 130 instructions per pair. FP64 step of 4096
+// three-species cells (2.1e6 particles) 6.11 -> 2.13 ms, relativistic beam of 2048 cells 6.45 -> 2.01 ms (2.06 and 1.93 without
+// the corrections); error against 64-bit results 1.3e-16 of the velocities.
 #pragma once
 
 #include "mcc_kernels.h"
@@ -211,6 +213,14 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
     st = sqrt(o * q);
 }
 
+// sqrt(x) from r = rsqrt(x), with one correction from the exactly formed residual x - y^2: half a unit of the last place, where
+// x r alone is off by up to one and a half. Two instructions instead of the dozen of a square root.
+__device__ __forceinline__ double root64(double x, double r)
+{
+    const double y = x * r;
+    return fma(fma(-y, y, x), 0.5 * r, y);
+}
+
 // Rotation of u (magnitude um) through (Theta, phi) about its own direction; returns du = u' - u.
 __device__ __forceinline__ void rotate64(double ux, double uy, double uz, double um, double st, double omc, double cp,
                                          double sp, double& dx, double& dy, double& dz)
@@ -223,7 +233,7 @@ __device__ __forceinline__ void rotate64(double ux, double uy, double uz, double
         const double zc = uz * sc, us = um * ss;
         dx = ax * zc - ay * us - ux * omc;
         dy = ay * zc + ax * us - uy * omc;
-        dz = -(p2 * rp) * sc - uz * omc;
+        dz = -root64(p2, rp) * sc - uz * omc;
     } else {
         dx = um * sc;
         dy = um * ss;
@@ -244,16 +254,18 @@ __device__ __forceinline__ bool pair64(const F64Tab& T, int method, double cw, c
     const double ux = vi[0] - vj[0], uy = vi[1] - vj[1], uz = vi[2] - vj[2];
     const double u2 = fma(uz, uz, fma(uy, uy, ux * ux));
     if (__double_as_longlong(u2) == 0) return false;
-    const double ru = rsqrt(u2);
+    const double ru = rsqrt(u2), um = root64(u2, ru);
+    // 1 / |u|^3: ru^3 (three roundings over three times that of ru), corrected once
+    const double u3 = u2 * um, r3 = ru * ru * ru;
     double st, omc, sp, cp, d0, d1;
-    angle64<TAPE>(T, method, cw * (ru * ru * ru), r, st, omc, pt != nullptr, d0, d1);
+    angle64<TAPE>(T, method, cw * fma(fma(-u3, r3, 1.0), r3, r3), r, st, omc, pt != nullptr, d0, d1);
     turn64(T, r.y, cp, sp);
     if (TAPE && pt) {
         const double x[kPairTape] = {ux, uy, uz, ru, st, omc, d0, d1, cp, sp};
 #pragma unroll
         for (int k = 0; k < kPairTape; ++k) pt[k * n] = x[k];
     }
-    rotate64(ux, uy, uz, u2 * ru, st, omc, cp, sp, du[0], du[1], du[2]);
+    rotate64(ux, uy, uz, um, st, omc, cp, sp, du[0], du[1], du[2]);
     return true;
 }
 
@@ -294,12 +306,11 @@ __device__ __forceinline__ bool rel_pair64(const F64Tab& T, int method, double c
         p2 += p[d] * p[d];
     }
     if (!(p2 > 0.0)) return false;
-    const double rp = rsqrt(p2);
-    const double pm = p2 * rp;
+    const double pm = root64(p2, rsqrt(p2));
     // v_rel* = |p*| (1 / (m_a gamma_a*) + 1 / (m_b gamma_b*)), m gamma* = sqrt(m^2 + |p*|^2 / c^2)
     const double pc = p2 * ic2;
     const double iv = rsqrt(fma(ma, ma, pc)) + rsqrt(fma(mb, mb, pc));
-    const double s = kw * (rp * rp * rp) / iv;
+    const double s = kw / (p2 * pm * iv);
     double st, omc, cp, sp, x0, x1, d[3];
     angle64<false>(T, method, s, r, st, omc, false, x0, x1);
     turn64(T, r.y, cp, sp);
