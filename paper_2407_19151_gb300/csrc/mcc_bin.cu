@@ -3,14 +3,15 @@
 //
 // histogram (atomic counts) -> exclusive scan -> scatter to the counted places (order within a segment arbitrary)
 // -> per-segment sort: by particle index, which restores the stable order, or straight by weight. The result does not
-// depend on the order in which the atomics were served. Lanes with equal keys in a row add once, which matters for nearly
-// binned input such as a re-bin after a particle push (a warp match over all lanes cost more than the atomics it saved on
-// shuffled input); the count's atomic also gives each particle its place in the segment, so the scatter needs none.
+// depend on the order in which the atomics were served. Lanes of a warp with equal keys add once (key_group); the count's
+// atomic also gives each particle its place in the segment, so the scatter needs none.
 // Segments of up to 512 entries are sorted by one warp in its slice of shared memory (warp barriers only), larger ones
-// by a whole CTA. What bounds it: atomics and random sectors on shuffled input (3.3e7 particles, 2e5 segments: 1.71 -> 1.14 ms,
-// of which count 0.46 -> 0.33, scatter 0.52 -> 0.35, index sorts 0.67 -> 0.40); the weight sorts after a push (1.7e7 particles,
-// 1e5 segments: 0.64 -> 0.29 ms). A two-pass radix sort of (key, index) pairs took 1.43 ms shuffled and lost on nearly
-// binned input, where a warp here has few atomics.
+// by a whole CTA. What bounds it: atomics and random sectors on shuffled input (3.3e7 particles, 2e5 segments: 1.64 ms with a
+// match in every warp, cursors and bitonic sorts, 1.09 so); the segment sorts after a push (17% moved: 0.92 -> 0.83 ms, 0.49 of
+// it the sorts; in weight order 1.63 -> 0.94). 1.34e8 particles: shuffled 7.6 -> 5.9 ms, after a push 3.49 -> 3.13, in weight
+// order 6.3 -> 3.5. Two thirds moved, which no push does, is the one input found where the network in every segment was
+// faster (0.97 against 1.10 ms). A two-pass radix sort of (key, index) pairs took 1.43 ms shuffled and lost on nearly binned
+// input, where a warp here has few atomics.
 #include <mutex>
 
 #include "mcc_kernels.h"
@@ -45,48 +46,58 @@ __device__ __forceinline__ long long bin_key(const int32_t* __restrict__ cell, c
     return (long long)c * S + s;
 }
 
-// Lanes of a warp with equal keys in a row: this lane's run starts at lane `lead` and is `len` lanes long.
-__device__ __forceinline__ void key_run(long long key, int& lead, int& len)
+// Lanes of a warp that count as one: this lane's group has `len` lanes, this one is number `rank`, the first is lane `lead`.
+// Either all lanes with equal keys (a warp match) or runs of equal keys in neighbouring lanes (two ballots). The match takes
+// time with the number of different keys, about 64 cycles of an SM for 32 of them, the atomics it saves take more: it is
+// taken when a warp's keys repeat, that is when at most kRunHeads runs begin (nearly binned input, such as a re-bin after
+// a push), when kSameKey lanes hold lane 0's key (species in turns within binned cells) or when there are few segments,
+// whose counters the atomics queue for. Shuffled input (32 runs of one lane) takes the runs. 3.3e7 particles, 2e5 segments,
+// count and scatter with cursors
+// in us: 17% moved by a push, 100 and 176 (runs alone 162 and 294); shuffled, count and scatter 330 and 350 (460 and 520 with
+// a match in every warp); 1e7 particles in 192 segments, 2360 and 1170 (runs alone 2650 and 1300).
+constexpr int kRunHeads = 28, kSameKey = 4;
+constexpr int64_t kFewSegments = 512;
+
+__device__ __forceinline__ void key_group(long long key, bool few, int& lead, int& rank, int& len)
 {
     const int lane = threadIdx.x & 31;
     const long long prev = __shfl_up_sync(0xffffffffu, key, 1);
     const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || key != prev);
+    const unsigned same0 = __ballot_sync(0xffffffffu, key == __shfl_sync(0xffffffffu, key, 0));
+    if (few || __popc(heads) <= kRunHeads || __popc(same0) >= kSameKey) {
+        const unsigned m = __match_any_sync(0xffffffffu, key);
+        lead = __ffs(m) - 1;
+        rank = __popc(m & ((1u << lane) - 1u));
+        len = __popc(m);
+        return;
+    }
     const unsigned upto = (2u << lane) - 1u;  // this lane and those below
     lead = 31 - __clz(heads & upto);
+    rank = lane - lead;
     const unsigned after = heads & ~upto;
     len = (after ? __ffs(after) - 1 : 32) - lead;
 }
 
-// All lanes of a warp run the same trips (the loop index is the warp's base), so the shuffles see the full warp. Four
-// elements per thread and iteration: their keys first, then their atomics, so that several are in flight.
+// All lanes of a warp run the same trips (the loop index is the warp's base), so the shuffles see the full warp. One element
+// per thread and iteration: four, a grid's stride apart, with their atomics in flight together took 202 / 208 us where one
+// takes 144 / 156 after a push (the counters of four places at once), and no less time on shuffled input.
 // PLACE: place[i] = the particle's place in its segment, in the order the atomics were served.
-constexpr int kBinUnroll = 4;
-
 template <bool PLACE>
 __global__ void __launch_bounds__(kBinThreads) k_hist(const int32_t* __restrict__ cell, const int32_t* __restrict__ species,
                                                       int64_t n, int32_t n_cells, int32_t S, int32_t* __restrict__ counts,
                                                       int32_t* __restrict__ place, int32_t* status)
 {
     const int lane = threadIdx.x & 31;
+    const bool few = (int64_t)n_cells * S <= kFewSegments;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += kBinUnroll * stride) {
-        long long key[kBinUnroll];
-        int lead[kBinUnroll], at[kBinUnroll];
-#pragma unroll
-        for (int u = 0; u < kBinUnroll; ++u) key[u] = bin_key(cell, species, base + u * stride + lane, n, n_cells, S, status);
-#pragma unroll
-        for (int u = 0; u < kBinUnroll; ++u) {
-            int len;
-            key_run(key[u], lead[u], len);
-            at[u] = 0;
-            if (key[u] >= 0 && lane == lead[u]) at[u] = atomicAdd(&counts[key[u]], len);
-        }
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+        const long long key = bin_key(cell, species, base + lane, n, n_cells, S, status);
+        int lead, rank, len, at = 0;
+        key_group(key, few, lead, rank, len);
+        if (key >= 0 && lane == lead) at = atomicAdd(&counts[key], len);
         if (PLACE) {
-#pragma unroll
-            for (int u = 0; u < kBinUnroll; ++u) {
-                const int a = __shfl_sync(0xffffffffu, at[u], lead[u]) + lane - lead[u];
-                if (key[u] >= 0) place[base + u * stride + lane] = a;
-            }
+            at = __shfl_sync(0xffffffffu, at, lead) + rank;
+            if (key >= 0) place[base + lane] = at;
         }
     }
 }
@@ -186,28 +197,20 @@ __global__ void __launch_bounds__(kBinThreads) k_scatter(const int32_t* __restri
                                                          const int32_t* __restrict__ place, int32_t* __restrict__ perm)
 {
     const int lane = threadIdx.x & 31;
+    const bool few = (int64_t)n_cells * S <= kFewSegments;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += kBinUnroll * stride) {
-        long long key[kBinUnroll];
-        int at[kBinUnroll];
-#pragma unroll
-        for (int u = 0; u < kBinUnroll; ++u) {
-            const int64_t i = base + u * stride + lane;
-            key[u] = bin_key(cell, species, i, n, n_cells, S, nullptr);
-            at[u] = PLACE && key[u] >= 0 ? place[i] : 0;
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
+        const long long key = bin_key(cell, species, base + lane, n, n_cells, S, nullptr);
+        int at = 0;
+        if (PLACE) {
+            if (key >= 0) at = place[base + lane];
+        } else {
+            int lead, rank, len;
+            key_group(key, few, lead, rank, len);
+            if (key >= 0 && lane == lead) at = atomicAdd(&cursor[key], len);
+            at = __shfl_sync(0xffffffffu, at, lead) + rank;
         }
-        if (!PLACE) {
-#pragma unroll
-            for (int u = 0; u < kBinUnroll; ++u) {
-                int lead, len;
-                key_run(key[u], lead, len);
-                if (key[u] >= 0 && lane == lead) at[u] = atomicAdd(&cursor[key[u]], len);
-                at[u] = __shfl_sync(0xffffffffu, at[u], lead) + lane - lead;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kBinUnroll; ++u)
-            if (key[u] >= 0) perm[offsets[key[u]] + at[u]] = (int32_t)(base + u * stride + lane);
+        if (key >= 0) perm[offsets[key] + at] = (int32_t)(base + lane);
     }
 }
 
@@ -252,8 +255,14 @@ __device__ __forceinline__ void warp_sort_smem(int n, Cmpx cmpx)
 // the count, zeroed before) for the CTA-wide sorts.
 // A segment in order already is left. Otherwise a counting sort on a linear map of the keys' top words (the indices) to n or
 // more buckets, then an insertion sort within a bucket. Indices of shuffled particles spread evenly, and so do weights over
-// decades, as the IEEE bits of a weight are nearly linear in its logarithm; a segment with a bucket above kBucketMost (after
-// a particle push most indices of a segment are neighbours) takes the bitonic network.
+// decades, as the IEEE bits of a weight are nearly linear in its logarithm. After a particle push most indices of a segment
+// are neighbours, those that stayed, and the rest come from anywhere: one bucket of the linear map would hold nearly all.
+// The map of such a segment (more than kBucketMost entries in the bucket of a middling one) has three pieces: half the buckets
+// for the 2.5 n indices around that entry, a quarter each for those below and above, by the logarithm of their distance (what
+// moved in comes from the next cells, rows and planes of the grid, orders of magnitude apart). A segment of which a third
+// comes from elsewhere, or one that still fills a bucket beyond kBucketMost, takes the bitonic network; up to 32 indices
+// take it in registers. 3.3e7 particles, 17% moved: 616 us by the network in every segment, 734 by a futile count and then
+// the network, 490 by three pieces.
 constexpr int kOrderWarps = 4;   // warps per CTA
 constexpr int kBucketMost = 12;  // longest bucket for the insertion sort
 
@@ -282,6 +291,18 @@ __global__ void __launch_bounds__(32 * kOrderWarps) k_segsort_warp(const int64_t
         if (n > kWarpSeg && lane == 0) large[1 + atomicAdd(&large[0], 1)] = (int32_t)seg;
         if (n < 2 || n > kWarpSeg) continue;
         int32_t* p = perm + b;
+        if (!WEIGHTED && n <= 32) {  // one index per lane: the network in registers, no shared memory
+            int32_t v = lane < n ? p[lane] : INT32_MAX;
+#pragma unroll
+            for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+                for (int j = k / 2; j > 0; j >>= 1) {
+                    const int32_t y = __shfl_xor_sync(0xffffffffu, v, j);
+                    v = ((lane & j) == 0) == ((lane & k) == 0) ? min(v, y) : max(v, y);
+                }
+            if (lane < n) p[lane] = v;
+            continue;
+        }
         uint32_t lo = 0xFFFFFFFFu, hi = 0u;
         for (int i = lane; i < n; i += 32) {
             const int32_t q = p[i];
@@ -296,24 +317,7 @@ __global__ void __launch_bounds__(32 * kOrderWarps) k_segsort_warp(const int64_t
         if (!__any_sync(0xffffffffu, out)) continue;
         lo = __reduce_min_sync(0xffffffffu, lo);
         hi = __reduce_max_sync(0xffffffffu, hi);
-        int lg = 5;
-        while ((1 << lg) < n) ++lg;
-        const int nb = 1 << lg, per = nb / 32;  // nb <= kWarpSeg
-        // bucket = (key - lo) nb / (hi - lo + 1), rounded down: below nb, and never decreasing in the key
-        const uint32_t span = hi - lo;
-        const uint32_t mult = span < (uint32_t)nb ? 0u : (uint32_t)(((uint64_t)nb << 32) / ((uint64_t)span + 1u));
-        auto bucket = [&](int i) -> int { return (int)(mult ? __umulhi(top(i) - lo, mult) : top(i) - lo); };
-        for (int i = lane; i < nb; i += 32) cnt[i] = 0;
-        __syncwarp();
-        for (int i = lane; i < n; i += 32) atomicAdd(&cnt[bucket(i)], 1u);
-        __syncwarp();
-        uint32_t sum = 0, most = 0;
-        for (int i = 0; i < per; ++i) {
-            const uint32_t x = cnt[lane * per + i];
-            sum += x;
-            most = max(most, x);
-        }
-        if (__reduce_max_sync(0xffffffffu, most) > kBucketMost) {
+        auto network = [&] {
             warp_sort_smem(n, [&](int x, int y) {
                 if (after(x, y)) {
                     const int32_t a = ib[x];
@@ -328,6 +332,57 @@ __global__ void __launch_bounds__(32 * kOrderWarps) k_segsort_warp(const int64_t
             });
             for (int i = lane; i < n; i += 32) p[i] = ib[i];
             __syncwarp();
+        };
+        int lg = 5;
+        while ((1 << lg) < n) ++lg;
+        const int nb = 1 << lg, per = nb / 32;  // nb <= kWarpSeg
+        // bucket = (key - lo) nb / (hi - lo + 1), rounded down: below nb, and never decreasing in the key
+        const uint32_t span = hi - lo;
+        // (a piece of width d with k buckets: (key - its start) k / d, the factor 0 where every key has a bucket of its own)
+        auto factor = [](uint32_t k, uint64_t d) { return d <= k ? 0u : (uint32_t)(((uint64_t)k << 32) / d); };
+        auto place = [](uint32_t x, uint32_t f) { return f ? __umulhi(x, f) : x; };
+        const uint32_t mult = factor((uint32_t)nb, (uint64_t)span + 1u);
+        uint32_t w0 = 0u, w1 = 0u, mw = 0u, side = 0u;  // side > 0: three pieces, side | 2 side | side buckets
+        if (!WEIGHTED) {
+            const uint32_t x = top(n / 4), y = top(n / 2), z = top(n - 1 - n / 4);
+            const uint32_t mid = max(min(x, y), min(max(x, y), z));
+            const uint32_t at = place(mid - lo, mult);
+            int share = 0;
+            for (int i = lane; i < n; i += 32) share += place(top(i) - lo, mult) == at;
+            if (__reduce_add_sync(0xffffffffu, share) > kBucketMost) {
+                const uint32_t half = (uint32_t)(n + n / 4);
+                w0 = mid - lo > half ? mid - half : lo;  // the window [w0, w1)
+                w1 = hi - mid >= half ? mid + half : hi + 1u;
+                int inside = 0;
+                for (int i = lane; i < n; i += 32) inside += top(i) >= w0 && top(i) < w1;
+                if (__reduce_add_sync(0xffffffffu, inside) < n - n / 3) {  // many from elsewhere, in clumps
+                    network();
+                    continue;
+                }
+                side = (uint32_t)nb / 4;
+                mw = factor(2 * side, (uint64_t)(w1 - w0));
+            }
+        }
+        // distance d = 1 .. 2^31 to a bucket below nb / 4: its exponent and leading bits, 31 octaves over nb / 4 buckets
+        auto octave = [&](uint32_t d) -> uint32_t { return (__float_as_uint((float)d) - 0x3F800000u) >> (30 - lg); };
+        auto bucket = [&](int i) -> int {
+            const uint32_t t = top(i);
+            if (WEIGHTED || side == 0u) return (int)place(t - lo, mult);
+            return (int)(t < w0 ? side - 1u - octave(w0 - t)
+                                : (t < w1 ? side + place(t - w0, mw) : 3 * side + octave(t - w1 + 1u)));
+        };
+        for (int i = lane; i < nb; i += 32) cnt[i] = 0;
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) atomicAdd(&cnt[bucket(i)], 1u);
+        __syncwarp();
+        uint32_t sum = 0, most = 0;
+        for (int i = 0; i < per; ++i) {
+            const uint32_t x = cnt[lane * per + i];
+            sum += x;
+            most = max(most, x);
+        }
+        if (__reduce_max_sync(0xffffffffu, most) > kBucketMost) {
+            network();
             continue;
         }
         uint32_t inc = sum;
