@@ -468,9 +468,14 @@ __global__ void __launch_bounds__(kBinThreads) k_segsort_w(const int64_t* __rest
 }
 
 // Four elements per thread and iteration, their permuted reads issued together (more reads in flight). A shuffled
-// permutation reads a whole sector per element, so what bounds it is how much of `in` stays in L2: the permutation and the
-// output, touched once, are marked to leave first (3.3e7 shuffled particles, three floats and a double: 1.56 -> 1.52 ms).
-template <class T>
+// permutation reads a whole sector per element, so what bounds it is how much of `in` stays in L2. STREAM: the permutation and
+// the output, touched once, are marked to leave first. Without / with, us, on one GPU: floats in nearly the output's order 90 /
+// 84 (33 million), 302 / 280 (134 million), shuffled 336 / 322 and 2663 / 2662; doubles in nearly the output's order 120 / 119
+// (33 million), 224 / 223 (67 million), but 425 / 501 (134 million), shuffled 560 / 555 and 3026 / 3040. Doubles go without
+// from 64 million on, where it gains nothing yet loses nothing.
+constexpr int64_t kStreamDoubles = 64'000'000;
+
+template <class T, bool STREAM>
 __global__ void k_gather(const T* __restrict__ in, const int32_t* __restrict__ perm, int64_t n, T* __restrict__ out)
 {
     constexpr int U = 4;
@@ -479,12 +484,15 @@ __global__ void k_gather(const T* __restrict__ in, const int32_t* __restrict__ p
         int32_t p[U];
         T v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) p[u] = base + u * stride < n ? __ldcs(perm + base + u * stride) : 0;
+        for (int u = 0; u < U; ++u) p[u] = base + u * stride < n ? (STREAM ? __ldcs(perm + base + u * stride) : perm[base + u * stride]) : 0;
 #pragma unroll
         for (int u = 0; u < U; ++u) v[u] = base + u * stride < n ? __ldg(in + p[u]) : T(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (base + u * stride < n) __stcs(out + base + u * stride, v[u]);
+            if (base + u * stride < n) {
+                if (STREAM) __stcs(out + base + u * stride, v[u]);
+                else out[base + u * stride] = v[u];
+            }
     }
 }
 
@@ -635,12 +643,13 @@ cudaError_t launch_gather(const void* in, const int32_t* perm, int64_t n, int el
 {
     if (n <= 0) return cudaSuccess;
     const int g = grid_for(n, kBinThreads);
-    if (elem_bytes == 8)
-        k_gather<uint64_t><<<g, kBinThreads, 0, st>>>(reinterpret_cast<const uint64_t*>(in), perm, n,
-                                                      reinterpret_cast<uint64_t*>(out));
-    else
-        k_gather<uint32_t><<<g, kBinThreads, 0, st>>>(reinterpret_cast<const uint32_t*>(in), perm, n,
-                                                      reinterpret_cast<uint32_t*>(out));
+    if (elem_bytes == 8) {
+        const auto kernel = n < kStreamDoubles ? k_gather<uint64_t, true> : k_gather<uint64_t, false>;
+        kernel<<<g, kBinThreads, 0, st>>>(reinterpret_cast<const uint64_t*>(in), perm, n, reinterpret_cast<uint64_t*>(out));
+    } else {
+        k_gather<uint32_t, true><<<g, kBinThreads, 0, st>>>(reinterpret_cast<const uint32_t*>(in), perm, n,
+                                                            reinterpret_cast<uint32_t*>(out));
+    }
     return cudaGetLastError();
 }
 

@@ -72,3 +72,12 @@ def test_nearly_binned(name):
     rperm, roff = O.bin_particles_weighted(cell, sp, w, C, S)
     np.testing.assert_array_equal(off.cpu().numpy(), roff)
     np.testing.assert_array_equal(perm.cpu().numpy(), rperm)
+
+
+@pytest.mark.parametrize("n", [63_999_999, 64_000_000])
+def test_gather_on_both_sides_of_the_streaming_line(n):
+    import paper_2407_19151_gb300 as mcc
+    g = torch.Generator(device="cuda").manual_seed(3)
+    perm = torch.randperm(n, device="cuda", generator=g).int()
+    x = torch.arange(n, device="cuda", dtype=torch.float64)
+    assert torch.equal(mcc.mcc_gather(x, perm), perm.double())
