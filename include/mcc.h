@@ -366,6 +366,23 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* particles, const int64_t* 
                    int32_t n_inter, const mcc_params* params, int32_t n_steps, int32_t max_cell,
                    int32_t* corr_pairs, int32_t* fail_count, void* ws, size_t ws_bytes, mcc_stream stream);
 
+/*
+ * mcc_step_fused_part: mcc_step_fused on some cells of a larger problem (a shard, or a chunk of a state that does not fit).
+ * How many threads run a cell follows from the number of cells of a call, how many of them are small and max_cell, and fixes the
+ * order of its float-float sums; with these of the whole problem in every part, the parts' results equal those of one call on the
+ * whole problem bit for bit (draws are keyed by the global cell id, params->cell_base).
+ *   whole_cells   cells of the whole problem, at least n_cells; 0: this call is the whole problem (mcc_step_fused)
+ *   whole_small   how many of them hold fewer than MCC_SMALL_CELL particles
+ *   max_cell      the bound for the whole problem
+ * Errors: MCC_ERR_INVALID_ARG for whole_cells below n_cells or whole_small outside [0, whole_cells]. Otherwise as mcc_step_fused.
+ */
+#define MCC_SMALL_CELL 128
+int mcc_step_fused_part(mcc_ctx* ctx, const mcc_particles* particles, const int64_t* offsets, int32_t n_cells,
+                        int32_t n_species, const mcc_species* sp, const double* lnL, const int32_t* interactions,
+                        int32_t n_inter, const mcc_params* params, int32_t n_steps, int32_t max_cell,
+                        int32_t* corr_pairs, int32_t* fail_count, void* ws, size_t ws_bytes, int32_t whole_cells,
+                        int32_t whole_small, mcc_stream stream);
+
 /* Particles staged on chip per cell by the one-CTA kernel of mcc_step_fused, which takes the cells above the
  * largest group class (0 = automatic: the largest tile with which four CTAs share an SM's shared memory, or the
  * largest cell if smaller). Cells above it run from the workspace slabs. */
@@ -377,8 +394,8 @@ int mcc_set_tile_cap(mcc_ctx* ctx, int32_t cap);
  * sixteen warps share an SM's shared memory); largest sets caps[4] (0 = as large as one CTA's shared memory
  * allows). Every capacity is capped by what one CTA's shared memory holds (44 bytes per particle). Both 0 is the
  * default; a call with few cells then runs its cells on larger groups than these classes say, and one with many small
- * cells runs those on half warps. Used by the autotuner; the step's results do not depend on it beyond the order of
- * float-float sums. */
+ * cells runs those on half warps (a part of a problem: mcc_step_fused_part). Used by the autotuner; the step's results do
+ * not depend on it beyond the order of float-float sums. */
 int mcc_set_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp, int32_t largest);
 
 /* The five class capacities mcc_step_fused uses for this precision and mode (caps_out: host int32[5]). */

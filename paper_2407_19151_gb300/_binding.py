@@ -73,6 +73,8 @@ class Params:
                                 # state before the store (fused step)
     launch_events: object = None  # optional list of 2 (GROUP_CLASSES + 1) torch.cuda.Event(enable_timing=True):
                                   # begin / end of each size class's kernel in the last step (fused step)
+    whole_cells: int = 0  # fused step on a part of a problem (cell_base its first cell): the cells of the whole problem,
+    whole_small: int = 0  # and those of fewer than SMALL_CELL particles; the parts then equal one call bit for bit
 
     def _c(self) -> _Params:
         return _Params(int(self.method), int(bool(self.relativistic)), float(self.dt), float(self.dV),
@@ -86,6 +88,7 @@ class Params:
 
 
 GROUP_CLASSES = 5  # size classes of the group kernels (MCC_GROUP_CLASSES)
+SMALL_CELL = 128   # MCC_SMALL_CELL
 _LIB = None
 _EVENT_ARRAYS = []
 
@@ -141,6 +144,9 @@ def lib():
         "mcc_step_fused": (C.c_int, [vp, P(_Particles), vp, C.c_int32, C.c_int32, P(_Species), P(C.c_double),
                                      P(C.c_int32), C.c_int32, P(_Params), C.c_int32, C.c_int32, vp, vp, vp,
                                      C.c_size_t, vp]),
+        "mcc_step_fused_part": (C.c_int, [vp, P(_Particles), vp, C.c_int32, C.c_int32, P(_Species), P(C.c_double),
+                                          P(C.c_int32), C.c_int32, P(_Params), C.c_int32, C.c_int32, vp, vp, vp,
+                                          C.c_size_t, C.c_int32, C.c_int32, vp]),
         "mcc_set_tile_cap": (C.c_int, [vp, C.c_int32]),
         "mcc_set_group_capacity": (C.c_int, [vp, C.c_int32, C.c_int32]),
         "mcc_group_capacities": (C.c_int, [vp, C.c_int32, C.c_int32, P(C.c_int32)]),
@@ -500,10 +506,10 @@ def mcc_step_fused(vx, vy, vz, w, offsets, n_cells, n_species, species, lnL, par
            "mcc_step_workspace_size")
     ws = ctx.workspace(("step", P.prec), nb.value)
     cp = params._c()
-    _check(lib().mcc_step_fused(ctx.handle, C.byref(P), _ptr(offsets), n_cells, n_species, _species(species),
-                                _lnL(lnL, n_species), flat, len(inter), C.byref(cp), int(n_steps), int(max_cell),
-                                _ptr(corr_pairs), _ptr(fail_count), _ptr(ws), nb.value,
-                                _stream(stream, vx.device)), "mcc_step_fused")
+    _check(lib().mcc_step_fused_part(ctx.handle, C.byref(P), _ptr(offsets), n_cells, n_species, _species(species),
+                                     _lnL(lnL, n_species), flat, len(inter), C.byref(cp), int(n_steps), int(max_cell),
+                                     _ptr(corr_pairs), _ptr(fail_count), _ptr(ws), nb.value, int(params.whole_cells),
+                                     int(params.whole_small), _stream(stream, vx.device)), "mcc_step_fused")
     return (corr_pairs, fail_count) if corr_pairs.numel() == fail_count.numel() == n_cells else \
         (corr_pairs[:n_cells], fail_count[:n_cells])
 

@@ -633,6 +633,7 @@ void group_caps(const mcc_ctx* ctx, bool f32, bool rel, int32_t caps[mcc::kGroup
         caps[k] = (int32_t)cap;
     }
 }
+static_assert(MCC_SMALL_CELL == mcc::kHalfCells, "the header's small cells are those of the half warps");
 // A call with few cells runs them on larger groups, as long as every warp is still resident: one visit is then shorter, and
 // one launch serves what would be several (the classes run one after another). Cells go up to class 3; class k is taken
 // while n_cells groups of it fit the GPU. Measured per step, 152 SMs, two species (us by group size 64 / 128 / 256 / 512):
@@ -689,16 +690,29 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
                    const mcc_params* p, int32_t n_steps, int32_t max_cell, int32_t* corr_pairs, int32_t* fail_count,
                    void* ws, size_t ws_bytes, mcc_stream stream)
 {
+    return mcc_step_fused_part(ctx, P, offsets, n_cells, n_species, sp, lnL, interactions, n_inter, p, n_steps, max_cell,
+                               corr_pairs, fail_count, ws, ws_bytes, 0, 0, stream);
+}
+
+int mcc_step_fused_part(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets, int32_t n_cells, int32_t n_species,
+                        const mcc_species* sp, const double* lnL, const int32_t* interactions, int32_t n_inter,
+                        const mcc_params* p, int32_t n_steps, int32_t max_cell, int32_t* corr_pairs, int32_t* fail_count,
+                        void* ws, size_t ws_bytes, int32_t whole_cells, int32_t whole_small, mcc_stream stream)
+{
     NvtxRange nvtx_("mcc_step_fused");
     if (!ctx || !P || !offsets || !sp || !lnL || !interactions || !valid_params(p) || n_steps < 0 || max_cell < 0)
         return MCC_ERR_INVALID_ARG;
     if (P->prec != MCC_F64 && P->prec != MCC_F32_MIXED) return MCC_ERR_INVALID_ARG;
     if (max_cell > MCC_MAX_SEGMENT) return MCC_ERR_TOO_LARGE;  // in-cell indices are 20-bit key fields
+    const bool part = whole_cells != 0;
+    if (part && (whole_cells < n_cells || whole_small < 0 || whole_small > whole_cells)) return MCC_ERR_INVALID_ARG;
     DeviceGuard g(ctx->device);
     StepArgs a;
     int rc = fill_args(a, ctx, P, offsets, n_cells, n_species, sp, lnL, interactions, n_inter, 0, p);
     if (rc != MCC_OK) return rc;
     if (n_cells == 0 || n_steps == 0) return MCC_OK;
+    // cells by whose number the call picks its groups
+    const int32_t pick_cells = part ? whole_cells : n_cells;
     a.corr_pairs = corr_pairs;
     a.fail_count = fail_count;
     a.resid = p->residual;
@@ -710,11 +724,13 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
     if (!ws || ws_bytes < need) return MCC_ERR_WORKSPACE;
     int32_t caps[mcc::kGroupClasses];
     group_caps(ctx, f32, rel, caps);
-    if (ctx->group_cap == 0) few_cells_caps(ctx, n_cells, max_cell, caps);
+    if (ctx->group_cap == 0) few_cells_caps(ctx, pick_cells, max_cell, caps);
     // two small cells to a warp, with automatic capacities, if they fill every warp's halves (a launch of its own costs the
     // time of a visit, 0.1 ms)
     int32_t half_min = 2 * mcc::kGroupWarpsPerSm * ctx->num_sms;
-    if (!f32 || ctx->group_cap > 0 || caps[0] < mcc::kHalfCells || n_cells < half_min) half_min = 0;
+    if (!f32 || ctx->group_cap > 0 || caps[0] < mcc::kHalfCells || pick_cells < half_min) half_min = 0;
+    // (the device counts the small cells of a whole problem; for a part the caller has)
+    if (part && half_min > 0) half_min = whole_small >= half_min ? 1 : 0;
     // the group kernels serve the mixed path; the FP64 path runs every cell on the one-CTA kernel
     const bool fallback = !f32 || max_cell > caps[mcc::kGroupClasses - 1];
     int32_t* order = reinterpret_cast<int32_t*>(ws);
@@ -795,7 +811,7 @@ int mcc_step_fused(mcc_ctx* ctx, const mcc_particles* P, const int64_t* offsets,
             big.rng.step = a.rng.step;
             big.step_add = a.step_add;
             const int cap = max_cell <= tile ? max_cell : tile;
-            const bool small = !f32 && max_cell <= mcc::kSmallCells && n_cells > 4 * ctx->num_sms;
+            const bool small = !f32 && max_cell <= mcc::kSmallCells && pick_cells > 4 * ctx->num_sms;
             rc = run_cells(ctx, big, f32, rel, small ? mcc::kFusedSmall : mcc::kFused, cap, S(stream), max_grid);
             if (rc != MCC_OK) return rc;
         }

@@ -2,8 +2,8 @@
 
 Cells are independent within a step and across steps (the collision acts per cell; positions are frozen), so the
 binned state splits into contiguous cell chunks. Chunk k is copied in on one stream, stepped ``n_steps`` times on a
-second (one mcc_step_fused call, random draws keyed by the global cell id, so the result equals the unchunked run bit
-for bit), and copied out on a third, while chunk k + 1 is already being copied in. With ``round_trips`` > 1 the state
+second (one mcc_step_fused call, random draws keyed by the global cell id and groups of threads picked by the whole
+problem, so the result equals the unchunked run bit for bit), and copied out on a third, while chunk k + 1 is already being copied in. With ``round_trips`` > 1 the state
 makes that many round trips through host memory: chunk k of round trip t + 1 is copied in as soon as its copy out of
 round trip t has landed, so the pipeline does not drain between round trips. Device memory is a ring of ``buffers``
 chunk-sized slots; only the transfers and the stream ordering live here, every step runs in the library's kernels.
@@ -16,7 +16,7 @@ import numpy as np
 import torch
 
 from . import _binding as B
-from .sharding import shard_cells, shard_view
+from .sharding import shard_cells, shard_view, whole_problem
 
 
 def step_host(vx, vy, vz, w, offsets, n_cells: int, n_species: int, species, lnL, params: B.Params,
@@ -45,6 +45,7 @@ def step_host(vx, vy, vz, w, offsets, n_cells: int, n_species: int, species, lnL
     # per-chunk counters on the device, accumulated over every step, copied out once at the end
     corr = [torch.zeros(max(c1 - c0, 1), dtype=torch.int32, device=dev) for c0, c1 in ranges]
     fail = [torch.zeros(max(c1 - c0, 1), dtype=torch.int32, device=dev) for c0, c1 in ranges]
+    whole = whole_problem(off, n_species, params)
     s_in, s_run, s_out = torch.cuda.Stream(dev), torch.cuda.Stream(dev), torch.cuda.Stream(dev)
     freed = [None] * nb                  # slot free again (its chunk copied out)
     landed = [None] * len(ranges)        # chunk's previous round trip back in host memory
@@ -68,7 +69,7 @@ def step_host(vx, vy, vz, w, offsets, n_cells: int, n_species: int, species, lnL
             with torch.cuda.stream(s_run):
                 s_run.wait_event(loaded)
                 p = dataclasses.replace(params, cell_base=int(params.cell_base) + c0,
-                                        step=int(params.step) + t * int(n_steps))
+                                        step=int(params.step) + t * int(n_steps), **whole)
                 B.mcc_step_fused(*(x[:n] for x in sl["v"]), sl["w"][:n], offs[k], c1 - c0, n_species, species, lnL,
                                  p, n_steps=n_steps, max_cell=max_cell, interactions=interactions,
                                  corr_pairs=corr[k], fail_count=fail[k], stream=s_run)

@@ -1,7 +1,7 @@
 """Sharding of the collision step across GPUs. Cells are independent within a step (the collision acts per cell,
 Sec. 2), so a problem splits into contiguous cell ranges with no exchange in the data path; every random draw is
-keyed by the global cell id (``Params.cell_base``), so the union of the shards equals the unsharded run bit for
-bit. The only collective is an optional all-reduce of per-species diagnostics."""
+keyed by the global cell id (``Params.cell_base``) and every shard picks its groups of threads by the whole problem
+(``Params.whole_cells``), so the union of the shards equals the unsharded run bit for bit. The only collective is an optional all-reduce of per-species diagnostics."""
 from __future__ import annotations
 
 import numpy as np
@@ -28,6 +28,16 @@ def shard_view(offsets, n_species: int, c0: int, c1: int):
     local = off[c0 * n_species: c1 * n_species + 1]
     p0, p1 = int(local[0]), int(local[-1])
     return local - p0, p0, p1
+
+
+def whole_problem(offsets, n_species: int, params) -> dict:
+    """Params.whole_cells / whole_small of a problem with these segment offsets, by which its parts pick their groups of
+    threads as one call on the whole would (as they are if the problem is itself a part)."""
+    if params.whole_cells:
+        return dict(whole_cells=params.whole_cells, whole_small=params.whole_small)
+    from ._binding import SMALL_CELL
+    counts = np.diff(np.asarray(offsets, dtype=np.int64)[::n_species])
+    return dict(whole_cells=len(counts), whole_small=int((counts < SMALL_CELL).sum()))
 
 
 def species_moments(vx, vy, vz, w, offsets, n_cells: int, n_species: int, m):
@@ -83,8 +93,9 @@ class CudaShard:
 class ShardedStep:
     """The collision step of one problem split over the ranks of a torch.distributed process group, one GPU per
     rank. Rank r owns the contiguous, particle-balanced cell range [c0, c1) of the global segment offsets
-    (shard_cells) and holds only those particles; step() runs the fused step on them with cell_base = c0, so every
-    draw is keyed by the global cell id and the union of the shards equals the unsharded run bit for bit. The data
+    (shard_cells) and holds only those particles; step() runs the fused step on them with cell_base = c0 and the whole
+    problem's cell counts, so every draw is keyed by the global cell id, every cell runs on as many threads as in the whole
+    problem, and the union of the shards equals the unsharded run bit for bit. The data
     path exchanges nothing (the collision acts per cell, Sec. 2); the one collective is the all-reduce (sum) of the
     per-species diagnostics (sum w, momentum, kinetic energy, count per species, and the failed corrections), once
     per call of step(). Without an initialised process group it runs the whole problem as one rank.
@@ -115,7 +126,8 @@ class ShardedStep:
         self.max_cell = int(counts.max()) if max_cell is None and len(counts) else int(max_cell or 0)
         self.species = list(species)
         self.lnL = lnL
-        self.params = dataclasses.replace(params, cell_base=int(params.cell_base) + self.c0)
+        self.params = dataclasses.replace(params, cell_base=int(params.cell_base) + self.c0,
+                                          **whole_problem(off, self.S, params))
         self.backend = backend if backend is not None else CudaShard()
         self.state = None
         self.fail = None
