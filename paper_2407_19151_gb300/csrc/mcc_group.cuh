@@ -599,6 +599,12 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
     }
     gsync<G>();
     if (!need) return;
+    // 2^lg <= ns buckets for the ns particles from s0. Their counters are halves of 32-bit words; in a full tile of odd capacity
+    // the last word's upper half is rho[0], which is stored while others still count, so that the last slot stays unused there.
+    auto buckets = [&](int s0, int ns) {
+        const int lg = 31 - __clz(ns);
+        return (t.cap & 1) && s0 + (1 << lg) == t.cap ? lg - 1 : lg;
+    };
     auto range = [&](int sp, uint32_t& lo, uint32_t& mult, int& lg) {
         uint32_t hi = sh.wrange[sp][0][1];
         lo = sh.wrange[sp][0][0];
@@ -606,8 +612,7 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
             lo = min(lo, sh.wrange[sp][w][0]);
             hi = max(hi, sh.wrange[sp][w][1]);
         }
-        const int ns = sh.off[sp + 1] - sh.off[sp];
-        lg = 31 - __clz(ns);  // 2^lg <= ns buckets
+        lg = buckets(sh.off[sp], sh.off[sp + 1] - sh.off[sp]);
         const uint32_t span = hi - lo;
         // floor(2^(32 + lg) / (span + 1)) from below: below 2^lg buckets, never decreasing in the key
         mult = span >> lg ? (uint32_t)(((uint64_t)1 << (32 + lg)) / ((uint64_t)span + 1u)) : 0u;
@@ -676,7 +681,7 @@ __device__ __noinline__ void gweight_order(const StepArgs& A, const GTile& t, GS
     for (int sp = 0; sp < S; ++sp) {
         if (!(need >> sp & 1u)) continue;
         const int s0 = sh.off[sp], ns = sh.off[sp + 1] - s0;
-        const int lg = 31 - __clz(ns);
+        const int lg = buckets(s0, ns);
         uint16_t* ord = t.rho + s0;
         const uint64_t* key = t.scr + s0;
         if (!(net >> sp & 1u)) {
