@@ -733,7 +733,7 @@ __device__ void correct_interaction(const StepArgs& A, const Tile<V>& t, Shared&
             V excl = __shfl_up_sync(0xffffffffu, inc, 1);
             if (lane == 0) excl = (V)0;
             const V tot = __shfl_sync(0xffffffffu, inc, 31);
-            const bool fast = tot >= Dabs;
+            const bool fast = A.max_corr_passes > 0 && tot >= Dabs;
             if (fast && valid && K > (V)0 && excl < Dabs) apply_pair(i, j, v1, v2, m1, m2, K, capv, excl);
             if (lane == 0) sh.fast = fast;
         }
