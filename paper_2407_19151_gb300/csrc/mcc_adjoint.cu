@@ -296,69 +296,83 @@ __device__ int energy_forward(const StepArgs& A, const Slab& sl, const Work& wk,
     done = none;
     const int passes = none ? 1 : A.max_corr_passes;
     bool stop = false;
+    static_assert(kWarps == 4, "the prefix sums below are those of the step kernel's four warps");
     for (int pass = 0; pass < passes && !stop; ++pass) {
         const int o = pass & 1, np = (ns - o) / 2;
         double carry = 0.0;
-        for (int base = 0; base < np && !stop; base += 32) {
-            const int m = base + lane;
-            int i = 0, j = 0;
-            double v1[3], v2[3], m1 = 1.0, m2 = 1.0, K = 0.0;
-            if (m < np) {
-                i = wk.rho[s0 + o + 2 * m];
-                j = wk.rho[s0 + o + 2 * m + 1];
-                ld3(wk.v, N, i, v1);
-                ld3(wk.v, N, j, v2);
-                m1 = msd * wk.w[i];
-                m2 = msd * wk.w[j];
-                K = pair_kecm<double, false>(A.c, m1, m2, v1, v2);
-            }
-            const bool ok = K > 0.0;
-            bool take;
-            double U = 0.0, capE = 0.0;
-            if (none) {
-                const unsigned b = __ballot_sync(0xffffffffu, ok);
-                take = ok && lane == __ffs(b) - 1;
-                stop = b != 0;
-            } else {
-                capE = ok ? A.fE * K : 0.0;
-                double inc = capE;
+        // Chunks of kThreads pairs as in the step kernel, 32 at a time. Its prefix sums: within a warp, then over its warps'
+        // totals, offsets t0, t1 + t0, (t2 + t1) + t0 and total (t3 + t2) + (t1 + t0), then the chunks before.
+        for (int chunk = 0; chunk < np && !stop; chunk += kThreads) {
+            double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
+            for (int grp = 0; grp < kWarps && chunk + 32 * grp < np && !stop; ++grp) {
+                const int m = chunk + 32 * grp + lane;
+                int i = 0, j = 0;
+                double v1[3], v2[3], m1 = 1.0, m2 = 1.0, K = 0.0;
+                if (m < np) {
+                    i = wk.rho[s0 + o + 2 * m];
+                    j = wk.rho[s0 + o + 2 * m + 1];
+                    ld3(wk.v, N, i, v1);
+                    ld3(wk.v, N, j, v2);
+                    m1 = msd * wk.w[i];
+                    m2 = msd * wk.w[j];
+                    K = pair_kecm<double, false>(A.c, m1, m2, v1, v2);
+                }
+                const bool ok = K > 0.0;
+                bool take;
+                double U = 0.0, capE = 0.0;
+                if (none) {
+                    const unsigned b = __ballot_sync(0xffffffffu, ok);
+                    take = ok && lane == __ffs(b) - 1;
+                    stop = b != 0;
+                } else {
+                    capE = ok ? A.fE * K : 0.0;
+                    double inc = capE;
 #pragma unroll
-                for (int q = 1; q < 32; q <<= 1) {
-                    const double y = __shfl_up_sync(0xffffffffu, inc, q);
-                    if (lane >= q) inc += y;
-                }
-                double excl = __shfl_up_sync(0xffffffffu, inc, 1);
-                excl = (lane ? excl : 0.0) + carry;
-                take = ok && excl < Dabs;
-                const double rem = Dabs - excl;
-                U = sgn * (rem < capE ? rem : capE);
-                carry += __shfl_sync(0xffffffffu, inc, 31);
-                stop = done = carry >= Dabs;
-            }
-            const unsigned b = __ballot_sync(0xffffffffu, take);
-            if (take) {
-                const int e = e0 + used + __popc(b & ((1u << lane) - 1u));
-                if (e < sl.E) {
-                    for (int k = 0; k < 3; ++k) {
-                        sl.ev[k * sl.E + e] = v1[k];
-                        sl.ev[(3 + k) * sl.E + e] = v2[k];
+                    for (int q = 1; q < 32; q <<= 1) {
+                        const double y = __shfl_up_sync(0xffffffffu, inc, q);
+                        if (lane >= q) inc += y;
                     }
-                    sl.ei[e] = i;
-                    sl.ej[e] = j;
-                    sl.eU[e] = U;
-                    sl.eK[e] = K;
-                    sl.ecap[e] = 2 * pass + (!none && fabs(U) == capE);
-                } else if (!none) {
-                    latch(A.status, kErrTooLarge);
+                    const double off = grp == 0 ? 0.0 : (grp == 1 ? t0 : (grp == 2 ? t1 + t0 : (t2 + t1) + t0));
+                    double excl = __shfl_up_sync(0xffffffffu, inc, 1);
+                    excl = (off + (lane ? excl : 0.0)) + carry;
+                    take = ok && excl < Dabs;
+                    const double rem = Dabs - excl;
+                    U = sgn * (rem < capE ? rem : capE);
+                    const double t = __shfl_sync(0xffffffffu, inc, 31);
+                    if (grp == 0) t0 = t;
+                    else if (grp == 1) t1 = t;
+                    else if (grp == 2) t2 = t;
+                    else t3 = t;
+                    // the step kernel's shortcut: the first 32 pairs absorb all of it
+                    if (pass == 0 && chunk == 0 && grp == 0) stop = done = t >= Dabs;
                 }
-                if (!none) {
-                    energy_pair<double, false>(A.c, m1, m2, K, v1, v2, U);
-                    st3(wk.v, N, i, v1);
-                    st3(wk.v, N, j, v2);
+                const unsigned b = __ballot_sync(0xffffffffu, take);
+                if (take) {
+                    const int e = e0 + used + __popc(b & ((1u << lane) - 1u));
+                    if (e < sl.E) {
+                        for (int k = 0; k < 3; ++k) {
+                            sl.ev[k * sl.E + e] = v1[k];
+                            sl.ev[(3 + k) * sl.E + e] = v2[k];
+                        }
+                        sl.ei[e] = i;
+                        sl.ej[e] = j;
+                        sl.eU[e] = U;
+                        sl.eK[e] = K;
+                        sl.ecap[e] = 2 * pass + (!none && fabs(U) == capE);
+                    } else if (!none) {
+                        latch(A.status, kErrTooLarge);
+                    }
+                    if (!none) {
+                        energy_pair<double, false>(A.c, m1, m2, K, v1, v2, U);
+                        st3(wk.v, N, i, v1);
+                        st3(wk.v, N, j, v2);
+                    }
                 }
+                used += __popc(b);
+                __syncwarp();
             }
-            used += __popc(b);
-            __syncwarp();
+            carry += (t3 + t2) + (t1 + t0);
+            if (!none && carry >= Dabs) stop = done = true;
         }
         Dabs -= carry;
     }
@@ -546,14 +560,14 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
                         const Acc<double>* r = accp(sh.red);
                         sh.W1[0] = r[0].x;
                         sh.W1[1] = r[2].x;
-                        sh.Sw = ms[0] * r[1].x + (intra ? 0.0 : ms[1] * r[3].x);
+                        sh.Sw = mass_sum(ms[0], r[1].x, ms[1], r[3].x, intra);
                     }
                     __syncthreads();
                     block_sum<double, 6>(mom, accp(sh.red_raw), accp(sh.red));
                     if (threadIdx.x == 0) {
                         const Acc<double>* r = accp(sh.red);
                         for (int k = 0; k < 3; ++k) {
-                            sh.S[k] = ms[0] * r[k].x + (intra ? 0.0 : ms[1] * r[3 + k].x);
+                            sh.S[k] = mass_sum(ms[0], r[k].x, ms[1], r[3 + k].x, intra);
                             sh.B[k] = sh.S[k] / sh.Sw;
                         }
                     }
@@ -582,33 +596,13 @@ __global__ void __launch_bounds__(kThreads, kAdjCtasPerSm) k_adjoint(const __gri
                     block_sum<double, 4>(acc, accp(sh.red_raw), accp(sh.red));
                     if (threadIdx.x == 0) {
                         const Acc<double>* r = accp(sh.red);
-                        const double dE = ms[0] * r[0].x + (intra ? 0.0 : ms[1] * r[2].x);
+                        const double dE = mass_sum(ms[0], r[0].x, ms[1], r[2].x, intra);
                         sh.dE = dE;
-                        sh.Es[0] = ms[0] * r[1].x;
-                        sh.Es[1] = intra ? 0.0 : ms[1] * r[3].x;
-                        double D0 = dE, D1 = 0.0;
-                        int fail = 0;
-                        if (!intra) {
-                            const bool c0 = na >= 2, c1 = nb >= 2;
-                            if (c0 && c1) {
-                                const double wa = sh.W1[0] / (double)na * sh.Es[0];
-                                const double wb = sh.W1[1] / (double)nb * sh.Es[1];
-                                const double den = wa + wb;
-                                if (den > 0.0) {
-                                    D0 = wa / den * dE;
-                                    D1 = dE - D0;
-                                } else if (dE != 0.0) {
-                                    fail = 1;
-                                }
-                            } else if (c0) {
-                                D0 = dE;
-                            } else if (c1) {
-                                D0 = 0.0;
-                                D1 = dE;
-                            } else if (dE != 0.0) {
-                                fail = 1;
-                            }
-                        }
+                        sh.Es[0] = __dmul_rn(ms[0], r[1].x);
+                        sh.Es[1] = intra ? 0.0 : __dmul_rn(ms[1], r[3].x);
+                        double D0, D1;
+                        const int fail = split64(intra, na, nb, split_weight64(sh.W1[0], na, sh.Es[0]),
+                                                 split_weight64(sh.W1[1], nb, sh.Es[1]), dE, D0, D1);
                         sh.zeroed[0] = fabs(D0) <= 0x1p-47 * sh.Es[0];
                         sh.zeroed[1] = fabs(D1) <= 0x1p-47 * (intra ? 0.0 : sh.Es[1]);
                         sh.D[0] = sh.zeroed[0] ? 0.0 : D0;

@@ -195,9 +195,7 @@ __device__ __forceinline__ void shift_coef(const StepArgs& A, const InterConst& 
     const int d = threadIdx.x;
     if (d >= 3) return;
     const double ma = A.m[ic.a], mb = A.m[ic.b];
-    const double Sw = ma * W2[ic.a].x + (intra ? 0.0 : mb * W2[ic.b].x);
-    const double S = ma * r[d].x + (intra ? 0.0 : mb * r[3 + d].x);
-    sh.B[d] = S / Sw;
+    sh.B[d] = mass_sum(ma, r[d].x, mb, r[3 + d].x, intra) / mass_sum(ma, W2[ic.a].x, mb, W2[ic.b].x, intra);
     sh.Bf[d] = (float)sh.B[d];
 }
 __device__ __forceinline__ void shift_coef(const StepArgs& A, const InterConst& ic, bool intra,
@@ -225,32 +223,12 @@ __device__ __forceinline__ void partition_coef(const StepArgs& A, const InterCon
     if (threadIdx.x >= 32) return;
     const double ma = A.m[ic.a], mb = A.m[ic.b];
     const bool b = threadIdx.x & 1;  // species of this lane's terms
-    const double E = b ? (intra ? 0.0 : mb * r[3].x) : ma * r[1].x;
-    const double wE = W1[b ? ic.b : ic.a].x / (double)(b ? nb : na) * E;
+    const double E = b ? (intra ? 0.0 : __dmul_rn(mb, r[3].x)) : __dmul_rn(ma, r[1].x);
+    const double wE = split_weight64(W1[b ? ic.b : ic.a].x, b ? nb : na, E);
     const double Ea = __shfl_sync(0xffffffffu, E, 0), Eb = __shfl_sync(0xffffffffu, E, 1);
     const double wa = __shfl_sync(0xffffffffu, wE, 0), wb = __shfl_sync(0xffffffffu, wE, 1);
-    const double dE = ma * r[0].x + (intra ? 0.0 : mb * r[2].x);
-    double D0 = dE, D1 = 0.0;
-    int fail = 0;
-    if (!intra) {
-        const bool can0 = na >= 2, can1 = nb >= 2;
-        if (can0 && can1) {
-            const double den = wa + wb;
-            if (den > 0.0) {
-                D0 = wa / den * dE;
-                D1 = dE - D0;
-            } else if (dE != 0.0) {
-                fail = 1;
-            }
-        } else if (can0) {
-            D0 = dE;
-        } else if (can1) {
-            D0 = 0.0;
-            D1 = dE;
-        } else if (dE != 0.0) {
-            fail = 1;
-        }
-    }
+    double D0, D1;
+    const int fail = split64(intra, na, nb, wa, wb, mass_sum(ma, r[0].x, mb, r[2].x, intra), D0, D1);
     if (threadIdx.x == 0) {
         sh.D[0] = fabs(D0) <= 0x1p-47 * Ea ? 0.0 : D0;
         sh.D[1] = fabs(D1) <= 0x1p-47 * Eb ? 0.0 : D1;

@@ -269,6 +269,38 @@ __device__ __forceinline__ bool pair64(const F64Tab& T, int method, double cw, c
     return true;
 }
 
+// The coefficients of a correction in double, shared by the step kernel and the adjoint's forward. Every product and sum is rounded
+// as written (the compiler contracts a product into a sum differently in the two kernels, and the crossing pairs' last bits
+// then differ).
+// m_a x_a + m_b x_b (the first alone for one species).
+__device__ __forceinline__ double mass_sum(double ma, double xa, double mb, double xb, bool intra)
+{
+    return fma(ma, xa, intra ? 0.0 : __dmul_rn(mb, xb));
+}
+// A species' weight in the split of Delta E (Eq. DeltaEs): mean weight times post-shift energy.
+__device__ __forceinline__ double split_weight64(double W1, int n, double E) { return __dmul_rn(W1 / (double)n, E); }
+// Delta E split between species a and b of weights wa and wb: a species with fewer than two particles takes no share. Returns 1 if
+// no species can take it.
+__device__ __forceinline__ int split64(bool intra, int na, int nb, double wa, double wb, double dE, double& D0, double& D1)
+{
+    D0 = dE;
+    D1 = 0.0;
+    if (intra) return 0;
+    const bool can0 = na >= 2, can1 = nb >= 2;
+    if (can0 && can1) {
+        const double den = __dadd_rn(wa, wb);
+        if (!(den > 0.0)) return dE != 0.0;
+        D0 = __dmul_rn(wa / den, dE);
+        D1 = __dsub_rn(dE, D0);
+    } else if (can1) {
+        D0 = 0.0;
+        D1 = dE;
+    } else if (!can0) {
+        return dE != 0.0;
+    }
+    return 0;
+}
+
 // Momentum change of particle i of a relativistic pair in the lab frame (proper velocities vi, vj, masses ma, mb): the
 // pair's centre-of-momentum frame (see rel_cm), s with |p*|^2 v_rel* in place of mu^2 u^3, the rotation of p* and the
 // boost of its change back. kw = kappa w_max N_min (halved for a triplet). False if p* vanishes.
