@@ -123,11 +123,11 @@ __device__ __forceinline__ double n97_rA(const F64Tab& T, double s, double& E, d
     return n97_poly(T.n97, s);
 }
 
-// A(s) for sample_angle: 0 where 1 - e^-s rounds to 1 (isotropic), infinite at s = 0.
+// A(s) for sample_angle: 0 where 1 - e^-s rounds to 1 or s is not a number (isotropic), infinite for s <= 0 (no scattering).
 __device__ __forceinline__ double n97_A(double s, const F64Tab& T)
 {
     double E, F;
-    if (s > 36.7) return 0.0;
+    if (!(s <= 36.7)) return 0.0;
     return s > 0.0 ? 1.0 / n97_rA<false>(T, s, E, F) : CUDART_INF;
 }
 
@@ -152,7 +152,8 @@ __device__ __forceinline__ double n97_W(const F64Tab& T, double s)
 // Polar angle of a pair, sin(Theta) and 1 - cos(Theta), from the scattering length s and the draws (r.x, r.w).
 // DERIV and want: also s times their derivatives in s.
 //  TA77: tan(Theta/2) = d = sqrt(s/2) g, g normal by Box-Muller; sin = 2 d / (1 + d^2), 1 - cos = 2 d^2 / (1 + d^2).
-//  N97:  1 - cos = -ln((1 - U) + U e^-2A) / A, 1 + cos = ln1p((1 - U) expm1(2A)) / A; s above 36.7 is isotropic.
+//  N97:  1 - cos = -ln((1 - U) + U e^-2A) / A, 1 + cos = ln1p((1 - U) expm1(2A)) / A; s above 36.7 is isotropic. What 1 - e^-s
+//        says beyond (as on the mixed path): no scattering for a negative s, isotropic if s is not a number.
 // The products whose rounding the two callers have to share are kept from being contracted.
 template <bool DERIV>
 __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, const uint4& r, double& st, double& omc,
@@ -163,7 +164,8 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
     if (method == 0) {
         double cs, sn;
         turn64(T, r.w, cs, sn);
-        const double d = sqrt(fmin(-s * ln64(T, U, 0.0), 1e200)) * cs;
+        const double t = -s * ln64(T, U, 0.0);  // bounded so that d^2 is finite
+        const double d = sqrt(from64(__double2hiint(t), 0x6974E718) ? 1e200 : t) * cs;
         const double d2 = __dmul_rn(d, d), q = 1.0 / (1.0 + d2);
         st = 2.0 * d * q;
         omc = 2.0 * d2 * q;
@@ -177,9 +179,13 @@ __device__ __forceinline__ void angle64(const F64Tab& T, int method, double s, c
     const double V = 1.0 - U;  // exact
     double o, q;
     const int hs = __double2hiint(s);
-    if (from64(hs, 0x40425800)) {  // s >= 36.69: isotropic
+    const uint32_t as = (uint32_t)hs & 0x7FFFFFFFu;
+    if (as >= 0x40425800u && (hs >= 0 || as > 0x7FF00000u)) {  // s >= 36.69 or not a number: isotropic
         o = 2.0 * U;
         q = 2.0 * V;
+    } else if (hs < 0) {  // s < 0, from a negative Coulomb logarithm: no scattering
+        o = 0.0;
+        q = 2.0;
     } else {
         double E, F;  // e^-2A, 1 - e^-2A
         const double rA = n97_rA<true>(T, s, E, F);
