@@ -26,7 +26,7 @@ struct NvtxRange {
 
 struct mcc_ctx {
     int device;
-    int32_t* dbuf;  // [0] status word, [1] work-queue counter, then the tables
+    int32_t* dbuf;  // [0] status word, [1] and [2] work-queue counters, [4..7] debug record, then the tables
     int64_t launches;
     int num_sms;
     size_t smem_optin;
@@ -36,11 +36,12 @@ struct mcc_ctx {
     int32_t group_top; // upper bound of the largest class; 0 = what one CTA's shared memory holds
     size_t smem_reserved;  // shared memory the system reserves per CTA
     // Attributes of the kernels, looked up once (each look-up costs about a microsecond of every call), and the last
-    // occupancy of each: launch shape << 8 | CTAs per SM in one word, so threads may share a context.
+    // occupancy of each (an unfused call has two shapes): launch shape << 8 | CTAs per SM in one word, so threads may share a
+    // context.
     size_t cell_static[2][2][mcc::kModes];  // [float][relativistic][mode]
     size_t group_static[2][mcc::kOrderClasses];
     size_t adjoint_static;
-    std::atomic<uint64_t> cell_occ[2][2][mcc::kModes], group_occ[2][mcc::kOrderClasses];
+    std::atomic<uint64_t> cell_occ[2][2][2][mcc::kModes], group_occ[2][mcc::kOrderClasses];
 };
 
 namespace mcc {
@@ -227,43 +228,53 @@ int cached_occupancy(std::atomic<uint64_t>& slot, uint64_t shape, F look_up)
     return b;
 }
 
-// Launch one cell-kernel pass over every cell (queue reset, persistent grid of at most max_grid CTAs).
-int run_cells(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, int cap, cudaStream_t st,
-              int max_grid = 1 << 30)
+// Launch one cell-kernel pass over every cell, with a persistent grid of at most max_grid CTAs that take cells from a.queue (zero
+// before). pass: 0, or 1 for the second launch of an unfused call, which may overlap the first.
+int launch_cells(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, int cap, cudaStream_t st, int max_grid, int pass)
 {
     const size_t per = mode == mcc::kPair ? mcc::pair_tile_bytes_per_particle() : mcc::tile_bytes_per_particle(f32);
     const size_t smem = (size_t)cap * per;
-    const int bps = cached_occupancy(ctx->cell_occ[f32][rel][mode], smem,
+    const int bps = cached_occupancy(ctx->cell_occ[pass][f32][rel][mode], smem,
                                      [&] { return mcc::cell_kernel_blocks_per_sm(f32, rel, mode, smem); });
     if (bps < 1) return MCC_ERR_CUDA;
     int grid = ctx->num_sms * bps;
     if (grid > max_grid) grid = max_grid;
     if (a.n_cells < grid) grid = a.n_cells > 0 ? a.n_cells : 1;
     a.cap = cap;
-    cudaError_t e = cudaMemsetAsync(ctx->dbuf + 1, 0, sizeof(int32_t), st);
-    if (e != cudaSuccess) return MCC_ERR_CUDA;
-    e = mcc::launch_cell(f32, rel, mode, a, grid, smem, st);
+    const cudaError_t e = mcc::launch_cell(f32, rel, mode, a, grid, smem, pass > 0, st);
     ctx->launches += 1;
     return cuda_status(e);
 }
 
+// The same with its queue reset before.
+int run_cells(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, int cap, cudaStream_t st, int max_grid)
+{
+    if (cudaMemsetAsync(ctx->dbuf + 1, 0, sizeof(int32_t), st) != cudaSuccess) return MCC_ERR_CUDA;
+    return launch_cells(ctx, a, f32, rel, mode, cap, st, max_grid, 0);
+}
+
 // An unfused call (one mode of the cell kernel over every cell). The caller gives no bound on its cells, and a tile for the
 // largest cell leaves one CTA per SM; so the cells that fit the tile of four CTAs per SM go first, with that tile, and the
-// larger ones in a second launch with the largest. 1000 cells of 400 particles, three interactions: 1.72 -> 1.16 ms.
+// larger ones in a second launch with the largest. 1000 cells of 400 particles, three interactions: 1.72 -> 1.16 ms. With no
+// more cells than SMs one launch with the largest tile holds them all; with more, one reset serves both queues and the second
+// launch overlaps the first. mcc_scatter, two launches one after another / so, us per call: FP64, 20 cells of 400 38 / 31, 1000 of
+// 400 110 / 107; float, 20 of 400 36 / 29, 100 of 2800 59 / 53, 200 of 1500 63 / 58, 500 of 1500 111 / 106 (one launch with the
+// largest tile for all cells: 43, 53, 58, 105; 1000 of 400 73 against 33).
 int run_split(mcc_ctx* ctx, StepArgs& a, bool f32, bool rel, int mode, cudaStream_t st)
 {
     const int cap = (int)(mode == mcc::kPair ? max_pair_tile_particles(ctx) : max_tile_particles(ctx, f32));
     int small = auto_tile(ctx, f32);
     if (mode == mcc::kPair)
         small = (int)((size_t)small * mcc::tile_bytes_per_particle(f32) / mcc::pair_tile_bytes_per_particle());
-    if (small < cap) {
-        a.more = 1;
-        const int rc = run_cells(ctx, a, f32, rel, mode, small, st);
-        if (rc != MCC_OK) return rc;
-        a.more = 0;
-        a.above = small;
-    }
-    return run_cells(ctx, a, f32, rel, mode, cap, st);
+    if (small >= cap || a.n_cells <= ctx->num_sms) return run_cells(ctx, a, f32, rel, mode, cap, st, 1 << 30);
+    if (cudaMemsetAsync(ctx->dbuf + 1, 0, 2 * sizeof(int32_t), st) != cudaSuccess) return MCC_ERR_CUDA;
+    a.more = 1;
+    const int rc = launch_cells(ctx, a, f32, rel, mode, small, st, 1 << 30, 0);
+    if (rc != MCC_OK) return rc;
+    a.more = 0;
+    a.above = small;
+    a.queue = ctx->dbuf + 2;
+    return launch_cells(ctx, a, f32, rel, mode, cap, st, 1 << 30, 1);
 }
 
 // Whether the adjoint's working arrays for cells of max_cell particles fit one CTA's shared memory.
@@ -318,7 +329,7 @@ int mcc_create(mcc_ctx** out, int device)
         for (int rel = 0; rel < 2; ++rel)
             for (int mode = 0; mode < mcc::kModes; ++mode) {
                 c->cell_static[f32][rel][mode] = mcc::cell_kernel_static_smem(f32, rel, mode);
-                c->cell_occ[f32][rel][mode] = 0;
+                for (int pass = 0; pass < 2; ++pass) c->cell_occ[pass][f32][rel][mode] = 0;
                 const cudaError_t e =
                     mcc::set_cell_smem_limit(f32, rel, mode, c->smem_optin - c->cell_static[f32][rel][mode]);
                 if (e != cudaSuccess) attr = e;

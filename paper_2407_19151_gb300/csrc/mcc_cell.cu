@@ -986,6 +986,8 @@ __global__ void __launch_bounds__(kThreads, MIN_BLOCKS) cell_kernel(const __grid
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ Shared sh;
+    // an unfused call's second launch (the cells above the first one's tile) may start where the first has finished
+    if (MODE != kFused) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (threadIdx.x == 0) sh.step = A.step_dev ? (uint32_t)(*A.step_dev + A.step_add) : A.rng.step;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1003,6 +1005,7 @@ __global__ void __launch_bounds__(kThreads, MIN_BLOCKS) cell_kernel(const __grid
         process_cell<V, REL, MODE>(A, c, dyn, sh);
         __syncthreads();
     }
+    if (MODE != kFused) asm volatile("griddepcontrol.wait;" ::: "memory");  // done only when the launch before it is
 }
 
 // Advance a step counter kept in device memory (after the steps of one call, so that a captured graph of the call
@@ -1235,8 +1238,8 @@ const void* group_kernel(bool f32, bool rel, int cls)
     return rel ? group_kernel_f32rel(cls) : group_kernel_f32(cls);
 }
 
-cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem, bool after,
-                         cudaStream_t st)
+// One launch; after: it may start before the one before it on the stream has finished.
+static cudaError_t launch(const void* kernel, const StepArgs& a, int grid, int threads, size_t smem, bool after, cudaStream_t st)
 {
     void* args[] = {const_cast<StepArgs*>(&a)};
     cudaLaunchAttribute attr;
@@ -1244,20 +1247,25 @@ cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int gri
     attr.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(groups * group_threads(cls));
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = after ? 1 : 0;
-    return cudaLaunchKernelExC(&cfg, group_kernel(f32, rel, cls), args);
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
+cudaError_t launch_group(bool f32, bool rel, int cls, const StepArgs& a, int grid, int groups, size_t smem, bool after,
+                         cudaStream_t st)
+{
+    return launch(group_kernel(f32, rel, cls), a, grid, groups * group_threads(cls), smem, after, st);
 }
 
 size_t pair_tile_bytes_per_particle() { return kPairTileBytesPerParticle; }
 
-cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, cudaStream_t st)
+cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, bool after, cudaStream_t st)
 {
-    void* args[] = {const_cast<StepArgs*>(&a)};
-    return cudaLaunchKernel(select_kernel(f32, rel, mode), dim3(grid), dim3(kThreads), args, smem, st);
+    return launch(select_kernel(f32, rel, mode), a, grid, kThreads, smem, after, st);
 }
 
 }  // namespace mcc

@@ -124,7 +124,8 @@ __host__ __device__ inline size_t group_smem(size_t shared_bytes, int cap)
 }
 
 // Kernel launches (defined in mcc_cell.cu / mcc_bin.cu).
-cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, cudaStream_t st);
+// after: the launch before it on the stream is the same unfused call's, and this one may overlap it
+cudaError_t launch_cell(bool f32, bool rel, int mode, const StepArgs& a, int grid, size_t smem, bool after, cudaStream_t st);
 cudaError_t launch_step_advance(uint64_t* step, uint64_t by, cudaStream_t st);
 // Cells ordered by group size class (largest class first; class kGroupClasses = cells above every class), largest
 // first within a class; class_off receives each class's [begin, end) in `order`.
