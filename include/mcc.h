@@ -394,9 +394,14 @@ int mcc_set_tile_cap(mcc_ctx* ctx, int32_t cap);
  * sixteen warps share an SM's shared memory); largest sets caps[4] (0 = as large as one CTA's shared memory
  * allows). Every capacity is capped by what one CTA's shared memory holds (44 bytes per particle). Both 0 is the
  * default; a call with few cells then runs its cells on larger groups than these classes say, and one with many small
- * cells runs those on half warps (a part of a problem: mcc_step_fused_part). Used by the autotuner; the step's results do
+ * cells runs those on half warps (a part of a problem: mcc_step_fused_part). The step's results do
  * not depend on it beyond the order of float-float sums. */
 int mcc_set_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp, int32_t largest);
+
+/* The capacity that "automatic" means (0 = the one with which sixteen warps share an SM's shared memory): unlike an explicit
+ * capacity it leaves a call with few cells its larger groups and one with many small cells its half warps. For the autotuner.
+ * Ends an explicit capacity; mcc_set_group_capacity ends it. */
+int mcc_tune_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp);
 
 /* The five class capacities mcc_step_fused uses for this precision and mode (caps_out: host int32[5]). */
 int mcc_group_capacities(mcc_ctx* ctx, int32_t prec, int32_t relativistic, int32_t* caps_out);

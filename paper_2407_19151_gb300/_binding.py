@@ -149,6 +149,7 @@ def lib():
                                           C.c_size_t, C.c_int32, C.c_int32, vp]),
         "mcc_set_tile_cap": (C.c_int, [vp, C.c_int32]),
         "mcc_set_group_capacity": (C.c_int, [vp, C.c_int32, C.c_int32]),
+        "mcc_tune_group_capacity": (C.c_int, [vp, C.c_int32]),
         "mcc_group_capacities": (C.c_int, [vp, C.c_int32, C.c_int32, P(C.c_int32)]),
         "mcc_sync_status": (C.c_int, [vp, vp]),
         "mcc_launch_count": (C.c_int64, [vp]),
@@ -206,6 +207,10 @@ class Context:
     def set_group_capacity(self, particles_per_warp: int, largest: int = 0):
         _check(lib().mcc_set_group_capacity(self.handle, int(particles_per_warp), int(largest)),
                "mcc_set_group_capacity")
+
+    def tune_group_capacity(self, particles_per_warp: int):
+        """The capacity that "automatic" means (0: the built-in one); calls of few or of small cells keep their own rules."""
+        _check(lib().mcc_tune_group_capacity(self.handle, int(particles_per_warp)), "mcc_tune_group_capacity")
 
     def group_capacities(self, prec: int = F32_MIXED, relativistic: bool = False) -> list[int]:
         caps = (C.c_int32 * GROUP_CLASSES)()

@@ -2,9 +2,11 @@
 
 Two knobs, both in the context (the step's results do not depend on them, only its speed):
 
-* the group capacity (particles per warp): the mixed path runs each cell on one CTA of 32 << k threads, k the
+* the group capacity (particles per warp): the mixed path runs each cell on a group of 32 << k threads, k the
   smallest size class whose capacity (capacity << k particles) holds the cell, so the capacity sets the class
-  thresholds, hence the threads per cell and the shared memory per CTA (resident CTAs per SM);
+  thresholds, hence the threads per cell and the shared memory per group (resident groups per SM). It stands for the
+  automatic capacity: calls with few cells keep their larger groups and calls with many small cells their half warps,
+  also those of other shapes on the same context;
 * the tile of the one-CTA kernel (particles staged in shared memory per cell), which serves the FP64 path and the
   cells above the largest group class.
 
@@ -97,7 +99,7 @@ def autotune(vx, vy, vz, w, offsets, n_cells: int, n_species: int, species, lnL,
     path = cache_path()
     hit = _CACHE.get(key) or (_load(path).get(key) if persist else None)
     if hit:
-        ctx.set_group_capacity(int(hit["group_cap"]))
+        ctx.tune_group_capacity(int(hit["group_cap"]))
         ctx.set_tile_cap(int(hit["tile_cap"]))
         _CACHE[key] = hit
         return dict(hit, cached=True)
@@ -125,7 +127,7 @@ def autotune(vx, vy, vz, w, offsets, n_cells: int, n_species: int, species, lnL,
     prec = B.F32_MIXED if f32 else B.F64
 
     def apply_group(cap):
-        ctx.set_group_capacity(cap)
+        ctx.tune_group_capacity(cap)
         return tuple(ctx.group_capacities(prec, rel))
 
     def apply_tile(cap):

@@ -33,6 +33,7 @@ struct mcc_ctx {
     size_t smem_per_sm;
     int32_t tile_cap;  // particles staged on chip per cell by the one-CTA kernel; 0 = automatic
     int32_t group_cap; // particles per warp of the group kernels' size classes; 0 = automatic
+    int32_t group_tuned;  // the automatic capacity, tuned; 0 = from the shared memory
     int32_t group_top; // upper bound of the largest class; 0 = what one CTA's shared memory holds
     size_t smem_reserved;  // shared memory the system reserves per CTA
     // Attributes of the kernels, looked up once (each look-up costs about a microsecond of every call), and the last
@@ -314,6 +315,7 @@ int mcc_create(mcc_ctx** out, int device)
     c->tile_cap = 0;
     c->group_cap = 0;
     c->group_top = 0;
+    c->group_tuned = 0;
     int optin = 0, sms = 0, per_sm = 0, reserved = 0;
     cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device);
     c->smem_reserved = (size_t)reserved;
@@ -629,6 +631,8 @@ void group_caps(const mcc_ctx* ctx, bool f32, bool rel, int32_t caps[mcc::kGroup
     size_t per_warp;
     if (ctx->group_cap > 0) {
         per_warp = (size_t)ctx->group_cap;
+    } else if (ctx->group_tuned > 0) {
+        per_warp = (size_t)ctx->group_tuned;
     } else {
         const size_t share = (group_budget(ctx, f32, rel, 0) / mcc::group_cta_warps(rel)) & ~(size_t)15;
         const size_t fixed = mcc::group_shared_bytes(0);
@@ -685,6 +689,16 @@ int mcc_set_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp, int32_t lar
     if (!ctx || particles_per_warp < 0 || largest < 0) return MCC_ERR_INVALID_ARG;
     ctx->group_cap = particles_per_warp;
     ctx->group_top = largest;
+    ctx->group_tuned = 0;
+    return MCC_OK;
+}
+
+int mcc_tune_group_capacity(mcc_ctx* ctx, int32_t particles_per_warp)
+{
+    if (!ctx || particles_per_warp < 0) return MCC_ERR_INVALID_ARG;
+    ctx->group_cap = 0;
+    ctx->group_top = 0;
+    ctx->group_tuned = particles_per_warp;
     return MCC_OK;
 }
 
