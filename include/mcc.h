@@ -129,7 +129,8 @@ int mcc_adjoint_workspace_size(mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, 
                                size_t* bytes);
 
 /* Bytes of one recorded tape of one interaction (tape = MCC_ADJOINT_RECORD / MCC_ADJOINT_REPLAY: one slab per cell,
- * about 250 bytes per particle of max_cell plus 80 bytes per possible energy pair). */
+ * about 140 bytes per particle of max_cell, 200 where a cell exceeds one CTA's shared memory, plus 76 bytes per possible
+ * energy pair). */
 int mcc_adjoint_tape_size(mcc_ctx* ctx, int32_t n_cells, int32_t max_cell, int32_t max_corr_passes, size_t* bytes);
 
 #define MCC_ADJOINT_RECOMPUTE 0

@@ -492,8 +492,8 @@ def default_interactions(n_species: int):
 
 def mcc_step_fused(vx, vy, vz, w, offsets, n_cells, n_species, species, lnL, params: Params, n_steps: int = 1,
                    max_cell: int | None = None, interactions=None, corr_pairs=None, fail_count=None, stream=None):
-    """n_steps whole collision steps in place (one persistent kernel launch per step). Returns the per-cell
-    accumulated (corr_pairs, fail_count) tensors."""
+    """n_steps whole collision steps in place (mixed path: one persistent kernel per cell size class and step; FP64: one per
+    step). Returns the per-cell accumulated (corr_pairs, fail_count) tensors."""
     ctx = context(vx.device)
     P = _particles(vx, vy, vz, w)
     inter = default_interactions(n_species) if interactions is None else [tuple(x) for x in interactions]

@@ -11,7 +11,7 @@ walks the segment backwards. Memory: checkpoint_every x interactions states of t
 
 Recorded tapes (float64, ``tape=True``, or ``tape=None`` when the tapes fit in half the free device memory): the
 forward runs every interaction through ``mcc_adjoint`` in recording mode, which keeps each cell's tape in device
-memory (about 250 bytes per particle per interaction plus the energy-pair reserve), and the backward is the reverse
+memory (about 140 bytes per particle per interaction plus the energy-pair reserve), and the backward is the reverse
 sweep alone, interaction by interaction from the last, with nothing recomputed. This trades memory for the
 backward's two recomputations of the forward (the replay and the recomputation inside each reverse call).
 

@@ -51,10 +51,9 @@ __device__ __forceinline__ long long bin_key(const int32_t* __restrict__ cell, c
 // time with the number of different keys, about 64 cycles of an SM for 32 of them, the atomics it saves take more: it is
 // taken when a warp's keys repeat, that is when at most kRunHeads runs begin (nearly binned input, such as a re-bin after
 // a push), when kSameKey lanes hold lane 0's key (species in turns within binned cells) or when there are few segments,
-// whose counters the atomics queue for. Shuffled input (32 runs of one lane) takes the runs. 3.3e7 particles, 2e5 segments,
-// count and scatter with cursors
-// in us: 17% moved by a push, 100 and 176 (runs alone 162 and 294); shuffled, count and scatter 330 and 350 (460 and 520 with
-// a match in every warp); 1e7 particles in 192 segments, 2360 and 1170 (runs alone 2650 and 1300).
+// whose counters the atomics queue for. Shuffled input (32 runs of one lane) takes the runs. Count, and scatter with cursors, us:
+// 3.3e7 particles in 2e5 segments, 17% moved by a push, 100 and 176 (runs alone 162 and 294), shuffled 330 and 350 (a match in
+// every warp 460 and 520); 1e7 particles in 192 segments 2360 and 1170 (runs alone 2650 and 1300).
 constexpr int kRunHeads = 28, kSameKey = 4;
 constexpr int64_t kFewSegments = 512;
 

@@ -14,8 +14,8 @@
 // The unfused C-ABI calls run single phases of the same code: PAIR writes the pair list, SCATTER the pair loop
 // (reading the list, writing the pre-scatter copy), CORRECT the moment correction (reading that copy).
 //
-// FP64 path: everything in double. Mixed path: float velocities and kinematics, float-float accumulation of the
-// per-cell sums, FP64 only for the per-cell coefficients (B, Delta E, its split) computed by one thread.
+// FP64 path: everything in double, the coefficients of a correction (B, Delta E, its split) spread over the first warp's lanes.
+// Mixed path: float velocities and kinematics, float-float sums, and the coefficients in float-float by one thread.
 #include "mcc_pair64.cuh"
 #include "mcc_perm.cuh"
 

@@ -84,16 +84,6 @@ __device__ __forceinline__ V u23(uint32_t r)
     return ((V)(r >> 9) + (V)0.5) * (V)(1.0 / 8388608.0);
 }
 
-// Permutation key of local index i: 44 random bits above the 20-bit index (distinct keys).
-__device__ __forceinline__ uint64_t perm_key(const RngKey& k, uint32_t cell, uint32_t inter, uint32_t side,
-                                             uint32_t i)
-{
-    const uint4 b = draw(k, i >> 1, cell, inter, side ? kTagPermB : kTagPermA);
-    const uint32_t hi = (i & 1u) ? b.z : b.x;
-    const uint32_t lo = (i & 1u) ? b.w : b.y;
-    return ((((uint64_t)hi << 32) | (uint64_t)lo) & ~kPermMask) | (uint64_t)i;
-}
-
 // Weight-descending order key: inverted IEEE bits of the (positive) weight truncated to 44 bits, then the rank in
 // the random permutation, so that weights equal to 2^-32 relative keep the random order.
 __device__ __forceinline__ uint64_t weight_key(double w, uint32_t rank)
@@ -157,13 +147,6 @@ __device__ __forceinline__ ff ff_div(ff a, ff b)
     const ff r = ff_sub(a, ff_mul(b, {q1, 0.f}));
     const float q2 = __fdiv_rn(r.hi, b.hi);
     return ff_fast_two_sum(q1, q2);
-}
-
-__device__ __forceinline__ ff ff_from_double(double x)
-{
-    const float hi = __double2float_rn(x);
-    const float lo = __double2float_rn(x - (double)hi);
-    return {hi, lo};
 }
 
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }

@@ -66,7 +66,6 @@ struct StepArgs {
     void* backup;
     int32_t* corr_pairs;
     int32_t* fail_count;
-    int32_t accumulate;
     // control
     int32_t* status;
     int32_t* queue;

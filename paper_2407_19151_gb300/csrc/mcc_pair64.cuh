@@ -10,7 +10,9 @@
 //   e^-2A       the same intervals: e^-2A below s = 2, 1 - e^-2A above (the smaller one, or nearly). Its polynomials lose
 //               relative precision towards s = 2^-5, where e^-2A is below 1e-16 of what it is added to
 //   ln u        u = 2^k m, ln m = -ln r_i + ln(m r_i) with tabulated r_i ~ 1/m (Tang, "Table-driven implementation of
-//               the logarithm function in IEEE floating-point arithmetic", 1990)
+//               the logarithm function in IEEE floating-point arithmetic", 1990); mantissas in [0.6875, 1.375), 128
+//               intervals and r_i = 1 next to 1 are the arrangement of the public log of Arm's Optimized Routines (the
+//               reciprocals, the logarithms and the Taylor terms are computed here);
 //               one logarithm per pair: of whichever of 1 - cos and 1 + cos is smaller, the other being 2 minus it
 //   azimuth     2 pi (k + 1/2) 2^-23 = nearest 1/256 turn, tabulated, + a remainder below pi/256 (addition theorem)
 // uniforms are assembled from their bits instead of converted, and comparisons are made on the bits (an FP64 comparison
