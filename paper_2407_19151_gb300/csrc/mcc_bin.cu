@@ -7,10 +7,10 @@
 // atomic also gives each particle its place in the segment, so the scatter needs none.
 // Segments of up to 512 entries are sorted by one warp in its slice of shared memory (warp barriers only), larger ones
 // by a whole CTA. What bounds it: atomics and random sectors on shuffled input (3.3e7 particles, 2e5 segments: 1.64 ms with a
-// match in every warp, cursors and bitonic sorts, 1.09 so); the segment sorts after a push (17% moved: 0.92 -> 0.83 ms, 0.49 of
-// it the sorts; in weight order 1.63 -> 0.94). 1.34e8 particles: shuffled 7.6 -> 5.9 ms, after a push 3.49 -> 3.13, in weight
-// order 6.3 -> 3.5. Two thirds moved, which no push does, is the one input found where the network in every segment was
-// faster (0.97 against 1.10 ms). A two-pass radix sort of (key, index) pairs took 1.43 ms shuffled and lost on nearly binned
+// match in every warp, cursors and bitonic sorts, 1.09 so); the segment sorts after a push (17% moved: 0.92 -> 0.81 ms, 0.47 of
+// it the sorts; in weight order 1.63 -> 0.94). 1.34e8 particles: shuffled 7.6 -> 5.9 ms, after a push 3.49 -> 3.05, in weight
+// order 6.3 -> 3.5. 60% moved, which no push does, is the one input found where the network in every segment was
+// faster (0.97 against 1.07 ms). A two-pass radix sort of (key, index) pairs took 1.43 ms shuffled and lost on nearly binned
 // input, where a warp here has few atomics.
 #include <mutex>
 
@@ -78,8 +78,10 @@ __device__ __forceinline__ void key_group(long long key, bool few, int& lead, in
 }
 
 // All lanes of a warp run the same trips (the loop index is the warp's base), so the shuffles see the full warp. One element
-// per thread and iteration: four, a grid's stride apart, with their atomics in flight together took 202 / 208 us where one
-// takes 144 / 156 after a push (the counters of four places at once), and no less time on shuffled input.
+// per thread and iteration: four, a grid's stride apart, with their atomics in flight together took 202 / 208 us (count / scatter)
+// where one takes 144 / 156 after a push (the counters of four places at once); on shuffled input they gain little (1.34e8
+// particles 5.79 against 5.92 ms, 3.3e7 1.09 against 1.10). Both kernels have to take the rows in the same order, or a segment's
+// places are written at different times (four in one of them only: 6.8 and 7.4 ms).
 // PLACE: place[i] = the particle's place in its segment, in the order the atomics were served.
 template <bool PLACE>
 __global__ void __launch_bounds__(kBinThreads) k_hist(const int32_t* __restrict__ cell, const int32_t* __restrict__ species,
@@ -256,14 +258,15 @@ __device__ __forceinline__ void warp_sort_smem(int n, Cmpx cmpx)
 // more buckets, then an insertion sort within a bucket. Indices of shuffled particles spread evenly, and so do weights over
 // decades, as the IEEE bits of a weight are nearly linear in its logarithm. After a particle push most indices of a segment
 // are neighbours, those that stayed, and the rest come from anywhere: one bucket of the linear map would hold nearly all.
-// The map of such a segment (more than kBucketMost entries in the bucket of a middling one) has three pieces: half the buckets
+// The map of such a segment (of 32 entries looked at, kCrowd in the bucket of a middling one) has three pieces: half the buckets
 // for the 2.5 n indices around that entry, a quarter each for those below and above, by the logarithm of their distance (what
 // moved in comes from the next cells, rows and planes of the grid, orders of magnitude apart). A segment of which a third
 // comes from elsewhere, or one that still fills a bucket beyond kBucketMost, takes the bitonic network; up to 32 indices
 // take it in registers. 3.3e7 particles, 17% moved: 616 us by the network in every segment, 734 by a futile count and then
-// the network, 490 by three pieces.
+// the network, 470 by three pieces.
 constexpr int kOrderWarps = 4;   // warps per CTA
 constexpr int kBucketMost = 12;  // longest bucket for the insertion sort
+constexpr int kCrowd = 8;        // of 32 entries looked at, in one bucket: a crowd
 
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(32 * kOrderWarps) k_segsort_warp(const int64_t* __restrict__ offsets, int64_t nk,
@@ -345,16 +348,12 @@ __global__ void __launch_bounds__(32 * kOrderWarps) k_segsort_warp(const int64_t
         if (!WEIGHTED) {
             const uint32_t x = top(n / 4), y = top(n / 2), z = top(n - 1 - n / 4);
             const uint32_t mid = max(min(x, y), min(max(x, y), z));
-            const uint32_t at = place(mid - lo, mult);
-            int share = 0;
-            for (int i = lane; i < n; i += 32) share += place(top(i) - lo, mult) == at;
-            if (__reduce_add_sync(0xffffffffu, share) > kBucketMost) {
+            const uint32_t at = place(mid - lo, mult), mine = top(lane * n >> 5);  // every lane an entry in turn
+            if (__popc(__ballot_sync(0xffffffffu, place(mine - lo, mult) == at)) >= kCrowd) {
                 const uint32_t half = (uint32_t)(n + n / 4);
                 w0 = mid - lo > half ? mid - half : lo;  // the window [w0, w1)
                 w1 = hi - mid >= half ? mid + half : hi + 1u;
-                int inside = 0;
-                for (int i = lane; i < n; i += 32) inside += top(i) >= w0 && top(i) < w1;
-                if (__reduce_add_sync(0xffffffffu, inside) < n - n / 3) {  // many from elsewhere, in clumps
+                if (__popc(__ballot_sync(0xffffffffu, mine >= w0 && mine < w1)) < 21) {  // many from elsewhere, in clumps
                     network();
                     continue;
                 }

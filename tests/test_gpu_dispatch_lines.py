@@ -49,13 +49,13 @@ def _step(mcc, wl, prec):
     return launches, err, corr.cpu().numpy(), fail.cpu().numpy(), ocorr, ofail
 
 
-# (cells per 152 SMs, largest cell, class from which the call runs)
-@pytest.mark.parametrize("n,largest,cls", [
-    (3, 700, 3), (304, 600, 3), (305, 600, 2), (608, 300, 2), (609, 300, 1), (1216, 150, 1), (1217, 150, 0),
-    (100, 511, 2), (100, 512, 3), (100, 255, 1), (100, 256, 2), (100, 127, 0), (100, 128, 1)])
-def test_few_cells(n, largest, cls):
+# (cells: so many per SM and so many more, largest cell, class from which the call runs)
+@pytest.mark.parametrize("per_sm,more,largest,cls", [
+    (0, 3, 700, 3), (2, 0, 600, 3), (2, 1, 600, 2), (4, 0, 300, 2), (4, 1, 300, 1), (8, 0, 150, 1), (8, 1, 150, 0),
+    (0, 100, 511, 2), (0, 100, 512, 3), (0, 100, 255, 1), (0, 100, 256, 2), (0, 100, 127, 0), (0, 100, 128, 1)])
+def test_few_cells(per_sm, more, largest, cls):
     import paper_2407_19151_gb300 as mcc
-    assert torch.cuda.get_device_properties(0).multi_processor_count == 152
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + more
     wl = _cells(_totals(n, largest) if n > 5 else [largest, 0, 1], "f32")
     caps = [-1] * cls + mcc.context(0).group_capacities()[cls:]
     launches, err, _, fail, _, ofail = _step(mcc, wl, "f32")
